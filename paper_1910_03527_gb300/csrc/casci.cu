@@ -44,6 +44,22 @@ __global__ void k_core_fock(int norb, const double *h1, const double *eri, const
     F[e] = v;
 }
 
+// The frozen core's share of dE/d(pq|rs) from the sums of rdm_one_body: for an occupied c and
+// active p, q, the weighted 1-RDM of the tuples without c.  (p or q = c: no such tuple.)
+__global__ void k_core_gradient(int norb, const uint8_t *occ, const double *core, double *grad_eri)
+{
+    const int e = blockIdx.x * blockDim.x + threadIdx.x, pq = e % (norb * norb), c = e / (norb * norb);
+    if (c >= norb || !occ[c]) return;
+    const int p = pq / norb, q = pq - p * norb;
+    if (p == c || q == c) return;
+    const double g = core[pq] + core[(size_t)(1 + c) * norb * norb + pq];
+    if (g == 0.0) return;
+    atomicAdd(&grad_eri[eri_index(norb, c, c, p, q)], g);
+    atomicAdd(&grad_eri[eri_index(norb, p, q, c, c)], g);
+    atomicAdd(&grad_eri[eri_index(norb, c, q, p, c)], -0.5 * g);
+    atomicAdd(&grad_eri[eri_index(norb, p, c, c, q)], -0.5 * g);
+}
+
 struct ClassifyArgs {
     int bucket_of_k[MBE_MAX_CAS + 1];
     int nbuckets;
@@ -178,18 +194,26 @@ static int run_casci(mbe_ctx *ctx, int norb, const double *h1, const double *eri
         a.cls[k].r = st->r;
         int64_t N = st->ns * st->ns;
         int b;
-        if (n <= WARP_MAX_N && N <= tu.warp_max_ndet && rdm != 2) {
+        // the sector solvers: energies in both precisions, density matrices in float64
+        const bool sector = sector_class(n, k) && o.s2_penalty == 0.0 && (rdm == 0 || o.precision == MBE_PREC_FP64);
+        if (n <= WARP_MAX_N && N <= tu.warp_max_ndet && (rdm != 2 || sector)) {
             int di = 0;
             while (DPL_SET[di] * 32 < N) ++di;
-            if (warp_bucket_of_dpl[di] < 0) {
-                warp_bucket_of_dpl[di] = (int)buckets.size();
-                buckets.push_back(Bucket{true, DPL_SET[di], 0, 0, 0});
+            // a bucket per class for the sector solvers, else one per determinants per lane
+            if (sector) {
+                buckets.push_back(Bucket{true, DPL_SET[di], 0, 0, 0, k});
+                b = (int)buckets.size() - 1;
+            } else {
+                if (warp_bucket_of_dpl[di] < 0) {
+                    warp_bucket_of_dpl[di] = (int)buckets.size();
+                    buckets.push_back(Bucket{true, DPL_SET[di], 0, 0, 0, -1});
+                }
+                b = warp_bucket_of_dpl[di];
             }
-            b = warp_bucket_of_dpl[di];
         } else {
             if (block_bucket < 0) {
                 block_bucket = (int)buckets.size();
-                buckets.push_back(Bucket{false, 0, 0, 0, 0});
+                buckets.push_back(Bucket{false, 0, 0, 0, 0, -1});
             }
             b = block_bucket;
             max_block_ns = std::max(max_block_ns, (int)st->ns);
@@ -221,6 +245,8 @@ static int run_casci(mbe_ctx *ctx, int norb, const double *h1, const double *eri
                    5 * align256((MAX_BUCKETS + 1) * 8) + (size_t)block_grid_n * slot_bytes +
                    (own_out ? align256((size_t)n_tuples * 8) + align256((size_t)n_tuples * 4) : 0) + 1024;
     if (split) bytes += align256((size_t)n_tuples * 8);
+    const size_t core_bytes = rdm == 2 ? (size_t)(1 + norb) * norb * norb * 8 : 0;
+    bytes += align256(core_bytes);
     void *ws = nullptr;
     int rc = workspace(ctx, bytes, &ws);
     if (rc) return rc;
@@ -246,6 +272,10 @@ static int run_casci(mbe_ctx *ctx, int norb, const double *h1, const double *eri
     a.weights = weights;
     a.grad_h1 = grad_h1;
     a.grad_eri = (rdm == 2) ? grad_eri : nullptr;
+    if (rdm == 2) {
+        a.core = bump.take<double>(core_bytes / 8);
+        MBE_CU(cudaMemsetAsync(a.core, 0, core_bytes, ctx->stream));
+    }
 
     a.F = F;
     a.perm = perm;
@@ -278,6 +308,11 @@ static int run_casci(mbe_ctx *ctx, int norb, const double *h1, const double *eri
             continue;
         }
         if ((rc = launch_warp_bucket(ctx, a, b, bk))) return rc;
+    }
+    if (rdm == 2) {
+        k_core_gradient<<<(norb * norb * norb + 255) / 256, 256, 0, ctx->stream>>>(norb, occ, a.core, grad_eri);
+        MBE_CU(cudaGetLastError());
+        ++ctx->launches;
     }
     return MBE_OK;
 }

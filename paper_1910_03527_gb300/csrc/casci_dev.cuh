@@ -89,6 +89,7 @@ struct BatchArgs {
     const double *weights;
     double *grad_h1;
     double *grad_eri;
+    double *core;  // rdm = 2: [1 + norb][norb^2], see rdm_one_body
 };
 
 // ------------------------------------------------------------------ group primitives
@@ -512,11 +513,11 @@ __device__ inline void eig3(const T (&G)[3][3], bool have_p, T (&y)[3])
             rotate3(A, Vv, 1, 2);
         }
     }
-    int m = 0;
-    if (A[1][1] < A[m][m]) m = 1;
-    if (A[2][2] < A[m][m]) m = 2;
+    // (selected by value: an indexed column would put the matrix in local memory)
+    const bool m1 = A[1][1] < A[0][0];
+    const bool m2 = A[2][2] < (m1 ? A[1][1] : A[0][0]);
 #pragma unroll
-    for (int i = 0; i < 3; ++i) y[i] = (T)Vv[i][m];
+    for (int i = 0; i < 3; ++i) y[i] = (T)(m2 ? Vv[i][2] : m1 ? Vv[i][1] : Vv[i][0]);
     if (!have_p) y[1] = (T)0;
     if constexpr (sizeof(T) == 8) {
         // float64 phase: one inverse-iteration step z = adj(G - theta I) y with
@@ -671,6 +672,22 @@ __device__ void rdm_accumulate(const Problem &pb, const double *c, double *g1, d
     }
 }
 
+// One element gc = w (gamma_pq - Phi's) of a tuple's weighted 1-RDM: into dE/dh, and into the
+// sums from which k_core_gradient forms the terms of the frozen core's two-electron
+// integrals.  Those need, for every occupied c outside A, gc at four places of dE/d(pq|rs);
+// here every tuple adds gc once to a.core[0][pq] and subtracts it from a.core[1 + c][pq] for
+// the few occupied c inside A, so the atomics per tuple no longer grow with the core (46
+// orbitals, order 4: 1,344 to 48 of them besides the n^4 of the active 2-RDM).
+__device__ inline void rdm_one_body(const BatchArgs &a, const int *A, int n, int p, int q, double gc)
+{
+    const size_t norb = a.norb, pq = A[p] * norb + A[q];
+    atomicAdd(&a.grad_h1[pq], gc);
+    if (!a.core || gc == 0.0) return;
+    atomicAdd(&a.core[pq], gc);
+    for (int i = 0; i < n; ++i)
+        if (a.occ[A[i]]) atomicAdd(&a.core[(1 + A[i]) * norb * norb + pq], -gc);
+}
+
 // Adds w * (dE_CAS(A)/dtheta - dE_Phi/dtheta) to the gradients from the active
 // density matrices accumulated by rdm_accumulate (Gamma = <E_pq E_rs> - d_qr gamma_ps).
 template <class G>
@@ -681,20 +698,7 @@ __device__ void rdm_flush(const BatchArgs &a, const Problem &pb, const double *g
     const int *A = pb.A;
     for (int e = tid; e < n * n; e += nt) {
         const int p = e / n, q = e - p * n;
-        const double dg = g1[e] - ((p == q && a.occ[A[p]]) ? 2.0 : 0.0);
-        atomicAdd(&a.grad_h1[A[p] * norb + A[q]], w * dg);
-        if (!g2 || dg == 0.0) continue;
-        const double gc = w * dg;
-        for (int c = 0; c < norb; ++c) {
-            if (!a.occ[c]) continue;
-            bool in_a = false;
-            for (int i = 0; i < n; ++i) in_a |= (A[i] == c);
-            if (in_a) continue;
-            atomicAdd(&a.grad_eri[eri_index(norb, c, c, A[p], A[q])], gc);
-            atomicAdd(&a.grad_eri[eri_index(norb, A[p], A[q], c, c)], gc);
-            atomicAdd(&a.grad_eri[eri_index(norb, c, A[q], A[p], c)], -0.5 * gc);
-            atomicAdd(&a.grad_eri[eri_index(norb, A[p], c, c, A[q])], -0.5 * gc);
-        }
+        rdm_one_body(a, A, n, p, q, w * (g1[e] - ((p == q && a.occ[A[p]]) ? 2.0 : 0.0)));
     }
     if (!g2) return;
     for (int e = tid; e < n * n * n * n; e += nt) {
@@ -2353,10 +2357,27 @@ struct Bucket {
     bool warp;
     int dpl;
     int max_ns, max_r, max_n;
+    int k;  // class of a sector-solver bucket, else -1
 };
+
+// String classes of the sector solvers (casci_sector.cuh): 2-6 orbitals, neither empty
+// nor full.  The S^2 penalty keeps the list-driven warp solver.
+constexpr int SECTOR_MAX_N = 6;
+inline bool sector_class(int n, int k) { return n >= 2 && n <= SECTOR_MAX_N && k >= 1 && k < n; }
+
+// Grid of a sector-solver launch: a persistent grid, or fewer blocks when the whole batch
+// has fewer tuples than warps in it.
+inline int sector_grid(const mbe_ctx *ctx, const BatchArgs &a, int per_sm)
+{
+    const int64_t need = (a.n_tuples + a.warps - 1) / a.warps;
+    return (int)std::min<int64_t>(need, (int64_t)ctx->sm_count * per_sm);
+}
 
 // Launchers of the solver kernels, one translation unit each (compiled in parallel).
 int launch_warp_bucket(mbe_ctx *ctx, const BatchArgs &a, int b, const Bucket &bk);       // casci_warp.cu
+int launch_sector_mixed(mbe_ctx *ctx, const BatchArgs &a, int b, int k);                 // casci_sector_mixed.cu
+int launch_sector64(mbe_ctx *ctx, const BatchArgs &a, int b, int k);                     // casci_sector64.cu
+int launch_sector64_redo(mbe_ctx *ctx, const BatchArgs &a, int b, int k);                // casci_sector64_redo.cu
 int launch_warp_mixed_dpl(mbe_ctx *ctx, const BatchArgs &a, int b, const MixLayout &L, int dpl);  // casci_mixed.cu
 int block_grid(mbe_ctx *ctx, int n, bool two_body, int *grid, size_t *smem);             // casci_block.cu
 int launch_block(mbe_ctx *ctx, const BatchArgs &a, int b, int grid, size_t smem);        // casci_block.cu

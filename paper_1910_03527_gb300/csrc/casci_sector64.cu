@@ -1,0 +1,44 @@
+// a5-a6 in float64 for tuples of 2-6 orbitals: the launches of the sector solver.
+#include "casci_sector64.cuh"
+
+namespace mbe {
+
+template <int N, int K>
+static int launch_class(mbe_ctx *ctx, const BatchArgs &a, int b)
+{
+    using C = Cls<N, K>;
+    const size_t smem = al16((int)sizeof(SectorTables<C>)) + sizeof(Sector64<C>) * a.warps;
+    MBE_CU(cudaFuncSetAttribute(k_sector64<C, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    int per_sm = 0;
+    MBE_CU(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_sector64<C, false>, a.warps * 32, smem));
+    if (per_sm < 1) per_sm = 1;
+    k_sector64<C, false><<<sector_grid(ctx, a, per_sm), a.warps * 32, smem, ctx->stream>>>(a, b);
+    MBE_CU(cudaGetLastError());
+    ++ctx->launches;
+    return MBE_OK;
+}
+
+int launch_sector64(mbe_ctx *ctx, const BatchArgs &a, int b, int k)
+{
+    switch (a.n * 8 + k) {
+    case 2 * 8 + 1: return launch_class<2, 1>(ctx, a, b);
+    case 3 * 8 + 1: return launch_class<3, 1>(ctx, a, b);
+    case 3 * 8 + 2: return launch_class<3, 2>(ctx, a, b);
+    case 4 * 8 + 1: return launch_class<4, 1>(ctx, a, b);
+    case 4 * 8 + 2: return launch_class<4, 2>(ctx, a, b);
+    case 4 * 8 + 3: return launch_class<4, 3>(ctx, a, b);
+    case 5 * 8 + 1: return launch_class<5, 1>(ctx, a, b);
+    case 5 * 8 + 2: return launch_class<5, 2>(ctx, a, b);
+    case 5 * 8 + 3: return launch_class<5, 3>(ctx, a, b);
+    case 5 * 8 + 4: return launch_class<5, 4>(ctx, a, b);
+    case 6 * 8 + 1: return launch_class<6, 1>(ctx, a, b);
+    case 6 * 8 + 2: return launch_class<6, 2>(ctx, a, b);
+    case 6 * 8 + 3: return launch_class<6, 3>(ctx, a, b);
+    case 6 * 8 + 4: return launch_class<6, 4>(ctx, a, b);
+    case 6 * 8 + 5: return launch_class<6, 5>(ctx, a, b);
+    }
+    set_error("casci_batch: no sector solver for the class (%d, %d)", a.n, k);
+    return MBE_EUNSUPPORTED;
+}
+
+}  // namespace mbe

@@ -38,8 +38,23 @@ static int launch_warp(mbe_ctx *ctx, const BatchArgs &a, int b, const Bucket &bk
     return tl.done();
 }
 
+// The same for a sector-solver bucket (one string class).
+static int launch_sector(mbe_ctx *ctx, const BatchArgs &a, int b, const Bucket &bk)
+{
+    TimedLaunch tl(ctx, a.order, 0, bk.dpl);
+    int rc;
+    if (a.pstate != nullptr) {
+        if ((rc = launch_sector_mixed(ctx, a, b, bk.k))) return rc;
+        if ((rc = launch_sector64_redo(ctx, a, b, bk.k))) return rc;
+    } else {
+        if ((rc = launch_sector64(ctx, a, b, bk.k))) return rc;
+    }
+    return tl.done();
+}
+
 int launch_warp_bucket(mbe_ctx *ctx, const BatchArgs &a, int b, const Bucket &bk)
 {
+    if (bk.k >= 0) return launch_sector(ctx, a, b, bk);
     switch (bk.dpl) {
     case 1: return launch_warp<1>(ctx, a, b, bk);
     case 2: return launch_warp<2>(ctx, a, b, bk);
