@@ -183,7 +183,7 @@ static int run_casci(mbe_ctx *ctx, int norb, const double *h1, const double *eri
     std::vector<Bucket> buckets;
     int warp_bucket_of_dpl[5] = {-1, -1, -1, -1, -1};
     int block_bucket = -1;
-    int max_block_ns = 0;
+    bool in_block[MBE_MAX_CAS + 1] = {};
     for (int k = 0; k <= n; ++k) {
         const StringTable *st = nullptr;
         int rc = get_table(ctx, n, k, &st);
@@ -216,7 +216,7 @@ static int run_casci(mbe_ctx *ctx, int norb, const double *h1, const double *eri
                 buckets.push_back(Bucket{false, 0, 0, 0, 0, -1});
             }
             b = block_bucket;
-            max_block_ns = std::max(max_block_ns, (int)st->ns);
+            in_block[k] = true;
         }
         Bucket &bk = buckets[b];
         bk.max_ns = std::max(bk.max_ns, (int)st->ns);
@@ -231,9 +231,8 @@ static int run_casci(mbe_ctx *ctx, int norb, const double *h1, const double *eri
     size_t block_smem_bytes = 0;
     size_t slot_bytes = 0;
     if (block_bucket >= 0) {
-        int rc = block_grid(ctx, n, rdm == 2, &block_grid_n, &block_smem_bytes);
+        int rc = block_grid(ctx, a, in_block, rdm, &block_grid_n, &block_smem_bytes, &slot_bytes);
         if (rc) return rc;
-        slot_bytes = slot_layout(max_block_ns, max_block_ns * max_block_ns).bytes;
     }
 
     const bool own_out = (eps_out == nullptr || status_out == nullptr);

@@ -1,81 +1,1147 @@
-// a5-a6, the block solver: one tuple CASCI of more than the warp solver's
-// determinants per thread block, vectors in a per-block slot of the workspace.
-#include "casci_dev.cuh"
+// a2-a7, the block solver: one tuple CASCI beyond the warp solvers per thread block.
+//
+// The Davidson's vectors lie in one spin-flip sector and are kept as their Ns (Ns + 1) / 2
+// elements with Ia <= Ib (orthonormal basis of the sector, as in casci_sector.cuh), in a
+// per-block slot of the workspace: half of the memory traffic of the vector algebra, which
+// with the sigma below is what bounds a tuple of 8 or 9 orbitals (46 vectors of up to 32 KB
+// in float32 per block do not fit in L2 for all blocks).
+//
+// sigma up to 9 orbitals (at most 126 strings): the whole coefficient matrix c sits in shared
+// memory, and per alpha string Ia the opposite-spin term is a dense product and a gather,
+//     T[p][J] = sum_x s_x V[p_x][p] c[J_x][J],   sigma[Ia][Ib] = sum_y s_y T[p_y][J_y].
+// The product is register-tiled (4 strings x 6 pairs per thread in float32: one 16-byte and
+// three 8-byte shared loads for 24 multiply-adds), where the double loop over both lists
+// gathers three values for every multiply-add; it does 2 P / R = 3.6 times more of them at
+// 9 orbitals, but near the rate of the pipe.  In float64 the same product runs on integers
+// (55-bit fixed point in two limbs, three wide integer multiply-adds per term, exact sums:
+// see casci_sector64.cuh), because a float64 multiply-add costs 36 integer ones here.
+// Beyond 9 orbitals c does not fit, and sigma walks both lists per element.
+#include "casci_sector.cuh"
 
 namespace mbe {
 
-__global__ void __launch_bounds__(CTA_THREADS, 2) k_casci_block(BatchArgs a, int bucket)
+constexpr int BLOCK_THREADS = 512;  // one block per SM: 128 registers a thread, up to 227 KB
+constexpr int GEMM_MAX_N = 9;       // orbitals up to which sigma is the tiled product
+constexpr int GEMM_T_BYTES = 48 * 1024;
+
+// Per-block slot of the workspace.
+struct BlockSlot {
+    size_t off_V, off_W, off_x, off_t, off_diag, off_Hs64, off_Hs32, off_x2, off_x0, off_full, vec, bytes;
+};
+
+__host__ __device__ inline int hs_stride(int ns) { return (ns + 3) / 4 * 4; }
+
+__host__ __device__ inline BlockSlot block_slot(int ns)
+{
+    BlockSlot L;
+    size_t o = 0;
+    const size_t vec = ((size_t)ns * (ns + 1) / 2 * 8 + 255) & ~(size_t)255;
+    const size_t mat = ((size_t)ns * hs_stride(ns) * 8 + 255) & ~(size_t)255;
+    L.vec = vec;
+    L.off_V = o; o += vec * MMAX;
+    L.off_W = o; o += vec * MMAX;
+    L.off_x = o; o += vec;
+    L.off_t = o; o += vec;
+    L.off_diag = o; o += vec;
+    L.off_x2 = o; o += vec;
+    L.off_x0 = o; o += vec;
+    L.off_Hs64 = o; o += mat;
+    L.off_Hs32 = o; o += mat / 2;
+    L.off_full = o; o += mat;  // the product C Hs, or the whole coefficient matrix
+    L.bytes = o;
+    return L;
+}
+
+// Shapes of the tiled sigma of one string class.
+struct GemmShape {
+    int cst;        // row stride of c and of T (strings, padded to 4)
+    int pst;        // row stride of the float32 V (pairs, padded to 6)
+    int rs;         // row stride of the lists
+    int np, tiles;  // pair groups, tiles per alpha string
+    int g;          // alpha strings per stage
+};
+
+template <typename T>
+__host__ __device__ inline GemmShape gemm_shape(int n, int ns, int r)
+{
+    GemmShape s;
+    const int P = n * (n + 1) / 2, tp = sizeof(T) == 8 ? 3 : 6;
+    s.cst = hs_stride(ns);
+    s.pst = (P + 5) / 6 * 6;
+    s.rs = r | 1;
+    s.np = (P + tp - 1) / tp;
+    s.tiles = s.np * (s.cst / 4);
+    s.g = BLOCK_THREADS / s.tiles;
+    const int fit = GEMM_T_BYTES / (P * s.cst * (int)sizeof(T));
+    if (s.g > fit) s.g = fit;
+    if (s.g > ns) s.g = ns;
+    if (s.g < 1) s.g = 1;
+    return s;
+}
+
+struct BlockMem {  // dynamic shared memory
+    int off_A, off_pp, off_h, off_V64, off_V32, off_red, off_G, off_J, off_ev, off_y, off_yp, off_r, off_misc,
+        off_hd, off_list, off_c, off_T, off_g1, bytes;
+};
+
+// gemm: the tiled sigma's lists, c (8 bytes an element) and T; else those are absent.
+// rdm: density matrices follow the solve.
+__host__ __device__ inline BlockMem block_mem(int n, bool gemm, int ns, int r, int rdm)
+{
+    BlockMem S;
+    const int P = n * (n + 1) / 2;
+    int o = 0;
+    S.off_A = o; o = al16(o + 4 * MBE_MAX_CAS);
+    S.off_pp = o; o = al16(o + 4 * P);
+    S.off_h = o; o = al16(o + 8 * n * n);
+    S.off_V64 = o; o = al16(o + 8 * P * P);
+    S.off_V32 = o; o = al16(o + 4 * P * ((P + 5) / 6 * 6));
+    S.off_red = o; o = al16(o + 8 * 32 * KRED);
+    S.off_G = o; o = al16(o + 8 * MMAX * MMAX);
+    S.off_J = o; o = al16(o + 4 * 4 * MMAX * MMAX);
+    S.off_ev = o; o = al16(o + 4 * MMAX);
+    S.off_y = o; o = al16(o + 8 * MMAX);
+    S.off_yp = o; o = al16(o + 8 * MMAX);
+    S.off_r = o; o = al16(o + 8 * MMAX);
+    S.off_misc = o; o = al16(o + 8 * 4);
+    S.off_g1 = o; o = al16(o + 8 * n * n);
+    S.off_hd = o; o = al16(o + (gemm ? 8 * ns : 0));
+    S.off_list = o; o = al16(o + (gemm ? 2 * ns * (r | 1) : 0));
+    S.off_c = o; o = al16(o + (gemm ? 8 * ns * hs_stride(ns) : 0));
+    S.off_T = o;
+    if (gemm) {
+        const GemmShape a = gemm_shape<float>(n, ns, r), b = gemm_shape<double>(n, ns, r);
+        const int ta = a.g * P * a.cst * 4, tb = b.g * P * b.cst * 8;
+        o = al16(o + (ta > tb ? ta : tb));
+    }
+    // the density matrices' vectors lie over c and T
+    const int d = rdm ? S.off_c + 8 * 33 * (n * n + 1) : 0;
+    S.bytes = al16(o > d ? o : d);
+    return S;
+}
+
+struct BlockProblem {
+    Problem pb;       // N: packed elements; diag: packed
+    bool gemm;
+    bool bad;         // an element of V or Hs is not finite (float64 sigma: fixed point cannot hold it)
+    int E;            // fixed-point exponent
+    char *smem;
+    BlockMem S;
+    double *full;     // [Ns][stride] scratch of the slot
+};
+
+__device__ __forceinline__ void ffma2(unsigned long long &d, unsigned long long a, unsigned long long b)
+{
+    asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(d) : "l"(a), "l"(b));
+}
+__device__ __forceinline__ unsigned long long dup2(float v)
+{
+    const unsigned long long u = __float_as_uint(v);
+    return u << 32 | u;
+}
+
+// The packed vector v as the whole matrix [Ns][ld] (elements with Ia != Ib scaled back).
+template <typename T>
+__device__ inline void expand_full(const Problem &pb, const T *v, T *full, int ld)
+{
+    int ia = 0, ib = 0;
+    tri_advance(ia, ib, threadIdx.x, pb.Ns);
+    for (int h = threadIdx.x; h < pb.N; h += blockDim.x) {
+        const T c = ia == ib ? v[h] : (T)0.70710678118654752 * v[h];
+        full[ia * ld + ib] = c;
+        full[ib * ld + ia] = pb.sector > 0 ? c : -c;
+        tri_advance(ia, ib, blockDim.x, pb.Ns);
+    }
+}
+
+// M = C Hs for the float32 product: 4 x 4 tiles, c from shared memory, Hs through L1.
+__device__ inline void same_spin(const Problem &pb, int ld, const float *c, const float *Hs, float *M)
+{
+    const int nt = ld / 4;
+    for (int q = threadIdx.x; q < nt * nt; q += blockDim.x) {
+        const int i0 = q / nt * 4, j0 = (q - q / nt * nt) * 4;
+        const float *c0 = c + i0 * ld, *c1 = c + (i0 + 1 < pb.Ns ? i0 + 1 : i0) * ld,
+                    *c2 = c + (i0 + 2 < pb.Ns ? i0 + 2 : i0) * ld, *c3 = c + (i0 + 3 < pb.Ns ? i0 + 3 : i0) * ld;
+        float4 a0 = make_float4(0, 0, 0, 0), a1 = a0, a2 = a0, a3 = a0;
+#pragma unroll 4
+        for (int J = 0; J < pb.Ns; ++J) {
+            const float4 h = *(const float4 *)(Hs + J * ld + j0);
+            const float x0 = c0[J], x1 = c1[J], x2 = c2[J], x3 = c3[J];
+            a0.x = fmaf(x0, h.x, a0.x); a0.y = fmaf(x0, h.y, a0.y); a0.z = fmaf(x0, h.z, a0.z); a0.w = fmaf(x0, h.w, a0.w);
+            a1.x = fmaf(x1, h.x, a1.x); a1.y = fmaf(x1, h.y, a1.y); a1.z = fmaf(x1, h.z, a1.z); a1.w = fmaf(x1, h.w, a1.w);
+            a2.x = fmaf(x2, h.x, a2.x); a2.y = fmaf(x2, h.y, a2.y); a2.z = fmaf(x2, h.z, a2.z); a2.w = fmaf(x2, h.w, a2.w);
+            a3.x = fmaf(x3, h.x, a3.x); a3.y = fmaf(x3, h.y, a3.y); a3.z = fmaf(x3, h.z, a3.z); a3.w = fmaf(x3, h.w, a3.w);
+        }
+        *(float4 *)(M + i0 * ld + j0) = a0;
+        if (i0 + 1 < pb.Ns) *(float4 *)(M + (i0 + 1) * ld + j0) = a1;
+        if (i0 + 2 < pb.Ns) *(float4 *)(M + (i0 + 2) * ld + j0) = a2;
+        if (i0 + 3 < pb.Ns) *(float4 *)(M + (i0 + 3) * ld + j0) = a3;
+    }
+}
+
+// The same on integers (Hs without its diagonal): 2 x 2 tiles, one int64 per element.
+__device__ inline void same_spin(const Problem &pb, int ld, const int2 *c, const int2 *Hs, long long *M)
+{
+    const int nt = ld / 2;
+    for (int q = threadIdx.x; q < nt * nt; q += blockDim.x) {
+        const int i0 = q / nt * 2, j0 = (q - q / nt * nt) * 2;
+        const int2 *c0 = c + i0 * ld, *c1 = c + (i0 + 1 < pb.Ns ? i0 + 1 : i0) * ld;
+        long long h00 = 0, h01 = 0, h10 = 0, h11 = 0, l00 = 0, l01 = 0, l10 = 0, l11 = 0;
+#pragma unroll 2
+        for (int J = 0; J < pb.Ns; ++J) {
+            const int4 h = *(const int4 *)(Hs + J * ld + j0);
+            const int2 a = c0[J], b = c1[J];
+            h00 += (long long)a.x * h.x; l00 += (long long)a.x * h.y; l00 += (long long)a.y * h.x;
+            h01 += (long long)a.x * h.z; l01 += (long long)a.x * h.w; l01 += (long long)a.y * h.z;
+            h10 += (long long)b.x * h.x; l10 += (long long)b.x * h.y; l10 += (long long)b.y * h.x;
+            h11 += (long long)b.x * h.z; l11 += (long long)b.x * h.w; l11 += (long long)b.y * h.z;
+        }
+        const long long half = 1LL << 27;
+        if (i0 < pb.Ns) {
+            M[i0 * ld + j0] = h00 + ((l00 + half) >> 28);
+            M[i0 * ld + j0 + 1] = h01 + ((l01 + half) >> 28);
+        }
+        if (i0 + 1 < pb.Ns) {
+            M[(i0 + 1) * ld + j0] = h10 + ((l10 + half) >> 28);
+            M[(i0 + 1) * ld + j0 + 1] = h11 + ((l11 + half) >> 28);
+        }
+    }
+}
+
+// One tile of T in float32: 4 strings x 6 pairs (pairs of pairs in one 64-bit register).
+__device__ __forceinline__ void gemm_tile(const Problem &pb, const GemmShape &s, const uint16_t *la, const float *c,
+                                          const float *V, int j0, int pg, float *T)
+{
+    unsigned long long a[4][3];
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int k = 0; k < 3; ++k) a[i][k] = 0ull;
+#pragma unroll 2
+    for (int x = 0; x < pb.R; ++x) {
+        const int e = la[x];
+        const float4 cv = *(const float4 *)(c + (e >> 7) * s.cst + j0);
+        const unsigned long long *v = (const unsigned long long *)(V + ((e >> 1) & 63) * s.pst + pg * 6);
+        const unsigned long long v0 = v[0], v1 = v[1], v2 = v[2];
+        const float cs[4] = {cv.x, cv.y, cv.z, cv.w};
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const unsigned long long d = dup2(flip_if(cs[i], e & 1));
+            ffma2(a[i][0], v0, d);
+            ffma2(a[i][1], v1, d);
+            ffma2(a[i][2], v2, d);
+        }
+    }
+#pragma unroll
+    for (int k = 0; k < 6; ++k) {
+        const int p = pg * 6 + k;
+        if (p < pb.P) {
+            float4 o;
+            o.x = __uint_as_float((unsigned)(a[0][k >> 1] >> (32 * (k & 1))));
+            o.y = __uint_as_float((unsigned)(a[1][k >> 1] >> (32 * (k & 1))));
+            o.z = __uint_as_float((unsigned)(a[2][k >> 1] >> (32 * (k & 1))));
+            o.w = __uint_as_float((unsigned)(a[3][k >> 1] >> (32 * (k & 1))));
+            *(float4 *)(T + p * s.cst + j0) = o;
+        }
+    }
+}
+
+// One tile of T in fixed point: 4 strings x 3 pairs.
+__device__ __forceinline__ void gemm_tile(const Problem &pb, const GemmShape &s, const uint16_t *la, const int2 *c,
+                                          const int2 *V, int j0, int pg, long long *T)
+{
+    long long hi[4][3], lo[4][3];
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int k = 0; k < 3; ++k) hi[i][k] = lo[i][k] = 0;
+    const int p0 = pg * 3, p1 = min(p0 + 1, pb.P - 1), p2 = min(p0 + 2, pb.P - 1);
+#pragma unroll 1
+    for (int x = 0; x < pb.R; ++x) {
+        const int e = la[x], m = -(e & 1);
+        const int4 c01 = *(const int4 *)(c + (e >> 7) * s.cst + j0), c23 = *(const int4 *)(c + (e >> 7) * s.cst + j0 + 2);
+        const int2 *v = V + ((e >> 1) & 63) * pb.P;
+        const int ch[4] = {c01.x, c01.z, c23.x, c23.z}, cl[4] = {c01.y, c01.w, c23.y, c23.w};
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            int2 w = v[k == 0 ? p0 : k == 1 ? p1 : p2];
+            w.x = (w.x ^ m) - m;
+            w.y = (w.y ^ m) - m;
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                hi[i][k] += (long long)w.x * ch[i];
+                lo[i][k] += (long long)w.x * cl[i];
+                lo[i][k] += (long long)w.y * ch[i];
+            }
+        }
+    }
+#pragma unroll
+    for (int k = 0; k < 3; ++k)
+        if (p0 + k < pb.P)
+#pragma unroll
+            for (int i = 0; i < 4; ++i) T[(p0 + k) * s.cst + j0 + i] = hi[i][k] + ((lo[i][k] + (1LL << 27)) >> 28);
+}
+
+// sigma of a packed sector vector, tiled product.
+template <typename T>
+__device__ __noinline__ void sigma_gemm(const BlockProblem &B, const T *src, T *dst)
+{
+    constexpr bool F64 = sizeof(T) == 8;
+    using E = typename std::conditional<F64, int2, float>::type;       // elements of c and V
+    using A = typename std::conditional<F64, long long, float>::type;  // sums
+    const Problem &pb = B.pb;
+    const int Ns = pb.Ns, tid = threadIdx.x, nt = blockDim.x, R = pb.R, sgn = pb.sector;
+    const GemmShape s = gemm_shape<T>(pb.n, Ns, R);
+    E *c = (E *)(B.smem + B.S.off_c);
+    A *Tm = (A *)(B.smem + B.S.off_T);
+    const uint16_t *list = (const uint16_t *)(B.smem + B.S.off_list);
+    const double *hd = (const double *)(B.smem + B.S.off_hd);
+    const E *V = (const E *)(B.smem + (F64 ? B.S.off_V64 : B.S.off_V32));
+    A *M = (A *)B.full;
+    {
+        int ia = 0, ib = 0;
+        tri_advance(ia, ib, tid, Ns);
+        for (int h = tid; h < pb.N; h += nt) {
+            if constexpr (F64) {
+                const int2 f = to_fixed(src[h], ia == ib ? 36028797018963968.0 : 0.70710678118654752 * 36028797018963968.0);
+                c[ia * s.cst + ib] = f;
+                c[ib * s.cst + ia] = sgn > 0 ? f : make_int2(-f.x, -f.y);
+            } else {
+                const float f = ia == ib ? src[h] : 0.70710678118654752f * src[h];
+                c[ia * s.cst + ib] = f;
+                c[ib * s.cst + ia] = sgn > 0 ? f : -f;
+            }
+            tri_advance(ia, ib, nt, Ns);
+        }
+        for (int q = tid; q < Ns * (s.cst - Ns); q += nt) c[q / (s.cst - Ns) * s.cst + Ns + q % (s.cst - Ns)] = E{};
+    }
+    __syncthreads();
+    same_spin(pb, s.cst, c, F64 ? (const E *)pb.Hs64 : (const E *)pb.Hs32, M);
+    const int nj = s.cst / 4;
+    for (int I0 = 0; I0 < Ns; I0 += s.g) {
+        const int gc = min(s.g, Ns - I0);
+        for (int q = tid; q < gc * s.tiles; q += nt) {
+            const int g = q / s.tiles, r = q - g * s.tiles, pg = r / nj, jj = r - pg * nj;
+            gemm_tile(pb, s, list + (I0 + g) * s.rs, c, V, 4 * jj, pg, Tm + g * pb.P * s.cst);
+        }
+        __syncthreads();  // (also orders M, written above, before its first use)
+        const int two = 2 * gc * Ns <= nt ? 1 : 0;  // two threads per element where they fit
+        for (int q0 = 0; q0 < (gc * Ns) << two; q0 += nt) {
+            const int q = q0 + tid, el = q >> two, g = el / Ns, Ib = el - g * Ns, Ia = I0 + g;
+            const bool on = g < gc && Ib >= Ia;
+            A acc = 0;
+            if (on) {
+                const A *t = Tm + g * pb.P * s.cst;
+                const uint16_t *lb = list + Ib * s.rs;
+                for (int y = two ? q & 1 : 0; y < R; y += 1 + two) {
+                    const int e = lb[y];
+                    const A v = t[((e >> 1) & 63) * s.cst + (e >> 7)];
+                    acc += e & 1 ? -v : v;
+                }
+            }
+            if (two) acc += __shfl_xor_sync(FULL, acc, 1);
+            if (on && !(two && (q & 1))) {
+                const A mt = M[Ib * s.cst + Ia];
+                const int h = Ia * Ns - Ia * (Ia - 1) / 2 + Ib - Ia;
+                acc += M[Ia * s.cst + Ib] + (sgn > 0 ? mt : -mt);
+                T v;
+                if constexpr (F64) {
+                    v = fma(hd[Ia] + hd[Ib], src[h], (double)acc * (pow2(B.E - 54) * (Ia == Ib ? 1.0 : 1.4142135623730951)));
+                    if (B.bad) v = __longlong_as_double(0x7ff8000000000000LL);
+                } else {
+                    v = Ia == Ib ? acc : 1.41421356f * acc;
+                }
+                dst[h] = sgn < 0 && Ia == Ib ? (T)0 : v;
+            }
+        }
+        __syncthreads();
+    }
+}
+
+// sigma of a packed sector vector; ends with a barrier.
+template <typename T>
+__device__ inline void sigma_block(const BlockProblem &B, const T *src, T *dst)
+{
+    const Problem &pb = B.pb;
+    if (B.gemm) sigma_gemm<T>(B, src, dst);
+    if (B.gemm && pb.s2mu == 0.0) return;
+    T *full = (T *)B.full;
+    expand_full<T>(pb, src, full, pb.Ns);
+    __syncthreads();
+    int ia = 0, ib = 0;
+    tri_advance(ia, ib, threadIdx.x, pb.Ns);
+    for (int h = threadIdx.x; h < pb.N; h += blockDim.x) {
+        T v = (T)0;
+        if (!(pb.sector < 0 && ia == ib)) {
+            if (!B.gemm) {
+                if constexpr (sizeof(T) == 4)
+                    v = sigma_elem_ashared<T>(pb, pb.V32, pb.Hs32, full, ia, ib);
+                else
+                    v = sigma_elem<T>(pb, pb.V64, pb.Hs64, full, ia * pb.Ns + ib);
+            }
+            if (pb.s2mu != 0.0) v += (T)pb.s2mu * s2_elem<T, T>(pb, full, ia, ib);
+            if (ia != ib) v *= (T)1.4142135623730951;
+        }
+        dst[h] = B.gemm ? dst[h] + v : v;
+        tri_advance(ia, ib, blockDim.x, pb.Ns);
+    }
+    __syncthreads();
+}
+
+// Lowest eigenpair of the m x m symmetric Rayleigh matrix G (shared memory, float64, row
+// stride MMAX) by the whole block: a float32 Jacobi on G - G00 I in round-robin order, m / 2
+// disjoint rotations at a time, one element of the matrix and of the eigenvectors per thread
+// (m - 1 steps per sweep, where rotating one pair after the other in one warp took m (m - 1)
+// / 2 of about the same length); in float64 then two Newton steps in that eigenbasis,
+// z = y - sum_{k != 0} e_k (e_k . r) / (theta_k - theta),  r = G y - theta y,
+// theta = y.G y, which make the lowest pair float64-accurate (one warp).
+// Output: y[0..m) (unit norm), y2 (the second lowest, which seeds the thick restart), and
+// misc[0] = theta; ends with a barrier.  buf: 4 MMAX^2 floats.
+template <bool REFINE>
+__device__ __noinline__ void small_eig_block(const double *G, int m, float *buf, float *ev, double *y, double *y2,
+                                             double *r, double *misc)
+{
+    const int tid = threadIdx.x, i = tid / MMAX, j = tid - i * MMAX, lane = tid & 31;
+    const bool on = i < m && j < m;
+    const double shift = G[0];
+    float *A = buf, *E = buf + MMAX * MMAX, *A2 = buf + 2 * MMAX * MMAX, *E2 = buf + 3 * MMAX * MMAX;
+    if (on) {
+        A[tid] = (float)(G[i * MMAX + j] - (i == j ? shift : 0.0));
+        E[tid] = i == j ? 1.0f : 0.0f;
+    }
+    __syncthreads();
+    const int M = m + (m & 1);  // an odd matrix gets an idle partner
+    // the rotation of row or column u with its partner: coefficients of itself and of the partner
+    auto rotation = [&](int u, int v, float &c, float &s) {
+        c = 1.f;
+        s = 0.f;
+        if (v >= m) return;
+        const int p = u < v ? u : v, q = u < v ? v : u;
+        const float apq = A[p * MMAX + q];
+        if (fabsf(apq) < 1e-36f) return;
+        const float th = (A[q * MMAX + q] - A[p * MMAX + p]) / (2.0f * apq);
+        float t = 1.0f / (fabsf(th) + sqrtf(th * th + 1.0f));
+        if (th < 0.0f) t = -t;
+        c = rsqrtf(t * t + 1.0f);
+        s = u < v ? -t * c : t * c;
+    };
+    for (int sweep = 0; sweep < 10 && m > 1; ++sweep) {
+        float dia = 0.f;
+        bool big = false;
+        if (on) {
+            for (int k = 0; k < m; ++k) dia += A[k * MMAX + k] * A[k * MMAX + k];
+            const float a = A[tid];
+            big = i != j && a * a > 1e-14f * dia && fabsf(a) > 1e-18f;
+        }
+        if (!__syncthreads_or(big)) break;
+        for (int step = 0; step < M - 1; ++step) {
+            if (on) {
+                auto partner = [&](int u) {
+                    if (u == M - 1) return step;
+                    if (u == step) return M - 1;
+                    const int v = 2 * step - u;
+                    return v < 0 ? v + M - 1 : v >= M - 1 ? v - (M - 1) : v;
+                };
+                const int pi = partner(i), pj = partner(j);
+                float ci, si, cj, sj;
+                rotation(i, pi, ci, si);
+                rotation(j, pj, cj, sj);
+                const int ui = pi < m ? pi : i, uj = pj < m ? pj : j;
+                const float a0 = cj * A[i * MMAX + j] + sj * A[i * MMAX + uj];
+                const float a1 = cj * A[ui * MMAX + j] + sj * A[ui * MMAX + uj];
+                A2[tid] = pi == j ? 0.0f : ci * a0 + si * a1;
+                E2[tid] = cj * E[i * MMAX + j] + sj * E[i * MMAX + uj];
+            }
+            __syncthreads();
+            float *z = A;
+            A = A2;
+            A2 = z;
+            z = E;
+            E = E2;
+            E2 = z;
+        }
+    }
+    if (tid < 32) {
+        float best = (lane < m) ? A[lane * MMAX + lane] : 3.0e38f;
+        int bi = lane;
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            float ov = __shfl_xor_sync(FULL, best, o);
+            int oi = __shfl_xor_sync(FULL, bi, o);
+            if (ov < best || (ov == best && oi < bi)) {
+                best = ov;
+                bi = oi;
+            }
+        }
+        float best2 = (lane < m && lane != bi) ? A[lane * MMAX + lane] : 3.0e38f;
+        int b2 = (lane < m && lane != bi) ? lane : 0x7fffffff;
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            float ov = __shfl_xor_sync(FULL, best2, o);
+            int oi = __shfl_xor_sync(FULL, b2, o);
+            if (ov < best2 || (ov == best2 && oi < b2)) {
+                best2 = ov;
+                b2 = oi;
+            }
+        }
+        if (lane < m) {
+            ev[lane] = A[lane * MMAX + lane];
+            y[lane] = (double)E[lane * MMAX + bi];
+            y2[lane] = (b2 < m) ? (double)E[lane * MMAX + b2] : 0.0;
+        }
+        __syncwarp();
+        double theta = shift + (double)best;
+        if (REFINE) {
+            for (int step = 0; step < 2; ++step) {
+                double g = 0.0, yi = (lane < m) ? y[lane] : 0.0;
+                if (lane < m)
+                    for (int k = 0; k < m; ++k) g += G[lane * MMAX + k] * y[k];
+                double yy = warp_sum(yi * yi), ygy = warp_sum(yi * g);
+                theta = ygy / yy;
+                if (lane < m) r[lane] = g - theta * yi;
+                __syncwarp();
+                // coefficient of eigenvector k (lane k)
+                double ck = 0.0;
+                if (lane < m && lane != bi) {
+                    for (int k = 0; k < m; ++k) ck += (double)E[k * MMAX + lane] * r[k];
+                    double den = shift + (double)ev[lane] - theta;
+                    ck = (fabs(den) > 1e-300) ? ck / den : 0.0;
+                }
+                __syncwarp();
+                if (lane < m) r[lane] = ck;  // reuse r for the coefficients
+                __syncwarp();
+                double z = yi;
+                if (lane < m)
+                    for (int k = 0; k < m; ++k) z -= (double)E[lane * MMAX + k] * r[k];
+                double zz = warp_sum(z * z);
+                if (lane < m) y[lane] = z / sqrt(zz);
+                __syncwarp();
+            }
+            double g = 0.0, yi = (lane < m) ? y[lane] : 0.0;
+            if (lane < m)
+                for (int k = 0; k < m; ++k) g += G[lane * MMAX + k] * y[k];
+            theta = warp_sum(yi * g);
+        }
+        if (lane == 0) misc[0] = theta;
+    }
+    __syncthreads();
+}
+
+// Sums of the first k of the values v[0..KRED) over the block; every thread gets the
+// totals.  Two barriers: the warps' sums, then one warp per value.  red: 32 * KRED elements.
+template <typename T>
+__device__ inline void block_sums(T (&v)[KRED], int k, T *red)
+{
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
+#pragma unroll
+    for (int i = 0; i < KRED; ++i)
+        if (i < k) v[i] = warp_sum(v[i]);
+    if (lane == 0)
+#pragma unroll
+        for (int i = 0; i < KRED; ++i)
+            if (i < k) red[w * KRED + i] = v[i];
+    __syncthreads();
+    T *tot = red + 31 * KRED;
+    for (int i = w; i < k; i += nw) {
+        const T s = warp_sum(lane < nw ? red[lane * KRED + i] : (T)0);
+        if (lane == 0) tot[i] = s;
+    }
+    __syncthreads();
+#pragma unroll
+    for (int i = 0; i < KRED; ++i)
+        if (i < k) v[i] = tot[i];
+}
+
+// The vectors are read and written 16 bytes at a time; the elements between N and the next
+// multiple of 16 bytes are zero in every vector (one in the diagonal).
+template <typename T>
+struct alignas(16) Pack {
+    static constexpr int L = 16 / sizeof(T);
+    T e[L];
+};
+
+// One Davidson phase in precision T on packed sector vectors.  V, W: MMAX vectors each,
+// leading dimension ld (elements).
+// Plain: x is the start vector in, the unit Ritz vector out.  Anchored (T =
+// float, anch): V[0] = x0 and W[0] = r0 = (H - shift) x0 are given (see struct
+// Anchor), every other basis vector is a correction whose image is the float32
+// sigma minus shift times it, the Ritz value is that of H - shift, the coupling
+// of x0 to a vector v is formed as v.r0, a thick restart keeps x0 and the
+// corrections of the two lowest Ritz vectors, and x returns the correction d of
+// the Ritz vector x0 + d.  steer: iterations without a 10% residual drop that end
+// the phase (0: none).
+template <typename T>
+__device__ __noinline__ PhaseOut davidson_block(const BlockProblem &B, T *Vp, T *Wp, size_t ld_, T *xp, T *tp, double tol,
+                                                int min_iter, int max_iter, int steer, double shift = 0.0,
+                                                bool anch = false, int mmax = MMAX)
+{
+    using K = Pack<T>;
+    constexpr int VL = K::L;
+    const Problem &pb = B.pb;
+    const BlockMem &S = B.S;
+    char *smem = B.smem;
+    const int tid = threadIdx.x, nt = blockDim.x, N = (pb.N + VL - 1) / VL;  // packs
+    const size_t ld = ld_ / VL;
+    K *V = (K *)Vp, *W = (K *)Wp, *x = (K *)xp, *tx = (K *)tp;
+    T *red = (T *)(smem + S.off_red);
+    double *G = (double *)(smem + S.off_G);
+    double *ys = (double *)(smem + S.off_y);
+    double *y2s = (double *)(smem + S.off_yp);
+    double *misc = (double *)(smem + S.off_misc);
+    PhaseOut o;
+    o.nsig = 0;
+    o.status = MBE_STATUS_OK;
+    o.dnorm = 0.0;
+    const T shT = (T)shift, shT_lo = (T)(shift - (double)shT);
+    T v[KRED];
+    auto dot = [&](const K &a, const K &b, T s) {
+#pragma unroll
+        for (int l = 0; l < VL; ++l) s = fma(a.e[l], b.e[l], s);
+        return s;
+    };
+    auto axpy = [&](T a, const K &b, K &c) {
+#pragma unroll
+        for (int l = 0; l < VL; ++l) c.e[l] = fma(a, b.e[l], c.e[l]);
+    };
+    auto scale = [&](T a, K *c) {
+        for (int d = tid; d < N; d += nt) {
+            K q = c[d];
+#pragma unroll
+            for (int l = 0; l < VL; ++l) q.e[l] *= a;
+            c[d] = q;
+        }
+    };
+    if (!anch) {
+        v[0] = 0;
+        for (int d = tid; d < N; d += nt) v[0] = dot(x[d], x[d], v[0]);
+        block_sums<T>(v, 1, red);
+        const T inv = (T)1 / sqrt(v[0]);
+        for (int d = tid; d < N; d += nt) {
+            K q = x[d];
+#pragma unroll
+            for (int l = 0; l < VL; ++l) q.e[l] *= inv;
+            V[d] = q;
+        }
+        __syncthreads();
+        sigma_block<T>(B, (const T *)V, (T *)W);
+        ++o.nsig;
+        v[0] = 0;
+        for (int d = tid; d < N; d += nt) v[0] = dot(V[d], W[d], v[0]);
+        block_sums<T>(v, 1, red);
+        if (tid == 0) G[0] = (double)v[0];
+    } else if (tid == 0) {
+        G[0] = 0.0;  // x0.r0 = 0: shift is x0's Rayleigh quotient
+    }
+    __syncthreads();
+    int m = 1;
+    double theta = 0.0;
+    T rn = 0;
+    T best = (T)3e38;
+    int stall = 0;
+    for (int it = 0;; ++it) {
+        small_eig_block<sizeof(T) == 8>(G, m, (float *)(smem + S.off_J), (float *)(smem + S.off_ev), ys, y2s,
+                                        (double *)(smem + S.off_r), misc);
+        theta = misc[0];
+        const T th = (T)theta;
+        K *tdst = (m < mmax) ? V + (size_t)m * ld : tx;
+        v[0] = 0;
+        v[1] = 0;
+        for (int d = tid; d < N; d += nt) {
+            K xs, hs, td;
+#pragma unroll
+            for (int l = 0; l < VL; ++l) xs.e[l] = hs.e[l] = 0;
+#pragma unroll 4
+            for (int i = 0; i < m; ++i) {
+                const T yi = (T)ys[i];
+                axpy(yi, V[(size_t)i * ld + d], xs);
+                axpy(yi, W[(size_t)i * ld + d], hs);
+            }
+#pragma unroll
+            for (int l = 0; l < VL; ++l) {
+                const T r = hs.e[l] - th * xs.e[l];
+                v[0] += r * r;
+                T den = (T)(pb.diag[d * VL + l] - shift) - th;
+                if (fabs(den) < (T)1e-4) den = den >= (T)0 ? (T)1e-4 : (T)-1e-4;
+                td.e[l] = r / den;
+                v[1] += td.e[l] * td.e[l];
+            }
+            tdst[d] = td;
+        }
+        block_sums<T>(v, 2, red);
+        rn = sqrt(v[0]);
+        const T t0n = sqrt(v[1]);
+        if (!isfinite(rn) || !isfinite(theta)) {
+            o.status = MBE_STATUS_NONFINITE;
+            break;
+        }
+        if (rn <= (T)tol && it >= min_iter) break;
+        if (it >= max_iter) {
+            o.status = MBE_STATUS_MAXITER;
+            break;
+        }
+        if (steer) {
+            if (rn < (T)0.9 * best) {
+                best = rn;
+                stall = 0;
+            } else if (++stall >= steer) {
+                break;
+            }
+        }
+        if (m == mmax) {
+            // Thick restart on the two lowest Ritz vectors (orthogonal by construction, so W
+            // stays consistent with H V); anchored: V[0] = x0, W[0] = r0 stay and the
+            // corrections of the two go to V[1], V[2] (both orthogonal to x0).
+            const int b = anch ? 1 : 0;
+            K *V0 = V + b * ld, *W0 = W + b * ld, *V1 = V0 + ld, *W1 = W0 + ld;
+            v[0] = 0;
+            for (int d = tid; d < N; d += nt) {
+                K u1, w1, u2, w2;
+#pragma unroll
+                for (int l = 0; l < VL; ++l) u1.e[l] = w1.e[l] = u2.e[l] = w2.e[l] = 0;
+#pragma unroll 2
+                for (int i = b; i < mmax; ++i) {
+                    const K vi = V[(size_t)i * ld + d], wi = W[(size_t)i * ld + d];
+                    axpy((T)ys[i], vi, u1);
+                    axpy((T)ys[i], wi, w1);
+                    axpy((T)y2s[i], vi, u2);
+                    axpy((T)y2s[i], wi, w2);
+                }
+                V0[d] = u1;
+                W0[d] = w1;
+                V1[d] = u2;
+                W1[d] = w2;
+                v[0] = dot(u1, u1, v[0]);
+            }
+            block_sums<T>(v, 1, red);
+            const T n0 = sqrt(v[0]);
+            if (anch) {
+                scale((T)1 / n0, V0);
+                scale((T)1 / n0, W0);
+            }
+            for (int pass = 0; pass < 2; ++pass) {
+                v[0] = 0;
+                for (int d = tid; d < N; d += nt) v[0] = dot(V0[d], V1[d], v[0]);
+                block_sums<T>(v, 1, red);
+                for (int d = tid; d < N; d += nt) {
+                    K q = V1[d], w = W1[d];
+                    axpy(-v[0], V0[d], q);
+                    axpy(-v[0], W0[d], w);
+                    V1[d] = q;
+                    W1[d] = w;
+                }
+            }
+            v[0] = 0;
+            for (int d = tid; d < N; d += nt) v[0] = dot(V1[d], V1[d], v[0]);
+            block_sums<T>(v, 1, red);
+            const T nn = sqrt(v[0]);
+            const bool keep = nn > (anch ? (T)1e-3 : (T)0.5);
+            if (keep) {
+                scale((T)1 / nn, V1);
+                scale((T)1 / nn, W1);
+            }
+            v[0] = v[1] = v[2] = v[3] = v[4] = 0;
+            for (int d = tid; d < N; d += nt) {
+                const K v0 = V0[d], w0 = W0[d];
+                v[0] = dot(v0, w0, v[0]);
+                if (anch) v[1] = dot(W[d], v0, v[1]);  // x0.(A u1) as u1.r0
+                if (keep) {
+                    const K v1 = V1[d], w1 = W1[d];
+                    v[2] = dot(v0, w1, v[2]);
+                    v[3] = dot(v1, w1, v[3]);
+                    if (anch) v[4] = dot(W[d], v1, v[4]);
+                }
+            }
+            block_sums<T>(v, 5, red);
+            if (tid == 0) {
+                G[b * MMAX + b] = (double)v[0];
+                if (anch) G[1] = G[MMAX] = (double)v[1];
+                if (keep) {
+                    G[b * MMAX + b + 1] = G[(b + 1) * MMAX + b] = (double)v[2];
+                    G[(b + 1) * MMAX + b + 1] = (double)v[3];
+                    if (anch) G[2] = G[2 * MMAX] = (double)v[4];
+                }
+                // the Ritz vector in the new basis
+                ys[b] = anch ? (double)n0 : 1.0;
+                ys[b + 1] = 0.0;
+            }
+            m = b + (keep ? 2 : 1);
+        }
+        // Correction: orthogonalise against V[0..m) into V[m]; a second pass when the first
+        // one cancelled (less than half of |t|^2 left; with more left, one pass is orthogonal
+        // to within a few rounding errors).
+        K *tv = V + (size_t)m * ld;
+        const K *tsrc = (tdst == tx) ? tx : tv;
+        T tn = t0n;
+        for (int pass = 0; pass < 2; ++pass) {
+#pragma unroll
+            for (int i = 0; i < KRED; ++i) v[i] = 0;
+            for (int d = tid; d < N; d += nt) {
+                const K td = (pass == 0) ? tsrc[d] : tv[d];
+#pragma unroll
+                for (int i = 0; i < MMAX; ++i)
+                    if (i < m) v[i] = dot(V[(size_t)i * ld + d], td, v[i]);
+            }
+            block_sums<T>(v, m, red);
+            T tt = 0;
+            for (int d = tid; d < N; d += nt) {
+                K td = (pass == 0) ? tsrc[d] : tv[d];
+#pragma unroll
+                for (int i = 0; i < MMAX; ++i)
+                    if (i < m) axpy(-v[i], V[(size_t)i * ld + d], td);
+                tv[d] = td;
+                tt = dot(td, td, tt);
+            }
+            v[0] = tt;
+            block_sums<T>(v, 1, red);
+            const T before = tn;
+            tn = sqrt(v[0]);
+            if (tn >= (T)0.70710678 * before) break;
+        }
+        if (!(tn > (T)1e-12 * t0n) || !(tn > (T)0)) {
+            // The correction lies in the current basis: nothing left to add.
+            if (!steer && rn > (T)tol) o.status = MBE_STATUS_MAXITER;
+            break;
+        }
+        scale((T)1 / tn, tv);
+        __syncthreads();
+        K *wv = W + (size_t)m * ld;
+        sigma_block<T>(B, (const T *)tv, (T *)wv);
+        ++o.nsig;
+#pragma unroll
+        for (int i = 0; i < KRED; ++i) v[i] = 0;
+        for (int d = tid; d < N; d += nt) {
+            K wd = wv[d];
+            const K td = tv[d];
+            if (anch) {
+#pragma unroll
+                for (int l = 0; l < VL; ++l) wd.e[l] = (wd.e[l] - shT * td.e[l]) - shT_lo * td.e[l];
+                wv[d] = wd;
+            }
+#pragma unroll
+            for (int i = 0; i < MMAX; ++i)
+                if (i < m) v[i] = (anch && i == 0) ? dot(W[d], td, v[i]) : dot(V[(size_t)i * ld + d], wd, v[i]);
+            v[MMAX] = dot(td, wd, v[MMAX]);
+        }
+        {
+            const T diag = v[MMAX];
+#pragma unroll
+            for (int i = 0; i <= MMAX; ++i)
+                if (i == m) v[i] = diag;
+        }
+        block_sums<T>(v, m + 1, red);
+        if (tid == 0)
+            for (int i = 0; i <= m; ++i) G[i * MMAX + m] = G[m * MMAX + i] = (double)v[i];
+        __syncthreads();
+        ++m;
+    }
+    // the Ritz vector; anchored: its correction d, scaled so that x0 keeps coefficient 1
+    __syncthreads();
+    const T inv0 = anch ? (T)(1.0 / ys[0]) : (T)1;
+    v[0] = 0;
+    for (int d = tid; d < N; d += nt) {
+        K u;
+#pragma unroll
+        for (int l = 0; l < VL; ++l) u.e[l] = 0;
+#pragma unroll 4
+        for (int i = anch ? 1 : 0; i < m; ++i) axpy((T)ys[i] * inv0, V[(size_t)i * ld + d], u);
+        x[d] = u;
+        v[0] = dot(u, u, v[0]);
+    }
+    block_sums<T>(v, 1, red);
+    if (anch) o.dnorm = (double)sqrt(v[0]);
+    o.lambda = theta;
+    o.rnorm = (double)rn;
+    return o;
+}
+
+// Element h of the sector's start vector in the packed basis (see sector_guess).
+__device__ inline double block_guess(int ia, int ib, int Ns, int h, int g, int sgn)
+{
+    const double z = GUESS_NOISE * guess_noise(ia * Ns + ib);
+    if (ia == ib) return sgn > 0 ? z + (h == g ? 2.0 : 0.0) : 0.0;
+    return 1.4142135623730951 * (z + (h == g ? 1.0 : 0.0));
+}
+
+template <typename T>
+__device__ inline void write_guess(const Problem &pb, int g, T *x)
+{
+    int ia = 0, ib = 0;
+    tri_advance(ia, ib, threadIdx.x, pb.Ns);
+    for (int h = threadIdx.x; h < pb.N; h += blockDim.x) {
+        x[h] = (T)block_guess(ia, ib, pb.Ns, h, g, pb.sector);
+        tri_advance(ia, ib, blockDim.x, pb.Ns);
+    }
+}
+
+// a2, a4: h_eff, V, Hs (Slater-Condon elements) and the packed diagonal, and for the tiled
+// sigma the lists, the padded float32 V and the fixed-point V and Hs (over the float64 ones).
+__device__ void block_setup(const BatchArgs &a, BlockProblem &B, const ClassInfo &ci)
+{
+    Problem &pb = B.pb;
+    const int tid = threadIdx.x, nt = blockDim.x, n = pb.n, P = pb.P, norb = a.norb, Ns = pb.Ns, st = pb.HSS;
+    double *red = (double *)(B.smem + B.S.off_red);
+    for (int e = tid; e < P; e += nt) {
+        int p = 0;
+        while ((p + 1) * (p + 2) / 2 <= e) ++p;
+        ((short *)pb.pp)[2 * e] = (short)p;
+        ((short *)pb.pp)[2 * e + 1] = (short)(e - p * (p + 1) / 2);
+    }
+    for (int e = tid; e < n * n; e += nt) {
+        const int x = e / n, y = e - x * n, gp = pb.A[x], gq = pb.A[y];
+        double v = a.F[gp * norb + gq];
+        for (int c = 0; c < n; ++c) {
+            const int gi = pb.A[c];
+            if (a.occ[gi])
+                v -= 2.0 * a.eri[eri_index(norb, gp, gq, gi, gi)] - a.eri[eri_index(norb, gp, gi, gi, gq)];
+        }
+        pb.h[e] = v;
+    }
+    __syncthreads();
+    const int vs = B.gemm ? (P + 5) / 6 * 6 : P;
+    double big = 0.0;
+    bool bad = false;
+    for (int e = tid; e < P * vs; e += nt) {
+        const int x = e / vs, y = e - x * vs;
+        double v = 0.0;
+        if (y < P) {
+            const int p = pb.pp[2 * x], q = pb.pp[2 * x + 1], r = pb.pp[2 * y], s = pb.pp[2 * y + 1];
+            v = a.eri[eri_index(norb, pb.A[p], pb.A[q], pb.A[r], pb.A[s])];
+            pb.V64[x * P + y] = v;
+            big = fmax(big, fabs(v));
+            bad = bad || !isfinite(v);
+        }
+        pb.V32[e] = (float)v;
+    }
+    if (B.gemm) {
+        uint16_t *list = (uint16_t *)(B.smem + B.S.off_list);
+        const int rs = pb.R | 1;
+        for (int e = tid; e < Ns * pb.R; e += nt) {
+            const int t = ci.table[e], I = e / pb.R;
+            list[I * rs + e - I * pb.R] = (uint16_t)(entry_J(t) << 7 | (t & 127));
+        }
+    }
+    __syncthreads();
+    auto H = [&](int p, int q) { return pb.h[p * n + q]; };
+    auto V = [&](int p, int q, int r, int s) { return pb.V64[pair_index(p, q) * P + pair_index(r, s)]; };
+    double *hd = (double *)(B.smem + B.S.off_hd);
+    {
+        int ia = 0, ib = 0;
+        tri_advance(ia, ib, tid, Ns);
+        for (int h = tid; h < pb.N; h += nt) {
+            const double v = string_element(pb.str[ia], pb.str[ib], H, V);
+            pb.Hs64[ia * st + ib] = pb.Hs64[ib * st + ia] = v;
+            pb.Hs32[ia * st + ib] = pb.Hs32[ib * st + ia] = (float)v;
+            if (ia != ib) big = fmax(big, fabs(v));
+            bad = bad || !isfinite(v);
+            tri_advance(ia, ib, nt, Ns);
+        }
+        for (int q = tid; q < Ns * (st - Ns); q += nt) {
+            const int at = q / (st - Ns) * st + Ns + q % (st - Ns);
+            pb.Hs64[at] = 0.0;
+            pb.Hs32[at] = 0.f;
+        }
+    }
+    B.bad = __syncthreads_or(bad);
+    {
+        int ia = 0, ib = 0;
+        tri_advance(ia, ib, tid, Ns);
+        for (int h = tid; h < pb.N; h += nt) {
+            double v = pb.Hs64[ia * st + ia] + pb.Hs64[ib * st + ib];
+            for (uint32_t sa = pb.str[ia]; sa; sa &= sa - 1u) {
+                const int p = __ffs((int)sa) - 1;
+                for (uint32_t sb = pb.str[ib]; sb; sb &= sb - 1u) v += V(p, p, __ffs((int)sb) - 1, __ffs((int)sb) - 1);
+            }
+            v += pb.s2mu * __popc(pb.str[ia] & ~pb.str[ib]);
+            pb.diag[h] = v;
+            tri_advance(ia, ib, nt, Ns);
+        }
+        if (tid < (4 - pb.N % 4) % 4) pb.diag[pb.N + tid] = 1.0;
+    }
+    if (B.gemm) {
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) big = fmax(big, __shfl_xor_sync(FULL, big, o));
+        if ((tid & 31) == 0) red[tid >> 5] = big;
+        __syncthreads();
+        B.E = fixed_exponent((tid & 31) < (nt >> 5) ? red[tid & 31] : 0.0);
+        const double scale = pow2(55 - B.E);
+        int2 *Vf = (int2 *)pb.V64, *Hf = (int2 *)pb.Hs64;
+        for (int e = tid; e < P * P; e += nt) Vf[e] = to_fixed(pb.V64[e], scale);
+        for (int e = tid; e < Ns * st; e += nt) {
+            const int I = e / st;
+            const double v = pb.Hs64[e];
+            if (e - I * st == I) hd[I] = v;
+            Hf[e] = e - I * st == I ? make_int2(0, 0) : to_fixed(v, scale);
+        }
+    }
+    __syncthreads();
+}
+
+// Spin-free density matrices of the packed unit vector x and their share of the gradients: the
+// Gram matrix of the vectors E_rs c (see sector_rdm), 32 elements of all of them in shared
+// memory at a time, the entries of the Gram matrix in registers.
+__device__ __noinline__ void block_rdm(const BatchArgs &a, const BlockProblem &B, const double *x, double w)
+{
+    constexpr int GE = 11;  // entries per thread: (n^2 + 1)(n^2 + 2) / 2 of them up to 10 orbitals
+    const Problem &pb = B.pb;
+    const int tid = threadIdx.x, nt = blockDim.x, n = pb.n, n2 = n * n, Ns = pb.Ns, lane = tid & 31;
+    const bool two = a.grad_eri != nullptr;
+    const int first = two ? 0 : n2 * (n2 + 1) / 2, ng = n2 * (n2 + 1) / 2 + n2;  // (without c.c)
+    double *D = (double *)(B.smem + B.S.off_c), *g1 = (double *)(B.smem + B.S.off_g1), *c = B.full;
+    expand_full<double>(pb, x, c, Ns);
+    double gram[GE];
+    int uv[GE];
+#pragma unroll
+    for (int i = 0; i < GE; ++i) {
+        const int q = first + tid + nt * i;
+        int v = (int)((sqrtf(8.f * q + 1.f) - 1.f) * 0.5f);
+        while ((v + 1) * (v + 2) / 2 <= q) ++v;
+        while (v * (v + 1) / 2 > q) --v;
+        uv[i] = q < ng ? v << 8 | (q - v * (v + 1) / 2) : -1;
+        gram[i] = 0.0;
+    }
+    __syncthreads();
+    const uint32_t full = (1u << n) - 1u;
+    int ia = 0, ib = 0;
+    tri_advance(ia, ib, lane, Ns);
+    // <I| E_rs = s <J| with |J> = s E_sr |I>: r occupied in I, s empty or r itself
+    auto entry = [&](int I, uint32_t st, int r, int s) {
+        const int at = __popc(st & ((1u << r) - 1u)) * (n - pb.k + 1) + __popc(~st & full & ((1u << s) - 1u)) + (r < s ? 1 : 0);
+        return pb.tab[I * pb.RS + at];
+    };
+    for (int h0 = 0; h0 < pb.N; h0 += 32) {
+        const bool on = h0 + lane < pb.N;
+        const int i = on ? ia : 0, j = on ? ib : 0;
+        const double wt = !on ? 0.0 : i == j ? 1.0 : 1.4142135623730951;
+        const uint32_t sa = pb.str[i], sb = pb.str[j];
+        for (int rs = tid >> 5; rs <= n2; rs += nt >> 5) {
+            double v = 0.0;
+            if (rs == n2) {
+                v = c[i * Ns + j];
+            } else {
+                const int r = rs / n, s = rs - r * n;
+                if ((sa >> r & 1u) && (r == s || !(sa >> s & 1u))) {
+                    const int q = entry(i, sa, r, s);
+                    v = flip_if(c[entry_J(q) * Ns + j], entry_neg(q));
+                }
+                if ((sb >> r & 1u) && (r == s || !(sb >> s & 1u))) {
+                    const int q = entry(j, sb, r, s);
+                    v += flip_if(c[i * Ns + entry_J(q)], entry_neg(q));
+                }
+            }
+            D[rs * 33 + lane] = wt * v;
+        }
+        __syncthreads();
+#pragma unroll
+        for (int q = 0; q < GE; ++q)
+            if (uv[q] >= 0) {
+                const double *du = D + (uv[q] & 255) * 33, *dv = D + (uv[q] >> 8) * 33;
+                double s = gram[q];
+#pragma unroll 8
+                for (int h = 0; h < 32; ++h) s = fma(du[h], dv[h], s);
+                gram[q] = s;
+            }
+        __syncthreads();
+        tri_advance(ia, ib, 32, Ns);
+    }
+#pragma unroll
+    for (int q = 0; q < GE; ++q)
+        if (uv[q] >= 0 && uv[q] >> 8 == n2) g1[uv[q] & 255] = gram[q];
+    __syncthreads();
+    for (int e = tid; e < n2; e += nt) {
+        const int p = e / n, q = e - p * n;
+        rdm_one_body(a, pb.A, n, p, q, w * (g1[e] - ((p == q && a.occ[pb.A[p]]) ? 2.0 : 0.0)));
+    }
+    if (two)
+#pragma unroll
+        for (int q = 0; q < GE; ++q)
+            if (uv[q] >= 0 && uv[q] >> 8 != n2) rdm_two_body(a, pb.A, n, uv[q] & 255, uv[q] >> 8, gram[q], g1, w);
+    __syncthreads();
+}
+
+__global__ void __launch_bounds__(BLOCK_THREADS, 1) k_casci_block(BatchArgs a, int bucket)
 {
     extern __shared__ __align__(16) char smem[];
-    const int n = a.n, P = n * (n + 1) / 2;
-    const BlockSmem S = block_smem(n, a.rdm == 2);
-    int *A = (int *)(smem + S.off_A);
-    double *red = (double *)(smem + S.off_red);
+    const int n = a.n, P = n * (n + 1) / 2, tid = threadIdx.x, nt = blockDim.x;
     __shared__ unsigned long long s_pos;
     char *slot = a.scratch + (size_t)blockIdx.x * a.slot_bytes;
     const int64_t begin = a.bucket_off[bucket];
     const int64_t cnt = a.bucket_off[bucket + 1] - begin;
+    int *A = (int *)smem;
     for (;;) {
-        if (threadIdx.x == 0) s_pos = atomicAdd(&a.counters[bucket], 1ULL);
+        if (tid == 0) s_pos = atomicAdd(&a.counters[bucket], 1ULL);
         __syncthreads();
-        unsigned long long pos = s_pos;
+        const unsigned long long pos = s_pos;
         __syncthreads();
         if ((int64_t)pos >= cnt) break;
         const int64_t t = a.perm[begin + (int64_t)pos];
-        if (threadIdx.x == 0) build_A(a, t, A);
+        if (tid == 0) build_A(a, t, A);
         __syncthreads();
         int k = 0;
-        for (int i = 0; i < n; ++i) k += a.occ[A[i]];
+        uint32_t mphi = 0;
+        for (int i = 0; i < n; ++i)
+            if (a.occ[A[i]]) {
+                ++k;
+                mphi |= 1u << i;
+            }
         const ClassInfo ci = a.cls[k];
-        Problem pb;
+        const BlockSlot L = block_slot(ci.ns);
+        BlockProblem B;
+        B.smem = smem;
+        B.S = block_mem(n, a.gemm, ci.ns, ci.r, a.rdm);
+        B.gemm = a.gemm;
+        B.E = 0;
+        B.full = (double *)(slot + L.off_full);
+        const BlockMem &S = B.S;
+        Problem &pb = B.pb;
         pb.n = n;
         pb.P = P;
         pb.k = k;
         pb.Ns = ci.ns;
-        pb.N = ci.ns * ci.ns;
+        pb.N = ci.ns * (ci.ns + 1) / 2;
         pb.R = ci.r;
         pb.RS = ci.r;
-        pb.HSS = odd_stride(ci.ns);
+        pb.HSS = hs_stride(ci.ns);
         pb.str = ci.strings;
         pb.tab = ci.table;
         pb.A = A;
         pb.pp = (const short *)(smem + S.off_pp);
         pb.h = (double *)(smem + S.off_h);
-        pb.hp = (double *)(smem + S.off_hp);
+        pb.hp = nullptr;
         pb.V64 = (double *)(smem + S.off_V64);
         pb.V32 = (float *)(smem + S.off_V32);
-        SlotLayout L = slot_layout(ci.ns, pb.N);
         pb.Hs64 = (double *)(slot + L.off_Hs64);
         pb.Hs32 = (float *)(slot + L.off_Hs32);
         pb.diag = (double *)(slot + L.off_diag);
         pb.c = nullptr;
         const bool mixed = a.precision == MBE_PREC_MIXED;
         pb.s2mu = a.s2mu;
-        setup_problem<BlockGroup>(a, pb, mixed);
-        uint32_t mphi = 0;
-        for (int i = 0; i < n; ++i)
-            if (a.occ[A[i]]) mphi |= 1u << i;
-        int iphi = string_rank(mphi);
-        double ephi = pb.diag[iphi * pb.Ns + iphi];
+        block_setup(a, B, ci);
+        const int iphi = string_rank(mphi);
+        const double ephi = pb.diag[iphi * pb.Ns - iphi * (iphi - 1) / 2];
         if (pb.N == 1) {
-            if (threadIdx.x == 0) store_result(a, t, pb.diag[0] - ephi - a.e_ref_corr, MBE_STATUS_OK, 0, 0);
+            if (tid == 0) store_result(a, t, pb.diag[0] - ephi - a.e_ref_corr, MBE_STATUS_OK, 0, 0);
             __syncthreads();
             continue;
         }
+        double *red = (double *)(smem + S.off_red);
         // start vectors: the lowest diagonal element (ties -> lowest index), and for
         // the P = -1 sector the lowest one with Ia != Ib
         double best = 1e300, best_o = 1e300;
         int bi = 0x7fffffff, bj = 0x7fffffff;
-        for (int d = threadIdx.x; d < pb.N; d += blockDim.x) {
-            const double v = pb.diag[d];
-            if (v < best || (v == best && d < bi)) {
-                best = v;
-                bi = d;
-            }
-            const int ia = d / pb.Ns;
-            if (ia != d - ia * pb.Ns && (v < best_o || (v == best_o && d < bj))) {
-                best_o = v;
-                bj = d;
+        {
+            int ia = 0, ib = 0;
+            tri_advance(ia, ib, tid, pb.Ns);
+            for (int d = tid; d < pb.N; d += nt) {
+                const double v = pb.diag[d];
+                if (v < best) {
+                    best = v;
+                    bi = d;
+                }
+                if (ia != ib && v < best_o) {
+                    best_o = v;
+                    bj = d;
+                }
+                tri_advance(ia, ib, nt, pb.Ns);
             }
         }
 #pragma unroll
@@ -93,18 +1159,19 @@ __global__ void __launch_bounds__(CTA_THREADS, 2) k_casci_block(BatchArgs a, int
                 bj = oi;
             }
         }
-        if ((threadIdx.x & 31) == 0) {
-            red[threadIdx.x >> 5] = best;
-            red[32 + (threadIdx.x >> 5)] = best_o;
-            ((int *)(red + 64))[threadIdx.x >> 5] = bi;
-            ((int *)(red + 64))[32 + (threadIdx.x >> 5)] = bj;
+        __syncthreads();
+        if ((tid & 31) == 0) {
+            red[tid >> 5] = best;
+            red[32 + (tid >> 5)] = best_o;
+            ((int *)(red + 64))[tid >> 5] = bi;
+            ((int *)(red + 64))[32 + (tid >> 5)] = bj;
         }
         __syncthreads();
         best = red[0];
         best_o = red[32];
         bi = ((int *)(red + 64))[0];
         bj = ((int *)(red + 64))[32];
-        for (int w = 1; w < (int)(blockDim.x >> 5); ++w) {
+        for (int w = 1; w < (nt >> 5); ++w) {
             double ov = red[w];
             int oi = ((int *)(red + 64))[w];
             if (ov < best || (ov == best && oi < bi)) {
@@ -118,41 +1185,47 @@ __global__ void __launch_bounds__(CTA_THREADS, 2) k_casci_block(BatchArgs a, int
                 bj = oi;
             }
         }
+        // The padding of the vectors (see Pack) is zero, and every operation on packs keeps it
+        // so; the float32 one is also overwritten by float64 vectors in the same place.
+        auto zero_padding = [&](bool f32) {
+            const int pad = f32 ? (4 - pb.N % 4) % 4 : pb.N % 2;
+            for (int q = tid; q < (2 * MMAX + 2) * pad; q += nt) {
+                const int v = q / pad, l = q - v * pad;
+                char *base = slot + (v < MMAX ? L.off_V + v * L.vec : v < 2 * MMAX ? L.off_W + (v - MMAX) * L.vec
+                                                              : v == 2 * MMAX ? L.off_x : L.off_t);
+                if (f32) ((float *)base)[pb.N + l] = 0.f; else ((double *)base)[pb.N + l] = 0.0;
+            }
+        };
+        zero_padding(false);
         __syncthreads();
-        double *x64 = (double *)(slot + L.off_x);
-        double *x2 = (double *)(slot + L.off_x2);
+        double *x64 = (double *)(slot + L.off_x), *x2 = (double *)(slot + L.off_x2);
+        float *x32 = (float *)(slot + L.off_x);
+        double *V64 = (double *)(slot + L.off_V), *W64 = (double *)(slot + L.off_W), *t64 = (double *)(slot + L.off_t);
+        float *V32 = (float *)V64, *W32 = (float *)W64, *t32 = (float *)t64;
         double lam = 0.0;
-        int status = MBE_STATUS_OK, n64 = 0, n32 = 0;
+        int status = MBE_STATUS_OK, n64 = 0, n32 = 0, won = 1;
         bool degen = false;
         // one copy of the sector's Davidson: two inlined copies, both hot on an SM,
         // overflow the instruction cache and slow every phase of every warp
 #pragma unroll 1
         for (int sector = 0; sector < 2; ++sector) {
             if (sector == 1 && (pb.Ns < 2 || status != MBE_STATUS_OK || a.even_only)) break;
-            const SectorGuess sg{sector == 0 ? bi : bj, sector == 0 ? 1 : -1};
+            const int g = sector == 0 ? bi : bj;
             if (sector == 1 && a.rdm)
-                for (int d = threadIdx.x; d < pb.N; d += blockDim.x) x2[d] = x64[d];
-            pb.sector = sg.sgn;
-            for (int d = threadIdx.x; d < pb.N; d += blockDim.x) x64[d] = sector_guess(d, pb.Ns, sg);
+                for (int d = tid; d < pb.N; d += nt) x2[d] = x64[d];
+            pb.sector = sector == 0 ? 1 : -1;
+            if (mixed) zero_padding(true);
             __syncthreads();
             bool lose = false, refined = false;
             if (mixed) {
-                float *x32 = (float *)(slot + L.off_x);
-                // narrow x in place (float view of the same region), bottom up
-                for (int base = 0; base < pb.N; base += blockDim.x) {
-                    int d = base + threadIdx.x;
-                    double v = (d < pb.N) ? x64[d] : 0.0;
-                    __syncthreads();
-                    if (d < pb.N) x32[d] = (float)v;
-                    __syncthreads();
-                }
+                write_guess<float>(pb, g, x32);
+                __syncthreads();
                 // the second sector: a pass to SECTOR_TOL, then one to tol_switch if undecided
                 PhaseOut o32;
                 for (int pass = 0; pass < 1 + sector; ++pass) {
                     const double tl = (sector == 0 || pass == 1) ? a.tol_switch : SECTOR_TOL;
-                    o32 = davidson_block<float>(pb, (float *)(slot + L.off_V), (float *)(slot + L.off_W), L.vec / 4,
-                                                x32, (float *)(slot + L.off_hx), (float *)(slot + L.off_t), smem, S,
-                                                tl, 0, a.max_iter, BLOCK_STALL, 0.0, false, a.block_basis);
+                    o32 = davidson_block<float>(B, V32, W32, L.vec / 4, x32, t32, tl, 0, a.max_iter, BLOCK_STALL, 0.0,
+                                                false, a.block_basis);
                     n32 += o32.nsig;
                     if (sector == 1)
                         lose = o32.status == MBE_STATUS_NONFINITE ||
@@ -166,74 +1239,79 @@ __global__ void __launch_bounds__(CTA_THREADS, 2) k_casci_block(BatchArgs a, int
                     // anchor x0, then the float32 Davidson on H - theta0 with x0 as its
                     // first basis vector; x0 <- x0 + d after each pass, re-anchoring while
                     // the residual stays above tol.
-                    for (int d = threadIdx.x; d < pb.N; d += blockDim.x) x0[d] = (double)x32[d];
+                    for (int d = tid; d < pb.N; d += nt) x0[d] = (double)x32[d];
                     __syncthreads();
-                    float *V0 = (float *)(slot + L.off_V), *W0 = (float *)(slot + L.off_W);
-                    double *s0 = (double *)(slot + L.off_hx);
                     bool done = false, bad = false;
                     double lam_s = 0.0;
                     for (int anc = 0; anc < BLOCK_ANCHORS && !done && !bad; ++anc) {
-                        sigma_block<double>(pb, pb.V64, pb.Hs64, x0, s0);
+                        // (the image over the basis, of which nothing is kept between anchors)
+                        double *s0 = W64 + (MMAX / 2) * (L.vec / 8);
+                        sigma_block<double>(B, x0, s0);
                         ++n64;
                         double q[KRED];
                         q[0] = q[1] = 0.0;
-                        for (int d = threadIdx.x; d < pb.N; d += blockDim.x) {
+                        for (int d = tid; d < pb.N; d += nt) {
                             q[0] += x0[d] * s0[d];
                             q[1] += x0[d] * x0[d];
                         }
-                        block_sum_n<double>(q, 2, red);
+                        block_sums<double>(q, 2, red);
                         const double th = q[0] / q[1], inv = 1.0 / sqrt(q[1]);
-                        for (int d = threadIdx.x; d < pb.N; d += blockDim.x) {
-                            V0[d] = (float)(x0[d] * inv);
-                            W0[d] = (float)((s0[d] - th * x0[d]) * inv);
+                        for (int d = tid; d < pb.N; d += nt) {
+                            V32[d] = (float)(x0[d] * inv);
+                            W32[d] = (float)((s0[d] - th * x0[d]) * inv);
                         }
                         __syncthreads();
-                        PhaseOut o = davidson_block<float>(pb, V0, W0, L.vec / 4, x32, (float *)(slot + L.off_hx),
-                                                           (float *)(slot + L.off_t), smem, S, a.tol, a.min_fp64,
-                                                           a.max_iter, BLOCK_ANCHOR_STALL, th, true, a.block_basis);
+                        zero_padding(true);  // (s0 lay over one W)
+                        __syncthreads();
+                        PhaseOut o = davidson_block<float>(B, V32, W32, L.vec / 4, x32, t32, a.tol, a.min_fp64, a.max_iter,
+                                                           BLOCK_ANCHOR_STALL, th, true, a.block_basis);
                         n32 += o.nsig;
                         lam_s = th + o.lambda;
                         bad = o.status == MBE_STATUS_NONFINITE;
                         done = !bad && o.rnorm <= a.tol && o.dnorm <= MIX_DMAX;
                         if (!bad)
-                            for (int d = threadIdx.x; d < pb.N; d += blockDim.x) x0[d] = x0[d] * inv + (double)x32[d];
+                            for (int d = tid; d < pb.N; d += nt) x0[d] = x0[d] * inv + (double)x32[d];
                         __syncthreads();
                     }
                     // the refined vector (or the start of the float64 fallback) as x64
-                    for (int d = threadIdx.x; d < pb.N; d += blockDim.x)
-                        x64[d] = bad ? sector_guess(d, pb.Ns, sg) : x0[d];
+                    if (bad)
+                        write_guess<double>(pb, g, x64);
+                    else
+                        for (int d = tid; d < pb.N; d += nt) x64[d] = x0[d];
                     __syncthreads();
                     if (done) {
                         refined = true;
                         if (sector == 1) degen = status == MBE_STATUS_OK && fabs(lam_s - lam) <= DEGEN_TOL;
-                        if (sector == 0) {
+                        if (sector == 0 || lam_s < lam) {
                             lam = lam_s;
                             status = MBE_STATUS_OK;
-                        } else if (lam_s < lam) {
-                            lam = lam_s;
-                            status = MBE_STATUS_OK;
+                            won = pb.sector;
                         } else {
                             lose = true;
                         }
                     }
+                } else if (finite) {
+                    for (int d = tid; d < pb.N; d += nt) x0[d] = (double)x32[d];
+                    __syncthreads();
+                    for (int d = tid; d < pb.N; d += nt) x64[d] = x0[d];
+                    __syncthreads();
                 } else {
-                    for (int d = threadIdx.x; d < pb.N; d += blockDim.x)
-                        x64[d] = finite ? (double)x32[d] : sector_guess(d, pb.Ns, sg);
+                    write_guess<double>(pb, g, x64);
                     __syncthreads();
                 }
-            } else if (sector == 1) {
-                PhaseOut o1 = davidson_block<double>(pb, (double *)(slot + L.off_V), (double *)(slot + L.off_W),
-                                                     L.vec / 8, x64, (double *)(slot + L.off_hx),
-                                                     (double *)(slot + L.off_t), smem, S, SECTOR_TOL, 0,
-                                                     a.max_iter, BLOCK_STALL, 0.0, false, a.block_basis);
-                n64 += o1.nsig;
-                lose = o1.status == MBE_STATUS_NONFINITE || sector_loses(o1.lambda, o1.rnorm, lam, 0.0);
+            } else {
+                write_guess<double>(pb, g, x64);
+                __syncthreads();
+                if (sector == 1) {
+                    PhaseOut o1 = davidson_block<double>(B, V64, W64, L.vec / 8, x64, t64, SECTOR_TOL, 0, a.max_iter,
+                                                         BLOCK_STALL, 0.0, false, a.block_basis);
+                    n64 += o1.nsig;
+                    lose = o1.status == MBE_STATUS_NONFINITE || sector_loses(o1.lambda, o1.rnorm, lam, 0.0);
+                }
             }
             if (!lose && !refined) {
-                PhaseOut o64 = davidson_block<double>(pb, (double *)(slot + L.off_V), (double *)(slot + L.off_W),
-                                                      L.vec / 8, x64, (double *)(slot + L.off_hx),
-                                                      (double *)(slot + L.off_t), smem, S, a.tol,
-                                                      mixed ? a.min_fp64 : 0, a.max_iter, 0, 0.0, false, a.block_basis);
+                PhaseOut o64 = davidson_block<double>(B, V64, W64, L.vec / 8, x64, t64, a.tol, mixed ? a.min_fp64 : 0,
+                                                      a.max_iter, 0, 0.0, false, a.block_basis);
                 n64 += o64.nsig;
                 if (sector == 0) {
                     lam = o64.lambda;
@@ -244,53 +1322,61 @@ __global__ void __launch_bounds__(CTA_THREADS, 2) k_casci_block(BatchArgs a, int
                     if (!lose) {
                         lam = o64.lambda;
                         status = o64.status;
+                        won = -1;
                     }
                 }
             }
             if (lose && a.rdm) {
                 __syncthreads();
-                for (int d = threadIdx.x; d < pb.N; d += blockDim.x) x64[d] = x2[d];
+                for (int d = tid; d < pb.N; d += nt) x64[d] = x2[d];
             }
             __syncthreads();
         }
-        if (threadIdx.x == 0) {
+        if (tid == 0) {
             double e = status == MBE_STATUS_NONFINITE ? __longlong_as_double(0x7ff8000000000000LL)
                                                       : lam - ephi - a.e_ref_corr;
             store_result(a, t, e, with_degeneracy(status, degen), n64, n32);
         }
         __syncthreads();
         if (a.rdm) {
-            double *g1 = (double *)(smem + S.off_g1);
-            double *g2 = (a.rdm == 2) ? (double *)(smem + S.off_g2) : nullptr;
-            for (int e = threadIdx.x; e < n * n; e += blockDim.x) g1[e] = 0.0;
-            if (g2)
-                for (int e = threadIdx.x; e < n * n * n * n; e += blockDim.x) g2[e] = 0.0;
-            __syncthreads();
-            rdm_accumulate<BlockGroup>(pb, x64, g1, g2);
-            __syncthreads();
-            rdm_flush<BlockGroup>(a, pb, g1, g2, a.weights ? a.weights[t] : 1.0);
-            __syncthreads();
+            pb.sector = won;
+            block_rdm(a, B, x64, a.weights ? a.weights[t] : 1.0);
         }
     }
 }
 
-int block_grid(mbe_ctx *ctx, int n, bool two_body, int *grid, size_t *smem)
+// Shared memory of a bucket's block launch, and whether its sigma is the tiled product.
+static size_t block_smem_bytes(const mbe_ctx *ctx, int n, const BatchArgs &a, const bool (&in)[MBE_MAX_CAS + 1], int rdm,
+                               int *gemm)
 {
-    BlockSmem S = block_smem(n, two_body);
-    *smem = (size_t)S.bytes;
+    size_t need[2] = {0, 0};
+    for (int k = 0; k <= n; ++k)
+        if (in[k])
+            for (int g = 0; g < 2; ++g)
+                if (g == 0 || n <= GEMM_MAX_N)
+                    need[g] = std::max(need[g], (size_t)block_mem(n, g, a.cls[k].ns, a.cls[k].r, rdm).bytes);
+    *gemm = n <= GEMM_MAX_N && need[1] <= ctx->smem_optin ? 1 : 0;
+    return need[*gemm];
+}
+
+int block_grid(mbe_ctx *ctx, BatchArgs &a, const bool (&in)[MBE_MAX_CAS + 1], int rdm, int *grid, size_t *smem,
+               size_t *slot)
+{
+    *smem = block_smem_bytes(ctx, a.n, a, in, rdm, &a.gemm);
     MBE_CHECK(*smem <= ctx->smem_optin, MBE_EUNSUPPORTED, "casci_batch: block solver needs %zu B shared memory",
               *smem);
     MBE_CU(cudaFuncSetAttribute(k_casci_block, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)*smem));
-    int per_sm = 0;
-    MBE_CU(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_casci_block, CTA_THREADS, *smem));
-    if (per_sm < 1) per_sm = 1;
-    *grid = ctx->sm_count * per_sm;
+    *grid = (int)std::min<int64_t>(ctx->sm_count, a.n_tuples);
+    int ns = 0;
+    for (int k = 0; k <= a.n; ++k)
+        if (in[k]) ns = std::max(ns, a.cls[k].ns);
+    *slot = block_slot(ns).bytes;
     return MBE_OK;
 }
 
 int launch_block(mbe_ctx *ctx, const BatchArgs &a, int b, int grid, size_t smem)
 {
-    k_casci_block<<<grid, CTA_THREADS, smem, ctx->stream>>>(a, b);
+    k_casci_block<<<grid, BLOCK_THREADS, smem, ctx->stream>>>(a, b);
     MBE_CU(cudaGetLastError());
     return MBE_OK;
 }

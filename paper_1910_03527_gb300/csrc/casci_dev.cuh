@@ -84,6 +84,7 @@ struct BatchArgs {
     int32_t *pstate;
     // tuned launch choices (mbe_tuning): warps per warp-solver block, block-solver basis
     int warps, block_basis;
+    int gemm;  // block solver: sigma by the tiled product
     // adjoint (casci_rdm_batch): 0 = energies only, 1 = + 1-RDM, 2 = + 1- and 2-RDM
     int rdm;
     const double *weights;
@@ -686,6 +687,23 @@ __device__ inline void rdm_one_body(const BatchArgs &a, const int *A, int n, int
     atomicAdd(&a.core[pq], gc);
     for (int i = 0; i < n; ++i)
         if (a.occ[A[i]]) atomicAdd(&a.core[(1 + A[i]) * norb * norb + pq], -gc);
+}
+
+// The two-electron gradient's share of one entry, G = <E_qp c|E_rs c> with qp = u, rs = v (and
+// its mirror image), of a tuple's density matrices: w / 2 (<E_pq E_rs> - d_qr gamma_ps - Phi's).
+__device__ inline void rdm_two_body(const BatchArgs &a, const int *A, int n, int u, int v, double G, const double *g1,
+                                    double w)
+{
+    for (int side = 0; side < (u == v ? 1 : 2); ++side) {
+        const int qp = side ? v : u, rs = side ? u : v;
+        const int q = qp / n, p = qp - q * n, r = rs / n, s = rs - r * n;
+        const bool op = a.occ[A[p]], oq = a.occ[A[q]], orr = a.occ[A[r]];
+        double phi = 0.0;
+        if (p == q && r == s && op && orr) phi += (p == r) ? 2.0 : 4.0;
+        if (p == s && q == r && p != q && op && oq) phi -= 2.0;
+        const double val = 0.5 * w * (G - (q == r ? g1[p * n + s] : 0.0) - phi);
+        if (val != 0.0) atomicAdd(&a.grad_eri[eri_index(a.norb, A[p], A[q], A[r], A[s])], val);
+    }
 }
 
 // Adds w * (dE_CAS(A)/dtheta - dE_Phi/dtheta) to the gradients from the active
@@ -1789,33 +1807,6 @@ constexpr int BLOCK_STALL = 3;
 constexpr int BLOCK_ANCHOR_STALL = 25;
 constexpr int BLOCK_ANCHORS = 8;
 
-// Per-block workspace slot: the Davidson basis V, its image W = H V, the Ritz
-// vector x and H x, a spare correction vector, the diagonal and Hs.
-struct SlotLayout {
-    size_t off_V, off_W, off_x, off_hx, off_t, off_diag, off_Hs64, off_Hs32, off_x2, off_x0, vec, bytes;
-};
-
-__host__ __device__ inline SlotLayout slot_layout(int ns, int N)
-{
-    SlotLayout L;
-    size_t o = 0;
-    size_t vec = ((size_t)N * 8 + 255) & ~(size_t)255;
-    int HSS = odd_stride(ns);
-    L.vec = vec;
-    L.off_V = o; o += vec * MMAX;
-    L.off_W = o; o += vec * MMAX;
-    L.off_x = o; o += vec;
-    L.off_hx = o; o += vec;
-    L.off_t = o; o += vec;
-    L.off_diag = o; o += vec;
-    L.off_Hs64 = o; o += ((size_t)ns * HSS * 8 + 255) & ~(size_t)255;
-    L.off_Hs32 = o; o += ((size_t)ns * HSS * 4 + 255) & ~(size_t)255;
-    L.off_x2 = o; o += vec;
-    L.off_x0 = o; o += vec;  // float64 anchor of the mixed refinement
-    L.bytes = o;
-    return L;
-}
-
 struct BlockSmem {  // dynamic shared memory of the block solver
     int off_A, off_pp, off_h, off_hp, off_V64, off_V32, off_red, off_G, off_A32, off_E32, off_ev, off_y,
         off_yp, off_r, off_misc, off_g1, off_g2, bytes;
@@ -1844,31 +1835,6 @@ __host__ __device__ inline BlockSmem block_smem(int n, bool two_body = false)
     S.off_g2 = o; o = al16(o + (two_body ? 8 * n * n * n * n : 0));
     S.bytes = o;
     return S;
-}
-
-// Sums of the first k of the values v[0..KRED) over the block; every thread gets
-// the totals.  red: >= 32 * KRED elements of T.
-template <typename T>
-__device__ inline void block_sum_n(T (&v)[KRED], int k, T *red)
-{
-    int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
-#pragma unroll
-    for (int i = 0; i < KRED; ++i)
-        if (i < k) v[i] = warp_sum(v[i]);
-    __syncthreads();
-    if (lane == 0)
-#pragma unroll
-        for (int i = 0; i < KRED; ++i)
-            if (i < k) red[w * KRED + i] = v[i];
-    __syncthreads();
-#pragma unroll
-    for (int i = 0; i < KRED; ++i)
-        if (i < k) {
-            T s = 0;
-            for (int j = 0; j < nw; ++j) s += red[j * KRED + i];
-            v[i] = s;
-        }
-    __syncthreads();
 }
 
 // Lowest eigenpair of the m x m symmetric Rayleigh matrix G (shared memory,
@@ -2001,331 +1967,6 @@ __device__ void small_eig_warp(const double *G, int m, float *A, float *E, float
     __syncwarp();
 }
 
-// One Davidson phase in precision T (block solver).  x: start vector in, Ritz
-// vector out.  V, W: MMAX vectors each, leading dimension ld (elements).
-// Block-wide sigma of a vector of one spin-flip sector: the elements with
-// Ia <= Ib are computed and mirrored (see sigma_warp); ends with a barrier.
-template <typename T>
-__device__ inline void sigma_block(const Problem &pb, const T *Vi, const T *Hs, const T *src, T *dst)
-{
-    const int Ns = pb.Ns, nh = Ns * (Ns + 1) / 2;
-    int ia = 0, ib = 0;
-    tri_advance(ia, ib, threadIdx.x, Ns);
-    for (int h = threadIdx.x; h < nh; h += blockDim.x) {
-        const int d = ia * Ns + ib, pd = ib * Ns + ia;
-        T v = (T)0;
-        if (!(pb.sector < 0 && ia == ib)) {
-            if constexpr (sizeof(T) == 4) v = sigma_elem_ashared<T>(pb, Vi, Hs, src, ia, ib);
-            else v = sigma_elem<T>(pb, Vi, Hs, src, d);
-        }
-        dst[d] = v;
-        if (pd != d) dst[pd] = pb.sector > 0 ? v : -v;
-        tri_advance(ia, ib, blockDim.x, Ns);
-    }
-    if (pb.s2mu != 0.0) add_s2_half<T, T>(pb, src, dst, threadIdx.x, blockDim.x);
-    __syncthreads();
-}
-
-// Plain: x is the start vector in, the unit Ritz vector out.  Anchored (T =
-// float, anch): V[0] = x0 and W[0] = r0 = (H - shift) x0 are given (see struct
-// Anchor), every other basis vector is a correction whose image is the float32
-// sigma minus shift times it, the Ritz value is that of H - shift, the coupling
-// of x0 to a vector v is formed as v.r0, a thick restart keeps x0 and the
-// corrections of the two lowest Ritz vectors, and x returns the correction d of
-// the Ritz vector x0 + d.  steer: iterations without a 10% residual drop that end
-// the phase (0: none).
-template <typename T>
-__device__ __noinline__ PhaseOut davidson_block(const Problem &pb, T *V, T *W, size_t ld, T *x, T *hx, T *tx, char *smem,
-                                   const BlockSmem &S, double tol, int min_iter, int max_iter, int steer,
-                                   double shift = 0.0, bool anch = false, int mmax = MMAX)
-{
-    const int tid = threadIdx.x, nt = blockDim.x, N = pb.N;
-    const T *Vi = sizeof(T) == 8 ? (const T *)pb.V64 : (const T *)pb.V32;
-    const T *Hs = sizeof(T) == 8 ? (const T *)pb.Hs64 : (const T *)pb.Hs32;
-    T *red = (T *)(smem + S.off_red);
-    double *G = (double *)(smem + S.off_G);
-    float *A32 = (float *)(smem + S.off_A32);
-    float *E32 = (float *)(smem + S.off_E32);
-    float *ev = (float *)(smem + S.off_ev);
-    double *ys = (double *)(smem + S.off_y);
-    double *y2s = (double *)(smem + S.off_yp);
-    double *rs = (double *)(smem + S.off_r);
-    double *misc = (double *)(smem + S.off_misc);
-    PhaseOut o;
-    o.nsig = 0;
-    o.status = MBE_STATUS_OK;
-    o.dnorm = 0.0;
-    const T shT = (T)shift, shT_lo = (T)(shift - (double)shT);
-    T v[KRED];
-    if (!anch) {
-        v[0] = 0;
-        for (int d = tid; d < N; d += nt) v[0] += x[d] * x[d];
-        block_sum_n<T>(v, 1, red);
-        T inv = (T)1 / sqrt(v[0]);
-        for (int d = tid; d < N; d += nt) V[d] = x[d] * inv;
-        __syncthreads();
-        sigma_block<T>(pb, Vi, Hs, V, W);
-        ++o.nsig;
-        v[0] = 0;
-        for (int d = tid; d < N; d += nt) v[0] += V[d] * W[d];
-        block_sum_n<T>(v, 1, red);
-        if (tid == 0) G[0] = (double)v[0];
-    } else if (tid == 0) {
-        G[0] = 0.0;  // x0.r0 = 0: shift is x0's Rayleigh quotient
-    }
-    __syncthreads();
-    int m = 1;
-    double theta = 0.0;
-    T rn = 0;
-    T best = (T)3e38;
-    int stall = 0;
-    for (int it = 0;; ++it) {
-        if (tid < 32) small_eig_warp<sizeof(T) == 8>(G, m, A32, E32, ev, ys, y2s, rs, misc);
-        __syncthreads();
-        theta = misc[0];
-        const T th = (T)theta;
-        T *tdst = (m < mmax) ? V + (size_t)m * ld : tx;
-        v[0] = 0;
-        v[1] = 0;
-        for (int d = tid; d < N; d += nt) {
-            T xs = 0, hs = 0;
-            for (int i = 0; i < m; ++i) {
-                T yi = (T)ys[i];
-                xs += yi * V[(size_t)i * ld + d];
-                hs += yi * W[(size_t)i * ld + d];
-            }
-            x[d] = xs;
-            hx[d] = hs;
-            T r = hs - th * xs;
-            v[0] += r * r;
-            const int pd = flip_det(d, pb.Ns);
-            T den = (T)(pb.diag[d < pd ? d : pd] - shift) - th;
-            if (fabs(den) < (T)1e-4) den = den >= (T)0 ? (T)1e-4 : (T)-1e-4;
-            const T td = r / den;
-            tdst[d] = td;
-            v[1] += td * td;
-        }
-        block_sum_n<T>(v, 2, red);
-        rn = sqrt(v[0]);
-        const T t0n = sqrt(v[1]);
-        if (!isfinite(rn) || !isfinite(theta)) {
-            o.status = MBE_STATUS_NONFINITE;
-            break;
-        }
-        if (rn <= (T)tol && it >= min_iter) break;
-        if (it >= max_iter) {
-            o.status = MBE_STATUS_MAXITER;
-            break;
-        }
-        if (steer) {
-            if (rn < (T)0.9 * best) {
-                best = rn;
-                stall = 0;
-            } else if (++stall >= steer) {
-                break;
-            }
-        }
-        if (m == mmax && anch) {
-            // Thick restart that keeps the anchor: V[0] = x0, W[0] = r0 stay; V[1], V[2]
-            // become the corrections of the two lowest Ritz vectors (both orthogonal
-            // to x0), orthonormalised.
-            for (int d = tid; d < N; d += nt) {
-                T u1 = 0, w1 = 0, u2 = 0, w2 = 0;
-                for (int i = 1; i < mmax; ++i) {
-                    const T vi = V[(size_t)i * ld + d], wi = W[(size_t)i * ld + d];
-                    u1 += (T)ys[i] * vi;
-                    w1 += (T)ys[i] * wi;
-                    u2 += (T)y2s[i] * vi;
-                    w2 += (T)y2s[i] * wi;
-                }
-                V[ld + d] = u1;
-                W[ld + d] = w1;
-                V[2 * ld + d] = u2;
-                W[2 * ld + d] = w2;
-            }
-            __syncthreads();
-            v[0] = 0;
-            for (int d = tid; d < N; d += nt) v[0] += V[ld + d] * V[ld + d];
-            block_sum_n<T>(v, 1, red);
-            const T i1 = (T)1 / sqrt(v[0]);
-            for (int d = tid; d < N; d += nt) {
-                V[ld + d] *= i1;
-                W[ld + d] *= i1;
-            }
-            __syncthreads();
-            for (int pass = 0; pass < 2; ++pass) {
-                v[0] = 0;
-                for (int d = tid; d < N; d += nt) v[0] += V[ld + d] * V[2 * ld + d];
-                block_sum_n<T>(v, 1, red);
-                for (int d = tid; d < N; d += nt) {
-                    V[2 * ld + d] -= v[0] * V[ld + d];
-                    W[2 * ld + d] -= v[0] * W[ld + d];
-                }
-            }
-            v[0] = 0;
-            for (int d = tid; d < N; d += nt) v[0] += V[2 * ld + d] * V[2 * ld + d];
-            block_sum_n<T>(v, 1, red);
-            int mnew = 2;
-            const T n2 = sqrt(v[0]);
-            if (n2 > (T)1e-3) {
-                const T i2 = (T)1 / n2;
-                for (int d = tid; d < N; d += nt) {
-                    V[2 * ld + d] *= i2;
-                    W[2 * ld + d] *= i2;
-                }
-                mnew = 3;
-            }
-            __syncthreads();
-            v[0] = v[1] = v[2] = v[3] = v[4] = 0;
-            for (int d = tid; d < N; d += nt) {
-                v[0] += W[d] * V[ld + d];  // x0.(A u1) as u1.r0
-                v[1] += V[ld + d] * W[ld + d];
-                if (mnew == 3) {
-                    v[2] += W[d] * V[2 * ld + d];
-                    v[3] += V[ld + d] * W[2 * ld + d];
-                    v[4] += V[2 * ld + d] * W[2 * ld + d];
-                }
-            }
-            block_sum_n<T>(v, 5, red);
-            if (tid == 0) {
-                G[1] = G[MMAX] = (double)v[0];
-                G[MMAX + 1] = (double)v[1];
-                if (mnew == 3) {
-                    G[2] = G[2 * MMAX] = (double)v[2];
-                    G[MMAX + 2] = G[2 * MMAX + 1] = (double)v[3];
-                    G[2 * MMAX + 2] = (double)v[4];
-                }
-            }
-            m = mnew;
-        } else if (m == mmax) {
-            // Thick restart on the two lowest Ritz vectors of the current basis
-            // (orthogonal by construction, so W stays consistent with H V).
-            for (int d = tid; d < N; d += nt) {
-                T x2 = 0, hx2 = 0;
-                for (int i = 0; i < mmax; ++i) {
-                    T yi = (T)y2s[i];
-                    x2 += yi * V[(size_t)i * ld + d];
-                    hx2 += yi * W[(size_t)i * ld + d];
-                }
-                V[d] = x[d];
-                W[d] = hx[d];
-                V[ld + d] = x2;
-                W[ld + d] = hx2;
-            }
-            __syncthreads();
-            for (int pass = 0; pass < 2; ++pass) {
-                v[0] = 0;
-                for (int d = tid; d < N; d += nt) v[0] += V[d] * V[ld + d];
-                block_sum_n<T>(v, 1, red);
-                for (int d = tid; d < N; d += nt) {
-                    V[ld + d] -= v[0] * V[d];
-                    W[ld + d] -= v[0] * W[d];
-                }
-            }
-            v[0] = 0;
-            for (int d = tid; d < N; d += nt) v[0] += V[ld + d] * V[ld + d];
-            block_sum_n<T>(v, 1, red);
-            int mnew = 1;
-            T nn = sqrt(v[0]);
-            if (nn > (T)0.5) {
-                T inv = (T)1 / nn;
-                for (int d = tid; d < N; d += nt) {
-                    V[ld + d] *= inv;
-                    W[ld + d] *= inv;
-                }
-                mnew = 2;
-            }
-            v[0] = v[1] = v[2] = 0;
-            for (int d = tid; d < N; d += nt) {
-                v[0] += V[d] * W[d];
-                if (mnew == 2) {
-                    v[1] += V[d] * W[ld + d];
-                    v[2] += V[ld + d] * W[ld + d];
-                }
-            }
-            block_sum_n<T>(v, 3, red);
-            if (tid == 0) {
-                G[0] = (double)v[0];
-                if (mnew == 2) {
-                    G[1] = G[MMAX] = (double)v[1];
-                    G[MMAX + 1] = (double)v[2];
-                }
-            }
-            m = mnew;
-        }
-        // Correction: orthogonalise against V[0..m) twice, into V[m].
-        T *tv = V + (size_t)m * ld;
-        const T *tsrc = (tdst == tx) ? tx : tv;
-        for (int pass = 0; pass < 2; ++pass) {
-#pragma unroll
-            for (int i = 0; i < KRED; ++i) v[i] = 0;
-            for (int d = tid; d < N; d += nt) {
-                T td = (pass == 0) ? tsrc[d] : tv[d];
-#pragma unroll
-                for (int i = 0; i < MMAX; ++i)
-                    if (i < m) v[i] += V[(size_t)i * ld + d] * td;
-            }
-            block_sum_n<T>(v, m, red);
-            for (int d = tid; d < N; d += nt) {
-                T td = (pass == 0) ? tsrc[d] : tv[d];
-#pragma unroll
-                for (int i = 0; i < MMAX; ++i)
-                    if (i < m) td -= v[i] * V[(size_t)i * ld + d];
-                tv[d] = td;
-            }
-        }
-        v[0] = 0;
-        for (int d = tid; d < N; d += nt) v[0] += tv[d] * tv[d];
-        block_sum_n<T>(v, 1, red);
-        T tn = sqrt(v[0]);
-        if (!(tn > (T)1e-12 * t0n) || !(tn > (T)0)) {
-            // The correction lies in the current basis: nothing left to add.
-            if (!steer && rn > (T)tol) o.status = MBE_STATUS_MAXITER;
-            break;
-        }
-        T tinv = (T)1 / tn;
-        for (int d = tid; d < N; d += nt) tv[d] *= tinv;
-        __syncthreads();
-        T *wv = W + (size_t)m * ld;
-        sigma_block<T>(pb, Vi, Hs, tv, wv);
-        ++o.nsig;
-#pragma unroll
-        for (int i = 0; i < KRED; ++i) v[i] = 0;
-        for (int d = tid; d < N; d += nt) {
-            T wd = wv[d];
-            if (anch) {
-                wd = (wd - shT * tv[d]) - shT_lo * tv[d];
-                wv[d] = wd;
-            }
-#pragma unroll
-            for (int i = 0; i < MMAX + 1; ++i)
-                if (i <= m) v[i] += (anch && i == 0) ? W[d] * tv[d] : V[(size_t)i * ld + d] * wd;
-        }
-        block_sum_n<T>(v, m + 1, red);
-        if (tid == 0)
-            for (int i = 0; i <= m; ++i) G[i * MMAX + m] = G[m * MMAX + i] = (double)v[i];
-        __syncthreads();
-        ++m;
-    }
-    if (anch) {
-        // the correction d of the Ritz vector, scaled so that x0 keeps coefficient 1
-        const T inv0 = (T)(1.0 / ys[0]);
-        v[0] = 0;
-        for (int d = tid; d < N; d += nt) {
-            T u = 0;
-            for (int i = 1; i < MMAX; ++i)
-                if (i < m) u += (T)ys[i] * V[(size_t)i * ld + d];
-            x[d] = u * inv0;
-            v[0] += x[d] * x[d];
-        }
-        block_sum_n<T>(v, 1, red);
-        o.dnorm = (double)sqrt(v[0]);
-    }
-    o.lambda = theta;
-    o.rnorm = (double)rn;
-    return o;
-}
-
 // Optional event pair around one solver launch (mbe_ctx_set_timing).
 struct TimedLaunch {
     mbe_ctx *ctx;
@@ -2379,7 +2020,8 @@ int launch_sector_mixed(mbe_ctx *ctx, const BatchArgs &a, int b, int k);        
 int launch_sector64(mbe_ctx *ctx, const BatchArgs &a, int b, int k);                     // casci_sector64.cu
 int launch_sector64_redo(mbe_ctx *ctx, const BatchArgs &a, int b, int k);                // casci_sector64_redo.cu
 int launch_warp_mixed_dpl(mbe_ctx *ctx, const BatchArgs &a, int b, const MixLayout &L, int dpl);  // casci_mixed.cu
-int block_grid(mbe_ctx *ctx, int n, bool two_body, int *grid, size_t *smem);             // casci_block.cu
+int block_grid(mbe_ctx *ctx, BatchArgs &a, const bool (&in)[MBE_MAX_CAS + 1], int rdm, int *grid, size_t *smem,
+               size_t *slot);                                                            // casci_block.cu
 int launch_block(mbe_ctx *ctx, const BatchArgs &a, int b, int grid, size_t smem);        // casci_block.cu
 __global__ void k_core_fock(int norb, const double *h1, const double *eri, const uint8_t *occ, double *F);
 

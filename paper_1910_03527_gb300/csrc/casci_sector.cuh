@@ -139,11 +139,11 @@ __device__ void build_tables(SectorTables<C> &T, const ClassInfo &ci)
 // ------------------------------------------------------------------ per-tuple set-up
 
 // One element of the one-spin string Hamiltonian by the Slater-Condon rules, from
-// h_eff over packed pairs and V over packed pairs of pairs: at most 2k - 1 additions per
-// element, where multiplying out sum E_pq E_rs takes R^2 per column.
-__host__ __device__ inline double string_element(uint32_t I, uint32_t J, const double *h, const double *Vp)
+// h(p, q) and V(p, q, r, s) = (pq|rs): at most k^2 additions, where multiplying out
+// sum E_pq E_rs takes R^2 per column.
+template <class H, class VF>
+__host__ __device__ inline double string_element(uint32_t I, uint32_t J, H h, VF V)
 {
-    auto V = [&](int p, int q, int r, int s) { return Vp[tri_index(pair_index(p, q), pair_index(r, s))]; };
     auto low = [](uint32_t s) {
         int b = 0;
 #ifdef __CUDA_ARCH__
@@ -167,7 +167,7 @@ __host__ __device__ inline double string_element(uint32_t I, uint32_t J, const d
     if (from == 0u) {
         for (uint32_t a = I; a; a &= a - 1u) {
             const int p = low(a);
-            v += h[pair_index(p, p)];
+            v += h(p, p);
             for (uint32_t b = a & (a - 1u); b; b &= b - 1u) {
                 const int q = low(b);
                 v += V(p, p, q, q) - V(p, q, p, q);
@@ -180,7 +180,7 @@ __host__ __device__ inline double string_element(uint32_t I, uint32_t J, const d
     to &= to - 1u;
     int neg = odd(I & between(p, a));
     if (from == 0u) {
-        v = h[pair_index(p, a)];
+        v = h(p, a);
         for (uint32_t c = I & J; c; c &= c - 1u) {
             const int r = low(c);
             v += V(p, a, r, r) - V(p, r, r, a);
@@ -258,10 +258,12 @@ __device__ SectorStart sector_setup(const BatchArgs &a, const SectorTables<C> &T
         dsum[e] = v;
     }
     __syncwarp();
+    auto hf = [&](int p, int q) { return h[pair_index(p, q)]; };
+    auto Vf = [&](int p, int q, int r, int s) { return Vp[tri_index(pair_index(p, q), pair_index(r, s))]; };
 #pragma unroll 1
     for (int e = lane; e < C::NH; e += 32) {
         const uchar2 ij = T.tri[e];
-        const double v = string_element(T.str[ij.x], T.str[ij.y], h, Vp);
+        const double v = string_element(T.str[ij.x], T.str[ij.y], hf, Vf);
         Hsp[e] = v;
         if (ij.x == ij.y) hd[ij.x] = v;
     }

@@ -341,7 +341,7 @@ __device__ __noinline__ void sector_rdm(const BatchArgs &a, const SectorTables<C
                                         const double (&x)[C::DH], double w)
 {
     constexpr int n = C::n, n2 = n * n, NV = n2 + 1, NG = NV * (NV + 1) / 2, GE = (NG + 31) / 32;
-    const int lane = threadIdx.x & 31, norb = a.norb;
+    const int lane = threadIdx.x & 31;
     double *D = W.m.r.D, *c = W.c.c;
 #pragma unroll
     for (int j = 0; j < C::DH; ++j) {
@@ -425,17 +425,7 @@ __device__ __noinline__ void sector_rdm(const BatchArgs &a, const SectorTables<C
         v -= v * (v + 1) / 2 > g ? 1 : 0;
         const int u = g - v * (v + 1) / 2;
         if (v >= n2 || u >= n2) continue;
-        for (int side = 0; side < (u == v ? 1 : 2); ++side) {
-            const int qp = side ? v : u, rs = side ? u : v;
-            const int q = qp / n, p = qp - q * n, r = rs / n, s = rs - r * n;
-            const double G = gram[i] - (q == r ? g1[p * n + s] : 0.0);
-            const bool op = a.occ[A[p]], oq = a.occ[A[q]], orr = a.occ[A[r]];
-            double phi = 0.0;
-            if (p == q && r == s && op && orr) phi += (p == r) ? 2.0 : 4.0;
-            if (p == s && q == r && p != q && op && oq) phi -= 2.0;
-            const double val = 0.5 * w * (G - phi);
-            if (val != 0.0) atomicAdd(&a.grad_eri[eri_index(norb, A[p], A[q], A[r], A[s])], val);
-        }
+        rdm_two_body(a, A, n, u, v, gram[i], g1, w);
     }
     __syncwarp();
 }

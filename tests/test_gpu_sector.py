@@ -1,0 +1,117 @@
+"""The sector solvers (tuples of 2-6 orbitals) and the block solver's tiled sigma.
+
+Every string class (n, k) of the sector solvers, and classes of 7-10 orbitals of
+the block solver on both sides of the size where its sigma changes form, against
+the oracle on random Hamiltonians, whose ground states lie in either spin-flip
+sector; the integrals also scaled up and down, since the float64 sigma is formed
+in fixed point with a scale taken from them.
+"""
+
+import itertools
+
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+
+pytestmark = pytest.mark.gpu
+
+from oracle import adjoint as oad  # noqa: E402
+from oracle import mbe as omb  # noqa: E402
+from workloads import random_system  # noqa: E402
+
+TOL = {"fp64": 1e-9, "mixed": 1e-8}  # E_h at integrals of order one; relative to their scale below
+
+
+@pytest.fixture(scope="module")
+def eng():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import paper_1910_03527_gb300 as e
+    e.build()
+    return e
+
+
+@pytest.fixture(scope="module")
+def ctx(eng):
+    c = eng.Context(0)
+    yield c
+    c.close()
+
+
+def dev(a):
+    return torch.tensor(np.ascontiguousarray(a), device="cuda")
+
+
+def _tuples(n, k, nocc, norb, count, rng):
+    """`count` tuples of n orbitals, k of them occupied."""
+    occ = list(itertools.combinations(range(nocc), k))
+    vir = list(itertools.combinations(range(nocc, norb), n - k))
+    got = {occ[rng.integers(len(occ))] + vir[rng.integers(len(vir))] for _ in range(4 * count)}
+    return sorted(got)[:count]
+
+
+def _check(eng, ctx, h1, eri, occ, tuples, prec, scale):
+    n = len(tuples[0])
+    opts = eng.Opts(precision=prec, tol=1e-7 * scale, tol_switch=1e-5 * scale)
+    eps, st, _ = ctx.casci_batch(dev(h1), dev(eri), dev(occ), [], 0.0, n, dev(np.array(tuples, dtype=np.int32)), opts)
+    e_phi = omb.phi_energy(h1, eri, occ)
+    want = np.array([omb.tuple_energy(h1, eri, occ, [], t, e_phi, 0.0) for t in tuples])
+    assert np.isin(st.cpu().numpy(), (0, 4)).all()
+    assert np.abs(eps.cpu().numpy() - want).max() <= TOL[prec] * scale
+
+
+@pytest.mark.parametrize("prec", ["fp64", "mixed"])
+@pytest.mark.parametrize("n,k", [(n, k) for n in range(2, 7) for k in range(1, n)])
+def test_sector_classes(eng, ctx, n, k, prec):
+    rng = np.random.default_rng(100 * n + k)
+    h1, eri, occ = random_system(12, 6, seed=10 * n + k, eri_scale=0.8)
+    _check(eng, ctx, h1, eri, occ, _tuples(n, k, 6, 12, 7, rng), prec, 1.0)
+
+
+@pytest.mark.parametrize("prec", ["fp64", "mixed"])
+@pytest.mark.parametrize("scale", [0.1, 37.0, 4096.0])
+@pytest.mark.parametrize("n,k", [(4, 2), (6, 3), (7, 3)])
+def test_scaled_integrals(eng, ctx, n, k, scale, prec):
+    rng = np.random.default_rng(5)
+    h1, eri, occ = random_system(12, 6, seed=3)
+    _check(eng, ctx, scale * h1, scale * eri, occ, _tuples(n, k, 6, 12, 4, rng), prec, scale)
+
+
+@pytest.mark.parametrize("prec", ["fp64", "mixed"])
+@pytest.mark.parametrize("n,k,count", [(7, 2, 5), (7, 3, 5), (7, 5, 5), (8, 3, 3), (8, 4, 3), (8, 6, 3), (9, 2, 3),
+                                       (9, 4, 1), (9, 7, 3), (10, 2, 3), (10, 8, 3)])
+def test_block_classes(eng, ctx, n, k, count, prec):
+    rng = np.random.default_rng(100 * n + k)
+    h1, eri, occ = random_system(18, 9, seed=10 * n + k, eri_scale=0.5)
+    _check(eng, ctx, h1, eri, occ, _tuples(n, k, 9, 18, count, rng), prec, 1.0)
+
+
+@pytest.mark.parametrize("prec", ["fp64", "mixed"])
+@pytest.mark.parametrize("n", [2, 4, 5, 6, 7])
+def test_density_matrices(eng, ctx, n, prec):
+    """Gradients of single tuples of every class against the oracle's density matrices."""
+    h1, eri, occ = random_system(9, 4, seed=n, eri_scale=0.3)
+    for k in range(max(1, n - 5), min(n, 5)):
+        t = tuple(range(4 - k, 4)) + tuple(range(4, 4 + n - k))
+        gh = torch.zeros((9, 9), dtype=torch.float64, device="cuda")
+        ge = torch.zeros((9,) * 4, dtype=torch.float64, device="cuda")
+        st = ctx.casci_rdm_batch(dev(h1), dev(eri), dev(occ), [], n, dev(np.array([t], dtype=np.int32)), None, gh, ge,
+                                 eng.Opts(precision=prec, tol=1e-10))
+        assert int(st[0]) == 0
+        _, wh, we = oad.cas_gradient(h1, eri, occ, list(t))
+        _, ph, pe = oad.cas_gradient(h1, eri, occ, [])
+        # (first order in the residual, 1e-10, over a gap of a few tenths)
+        assert np.abs(gh.cpu().numpy() - (wh - ph)).max() <= 1e-8
+        assert np.abs(ge.cpu().numpy() - (we - pe)).max() <= 1e-8
+
+
+def test_integrals_that_are_not_finite(eng, ctx):
+    h1, eri, occ = random_system(12, 6, seed=3)
+    for n, t in ((4, (4, 5, 6, 7)), (6, (3, 4, 5, 6, 7, 8)), (7, (3, 4, 5, 6, 7, 8, 9))):
+        bad = eri.copy()
+        bad[6, 6, 6, 6] = np.nan
+        for prec in ("fp64", "mixed"):
+            eps, st, _ = ctx.casci_batch(dev(h1), dev(bad), dev(occ), [], 0.0, n, dev(np.array([t], dtype=np.int32)),
+                                         eng.Opts(precision=prec))
+            assert int(st[0]) == 2 and np.isnan(float(eps[0]))
