@@ -487,6 +487,10 @@ __device__ inline void rotate3(float (&A)[3][3], float (&Vv)[3][3], int p, int q
     }
 }
 
+// Out of line: each float64 division and square root is a few hundred bytes of code.
+static __device__ __noinline__ double div64(double a, double b) { return a / b; }
+static __device__ __noinline__ double inv_sqrt64(double a) { return 1.0 / sqrt(a); }
+
 template <typename T>
 __device__ inline void eig3(const T (&G)[3][3], bool have_p, T (&y)[3])
 {
@@ -505,6 +509,7 @@ __device__ inline void eig3(const T (&G)[3][3], bool have_p, T (&y)[3])
         rotate3(A, Vv, 0, 2);
         A[1][1] = 3.0e38f;
     } else {
+#pragma unroll 1
         for (int sweep = 0; sweep < 6; ++sweep) {
             float off = fabsf(A[0][1]) + fabsf(A[0][2]) + fabsf(A[1][2]);
             float dia = fabsf(A[0][0]) + fabsf(A[1][1]) + fabsf(A[2][2]);
@@ -538,7 +543,7 @@ __device__ inline void eig3(const T (&G)[3][3], bool have_p, T (&y)[3])
         for (int i = 0; i < 3; ++i)
 #pragma unroll
             for (int j = 0; j < 3; ++j) th += y[i] * Gm[i][j] * y[j];
-        th /= nrm;
+        th = div64(th, nrm);
         T M[3][3];
 #pragma unroll
         for (int i = 0; i < 3; ++i)
@@ -559,12 +564,12 @@ __device__ inline void eig3(const T (&G)[3][3], bool have_p, T (&y)[3])
         for (int i = 0; i < 3; ++i) z[i] = adj[i][0] * y[0] + adj[i][1] * y[1] + adj[i][2] * y[2];
         T zz = z[0] * z[0] + z[1] * z[1] + z[2] * z[2];
         if (zz > (T)1e-280 && isfinite(zz)) {
-            T inv = (T)1 / sqrt(zz);
+            T inv = inv_sqrt64(zz);
             T sgn = (z[0] * y[0] + z[1] * y[1] + z[2] * y[2]) < (T)0 ? -inv : inv;
 #pragma unroll
             for (int i = 0; i < 3; ++i) y[i] = z[i] * sgn;
         } else {
-            T inv = (T)1 / sqrt(nrm);
+            T inv = inv_sqrt64(nrm);
 #pragma unroll
             for (int i = 0; i < 3; ++i) y[i] *= inv;
         }

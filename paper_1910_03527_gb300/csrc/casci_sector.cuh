@@ -102,6 +102,16 @@ __device__ __forceinline__ void static_for(F f)
     static_for_(f, std::make_integer_sequence<int, COUNT>{});
 }
 
+// v, hidden from the optimiser.  A condition that never changes inside the Davidson loop
+// (plain or anchored, the sector's sign) makes the compiler write one copy of the loop for each
+// of its values, sigma included; on an SM all copies are hot, and the instruction cache is what
+// these kernels wait for.
+__device__ __forceinline__ int opaque(int v)
+{
+    asm volatile("" : "+r"(v));
+    return v;
+}
+
 // ------------------------------------------------------------------ block-wide tables
 
 // Tables of the class, built once per block: the replacement lists (J << 8 | pair << 1
@@ -119,18 +129,23 @@ struct SectorTables {
 template <class C>
 __device__ void build_tables(SectorTables<C> &T, const ClassInfo &ci)
 {
+#pragma unroll 1
     for (int i = threadIdx.x; i < C::NS * C::R; i += blockDim.x) {
         const int e = ci.table[i];
         T.list[i] = (uint16_t)(entry_J(e) << 8 | (e & 0xff));
     }
+#pragma unroll 1
     for (int i = threadIdx.x; i < C::NS; i += blockDim.x) {
         T.str[i] = ci.strings[i];
+#pragma unroll 1
         for (int j = i; j < C::NS; ++j)
             T.tri[i * C::NS - i * (i - 1) / 2 + j - i] = make_uchar2((unsigned char)i, (unsigned char)j);
     }
+#pragma unroll 1
     for (int x = threadIdx.x; x < C::P; x += blockDim.x) {
         const int a = C::pair_hi(x);
         T.pq[x] = make_uchar2((unsigned char)a, (unsigned char)(x - a * (a + 1) / 2));
+#pragma unroll 1
         for (int y = 0; y <= x; ++y) T.ptri[x * (x + 1) / 2 + y] = make_uchar2((unsigned char)x, (unsigned char)y);
     }
     __syncthreads();
@@ -155,7 +170,11 @@ __host__ __device__ inline double string_element(uint32_t I, uint32_t J, H h, VF
     };
     auto odd = [](uint32_t s) {
         int c = 0;
+#ifdef __CUDA_ARCH__
+        c = __popc(s) & 1;
+#else
         for (; s; s &= s - 1u) c ^= 1;
+#endif
         return c;
     };
     auto between = [](int a, int b) {
@@ -165,9 +184,11 @@ __host__ __device__ inline double string_element(uint32_t I, uint32_t J, H h, VF
     uint32_t from = I & ~J, to = J & ~I;
     double v = 0.0;
     if (from == 0u) {
+#pragma unroll 1
         for (uint32_t a = I; a; a &= a - 1u) {
             const int p = low(a);
             v += h(p, p);
+#pragma unroll 1
             for (uint32_t b = a & (a - 1u); b; b &= b - 1u) {
                 const int q = low(b);
                 v += V(p, p, q, q) - V(p, q, p, q);
@@ -181,6 +202,7 @@ __host__ __device__ inline double string_element(uint32_t I, uint32_t J, H h, VF
     int neg = odd(I & between(p, a));
     if (from == 0u) {
         v = h(p, a);
+#pragma unroll 1
         for (uint32_t c = I & J; c; c &= c - 1u) {
             const int r = low(c);
             v += V(p, a, r, r) - V(p, r, r, a);
@@ -229,7 +251,7 @@ __device__ SectorStart sector_setup(const BatchArgs &a, const SectorTables<C> &T
 {
     const int lane = threadIdx.x & 31;
     const size_t norb = a.norb;
-#pragma unroll 4
+#pragma unroll 2
     for (int e = lane; e < C::PT; e += 32) {
         const uchar2 xy = T.ptri[e], pq = T.pq[xy.x], rs = T.pq[xy.y];
         Vp[e] = a.eri[eri_index(a.norb, A[pq.x], A[pq.y], A[rs.x], A[rs.y])];
@@ -242,15 +264,18 @@ __device__ SectorStart sector_setup(const BatchArgs &a, const SectorTables<C> &T
     if (lane < C::P) {
         const int p = T.pq[lane].x, q = T.pq[lane].y;
         double v = a.F[A[p] * norb + A[q]];
+#pragma unroll 1
         for (uint32_t m = mphi; m; m &= m - 1u) {
             const int i = __ffs((int)m) - 1;
             v -= 2.0 * Vp[tri_index(lane, pair_index(i, i))] - Vp[tri_index(pair_index(p, i), pair_index(i, q))];
         }
         h[lane] = v;
     }
+#pragma unroll 1
     for (int e = lane; e < C::NS * C::n; e += 32) {  // sum_{p in I} (pp|qq)
         const int I = e / C::n, q = e - I * C::n;
         double v = 0.0;
+#pragma unroll 1
         for (uint32_t m = T.str[I]; m; m &= m - 1u) {
             const int p = __ffs((int)m) - 1;
             v += Vp[tri_index(pair_index(p, p), pair_index(q, q))];
@@ -275,6 +300,7 @@ __device__ SectorStart sector_setup(const BatchArgs &a, const SectorTables<C> &T
     for (int e = lane; e < C::NH; e += 32) {
         const uchar2 ij = T.tri[e];
         double v = hd[ij.x] + hd[ij.y];
+#pragma unroll 1
         for (uint32_t m = T.str[ij.y]; m; m &= m - 1u) v += dsum[ij.x * C::n + __ffs((int)m) - 1];
         diag[e] = v;
         if (v < best) {
@@ -362,86 +388,119 @@ __device__ __forceinline__ void sector_rounds(AB ab, ROW row, FLUSH flush)
 template <class C>
 __device__ __forceinline__ int c_at(int J, int m) { return ((m >> 1) * C::NS + J) * 2 + (m & 1); }
 
-// Writes the packed sector vector t as the full coefficient matrix.
-template <class C, typename T>
-__device__ __forceinline__ void expand(const SectorTables<C> &Tb, const T (&t)[C::DH], int sgn, T *cm)
+// Two float32 values in one register pair, for fma.rn.f32x2: one instruction for two
+// multiply-adds (the rate of the pipe is the same, but these kernels wait for instructions).
+__device__ __forceinline__ uint64_t pack2(float x, float y)
 {
+    return (uint64_t)__float_as_uint(y) << 32 | __float_as_uint(x);
+}
+__device__ __forceinline__ float2 unpack2(uint64_t v)
+{
+    return make_float2(__uint_as_float((uint32_t)v), __uint_as_float((uint32_t)(v >> 32)));
+}
+__device__ __forceinline__ void ffma2(uint64_t &d, uint64_t a, uint64_t b)
+{
+    asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(d) : "l"(a), "l"(b));
+}
+
+// sector_rounds for the float32 sigma, which takes list entries and rows of Hs two at a time:
+// ab(Ib, y) does entries y and y + 1 (y + 1 = R: the zero row), row(Ib, j) rows 2j and 2j + 1.
+template <class C, class AB, class ROW, class FLUSH>
+__device__ __forceinline__ void sector_rounds2(AB ab, ROW row, FLUSH flush)
+{
+    const int lane = threadIdx.x & 31;
+    if constexpr (C::HELP) {
+        const bool main = lane < C::NS;
+#pragma unroll 1
+        for (int ph = 0; ph < 2; ++ph) {
+            const int Ib = main ? lane : lane - C::NS + 12 * ph;
+            if (Ib < C::NS) {
+#pragma unroll 1
+                for (int r = 0; r < 2; ++r) {
+                    ab(Ib, (main ? 4 * ph : 8) + 2 * r);
+                    row(Ib, main ? 4 * ph + 2 * r : 8 + r);
+                    if (main) row(Ib, 4 * ph + 2 * r + 1);
+                }
+                if (!main) flush(Ib, 1);
+            }
+        }
+        if (main) flush(lane, 0);
+    } else {
+        const int part = lane / C::NS, Ib = lane - part * C::NS;
+        if (part < C::L) {
+#pragma unroll 1
+            for (int y = 2 * part; y < C::R; y += 2 * C::L) ab(Ib, y);
+#pragma unroll 1
+            for (int j = part; j < C::NSH; j += C::L) row(Ib, j);
+            flush(Ib, part);
+        }
+    }
+}
+
+// sigma of the packed vector t.  cm: c[J][m] at m NS + J.  Vs: [P][2P + 1], 1/2 V with rows (of
+// the second index) 2 pair + neg, the sign applied, and a zero row.  Hs2: [NSH][NSP] pairs of
+// rows of Hs.
+template <class C>
+__device__ __forceinline__ void sigma_sector(const SectorTables<C> &Tb, const float *Vs, const float2 *Hs2, float *cm,
+                                             float *S, int sgn, const float (&t)[C::DH], float (&out)[C::DH])
+{
+    constexpr int VR = 2 * C::P + 1;
     const int lane = threadIdx.x & 31;
 #pragma unroll
     for (int j = 0; j < C::DH; ++j) {
         const int e = lane + 32 * j;
         if (e < C::NH) {
             const uchar2 ij = Tb.tri[e];
-            const T v = ij.x == ij.y ? t[j] : (T)0.70710678118654752 * t[j];
-            cm[c_at<C>(ij.x, ij.y)] = v;
-            cm[c_at<C>(ij.y, ij.x)] = sgn > 0 ? v : -v;
+            const float v = ij.x == ij.y ? t[j] : 0.70710678f * t[j];
+            cm[ij.y * C::NS + ij.x] = v;
+            cm[ij.x * C::NS + ij.y] = (float)sgn * v;
         }
     }
-}
-
-// V2: [PH][2P] pairs of columns of 1/2 V, rows 2 pair + neg with the sign applied.
-template <class C>
-__device__ __forceinline__ void sigma_sector(const SectorTables<C> &Tb, const float2 *V2, const float *Hs, float *cm,
-                                             float *S, int sgn, const float (&t)[C::DH], float (&out)[C::DH])
-{
-    const int lane = threadIdx.x & 31;
-    expand<C, float>(Tb, t, sgn, cm);
     __syncwarp();
-    const float2 *cm2 = (const float2 *)cm;
-    float acc[C::NSP];
+    uint64_t acc[C::NS];
 #pragma unroll
-    for (int i = 0; i < C::NSP; ++i) acc[i] = 0.f;
-    sector_rounds<C>(
+    for (int i = 0; i < C::NS; ++i) acc[i] = 0ull;
+    const int flip = (1 - sgn) >> 1;  // (row J_y is read as column J_y: sgn times it)
+    sector_rounds2<C>(
         [&](int Ib, int y) {
-            // (row J_y read as column J_y: sgn times it)
-            const int e = Tb.list[Ib * C::R + y], J = e >> 8, row = (e & 255) ^ (sgn < 0 ? 1 : 0);
-            float c[2 * C::NSH];
-#pragma unroll
-            for (int m = 0; m < C::NSH; ++m) {
-                const float2 v = cm2[m * C::NS + J];
-                c[2 * m] = v.x;
-                c[2 * m + 1] = v.y;
+            const int e0 = Tb.list[Ib * C::R + y], J0 = e0 >> 8, row0 = (e0 & 255) ^ flip;
+            int J1 = 0, row1 = 2 * C::P;
+            if (C::R % 2 == 0 || y + 1 < C::R) {
+                const int e1 = Tb.list[Ib * C::R + y + 1];
+                J1 = e1 >> 8;
+                row1 = (e1 & 255) ^ flip;
             }
-            static_for<C::PH>([&](auto ph) {
-                const float2 v2 = V2[ph * 2 * C::P + row];
-                static_for<2>([&](auto half) {
-                    constexpr int p = 2 * decltype(ph)::value + decltype(half)::value;
-                    if constexpr (p < C::P) {
-                        const float v = decltype(half)::value ? v2.y : v2.x;
-                        static_for<C::NS>([&](auto I) {
-                            constexpr int a = C::pair_hi(p), b = C::pair_lo(p);
-                            constexpr int Jx = C::target(decltype(I)::value, a, b);
-                            if constexpr (Jx >= 0) {
-                                if constexpr (C::negative(decltype(I)::value, a, b))
-                                    acc[I] = fmaf(-v, c[Jx], acc[I]);
-                                else
-                                    acc[I] = fmaf(v, c[Jx], acc[I]);
-                            }
-                        });
-                    }
+            uint64_t c[C::NS];
+#pragma unroll
+            for (int m = 0; m < C::NS; ++m) c[m] = pack2(cm[m * C::NS + J0], cm[m * C::NS + J1]);
+            static_for<C::P>([&](auto p) {
+                const float v0 = Vs[p * VR + row0], v1 = Vs[p * VR + row1];
+                const uint64_t v = pack2(v0, v1), w = pack2(-v0, -v1);
+                static_for<C::NS>([&](auto I) {
+                    constexpr int a = C::pair_hi(decltype(p)::value), b = C::pair_lo(decltype(p)::value);
+                    constexpr int Jx = C::target(decltype(I)::value, a, b);
+                    if constexpr (Jx >= 0) ffma2(acc[I], C::negative(decltype(I)::value, a, b) ? w : v, c[Jx]);
                 });
             });
         },
-        [&](int Ib, int J) {
-            float c = cm[c_at<C>(Ib, J)];
-            c = sgn > 0 ? c : -c;
-            const float4 *hs = (const float4 *)(Hs + J * C::NSP);
+        [&](int Ib, int j) {
+            const int J1 = 2 * j + 1 < C::NS ? 2 * j + 1 : 2 * j;
+            const uint64_t c = pack2((float)sgn * cm[2 * j * C::NS + Ib], (float)sgn * cm[J1 * C::NS + Ib]);
+            const ulonglong2 *hs = (const ulonglong2 *)(Hs2 + j * C::NSP);
 #pragma unroll
-            for (int i = 0; i < C::NSP / 4; ++i) {
-                if (4 * i >= C::NS) break;
-                const float4 v = hs[i];
-                acc[4 * i] = fmaf(c, v.x, acc[4 * i]);
-                acc[4 * i + 1] = fmaf(c, v.y, acc[4 * i + 1]);
-                acc[4 * i + 2] = fmaf(c, v.z, acc[4 * i + 2]);
-                acc[4 * i + 3] = fmaf(c, v.w, acc[4 * i + 3]);
+            for (int i = 0; i < (C::NS + 1) / 2; ++i) {
+                const ulonglong2 v = hs[i];
+                ffma2(acc[2 * i], c, v.x);
+                if (2 * i + 1 < C::NS) ffma2(acc[2 * i + 1 < C::NS ? 2 * i + 1 : 0], c, v.y);
             }
         },
         [&](int Ib, int part) {
-            float4 *s = (float4 *)(S + (part * C::NS + Ib) * C::NSP);
+            float *s = S + (part * C::NS + Ib) * C::NSP;
 #pragma unroll
-            for (int i = 0; i < C::NSP / 4; ++i) {
-                s[i] = make_float4(acc[4 * i], acc[4 * i + 1], acc[4 * i + 2], acc[4 * i + 3]);
-                acc[4 * i] = acc[4 * i + 1] = acc[4 * i + 2] = acc[4 * i + 3] = 0.f;
+            for (int i = 0; i < C::NS; ++i) {
+                const float2 v = unpack2(acc[i]);
+                s[i] = v.x + v.y;
+                acc[i] = 0ull;
             }
         });
     __syncwarp();
@@ -457,8 +516,8 @@ __device__ __forceinline__ void sigma_sector(const SectorTables<C> &Tb, const fl
                 u += S[(p * C::NS + ij.y) * C::NSP + ij.x];
                 w += S[(p * C::NS + ij.x) * C::NSP + ij.y];
             }
-            const float v = sgn > 0 ? u + w : u - w;
-            out[j] = ij.x == ij.y ? (sgn > 0 ? v : 0.f) : 1.41421356f * v;
+            const float v = fmaf((float)sgn, w, u);  // (zero on the diagonal of the odd sector)
+            out[j] = ij.x == ij.y ? v : 1.41421356f * v;
         }
     }
     __syncwarp();
@@ -471,86 +530,100 @@ __device__ __forceinline__ void sigma_sector(const SectorTables<C> &Tb, const fl
 // so V and Hs are kept as 55-bit fixed-point numbers in two limbs (to_fixed) and the anchor
 // as integers c 2^28: each term is two 32 x 32 + 64 -> 64 bit multiply-adds, exact.  The sums
 // cannot overflow: by Cauchy-Schwarz the absolute terms of one element add up to at most
-// (12 * 3 + 5) |c| |V|max < 2^5.4 * 2^28 * 2^27 for a unit vector (a list of 12 entries holds
+// (12 * 3 + 9) |c| |V|max < 2^5.5 * 2^28 * 2^27 for a unit vector (a list of 12 entries holds
 // its own string 3 times, every other string once).  The result is rounded once, to 2^-55 of
-// the largest element of V and Hs.  The diagonal of Hs
+// the largest element of V and Hs.  Taken once or twice per tuple, so the loops are kept rolled:
+// unrolled like the float32 sigma they were 37 KB of code for the same number of instructions.  The diagonal of Hs
 // is left to the caller (it would set the scale).
 template <class C>
 __device__ __forceinline__ void sigma_anchor(const SectorTables<C> &Tb, const int2 *Vf, const int2 *Hsf, const int *cm,
                                              long long *S, int sgn)
 {
     const int lane = threadIdx.x & 31;
-    const int2 *cm2 = (const int2 *)cm;
-    constexpr int ST = C::NS | 1;
-    if (lane < C::NS) {
-        const int Ib = lane;
-        long long hi[C::NS], lo[C::NS];
-#pragma unroll
-        for (int i = 0; i < C::NS; ++i) hi[i] = lo[i] = 0;
 #pragma unroll 1
-        for (int y = 0; y < C::R; ++y) {
-            const int e = Tb.list[Ib * C::R + y], J = e >> 8, pr = (e & 255) >> 1, m = -((e & 1) ^ (sgn < 0 ? 1 : 0));
-            int c[2 * C::NSH];
-#pragma unroll
-            for (int i = 0; i < C::NSH; ++i) {
-                const int2 v = cm2[i * C::NS + J];
-                c[2 * i] = (v.x ^ m) - m;
-                c[2 * i + 1] = (v.y ^ m) - m;
+    for (int h = lane; h < C::NH; h += 32) {
+        const uchar2 ij = Tb.tri[h];
+        long long hi = 0, lo = 0;
+        const uint16_t *la = Tb.list + ij.x * C::R, *lb = Tb.list + ij.y * C::R;
+#pragma unroll 1
+        for (int x = 0; x < C::R; ++x) {
+            const int ea = la[x];
+            const int2 *v = Vf + ((ea & 255) >> 1) * C::P;
+            const int *c = cm + (ea >> 8) * C::NS;
+#pragma unroll 2
+            for (int y = 0; y < C::R; ++y) {
+                const int eb = lb[y], m = -((ea ^ eb) & 1);
+                const int2 w = v[(eb & 255) >> 1];
+                const int q = (c[eb >> 8] ^ m) - m;
+                hi += (long long)w.x * q;
+                lo += (long long)w.y * q;
             }
-            static_for<C::P>([&](auto p) {
-                const int2 v = Vf[tri_index(pr, p)];
-                static_for<C::NS>([&](auto I) {
-                    constexpr int a = C::pair_hi(decltype(p)::value), b = C::pair_lo(decltype(p)::value);
-                    constexpr int Jx = C::target(decltype(I)::value, a, b);
-                    if constexpr (Jx >= 0) {
-                        constexpr bool neg = C::negative(decltype(I)::value, a, b);
-                        hi[I] += (long long)(neg ? -v.x : v.x) * c[Jx];
-                        lo[I] += (long long)(neg ? -v.y : v.y) * c[Jx];
-                    }
-                });
-            });
         }
-#pragma unroll 1
-        for (int J = 0; J < C::NS; ++J) {
-            int c = cm[c_at<C>(Ib, J)];
-            c = sgn > 0 ? c : -c;
-            static_for<C::NS>([&](auto I) {
-                const int r = J < I ? J : (int)I, s = J < I ? (int)I : J;
-                const int2 v = Hsf[r * C::NS - r * (r - 1) / 2 + s - r];
-                hi[I] += (long long)v.x * c;
-                lo[I] += (long long)v.y * c;
-            });
+#pragma unroll 2
+        for (int J = 0; J < C::NS; ++J) {  // (Hs C)[Ia][Ib] + (C Hs)[Ia][Ib], without the diagonal of Hs
+            const int r = min(ij.x, J), s = max(ij.x, J), t = min(ij.y, J), u = max(ij.y, J);
+            const int2 a = Hsf[r * C::NS - r * (r - 1) / 2 + s - r], b = Hsf[t * C::NS - t * (t - 1) / 2 + u - t];
+            const int p = cm[J * C::NS + ij.y], q = cm[ij.x * C::NS + J];
+            hi += (long long)a.x * p;
+            lo += (long long)a.y * p;
+            hi += (long long)b.x * q;
+            lo += (long long)b.y * q;
         }
-#pragma unroll
-        for (int i = 0; i < C::NS; ++i) S[Ib * ST + i] = hi[i] + ((lo[i] + (1LL << 27)) >> 28);
+        S[h] = hi + ((lo + (1LL << 27)) >> 28);
     }
     __syncwarp();
+}
+
+// Sums of the K (a power of two) values over the warp; every lane gets all totals.  Each
+// step halves the values that a lane carries, so K = 8 takes 9 additions instead of 40.
+template <int K, typename T>
+__device__ __forceinline__ void warp_sum_n(T (&v)[K])
+{
+    const int lane = threadIdx.x & 31;
+    int o = 16;
+#pragma unroll
+    for (int m = K / 2; m >= 1; m >>= 1) {
+        const bool up = lane & o;
+#pragma unroll
+        for (int i = 0; i < m; ++i) {
+            const T send = up ? v[i] : v[i + m];
+            const T keep = up ? v[i + m] : v[i];
+            v[i] = keep + __shfl_xor_sync(FULL, send, o);
+        }
+        o >>= 1;
+    }
+#pragma unroll
+    for (; o > 0; o >>= 1) v[0] += __shfl_xor_sync(FULL, v[0], o);
+    const T s = v[0];
+    // value i was kept by the lanes whose leading bits spell i
+#pragma unroll
+    for (int i = 0; i < K; ++i) v[i] = __shfl_sync(FULL, s, i * (32 / K));
 }
 
 // ------------------------------------------------------------------ Davidson on packed sector vectors
 
 // The warp solver's Davidson (davidson_warp, plain and anchored) on packed vectors; sigma(t,
-// ht) forms the image of t.
+// ht) forms the image of t.  The dot products of a stage are reduced together, and the second
+// orthogonalisation pass is taken only when the first one cancelled (less than half of |t|^2
+// left; with more left, one pass is orthogonal to within a few rounding errors).
 template <class C, class SIGMA>
 __device__ __forceinline__ PhaseOut davidson_sector(SIGMA sigma, const float *dg, float (&x)[C::DH], double tol,
-                                                    int min_iter, int max_iter, const Anchor *an)
+                                                    int min_iter, int max_iter, const Anchor &an, bool anchored)
 {
     constexpr int DH = C::DH;
     const int lane = threadIdx.x & 31;
-    const bool anch = an != nullptr;
-    const float *x0s = anch ? an->x0 : nullptr, *r0s = anch ? an->r0 : nullptr;
-    const float shift = anch ? an->shift : 0.f, shift_lo = anch ? an->shift_lo : 0.f;
-    const float x0x0 = anch ? an->x0x0 : 0.f;
+    const float *x0s = an.x0, *r0s = an.r0;
+    const float shift = an.shift, shift_lo = an.shift_lo, x0x0 = an.x0x0;  // (shift 0 when plain)
     float hx[DH], p[DH], hp[DH], t[DH], ht[DH], x0[DH], r0[DH];
     PhaseOut o;
     o.nsig = 0;
     o.status = MBE_STATUS_OK;
     o.dnorm = 0.0;
     float lam = 0.f;
-    bool first = !anch;
+    int first = opaque(!anchored);
 #pragma unroll
     for (int j = 0; j < DH; ++j) p[j] = hp[j] = hx[j] = 0.f;
-    if (!anch) {
+    if (!anchored) {
         float s = 0.f;
 #pragma unroll
         for (int j = 0; j < DH; ++j) s += x[j] * x[j];
@@ -566,26 +639,32 @@ __device__ __forceinline__ PhaseOut davidson_sector(SIGMA sigma, const float *dg
     float best = 3e38f, rn = 0.f, xx = 1.f;
     int stall = 0;
     for (int it = 0;;) {
+        const bool anch = opaque(anchored);
         if (!first) {
-            float rr = 0.f, t0n = 0.f;
+            float v[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};  // |r|^2, x.t, p.t, |t|^2, |x|^2
 #pragma unroll
             for (int j = 0; j < DH; ++j) {
                 const int e = lane + 32 * j;
-                t[j] = x0[j] = r0[j] = 0.f;
+                t[j] = x0[j] = 0.f;
                 if (e < C::NH) {
+                    float r0j = 0.f;
                     if (anch) {
                         x0[j] = x0s[e];
-                        r0[j] = r0s[e];
+                        r0j = r0s[e];
                     }
-                    const float r = (r0[j] + hx[j]) - lam * (x0[j] + x[j]);
-                    rr += r * r;
+                    const float xj = x0[j] + x[j], r = (r0j + hx[j]) - lam * xj;
                     float den = dg[e] - shift - lam;
                     if (fabsf(den) < 1e-4f) den = den >= 0.f ? 1e-4f : -1e-4f;
-                    t[j] = r / den;
-                    t0n += t[j] * t[j];
+                    t[j] = __fdividef(r, den);
+                    v[0] += r * r;
+                    v[1] += xj * t[j];
+                    v[2] += p[j] * t[j];
+                    v[3] += t[j] * t[j];
+                    v[4] += xj * xj;
                 }
             }
-            rn = sqrtf(warp_sum(rr));
+            warp_sum_n<8>(v);
+            rn = sqrtf(v[0]);
             if (!isfinite(rn) || !isfinite(lam)) {
                 o.status = MBE_STATUS_NONFINITE;
                 break;
@@ -601,35 +680,35 @@ __device__ __forceinline__ PhaseOut davidson_sector(SIGMA sigma, const float *dg
             } else if (++stall >= 3) {
                 break;
             }
-            if (anch) {
-                float s = 0.f;
+            if (anch) xx = v[4];
+            // orthonormalise t against x and p
+            float ax = v[1] / xx, ap = v[2], tt = 0.f;
+#pragma unroll
+            for (int j = 0; j < DH; ++j) {
+                t[j] -= ax * (x0[j] + x[j]) + ap * p[j];
+                tt += t[j] * t[j];
+            }
+            tt = warp_sum(tt);
+            if (!(tt >= 0.5f * v[3])) {
+                float w[2] = {0.f, 0.f};
 #pragma unroll
                 for (int j = 0; j < DH; ++j) {
-                    const float xj = x0[j] + x[j];
-                    s += xj * xj;
+                    w[0] += (x0[j] + x[j]) * t[j];
+                    w[1] += p[j] * t[j];
                 }
-                t0n = sqrtf(warp_sum(t0n));
-                xx = warp_sum(s);
-            }
-            // orthonormalise t against x and p (two passes)
-#pragma unroll 1
-            for (int pass = 0; pass < 2; ++pass) {
-                float ax = 0.f, ap = 0.f;
+                warp_sum_n<2>(w);
+                ax = w[0] / xx;
+                ap = w[1];
+                tt = 0.f;
 #pragma unroll
                 for (int j = 0; j < DH; ++j) {
-                    ax += (x0[j] + x[j]) * t[j];
-                    ap += p[j] * t[j];
+                    t[j] -= ax * (x0[j] + x[j]) + ap * p[j];
+                    tt += t[j] * t[j];
                 }
-                ax = warp_sum(ax) / xx;
-                ap = warp_sum(ap);
-#pragma unroll
-                for (int j = 0; j < DH; ++j) t[j] -= ax * (x0[j] + x[j]) + ap * p[j];
+                tt = warp_sum(tt);
             }
-            float tt = 0.f;
-#pragma unroll
-            for (int j = 0; j < DH; ++j) tt += t[j] * t[j];
-            const float tn = sqrtf(warp_sum(tt));
-            if (anch ? !(tn > 1e-4f * t0n) : !(tn > tiny_norm<float>())) break;  // nothing left to add
+            const float tn = sqrtf(tt);
+            if (anch ? !(tn > 1e-4f * sqrtf(v[3])) : !(tn > tiny_norm<float>())) break;  // nothing left to add
             const float tinv = 1.f / tn;
 #pragma unroll
             for (int j = 0; j < DH; ++j) t[j] *= tinv;
@@ -644,32 +723,33 @@ __device__ __forceinline__ PhaseOut davidson_sector(SIGMA sigma, const float *dg
                 xh += x[j] * ht[j];
             }
             lam = warp_sum(xh);
-            first = false;
+            first = opaque(0);
             continue;
         }
         ++it;
         // G = [x p t]^T A [x p t]; a coupling x.(A v) is formed as v.r0 + d.(A v)
-        float g00 = 0.f, g01 = 0.f, g02 = 0.f, g11 = 0.f, g12 = 0.f, g22 = 0.f;
+        float g[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
 #pragma unroll
         for (int j = 0; j < DH; ++j) {
             const int e = lane + 32 * j;
             r0[j] = anch && e < C::NH ? r0s[e] : 0.f;
-            if (anch) ht[j] = (ht[j] - shift * t[j]) - shift_lo * t[j];
-            g00 += x[j] * (2.f * r0[j] + hx[j]);
-            g01 += p[j] * r0[j] + x[j] * hp[j];
-            g02 += t[j] * r0[j] + x[j] * ht[j];
-            g11 += p[j] * hp[j];
-            g12 += p[j] * ht[j];
-            g22 += t[j] * ht[j];
+            ht[j] = (ht[j] - shift * t[j]) - shift_lo * t[j];
+            g[0] += x[j] * (2.f * r0[j] + hx[j]);
+            g[1] += p[j] * r0[j] + x[j] * hp[j];
+            g[2] += t[j] * r0[j] + x[j] * ht[j];
+            g[3] += p[j] * hp[j];
+            g[4] += p[j] * ht[j];
+            g[5] += t[j] * ht[j];
         }
+        warp_sum_n<8>(g);
         float G[3][3];
         const float sx = anch ? 1.f / sqrtf(xx) : 1.f;
-        G[0][0] = warp_sum(g00) * sx * sx;
-        G[0][1] = G[1][0] = warp_sum(g01) * sx;
-        G[0][2] = G[2][0] = warp_sum(g02) * sx;
-        G[1][1] = warp_sum(g11);
-        G[1][2] = G[2][1] = warp_sum(g12);
-        G[2][2] = warp_sum(g22);
+        G[0][0] = g[0] * sx * sx;
+        G[0][1] = G[1][0] = g[1] * sx;
+        G[0][2] = G[2][0] = g[2] * sx;
+        G[1][1] = g[3];
+        G[1][2] = G[2][1] = g[4];
+        G[2][2] = g[5];
         float y[3];
         eig3<float>(G, have_p, y);
         const float y0 = y[0] * sx, y1 = y[1], y2 = y[2];
@@ -681,7 +761,7 @@ __device__ __forceinline__ PhaseOut davidson_sector(SIGMA sigma, const float *dg
         q0 *= zi;
         q1 *= zi;
         q2 *= zi;
-        float nxx = 0.f, nxh = 0.f, nxr = 0.f, nx0 = 0.f;
+        float n[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
         for (int j = 0; j < DH; ++j) {
             const int e = lane + 32 * j;
@@ -692,24 +772,21 @@ __device__ __forceinline__ PhaseOut davidson_sector(SIGMA sigma, const float *dg
             hp[j] = q0 * (r0[j] + hx[j]) + q1 * hp[j] + q2 * ht[j];
             x[j] = nx;
             hx[j] = nhx;
-            nxx += nx * nx;
-            nxh += nx * nhx;
-            nxr += nx * r0[j];
-            nx0 += nx * x0[j];
+            n[0] += nx * nx;
+            n[1] += nx * nhx;
+            n[2] += nx * r0[j];
+            n[3] += nx * x0[j];
         }
-        nxx = warp_sum(nxx);
-        nxh = warp_sum(nxh);
+        warp_sum_n<4>(n);
         float sc;
         if (anch) {
-            nxr = warp_sum(nxr);
-            nx0 = warp_sum(nx0);
             sc = 1.f / y0;
             // mu = (x.Ax) / (x.x), x = x0 + sc nx, A x = r0 + sc A nx, x0.r0 = 0
-            lam = (sc * 2.f * nxr + sc * sc * nxh) / (x0x0 + sc * 2.f * nx0 + sc * sc * nxx);
-            o.dnorm = (double)(fabsf(sc) * sqrtf(nxx));
+            lam = (sc * 2.f * n[2] + sc * sc * n[1]) / (x0x0 + sc * 2.f * n[3] + sc * sc * n[0]);
+            o.dnorm = (double)(fabsf(sc) * sqrtf(n[0]));
         } else {
-            sc = 1.f / sqrtf(nxx);
-            lam = nxh / nxx;
+            sc = 1.f / sqrtf(n[0]);
+            lam = n[1] / n[0];
         }
 #pragma unroll
         for (int j = 0; j < DH; ++j) {
@@ -727,12 +804,12 @@ __device__ __forceinline__ PhaseOut davidson_sector(SIGMA sigma, const float *dg
 // Shared memory of one warp of the mixed sector solver.
 template <class C>
 struct SectorMixed {
-    long long Vf[C::PT];   // float64 V during set-up, then fixed point (1/2 V)
+    int2 Vf[C::P * C::P];  // float64 V (packed) during set-up, then fixed point
     long long Hsf[C::NH];  // float64 Hs during set-up, then fixed point (off-diagonal)
     double hd[C::NS];      // diagonal of Hs
     union {                // sigma partial sums; set-up scratch
         alignas(16) float S[C::L * C::NS * C::NSP];
-        long long S64[C::NS * (C::NS | 1)];
+        long long S64[C::NH];
         struct {
             double diag[C::NH], h[C::P];
         } su;
@@ -742,9 +819,15 @@ struct SectorMixed {
         int cmi[2 * C::NSH * C::NS];
         double dsum[C::NS * C::n];
     } c;
-    alignas(16) float Hs32[C::NS * C::NSP];
-    float2 V2[C::PH * 2 * C::P];
-    float dg[C::NH], x0[C::NH], r0[C::NH];
+    alignas(16) float2 Hs2[C::NSH * C::NSP];  // rows of Hs in pairs
+    float Vs[C::P * (2 * C::P + 1)];          // 1/2 V, both signs
+    float dg[C::NH];
+    union {
+        struct {
+            float x0[C::NH], r0[C::NH];
+        };
+        double Vp[C::PT];  // set-up: float64 V
+    };
     int A[8];
 };
 
@@ -770,33 +853,46 @@ __global__ void __launch_bounds__(SECTOR_WARPS * 32, C::DH > 4 ? 3 : 4) k_sector
         const int64_t t = a.perm[begin + (int64_t)pos];
         if (lane == 0) build_A(a, t, W.A);
         __syncwarp();
-        double *Vp = (double *)W.Vf, *Hsp = (double *)W.Hsf;
+        double *Vp = W.Vp, *Hsp = (double *)W.Hsf;
         const SectorStart st =
             sector_setup<C>(a, T, W.A, Vp, Hsp, W.hd, W.s.su.h, W.c.dsum, W.s.su.diag);
         double vmax = 0.0;
+#pragma unroll 1
         for (int e = lane; e < C::PT; e += 32) {
             const uchar2 xy = T.ptri[e];
-            const double v = 0.5 * Vp[e];
-            const float f = (float)v;
-            float *col = (float *)&W.V2[(xy.y >> 1) * 2 * C::P] + (xy.y & 1);
-            col[4 * xy.x] = f;
-            col[4 * xy.x + 2] = -f;
-            col = (float *)&W.V2[(xy.x >> 1) * 2 * C::P] + (xy.x & 1);
-            col[4 * xy.y] = f;
-            col[4 * xy.y + 2] = -f;
+            const double v = Vp[e];
+            const float f = 0.5f * (float)v;
+            constexpr int VR = 2 * C::P + 1;
+            float *s = W.Vs + xy.y * VR + 2 * xy.x;
+            s[0] = f;
+            s[1] = -f;
+            s = W.Vs + xy.x * VR + 2 * xy.y;
+            s[0] = f;
+            s[1] = -f;
             vmax = fmax(vmax, fabs(v));
         }
+#pragma unroll 1
         for (int e = lane; e < C::NH; e += 32) {
             const uchar2 ij = T.tri[e];
             const double v = Hsp[e];
-            W.Hs32[ij.x * C::NSP + ij.y] = W.Hs32[ij.y * C::NSP + ij.x] = (float)v;
+            float *hs = (float *)W.Hs2;
+            hs[((ij.x >> 1) * C::NSP + ij.y) * 2 + (ij.x & 1)] = (float)v;
+            hs[((ij.y >> 1) * C::NSP + ij.x) * 2 + (ij.y & 1)] = (float)v;
             if (ij.x != ij.y) vmax = fmax(vmax, fabs(v));
             W.dg[e] = (float)W.s.su.diag[e];
         }
+        for (int p = lane; p < C::P; p += 32) W.Vs[p * (2 * C::P + 1) + 2 * C::P] = 0.f;
+        if (C::NS & 1)  // the last row's partner
+            for (int i = lane; i < C::NS; i += 32) W.Hs2[(C::NSH - 1) * C::NSP + i].y = 0.f;
         const int E = fixed_exponent(vmax);
         const double scale = pow2(55 - E);
         __syncwarp();
-        for (int e = lane; e < C::PT; e += 32) ((int2 *)W.Vf)[e] = to_fixed(0.5 * Vp[e], scale);
+#pragma unroll 1
+        for (int e = lane; e < C::PT; e += 32) {
+            const uchar2 xy = T.ptri[e];
+            W.Vf[xy.x * C::P + xy.y] = W.Vf[xy.y * C::P + xy.x] = to_fixed(Vp[e], scale);
+        }
+#pragma unroll 1
         for (int e = lane; e < C::NH; e += 32) {
             const uchar2 ij = T.tri[e];
             ((int2 *)W.Hsf)[e] = ij.x == ij.y ? make_int2(0, 0) : to_fixed(Hsp[e], scale);
@@ -808,9 +904,9 @@ __global__ void __launch_bounds__(SECTOR_WARPS * 32, C::DH > 4 ? 3 : 4) k_sector
         // one copy of the sector's Davidson: two inlined copies, both hot on an SM,
         // overflow the instruction cache and slow every phase of every warp
 #pragma unroll 1
-        for (int sector = 0; sector < 2 && !redo; ++sector) {
+        for (int sector = opaque(0); sector < 2 && !redo; ++sector) {
             if (sector == 1 && a.even_only) break;
-            const int sgn = sector == 0 ? 1 : -1, g = sector == 0 ? st.g : st.go;
+            const int sgn = opaque(sector == 0 ? 1 : -1), g = sector == 0 ? st.g : st.go;
             float xv[C::DH];
 #pragma unroll
             for (int j = 0; j < C::DH; ++j) {
@@ -818,7 +914,7 @@ __global__ void __launch_bounds__(SECTOR_WARPS * 32, C::DH > 4 ? 3 : 4) k_sector
                 xv[j] = e < C::NH ? packed_guess<C, float>(T.tri[e], e, g, sgn) : 0.f;
             }
             auto sigma = [&](const float(&tv)[C::DH], float(&out)[C::DH]) {
-                sigma_sector<C>(T, W.V2, W.Hs32, W.c.cm, W.s.S, sgn, tv, out);
+                sigma_sector<C>(T, W.Vs, W.Hs2, W.c.cm, W.s.S, sgn, tv, out);
             };
             // plain float32 passes (the first sector one to tol_switch; the second one
             // to SECTOR_TOL, then tol_switch, decided against the first's float32
@@ -828,10 +924,10 @@ __global__ void __launch_bounds__(SECTOR_WARPS * 32, C::DH > 4 ? 3 : 4) k_sector
             double th = 0.0, lam_s = 0.0;
             Anchor an{W.x0, W.r0, 0.f, 0.f, 1.f};
             for (;;) {
-                const bool anchored = anchors > 0;
+                const bool anchored = opaque(anchors) > 0;
                 const double tl = anchored ? a.tol : ((sector == 0 || passes == 1) ? a.tol_switch : SECTOR_TOL);
-                const PhaseOut o = davidson_sector<C>(sigma, W.dg, xv, tl, anchored ? a.min_fp64 : 0, a.max_iter,
-                                                      anchored ? &an : nullptr);
+                const PhaseOut o = davidson_sector<C>(sigma, W.dg, xv, tl, anchored ? a.min_fp64 : 0, a.max_iter, an,
+                                                      anchored);
                 n32 += o.nsig;
                 if (!anchored) {
                     const bool finite = o.status != MBE_STATUS_NONFINITE;
@@ -884,12 +980,12 @@ __global__ void __launch_bounds__(SECTOR_WARPS * 32, C::DH > 4 ? 3 : 4) k_sector
                         const uchar2 ij = T.tri[e];
                         const float f = xv[j] * inv * (ij.x == ij.y ? 268435456.f : 0.70710678f * 268435456.f);
                         const int q = __float2int_rn(fminf(fmaxf(f, -268435456.f), 268435456.f));
-                        W.c.cmi[c_at<C>(ij.x, ij.y)] = q;
-                        W.c.cmi[c_at<C>(ij.y, ij.x)] = sgn > 0 ? q : -q;
+                        W.c.cmi[ij.x * C::NS + ij.y] = q;
+                        W.c.cmi[ij.y * C::NS + ij.x] = sgn * q;
                     }
                 }
                 __syncwarp();
-                sigma_anchor<C>(T, (const int2 *)W.Vf, (const int2 *)W.Hsf, W.c.cmi, W.s.S64, sgn);
+                sigma_anchor<C>(T, W.Vf, (const int2 *)W.Hsf, W.c.cmi, W.s.S64, sgn);
                 ++n64;
                 double xs = 0.0, xx = 0.0;
                 double s0[C::DH], c0[C::DH];
@@ -899,11 +995,9 @@ __global__ void __launch_bounds__(SECTOR_WARPS * 32, C::DH > 4 ? 3 : 4) k_sector
                     s0[j] = c0[j] = 0.0;
                     if (e < C::NH) {
                         const uchar2 ij = T.tri[e];
-                        constexpr int ST = C::NS | 1;
-                        const long long u = W.s.S64[ij.y * ST + ij.x], w = W.s.S64[ij.x * ST + ij.y];
                         const double wt = ij.x == ij.y ? 1.0 : 1.4142135623730951;
-                        c0[j] = (double)W.c.cmi[c_at<C>(ij.x, ij.y)] * (wt * pow2(-28));
-                        s0[j] = fma(W.hd[ij.x] + W.hd[ij.y], c0[j], (double)(sgn > 0 ? u + w : u - w) * (wt * pow2(E - 55)));
+                        c0[j] = (double)W.c.cmi[ij.x * C::NS + ij.y] * (wt * pow2(-28));
+                        s0[j] = fma(W.hd[ij.x] + W.hd[ij.y], c0[j], ij.x == ij.y && sgn < 0 ? 0.0 : (double)W.s.S64[e] * (wt * pow2(E - 55)));
                         xs = fma(c0[j], s0[j], xs);
                         xx = fma(c0[j], c0[j], xx);
                     }

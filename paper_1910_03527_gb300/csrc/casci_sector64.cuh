@@ -13,31 +13,6 @@
 
 namespace mbe {
 
-// Sums of the K (a power of two) values over the warp; every lane gets all totals.  Each
-// step halves the values that a lane carries, so K = 8 takes 9 additions instead of 40.
-template <int K>
-__device__ __forceinline__ void warp_sum_n(double (&v)[K])
-{
-    const int lane = threadIdx.x & 31;
-    int o = 16;
-#pragma unroll
-    for (int m = K / 2; m >= 1; m >>= 1) {
-        const bool up = lane & o;
-#pragma unroll
-        for (int i = 0; i < m; ++i) {
-            const double send = up ? v[i] : v[i + m];
-            const double keep = up ? v[i + m] : v[i];
-            v[i] = keep + __shfl_xor_sync(FULL, send, o);
-        }
-        o >>= 1;
-    }
-    for (; o > 0; o >>= 1) v[0] += __shfl_xor_sync(FULL, v[0], o);
-    const double s = v[0];
-    // value i was kept by the lanes whose leading bits spell i
-#pragma unroll
-    for (int i = 0; i < K; ++i) v[i] = __shfl_sync(FULL, s, i * (32 / K));
-}
-
 // Shared memory of one warp.
 template <class C>
 struct Sector64 {
@@ -80,7 +55,7 @@ __device__ __forceinline__ void sigma_sector64(const SectorTables<C> &Tb, Sector
             const int2 f = to_fixed(t[j], w);
             int2 *ci = (int2 *)W.c.ci;
             ci[c_at<C>(ij.x, ij.y)] = f;
-            ci[c_at<C>(ij.y, ij.x)] = sgn > 0 ? f : make_int2(-f.x, -f.y);
+            ci[c_at<C>(ij.y, ij.x)] = make_int2(sgn * f.x, sgn * f.y);
         }
     }
     __syncwarp();
@@ -89,7 +64,7 @@ __device__ __forceinline__ void sigma_sector64(const SectorTables<C> &Tb, Sector
     for (int i = 0; i < C::NS; ++i) hi[i] = lo[i] = 0;
     sector_rounds<C>(
         [&](int Ib, int y) {
-            const int e = Tb.list[Ib * C::R + y], J = e >> 8, pr = (e & 255) >> 1, m = -((e & 1) ^ (sgn < 0 ? 1 : 0));
+            const int e = Tb.list[Ib * C::R + y], J = e >> 8, pr = (e & 255) >> 1, m = -((e & 1) ^ ((1 - sgn) >> 1));
             int ch[2 * C::NSH], cl[2 * C::NSH];
 #pragma unroll
             for (int i = 0; i < C::NSH; ++i) {
@@ -116,7 +91,7 @@ __device__ __forceinline__ void sigma_sector64(const SectorTables<C> &Tb, Sector
         },
         [&](int Ib, int J) {
             int2 c = ((const int2 *)W.c.ci)[c_at<C>(Ib, J)];
-            c = sgn > 0 ? c : make_int2(-c.x, -c.y);
+            c = make_int2(sgn * c.x, sgn * c.y);
             const int4 *hs = (const int4 *)(W.m.s.Hsf + J * C::NSP);
 #pragma unroll
             for (int i = 0; i < C::NSP / 2; ++i) {
@@ -154,7 +129,7 @@ __device__ __forceinline__ void sigma_sector64(const SectorTables<C> &Tb, Sector
                 w += W.m.s.u.S[(p * C::NS + ij.x) * ST + ij.y];
             }
             const double wt = ij.x == ij.y ? unit : 1.4142135623730951 * unit;
-            out[j] = fma(W.hd[ij.x] + W.hd[ij.y], t[j], (double)(sgn > 0 ? u + w : u - w) * wt);
+            out[j] = fma(W.hd[ij.x] + W.hd[ij.y], t[j], (double)(u + sgn * w) * wt);
         }
     }
     __syncwarp();
@@ -167,7 +142,7 @@ __device__ __forceinline__ void sigma_sector64(const SectorTables<C> &Tb, Sector
 // with a Newton step (relative error 4e-15), and x is rescaled only when its norm has drifted.
 template <class C, class SIGMA>
 __device__ __forceinline__ PhaseOut davidson_sector64(SIGMA sigma, const double *dg, double (&x)[C::DH], double tol,
-                                                      int min_iter, int max_iter, bool steer)
+                                                      int min_iter, int max_iter, bool steered)
 {
     constexpr int DH = C::DH;
     const int lane = threadIdx.x & 31;
@@ -178,12 +153,13 @@ __device__ __forceinline__ PhaseOut davidson_sector64(SIGMA sigma, const double 
     o.dnorm = 0.0;
     double lam = 0.0, rn = 0.0, best = 1e300;
     int stall = 0;
-    bool first = true, have_p = false;
+    int first = opaque(1);
+    bool have_p = false;
     {
         double s = 0.0;
 #pragma unroll
         for (int j = 0; j < DH; ++j) s = fma(x[j], x[j], s);
-        s = 1.0 / sqrt(warp_sum(s));
+        s = inv_sqrt64(warp_sum(s));
 #pragma unroll
         for (int j = 0; j < DH; ++j) {
             t[j] = x[j] = x[j] * s;
@@ -191,6 +167,7 @@ __device__ __forceinline__ PhaseOut davidson_sector64(SIGMA sigma, const double 
         }
     }
     for (int it = 0;;) {
+        const bool steer = opaque(steered);
         if (!first) {
             double v[4] = {0.0, 0.0, 0.0, 0.0};  // |r|^2, x.t, p.t, |t|^2
 #pragma unroll
@@ -257,7 +234,7 @@ __device__ __forceinline__ PhaseOut davidson_sector64(SIGMA sigma, const double 
                 if (!steer && rn > tol) o.status = MBE_STATUS_MAXITER;
                 break;
             }
-            const double tinv = 1.0 / tn;
+            const double tinv = div64(1.0, tn);
 #pragma unroll
             for (int j = 0; j < DH; ++j) t[j] *= tinv;
         }
@@ -271,7 +248,7 @@ __device__ __forceinline__ PhaseOut davidson_sector64(SIGMA sigma, const double 
                 xh = fma(x[j], ht[j], xh);
             }
             lam = warp_sum(xh);
-            first = false;
+            first = opaque(0);
             continue;
         }
         ++it;
@@ -299,7 +276,7 @@ __device__ __forceinline__ PhaseOut davidson_sector64(SIGMA sigma, const double 
         double q0 = -w2 * y[0], q1 = y[1] - w2 * y[1], q2 = y[2] - w2 * y[2];
         const double zn = sqrt(q0 * q0 + q1 * q1 + q2 * q2);
         have_p = zn > tiny_norm<double>() * 1e-3;
-        const double zi = have_p ? 1.0 / zn : 0.0;
+        const double zi = have_p ? div64(1.0, zn) : 0.0;
         q0 *= zi;
         q1 *= zi;
         q2 *= zi;
@@ -316,9 +293,9 @@ __device__ __forceinline__ PhaseOut davidson_sector64(SIGMA sigma, const double 
             n[1] = fma(nx, nhx, n[1]);
         }
         warp_sum_n<2>(n);
-        lam = n[1] / n[0];
+        lam = div64(n[1], n[0]);
         if (!(fabs(n[0] - 1.0) <= 4e-15)) {
-            const double sc = 1.0 / sqrt(n[0]);
+            const double sc = inv_sqrt64(n[0]);
 #pragma unroll
             for (int j = 0; j < DH; ++j) {
                 x[j] *= sc;
@@ -455,10 +432,12 @@ __global__ void __launch_bounds__(SECTOR_WARPS * 32, C::DH > 4 ? 2 : 3) k_sector
         const SectorStart st = sector_setup<C>(a, T, W.A, Vp, Hsp, W.hd, W.m.s.u.su.h, W.m.s.u.su.dsum, W.dg);
         double vmax = 0.0;
         bool bad = false;
+#pragma unroll 1
         for (int e = lane; e < C::PT; e += 32) {
             vmax = fmax(vmax, 0.5 * fabs(Vp[e]));
             bad = bad || !isfinite(Vp[e]);
         }
+#pragma unroll 1
         for (int e = lane; e < C::NH; e += 32) {
             const uchar2 ij = T.tri[e];
             if (ij.x != ij.y) vmax = fmax(vmax, fabs(Hsp[e]));
@@ -466,10 +445,12 @@ __global__ void __launch_bounds__(SECTOR_WARPS * 32, C::DH > 4 ? 2 : 3) k_sector
         }
         const int E = fixed_exponent(vmax);
         const double scale = pow2(55 - E);
+#pragma unroll 1
         for (int e = lane; e < C::PT; e += 32) {
             const uchar2 xy = T.ptri[e];
             W.m.s.Vf[xy.x * C::P + xy.y] = W.m.s.Vf[xy.y * C::P + xy.x] = to_fixed(0.5 * Vp[e], scale);
         }
+#pragma unroll 1
         for (int e = lane; e < C::NH; e += 32) {
             const uchar2 ij = T.tri[e];
             const int2 f = ij.x == ij.y ? make_int2(0, 0) : to_fixed(Hsp[e], scale);
@@ -485,9 +466,9 @@ __global__ void __launch_bounds__(SECTOR_WARPS * 32, C::DH > 4 ? 2 : 3) k_sector
         bool degen = false;
         const int n32 = REDO ? a.pstate[2 * t + 1] : 0;  // the mixed solver's float32 work
 #pragma unroll 1
-        for (int sector = 0; sector < 2; ++sector) {
+        for (int sector = opaque(0); sector < 2; ++sector) {
             if (sector == 1 && (status != MBE_STATUS_OK || a.even_only)) break;
-            const int sgn = sector == 0 ? 1 : -1, g = sector == 0 ? st.g : st.go;
+            const int sgn = opaque(sector == 0 ? 1 : -1), g = sector == 0 ? st.g : st.go;
 #pragma unroll
             for (int j = 0; j < C::DH; ++j) {
                 const int e = lane + 32 * j;
@@ -501,7 +482,7 @@ __global__ void __launch_bounds__(SECTOR_WARPS * 32, C::DH > 4 ? 2 : 3) k_sector
             // one call site keeps the kernel within the instruction cache
             bool lose = false;
 #pragma unroll 1
-            for (int pass = sector == 1 ? 0 : 1; pass < 2 && !lose; ++pass) {
+            for (int pass = opaque(sector == 1 ? 0 : 1); pass < 2 && !lose; ++pass) {
                 const bool decide = pass == 0;
                 const PhaseOut o = davidson_sector64<C>(sigma, W.dg, x, decide ? SECTOR_TOL : a.tol, 0, a.max_iter, decide);
                 n64 += o.nsig;
