@@ -20,6 +20,15 @@
 
 namespace mbe {
 
+// The block's dynamic shared memory.  Named by its symbol wherever it is read: through a pointer
+// kept in a struct the compiler loses the address space, and the tiled product took twice as
+// many instructions (generic loads with 64-bit addresses).
+__device__ __forceinline__ char *block_shared()
+{
+    extern __shared__ __align__(16) char smem[];
+    return smem;
+}
+
 constexpr int BLOCK_THREADS = 512;  // one block per SM: 128 registers a thread, up to 227 KB
 constexpr int GEMM_MAX_N = 9;       // orbitals up to which sigma is the tiled product
 constexpr int GEMM_T_BYTES = 48 * 1024;
@@ -54,7 +63,8 @@ __host__ __device__ inline BlockSlot block_slot(int ns)
 
 // Shapes of the tiled sigma of one string class.
 struct GemmShape {
-    int cst;        // row stride of c and of T (strings, padded to 4)
+    int cst;        // row stride of T and of the fixed-point c (strings, padded to 4)
+    int fst;        // row stride of the float32 c (not a multiple of 32: its columns are written too)
     int pst;        // row stride of the float32 V (pairs, padded to 6)
     int rs;         // row stride of the lists
     int np, tiles;  // pair groups, tiles per alpha string
@@ -67,6 +77,7 @@ __host__ __device__ inline GemmShape gemm_shape(int n, int ns, int r)
     GemmShape s;
     const int P = n * (n + 1) / 2, tp = sizeof(T) == 8 ? 3 : 6;
     s.cst = hs_stride(ns);
+    s.fst = s.cst % 32 == 0 ? s.cst + 4 : s.cst;
     s.pst = (P + 5) / 6 * 6;
     s.rs = r | 1;
     s.np = (P + tp - 1) / tp;
@@ -75,6 +86,7 @@ __host__ __device__ inline GemmShape gemm_shape(int n, int ns, int r)
     const int fit = GEMM_T_BYTES / (P * s.cst * (int)sizeof(T));
     if (s.g > fit) s.g = fit;
     if (s.g > ns) s.g = ns;
+    if (s.g > 1) s.g &= ~1;  // (strings are taken in pairs)
     if (s.g < 1) s.g = 1;
     return s;
 }
@@ -107,7 +119,13 @@ __host__ __device__ inline BlockMem block_mem(int n, bool gemm, int ns, int r, i
     S.off_g1 = o; o = al16(o + 8 * n * n);
     S.off_hd = o; o = al16(o + (gemm ? 8 * ns : 0));
     S.off_list = o; o = al16(o + (gemm ? 2 * ns * (r | 1) : 0));
-    S.off_c = o; o = al16(o + (gemm ? 8 * ns * hs_stride(ns) : 0));
+    S.off_c = o;
+    if (gemm) {
+        // fixed point: c; float32: c, V twice over with both signs, list offsets (see sigma_gemm)
+        const GemmShape a = gemm_shape<float>(n, ns, r);
+        const int f = al16(4 * ns * a.fst) + 16 * P * a.pst + 4 * ns * r;
+        o = al16(o + (f > 8 * ns * a.cst ? f : 8 * ns * a.cst));
+    }
     S.off_T = o;
     if (gemm) {
         const GemmShape a = gemm_shape<float>(n, ns, r), b = gemm_shape<double>(n, ns, r);
@@ -125,18 +143,13 @@ struct BlockProblem {
     bool gemm;
     bool bad;         // an element of V or Hs is not finite (float64 sigma: fixed point cannot hold it)
     int E;            // fixed-point exponent
-    char *smem;
     BlockMem S;
     double *full;     // [Ns][stride] scratch of the slot
 };
 
-__device__ __forceinline__ void ffma2(unsigned long long &d, unsigned long long a, unsigned long long b)
+__device__ __forceinline__ uint64_t dup2(float v)
 {
-    asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(d) : "l"(a), "l"(b));
-}
-__device__ __forceinline__ unsigned long long dup2(float v)
-{
-    const unsigned long long u = __float_as_uint(v);
+    const uint64_t u = __float_as_uint(v);
     return u << 32 | u;
 }
 
@@ -154,33 +167,47 @@ __device__ inline void expand_full(const Problem &pb, const T *v, T *full, int l
     }
 }
 
-// M = C Hs for the float32 product: 4 x 4 tiles, c from shared memory, Hs through L1.
-__device__ inline void same_spin(const Problem &pb, int ld, const float *c, const float *Hs, float *M)
+// M = C Hs for the float32 product: 8 x 4 tiles, c from shared memory by its rows (C[i][J] is
+// sgn C[J][i]), Hs through L1.
+__device__ inline void same_spin(const Problem &pb, int ld, int fst, const float *c, const float *Hs, float *M)
 {
-    const int nt = ld / 4;
-    for (int q = threadIdx.x; q < nt * nt; q += blockDim.x) {
-        const int i0 = q / nt * 4, j0 = (q - q / nt * nt) * 4;
-        const float *c0 = c + i0 * ld, *c1 = c + (i0 + 1 < pb.Ns ? i0 + 1 : i0) * ld,
-                    *c2 = c + (i0 + 2 < pb.Ns ? i0 + 2 : i0) * ld, *c3 = c + (i0 + 3 < pb.Ns ? i0 + 3 : i0) * ld;
-        float4 a0 = make_float4(0, 0, 0, 0), a1 = a0, a2 = a0, a3 = a0;
+    const int nj = ld / 4, ni = (pb.Ns + 7) / 8;
+    for (int q = threadIdx.x; q < ni * nj; q += blockDim.x) {
+        const int i0 = q / nj * 8, j0 = (q - q / nj * nj) * 4;
+        const int i1 = i0 + 4 < fst ? i0 + 4 : i0;  // (past the last string: not stored)
+        uint64_t a[4][4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+#pragma unroll
+            for (int j = 0; j < 4; ++j) a[i][j] = 0ull;
 #pragma unroll 4
         for (int J = 0; J < pb.Ns; ++J) {
             const float4 h = *(const float4 *)(Hs + J * ld + j0);
-            const float x0 = c0[J], x1 = c1[J], x2 = c2[J], x3 = c3[J];
-            a0.x = fmaf(x0, h.x, a0.x); a0.y = fmaf(x0, h.y, a0.y); a0.z = fmaf(x0, h.z, a0.z); a0.w = fmaf(x0, h.w, a0.w);
-            a1.x = fmaf(x1, h.x, a1.x); a1.y = fmaf(x1, h.y, a1.y); a1.z = fmaf(x1, h.z, a1.z); a1.w = fmaf(x1, h.w, a1.w);
-            a2.x = fmaf(x2, h.x, a2.x); a2.y = fmaf(x2, h.y, a2.y); a2.z = fmaf(x2, h.z, a2.z); a2.w = fmaf(x2, h.w, a2.w);
-            a3.x = fmaf(x3, h.x, a3.x); a3.y = fmaf(x3, h.y, a3.y); a3.z = fmaf(x3, h.z, a3.z); a3.w = fmaf(x3, h.w, a3.w);
+            const ulonglong2 c0 = *(const ulonglong2 *)(c + J * fst + i0), c1 = *(const ulonglong2 *)(c + J * fst + i1);
+            const uint64_t cc[4] = {c0.x, c0.y, c1.x, c1.y};
+            const uint64_t hh[4] = {dup2(h.x), dup2(h.y), dup2(h.z), dup2(h.w)};
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+#pragma unroll
+                for (int j = 0; j < 4; ++j) ffma2(a[i][j], cc[i], hh[j]);
         }
-        *(float4 *)(M + i0 * ld + j0) = a0;
-        if (i0 + 1 < pb.Ns) *(float4 *)(M + (i0 + 1) * ld + j0) = a1;
-        if (i0 + 2 < pb.Ns) *(float4 *)(M + (i0 + 2) * ld + j0) = a2;
-        if (i0 + 3 < pb.Ns) *(float4 *)(M + (i0 + 3) * ld + j0) = a3;
+        const float sg = pb.sector > 0 ? 1.f : -1.f;
+#pragma unroll
+        for (int i = 0; i < 8; ++i)
+            if (i0 + i < pb.Ns) {
+                float4 o;
+                const int h = 32 * (i & 1);
+                o.x = sg * __uint_as_float((uint32_t)(a[i >> 1][0] >> h));
+                o.y = sg * __uint_as_float((uint32_t)(a[i >> 1][1] >> h));
+                o.z = sg * __uint_as_float((uint32_t)(a[i >> 1][2] >> h));
+                o.w = sg * __uint_as_float((uint32_t)(a[i >> 1][3] >> h));
+                *(float4 *)(M + (i0 + i) * ld + j0) = o;
+            }
     }
 }
 
 // The same on integers (Hs without its diagonal): 2 x 2 tiles, one int64 per element.
-__device__ inline void same_spin(const Problem &pb, int ld, const int2 *c, const int2 *Hs, long long *M)
+__device__ inline void same_spin(const Problem &pb, int ld, int, const int2 *c, const int2 *Hs, long long *M)
 {
     const int nt = ld / 2;
     for (int q = threadIdx.x; q < nt * nt; q += blockDim.x) {
@@ -208,42 +235,38 @@ __device__ inline void same_spin(const Problem &pb, int ld, const int2 *c, const
     }
 }
 
-// One tile of T in float32: 4 strings x 6 pairs (pairs of pairs in one 64-bit register).
-__device__ __forceinline__ void gemm_tile(const Problem &pb, const GemmShape &s, const uint16_t *la, const float *c,
-                                          const float *V, int j0, int pg, float *T)
+// One tile of T in float32: 4 strings x 6 pairs, two strings per instruction (fma.rn.f32x2).
+// Per list entry one offset pair, the four strings and six pairs (V holds each value twice).
+__device__ __forceinline__ void gemm_tile(const Problem &pb, const GemmShape &s, const uint32_t *la, const char *c,
+                                          const char *V, int j0, int pg, float *T)
 {
-    unsigned long long a[4][3];
+    uint64_t a[6][2];
 #pragma unroll
-    for (int i = 0; i < 4; ++i)
-#pragma unroll
-        for (int k = 0; k < 3; ++k) a[i][k] = 0ull;
-#pragma unroll 2
+    for (int k = 0; k < 6; ++k) a[k][0] = a[k][1] = 0ull;
+    c += 4 * j0;
+    V += 48 * pg;
+#pragma unroll 4
     for (int x = 0; x < pb.R; ++x) {
-        const int e = la[x];
-        const float4 cv = *(const float4 *)(c + (e >> 7) * s.cst + j0);
-        const unsigned long long *v = (const unsigned long long *)(V + ((e >> 1) & 63) * s.pst + pg * 6);
-        const unsigned long long v0 = v[0], v1 = v[1], v2 = v[2];
-        const float cs[4] = {cv.x, cv.y, cv.z, cv.w};
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            const unsigned long long d = dup2(flip_if(cs[i], e & 1));
-            ffma2(a[i][0], v0, d);
-            ffma2(a[i][1], v1, d);
-            ffma2(a[i][2], v2, d);
-        }
+        const uint32_t e = la[x];
+        const ulonglong2 cv = *(const ulonglong2 *)(c + ((e & 0xffffu) << 4));
+        const ulonglong2 *v = (const ulonglong2 *)(V + (e >> 16 << 4));
+        const ulonglong2 v0 = v[0], v1 = v[1], v2 = v[2];
+        ffma2(a[0][0], v0.x, cv.x);
+        ffma2(a[0][1], v0.x, cv.y);
+        ffma2(a[1][0], v0.y, cv.x);
+        ffma2(a[1][1], v0.y, cv.y);
+        ffma2(a[2][0], v1.x, cv.x);
+        ffma2(a[2][1], v1.x, cv.y);
+        ffma2(a[3][0], v1.y, cv.x);
+        ffma2(a[3][1], v1.y, cv.y);
+        ffma2(a[4][0], v2.x, cv.x);
+        ffma2(a[4][1], v2.x, cv.y);
+        ffma2(a[5][0], v2.y, cv.x);
+        ffma2(a[5][1], v2.y, cv.y);
     }
 #pragma unroll
-    for (int k = 0; k < 6; ++k) {
-        const int p = pg * 6 + k;
-        if (p < pb.P) {
-            float4 o;
-            o.x = __uint_as_float((unsigned)(a[0][k >> 1] >> (32 * (k & 1))));
-            o.y = __uint_as_float((unsigned)(a[1][k >> 1] >> (32 * (k & 1))));
-            o.z = __uint_as_float((unsigned)(a[2][k >> 1] >> (32 * (k & 1))));
-            o.w = __uint_as_float((unsigned)(a[3][k >> 1] >> (32 * (k & 1))));
-            *(float4 *)(T + p * s.cst + j0) = o;
-        }
-    }
+    for (int k = 0; k < 6; ++k)
+        if (pg * 6 + k < pb.P) *(ulonglong2 *)(T + (pg * 6 + k) * s.cst + j0) = make_ulonglong2(a[k][0], a[k][1]);
 }
 
 // One tile of T in fixed point: 4 strings x 3 pairs.
@@ -292,55 +315,83 @@ __device__ __noinline__ void sigma_gemm(const BlockProblem &B, const T *src, T *
     const Problem &pb = B.pb;
     const int Ns = pb.Ns, tid = threadIdx.x, nt = blockDim.x, R = pb.R, sgn = pb.sector;
     const GemmShape s = gemm_shape<T>(pb.n, Ns, R);
-    E *c = (E *)(B.smem + B.S.off_c);
-    A *Tm = (A *)(B.smem + B.S.off_T);
-    const uint16_t *list = (const uint16_t *)(B.smem + B.S.off_list);
-    const double *hd = (const double *)(B.smem + B.S.off_hd);
-    const E *V = (const E *)(B.smem + (F64 ? B.S.off_V64 : B.S.off_V32));
+    E *c = (E *)(block_shared() + B.S.off_c);
+    A *Tm = (A *)(block_shared() + B.S.off_T);
+    const uint16_t *list = (const uint16_t *)(block_shared() + B.S.off_list);
+    const double *hd = (const double *)(block_shared() + B.S.off_hd);
     A *M = (A *)B.full;
+    const int cld = F64 ? s.cst : s.fst;
+    // float32: behind c, V with every value twice (rows 2 pair + neg), and the lists as offsets
+    // of the rows of c (low half) and V (high half) in units of 16 bytes
+    char *Vd = block_shared() + B.S.off_c + al16(4 * Ns * s.fst);
+    uint32_t *list32 = (uint32_t *)(Vd + 16 * pb.P * s.pst);
     {
         int ia = 0, ib = 0;
         tri_advance(ia, ib, tid, Ns);
         for (int h = tid; h < pb.N; h += nt) {
             if constexpr (F64) {
                 const int2 f = to_fixed(src[h], ia == ib ? 36028797018963968.0 : 0.70710678118654752 * 36028797018963968.0);
-                c[ia * s.cst + ib] = f;
-                c[ib * s.cst + ia] = sgn > 0 ? f : make_int2(-f.x, -f.y);
+                c[ia * cld + ib] = f;
+                c[ib * cld + ia] = sgn > 0 ? f : make_int2(-f.x, -f.y);
             } else {
                 const float f = ia == ib ? src[h] : 0.70710678118654752f * src[h];
-                c[ia * s.cst + ib] = f;
-                c[ib * s.cst + ia] = sgn > 0 ? f : -f;
+                c[ia * cld + ib] = f;
+                c[ib * cld + ia] = sgn > 0 ? f : -f;
             }
             tri_advance(ia, ib, nt, Ns);
         }
-        for (int q = tid; q < Ns * (s.cst - Ns); q += nt) c[q / (s.cst - Ns) * s.cst + Ns + q % (s.cst - Ns)] = E{};
+        for (int q = tid; q < Ns * (cld - Ns); q += nt) c[q / (cld - Ns) * cld + Ns + q % (cld - Ns)] = E{};
+        if constexpr (!F64) {
+            const float *V32 = (const float *)(block_shared() + B.S.off_V32);
+            for (int q = tid; q < pb.P * s.pst; q += nt) {
+                const int x = q / s.pst, y = q - x * s.pst;
+                ((float2 *)Vd)[2 * x * s.pst + y] = make_float2(V32[q], V32[q]);
+                ((float2 *)Vd)[(2 * x + 1) * s.pst + y] = make_float2(-V32[q], -V32[q]);
+            }
+            for (int q = tid; q < Ns * R; q += nt) {
+                const int e = list[q / R * s.rs + q % R];
+                list32[q] = (uint32_t)((e >> 7) * (s.fst / 4)) | (uint32_t)((e & 127) * (s.pst / 2)) << 16;
+            }
+        }
     }
     __syncthreads();
-    same_spin(pb, s.cst, c, F64 ? (const E *)pb.Hs64 : (const E *)pb.Hs32, M);
+    same_spin(pb, s.cst, cld, c, F64 ? (const E *)pb.Hs64 : (const E *)pb.Hs32, M);
     const int nj = s.cst / 4;
+    // Strings are taken from both ends of the list, so that each pair of them has Ns + 1 elements
+    // with Ia <= Ib.
     for (int I0 = 0; I0 < Ns; I0 += s.g) {
         const int gc = min(s.g, Ns - I0);
+        auto string = [&](int i) { return i & 1 ? Ns - 1 - (i >> 1) : i >> 1; };
         for (int q = tid; q < gc * s.tiles; q += nt) {
-            const int g = q / s.tiles, r = q - g * s.tiles, pg = r / nj, jj = r - pg * nj;
-            gemm_tile(pb, s, list + (I0 + g) * s.rs, c, V, 4 * jj, pg, Tm + g * pb.P * s.cst);
+            const int g = q / s.tiles, r = q - g * s.tiles, pg = r / nj, jj = r - pg * nj, Ia = string(I0 + g);
+            if constexpr (F64)
+                gemm_tile(pb, s, list + Ia * s.rs, c, (const int2 *)(block_shared() + B.S.off_V64), 4 * jj, pg,
+                          Tm + g * pb.P * s.cst);
+            else
+                gemm_tile(pb, s, list32 + Ia * R, (const char *)c, Vd, 4 * jj, pg, Tm + g * pb.P * s.cst);
         }
         __syncthreads();  // (also orders M, written above, before its first use)
-        const int two = 2 * gc * Ns <= nt ? 1 : 0;  // two threads per element where they fit
-        for (int q0 = 0; q0 < (gc * Ns) << two; q0 += nt) {
-            const int q = q0 + tid, el = q >> two, g = el / Ns, Ib = el - g * Ns, Ia = I0 + g;
-            const bool on = g < gc && Ib >= Ia;
+        const int n1 = Ns + 1, ne = (gc + 1) / 2 * n1;
+        int split = 0;  // 2^split threads per element, where they fit
+        while (split < 3 && (ne << (split + 1)) <= nt) ++split;
+        for (int q0 = 0; q0 < ne << split; q0 += nt) {
+            const int q = q0 + tid, el = q >> split, pr = el / n1, r = el - pr * n1;
+            const int first = string(I0 + 2 * pr), len = Ns - first;  // elements of the pair's first string
+            const int g = 2 * pr + (r < len ? 0 : 1), Ia = r < len ? first : string(I0 + g), Ib = Ia + r - (r < len ? 0 : len);
+            const bool on = g < gc && Ib < Ns;
             A acc = 0;
             if (on) {
                 const A *t = Tm + g * pb.P * s.cst;
                 const uint16_t *lb = list + Ib * s.rs;
-                for (int y = two ? q & 1 : 0; y < R; y += 1 + two) {
+#pragma unroll 4
+                for (int y = q & ((1 << split) - 1); y < R; y += 1 << split) {
                     const int e = lb[y];
                     const A v = t[((e >> 1) & 63) * s.cst + (e >> 7)];
                     acc += e & 1 ? -v : v;
                 }
             }
-            if (two) acc += __shfl_xor_sync(FULL, acc, 1);
-            if (on && !(two && (q & 1))) {
+            for (int o = 1; o < 1 << split; o <<= 1) acc += __shfl_xor_sync(FULL, acc, o);
+            if (on && (q & ((1 << split) - 1)) == 0) {
                 const A mt = M[Ib * s.cst + Ia];
                 const int h = Ia * Ns - Ia * (Ia - 1) / 2 + Ib - Ia;
                 acc += M[Ia * s.cst + Ib] + (sgn > 0 ? mt : -mt);
@@ -360,7 +411,7 @@ __device__ __noinline__ void sigma_gemm(const BlockProblem &B, const T *src, T *
 
 // sigma of a packed sector vector; ends with a barrier.
 template <typename T>
-__device__ inline void sigma_block(const BlockProblem &B, const T *src, T *dst)
+__device__ __noinline__ void sigma_block(const BlockProblem &B, const T *src, T *dst)
 {
     const Problem &pb = B.pb;
     if (B.gemm) sigma_gemm<T>(B, src, dst);
@@ -390,17 +441,22 @@ __device__ inline void sigma_block(const BlockProblem &B, const T *src, T *dst)
 
 // Lowest eigenpair of the m x m symmetric Rayleigh matrix G (shared memory, float64, row
 // stride MMAX) by the whole block: a float32 Jacobi on G - G00 I in round-robin order, m / 2
-// disjoint rotations at a time, one element of the matrix and of the eigenvectors per thread
-// (m - 1 steps per sweep, where rotating one pair after the other in one warp took m (m - 1)
+// disjoint rotations at a time (one lane each), then one element of the matrix and of the
+// eigenvectors per thread (m - 1 steps per sweep, where rotating one pair after the other in one warp took m (m - 1)
 // / 2 of about the same length); in float64 then two Newton steps in that eigenbasis,
 // z = y - sum_{k != 0} e_k (e_k . r) / (theta_k - theta),  r = G y - theta y,
 // theta = y.G y, which make the lowest pair float64-accurate (one warp).
 // Output: y[0..m) (unit norm), y2 (the second lowest, which seeds the thick restart), and
-// misc[0] = theta; ends with a barrier.  buf: 4 MMAX^2 floats.
+// misc[0] = theta; ends with a barrier.
 template <bool REFINE>
-__device__ __noinline__ void small_eig_block(const double *G, int m, float *buf, float *ev, double *y, double *y2,
-                                             double *r, double *misc)
+__device__ __noinline__ void small_eig_block(const BlockMem &S, int m)
 {
+    char *smem = block_shared();
+    const double *G = (const double *)(smem + S.off_G);
+    float *buf = (float *)(smem + S.off_J), *ev = (float *)(smem + S.off_ev);
+    double *y = (double *)(smem + S.off_y), *y2 = (double *)(smem + S.off_yp), *r = (double *)(smem + S.off_r),
+           *misc = (double *)(smem + S.off_misc);
+    __shared__ float2 rot[MMAX + 1];
     const int tid = threadIdx.x, i = tid / MMAX, j = tid - i * MMAX, lane = tid & 31;
     const bool on = i < m && j < m;
     const double shift = G[0];
@@ -411,20 +467,6 @@ __device__ __noinline__ void small_eig_block(const double *G, int m, float *buf,
     }
     __syncthreads();
     const int M = m + (m & 1);  // an odd matrix gets an idle partner
-    // the rotation of row or column u with its partner: coefficients of itself and of the partner
-    auto rotation = [&](int u, int v, float &c, float &s) {
-        c = 1.f;
-        s = 0.f;
-        if (v >= m) return;
-        const int p = u < v ? u : v, q = u < v ? v : u;
-        const float apq = A[p * MMAX + q];
-        if (fabsf(apq) < 1e-36f) return;
-        const float th = (A[q * MMAX + q] - A[p * MMAX + p]) / (2.0f * apq);
-        float t = 1.0f / (fabsf(th) + sqrtf(th * th + 1.0f));
-        if (th < 0.0f) t = -t;
-        c = rsqrtf(t * t + 1.0f);
-        s = u < v ? -t * c : t * c;
-    };
     for (int sweep = 0; sweep < 10 && m > 1; ++sweep) {
         float dia = 0.f;
         bool big = false;
@@ -435,22 +477,38 @@ __device__ __noinline__ void small_eig_block(const double *G, int m, float *buf,
         }
         if (!__syncthreads_or(big)) break;
         for (int step = 0; step < M - 1; ++step) {
+            auto partner = [&](int u) {
+                if (u == M - 1) return step;
+                if (u == step) return M - 1;
+                const int v = 2 * step - u;
+                return v < 0 ? v + M - 1 : v >= M - 1 ? v - (M - 1) : v;
+            };
+            // the rotations of the step, one lane each: coefficients of a row itself and of its partner
+            if (tid < M) {
+                const int v = partner(tid);
+                if (tid < v) {
+                    float c = 1.f, sn = 0.f;
+                    const float apq = v < m ? A[tid * MMAX + v] : 0.f;
+                    if (fabsf(apq) >= 1e-36f) {
+                        const float th = (A[v * MMAX + v] - A[tid * MMAX + tid]) / (2.0f * apq);
+                        float t = 1.0f / (fabsf(th) + sqrtf(th * th + 1.0f));
+                        if (th < 0.0f) t = -t;
+                        c = rsqrtf(t * t + 1.0f);
+                        sn = t * c;
+                    }
+                    rot[tid] = make_float2(c, -sn);
+                    rot[v] = make_float2(c, sn);
+                }
+            }
+            __syncthreads();
             if (on) {
-                auto partner = [&](int u) {
-                    if (u == M - 1) return step;
-                    if (u == step) return M - 1;
-                    const int v = 2 * step - u;
-                    return v < 0 ? v + M - 1 : v >= M - 1 ? v - (M - 1) : v;
-                };
                 const int pi = partner(i), pj = partner(j);
-                float ci, si, cj, sj;
-                rotation(i, pi, ci, si);
-                rotation(j, pj, cj, sj);
+                const float2 ri = rot[i], rj = rot[j];
                 const int ui = pi < m ? pi : i, uj = pj < m ? pj : j;
-                const float a0 = cj * A[i * MMAX + j] + sj * A[i * MMAX + uj];
-                const float a1 = cj * A[ui * MMAX + j] + sj * A[ui * MMAX + uj];
-                A2[tid] = pi == j ? 0.0f : ci * a0 + si * a1;
-                E2[tid] = cj * E[i * MMAX + j] + sj * E[i * MMAX + uj];
+                const float a0 = rj.x * A[i * MMAX + j] + rj.y * A[i * MMAX + uj];
+                const float a1 = rj.x * A[ui * MMAX + j] + rj.y * A[ui * MMAX + uj];
+                A2[tid] = pi == j ? 0.0f : ri.x * a0 + ri.y * a1;
+                E2[tid] = rj.x * E[i * MMAX + j] + rj.y * E[i * MMAX + uj];
             }
             __syncthreads();
             float *z = A;
@@ -527,19 +585,45 @@ __device__ __noinline__ void small_eig_block(const double *G, int m, float *buf,
     __syncthreads();
 }
 
-// Sums of the first k of the values v[0..KRED) over the block; every thread gets the
-// totals.  Two barriers: the warps' sums, then one warp per value.  red: 32 * KRED elements.
-template <typename T>
-__device__ inline void block_sums(T (&v)[KRED], int k, T *red)
+// Sums of K values over the block; every thread gets the totals.  Two barriers.
+template <int K, typename T>
+__device__ __forceinline__ void block_sums(T (&v)[K], T *red)
 {
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
 #pragma unroll
-    for (int i = 0; i < KRED; ++i)
-        if (i < k) v[i] = warp_sum(v[i]);
+    for (int i = 0; i < K; ++i) v[i] = warp_sum(v[i]);
     if (lane == 0)
 #pragma unroll
-        for (int i = 0; i < KRED; ++i)
-            if (i < k) red[w * KRED + i] = v[i];
+        for (int i = 0; i < K; ++i) red[w * KRED + i] = v[i];
+    __syncthreads();
+    T *tot = red + 31 * KRED;
+    if (w < K) {
+        const T s = warp_sum(lane < nw ? red[lane * KRED + w] : (T)0);
+        if (lane == 0) tot[w] = s;
+    }
+    __syncthreads();
+#pragma unroll
+    for (int i = 0; i < K; ++i) v[i] = tot[i];
+}
+
+// The same for the first k <= KRED of the values of v, which end up in tot[0..k) (shared).  A
+// warp folds the values and its lanes at the same time: 31 exchanges, after which lane i holds
+// the sum of value i.
+template <typename T>
+__device__ __forceinline__ const T *block_sums_many(T (&v)[32], int k, T *red)
+{
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
+#pragma unroll
+    for (int m = 16; m >= 1; m >>= 1) {
+        const bool up = lane & m;
+#pragma unroll
+        for (int i = 0; i < m; ++i) {
+            const T send = up ? v[i] : v[i + m];
+            const T keep = up ? v[i + m] : v[i];
+            v[i] = keep + __shfl_xor_sync(FULL, send, m);
+        }
+    }
+    if (lane < KRED) red[w * KRED + lane] = v[0];
     __syncthreads();
     T *tot = red + 31 * KRED;
     for (int i = w; i < k; i += nw) {
@@ -547,9 +631,7 @@ __device__ inline void block_sums(T (&v)[KRED], int k, T *red)
         if (lane == 0) tot[i] = s;
     }
     __syncthreads();
-#pragma unroll
-    for (int i = 0; i < KRED; ++i)
-        if (i < k) v[i] = tot[i];
+    return tot;
 }
 
 // The vectors are read and written 16 bytes at a time; the elements between N and the next
@@ -573,13 +655,14 @@ struct alignas(16) Pack {
 template <typename T>
 __device__ __noinline__ PhaseOut davidson_block(const BlockProblem &B, T *Vp, T *Wp, size_t ld_, T *xp, T *tp, double tol,
                                                 int min_iter, int max_iter, int steer, double shift = 0.0,
-                                                bool anch = false, int mmax = MMAX)
+                                                bool anchored = false, int mmax = MMAX)
 {
     using K = Pack<T>;
+    bool anch = anchored;
     constexpr int VL = K::L;
     const Problem &pb = B.pb;
     const BlockMem &S = B.S;
-    char *smem = B.smem;
+    char *smem = block_shared();
     const int tid = threadIdx.x, nt = blockDim.x, N = (pb.N + VL - 1) / VL;  // packs
     const size_t ld = ld_ / VL;
     K *V = (K *)Vp, *W = (K *)Wp, *x = (K *)xp, *tx = (K *)tp;
@@ -593,7 +676,7 @@ __device__ __noinline__ PhaseOut davidson_block(const BlockProblem &B, T *Vp, T 
     o.status = MBE_STATUS_OK;
     o.dnorm = 0.0;
     const T shT = (T)shift, shT_lo = (T)(shift - (double)shT);
-    T v[KRED];
+    T v1[1], v2[2];
     auto dot = [&](const K &a, const K &b, T s) {
 #pragma unroll
         for (int l = 0; l < VL; ++l) s = fma(a.e[l], b.e[l], s);
@@ -612,10 +695,10 @@ __device__ __noinline__ PhaseOut davidson_block(const BlockProblem &B, T *Vp, T 
         }
     };
     if (!anch) {
-        v[0] = 0;
-        for (int d = tid; d < N; d += nt) v[0] = dot(x[d], x[d], v[0]);
-        block_sums<T>(v, 1, red);
-        const T inv = (T)1 / sqrt(v[0]);
+        v1[0] = 0;
+        for (int d = tid; d < N; d += nt) v1[0] = dot(x[d], x[d], v1[0]);
+        block_sums(v1, red);
+        const T inv = (T)1 / sqrt(v1[0]);
         for (int d = tid; d < N; d += nt) {
             K q = x[d];
 #pragma unroll
@@ -625,10 +708,10 @@ __device__ __noinline__ PhaseOut davidson_block(const BlockProblem &B, T *Vp, T 
         __syncthreads();
         sigma_block<T>(B, (const T *)V, (T *)W);
         ++o.nsig;
-        v[0] = 0;
-        for (int d = tid; d < N; d += nt) v[0] = dot(V[d], W[d], v[0]);
-        block_sums<T>(v, 1, red);
-        if (tid == 0) G[0] = (double)v[0];
+        v1[0] = 0;
+        for (int d = tid; d < N; d += nt) v1[0] = dot(V[d], W[d], v1[0]);
+        block_sums(v1, red);
+        if (tid == 0) G[0] = (double)v1[0];
     } else if (tid == 0) {
         G[0] = 0.0;  // x0.r0 = 0: shift is x0's Rayleigh quotient
     }
@@ -639,13 +722,12 @@ __device__ __noinline__ PhaseOut davidson_block(const BlockProblem &B, T *Vp, T 
     T best = (T)3e38;
     int stall = 0;
     for (int it = 0;; ++it) {
-        small_eig_block<sizeof(T) == 8>(G, m, (float *)(smem + S.off_J), (float *)(smem + S.off_ev), ys, y2s,
-                                        (double *)(smem + S.off_r), misc);
+        anch = opaque(anchored);
+        small_eig_block<sizeof(T) == 8>(S, m);
         theta = misc[0];
         const T th = (T)theta;
         K *tdst = (m < mmax) ? V + (size_t)m * ld : tx;
-        v[0] = 0;
-        v[1] = 0;
+        v2[0] = v2[1] = 0;
         for (int d = tid; d < N; d += nt) {
             K xs, hs, td;
 #pragma unroll
@@ -659,17 +741,17 @@ __device__ __noinline__ PhaseOut davidson_block(const BlockProblem &B, T *Vp, T 
 #pragma unroll
             for (int l = 0; l < VL; ++l) {
                 const T r = hs.e[l] - th * xs.e[l];
-                v[0] += r * r;
+                v2[0] += r * r;
                 T den = (T)(pb.diag[d * VL + l] - shift) - th;
                 if (fabs(den) < (T)1e-4) den = den >= (T)0 ? (T)1e-4 : (T)-1e-4;
                 td.e[l] = r / den;
-                v[1] += td.e[l] * td.e[l];
+                v2[1] += td.e[l] * td.e[l];
             }
             tdst[d] = td;
         }
-        block_sums<T>(v, 2, red);
-        rn = sqrt(v[0]);
-        const T t0n = sqrt(v[1]);
+        block_sums(v2, red);
+        rn = sqrt(v2[0]);
+        const T t0n = sqrt(v2[1]);
         if (!isfinite(rn) || !isfinite(theta)) {
             o.status = MBE_STATUS_NONFINITE;
             break;
@@ -693,7 +775,7 @@ __device__ __noinline__ PhaseOut davidson_block(const BlockProblem &B, T *Vp, T 
             // corrections of the two go to V[1], V[2] (both orthogonal to x0).
             const int b = anch ? 1 : 0;
             K *V0 = V + b * ld, *W0 = W + b * ld, *V1 = V0 + ld, *W1 = W0 + ld;
-            v[0] = 0;
+            v1[0] = 0;
             for (int d = tid; d < N; d += nt) {
                 K u1, w1, u2, w2;
 #pragma unroll
@@ -710,55 +792,55 @@ __device__ __noinline__ PhaseOut davidson_block(const BlockProblem &B, T *Vp, T 
                 W0[d] = w1;
                 V1[d] = u2;
                 W1[d] = w2;
-                v[0] = dot(u1, u1, v[0]);
+                v1[0] = dot(u1, u1, v1[0]);
             }
-            block_sums<T>(v, 1, red);
-            const T n0 = sqrt(v[0]);
+            block_sums(v1, red);
+            const T n0 = sqrt(v1[0]);
             if (anch) {
                 scale((T)1 / n0, V0);
                 scale((T)1 / n0, W0);
             }
             for (int pass = 0; pass < 2; ++pass) {
-                v[0] = 0;
-                for (int d = tid; d < N; d += nt) v[0] = dot(V0[d], V1[d], v[0]);
-                block_sums<T>(v, 1, red);
+                v1[0] = 0;
+                for (int d = tid; d < N; d += nt) v1[0] = dot(V0[d], V1[d], v1[0]);
+                block_sums(v1, red);
                 for (int d = tid; d < N; d += nt) {
                     K q = V1[d], w = W1[d];
-                    axpy(-v[0], V0[d], q);
-                    axpy(-v[0], W0[d], w);
+                    axpy(-v1[0], V0[d], q);
+                    axpy(-v1[0], W0[d], w);
                     V1[d] = q;
                     W1[d] = w;
                 }
             }
-            v[0] = 0;
-            for (int d = tid; d < N; d += nt) v[0] = dot(V1[d], V1[d], v[0]);
-            block_sums<T>(v, 1, red);
-            const T nn = sqrt(v[0]);
+            v1[0] = 0;
+            for (int d = tid; d < N; d += nt) v1[0] = dot(V1[d], V1[d], v1[0]);
+            block_sums(v1, red);
+            const T nn = sqrt(v1[0]);
             const bool keep = nn > (anch ? (T)1e-3 : (T)0.5);
             if (keep) {
                 scale((T)1 / nn, V1);
                 scale((T)1 / nn, W1);
             }
-            v[0] = v[1] = v[2] = v[3] = v[4] = 0;
+            T q[5] = {0, 0, 0, 0, 0};
             for (int d = tid; d < N; d += nt) {
-                const K v0 = V0[d], w0 = W0[d];
-                v[0] = dot(v0, w0, v[0]);
-                if (anch) v[1] = dot(W[d], v0, v[1]);  // x0.(A u1) as u1.r0
+                const K a0 = V0[d], b0 = W0[d];
+                q[0] = dot(a0, b0, q[0]);
+                if (anch) q[1] = dot(W[d], a0, q[1]);  // x0.(A u1) as u1.r0
                 if (keep) {
-                    const K v1 = V1[d], w1 = W1[d];
-                    v[2] = dot(v0, w1, v[2]);
-                    v[3] = dot(v1, w1, v[3]);
-                    if (anch) v[4] = dot(W[d], v1, v[4]);
+                    const K a1 = V1[d], b1 = W1[d];
+                    q[2] = dot(a0, b1, q[2]);
+                    q[3] = dot(a1, b1, q[3]);
+                    if (anch) q[4] = dot(W[d], a1, q[4]);
                 }
             }
-            block_sums<T>(v, 5, red);
+            block_sums(q, red);
             if (tid == 0) {
-                G[b * MMAX + b] = (double)v[0];
-                if (anch) G[1] = G[MMAX] = (double)v[1];
+                G[b * MMAX + b] = (double)q[0];
+                if (anch) G[1] = G[MMAX] = (double)q[1];
                 if (keep) {
-                    G[b * MMAX + b + 1] = G[(b + 1) * MMAX + b] = (double)v[2];
-                    G[(b + 1) * MMAX + b + 1] = (double)v[3];
-                    if (anch) G[2] = G[2 * MMAX] = (double)v[4];
+                    G[b * MMAX + b + 1] = G[(b + 1) * MMAX + b] = (double)q[2];
+                    G[(b + 1) * MMAX + b + 1] = (double)q[3];
+                    if (anch) G[2] = G[2 * MMAX] = (double)q[4];
                 }
                 // the Ritz vector in the new basis
                 ys[b] = anch ? (double)n0 : 1.0;
@@ -772,29 +854,35 @@ __device__ __noinline__ PhaseOut davidson_block(const BlockProblem &B, T *Vp, T 
         K *tv = V + (size_t)m * ld;
         const K *tsrc = (tdst == tx) ? tx : tv;
         T tn = t0n;
+#pragma unroll 1
         for (int pass = 0; pass < 2; ++pass) {
+            const K *src = pass == 0 ? tsrc : tv;
+            T v[32];
 #pragma unroll
-            for (int i = 0; i < KRED; ++i) v[i] = 0;
+            for (int i = 0; i < 32; ++i) v[i] = 0;
             for (int d = tid; d < N; d += nt) {
-                const K td = (pass == 0) ? tsrc[d] : tv[d];
+                const K td = src[d];
 #pragma unroll
                 for (int i = 0; i < MMAX; ++i)
                     if (i < m) v[i] = dot(V[(size_t)i * ld + d], td, v[i]);
             }
-            block_sums<T>(v, m, red);
-            T tt = 0;
+            const T *tot = block_sums_many(v, m, red);
+            T c[MMAX];
+#pragma unroll
+            for (int i = 0; i < MMAX; ++i) c[i] = i < m ? -tot[i] : (T)0;
+            v1[0] = 0;
             for (int d = tid; d < N; d += nt) {
-                K td = (pass == 0) ? tsrc[d] : tv[d];
+                K td = src[d];
 #pragma unroll
                 for (int i = 0; i < MMAX; ++i)
-                    if (i < m) axpy(-v[i], V[(size_t)i * ld + d], td);
+                    if (i < m) axpy(c[i], V[(size_t)i * ld + d], td);
                 tv[d] = td;
-                tt = dot(td, td, tt);
+                v1[0] = dot(td, td, v1[0]);
             }
-            v[0] = tt;
-            block_sums<T>(v, 1, red);
+            __syncthreads();  // (tot is read before the next sums)
+            block_sums(v1, red);
             const T before = tn;
-            tn = sqrt(v[0]);
+            tn = sqrt(v1[0]);
             if (tn >= (T)0.70710678 * before) break;
         }
         if (!(tn > (T)1e-12 * t0n) || !(tn > (T)0)) {
@@ -807,8 +895,9 @@ __device__ __noinline__ PhaseOut davidson_block(const BlockProblem &B, T *Vp, T 
         K *wv = W + (size_t)m * ld;
         sigma_block<T>(B, (const T *)tv, (T *)wv);
         ++o.nsig;
+        T v[32];
 #pragma unroll
-        for (int i = 0; i < KRED; ++i) v[i] = 0;
+        for (int i = 0; i < 32; ++i) v[i] = 0;
         for (int d = tid; d < N; d += nt) {
             K wd = wv[d];
             const K td = tv[d];
@@ -819,25 +908,22 @@ __device__ __noinline__ PhaseOut davidson_block(const BlockProblem &B, T *Vp, T 
             }
 #pragma unroll
             for (int i = 0; i < MMAX; ++i)
-                if (i < m) v[i] = (anch && i == 0) ? dot(W[d], td, v[i]) : dot(V[(size_t)i * ld + d], wd, v[i]);
+                if (i < m) v[i] = dot(V[(size_t)i * ld + d], wd, v[i]);
             v[MMAX] = dot(td, wd, v[MMAX]);
+            if (anch) v[MMAX + 1] = dot(W[d], td, v[MMAX + 1]);  // x0.(A t) as t.r0
         }
-        {
-            const T diag = v[MMAX];
-#pragma unroll
-            for (int i = 0; i <= MMAX; ++i)
-                if (i == m) v[i] = diag;
+        const T *tot = block_sums_many(v, MMAX + 2, red);
+        if (tid <= m) {
+            const double g = tid == m ? (double)tot[MMAX] : anch && tid == 0 ? (double)tot[MMAX + 1] : (double)tot[tid];
+            G[tid * MMAX + m] = G[m * MMAX + tid] = g;
         }
-        block_sums<T>(v, m + 1, red);
-        if (tid == 0)
-            for (int i = 0; i <= m; ++i) G[i * MMAX + m] = G[m * MMAX + i] = (double)v[i];
         __syncthreads();
         ++m;
     }
     // the Ritz vector; anchored: its correction d, scaled so that x0 keeps coefficient 1
     __syncthreads();
     const T inv0 = anch ? (T)(1.0 / ys[0]) : (T)1;
-    v[0] = 0;
+    v1[0] = 0;
     for (int d = tid; d < N; d += nt) {
         K u;
 #pragma unroll
@@ -845,10 +931,10 @@ __device__ __noinline__ PhaseOut davidson_block(const BlockProblem &B, T *Vp, T 
 #pragma unroll 4
         for (int i = anch ? 1 : 0; i < m; ++i) axpy((T)ys[i] * inv0, V[(size_t)i * ld + d], u);
         x[d] = u;
-        v[0] = dot(u, u, v[0]);
+        v1[0] = dot(u, u, v1[0]);
     }
-    block_sums<T>(v, 1, red);
-    if (anch) o.dnorm = (double)sqrt(v[0]);
+    block_sums(v1, red);
+    if (anch) o.dnorm = (double)sqrt(v1[0]);
     o.lambda = theta;
     o.rnorm = (double)rn;
     return o;
@@ -879,7 +965,7 @@ __device__ void block_setup(const BatchArgs &a, BlockProblem &B, const ClassInfo
 {
     Problem &pb = B.pb;
     const int tid = threadIdx.x, nt = blockDim.x, n = pb.n, P = pb.P, norb = a.norb, Ns = pb.Ns, st = pb.HSS;
-    double *red = (double *)(B.smem + B.S.off_red);
+    double *red = (double *)(block_shared() + B.S.off_red);
     for (int e = tid; e < P; e += nt) {
         int p = 0;
         while ((p + 1) * (p + 2) / 2 <= e) ++p;
@@ -913,7 +999,7 @@ __device__ void block_setup(const BatchArgs &a, BlockProblem &B, const ClassInfo
         pb.V32[e] = (float)v;
     }
     if (B.gemm) {
-        uint16_t *list = (uint16_t *)(B.smem + B.S.off_list);
+        uint16_t *list = (uint16_t *)(block_shared() + B.S.off_list);
         const int rs = pb.R | 1;
         for (int e = tid; e < Ns * pb.R; e += nt) {
             const int t = ci.table[e], I = e / pb.R;
@@ -923,7 +1009,7 @@ __device__ void block_setup(const BatchArgs &a, BlockProblem &B, const ClassInfo
     __syncthreads();
     auto H = [&](int p, int q) { return pb.h[p * n + q]; };
     auto V = [&](int p, int q, int r, int s) { return pb.V64[pair_index(p, q) * P + pair_index(r, s)]; };
-    double *hd = (double *)(B.smem + B.S.off_hd);
+    double *hd = (double *)(block_shared() + B.S.off_hd);
     {
         int ia = 0, ib = 0;
         tri_advance(ia, ib, tid, Ns);
@@ -986,7 +1072,7 @@ __device__ __noinline__ void block_rdm(const BatchArgs &a, const BlockProblem &B
     const int tid = threadIdx.x, nt = blockDim.x, n = pb.n, n2 = n * n, Ns = pb.Ns, lane = tid & 31;
     const bool two = a.grad_eri != nullptr;
     const int first = two ? 0 : n2 * (n2 + 1) / 2, ng = n2 * (n2 + 1) / 2 + n2;  // (without c.c)
-    double *D = (double *)(B.smem + B.S.off_c), *g1 = (double *)(B.smem + B.S.off_g1), *c = B.full;
+    double *D = (double *)(block_shared() + B.S.off_c), *g1 = (double *)(block_shared() + B.S.off_g1), *c = B.full;
     expand_full<double>(pb, x, c, Ns);
     double gram[GE];
     int uv[GE];
@@ -1060,7 +1146,7 @@ __device__ __noinline__ void block_rdm(const BatchArgs &a, const BlockProblem &B
 
 __global__ void __launch_bounds__(BLOCK_THREADS, 1) k_casci_block(BatchArgs a, int bucket)
 {
-    extern __shared__ __align__(16) char smem[];
+    char *smem = block_shared();
     const int n = a.n, P = n * (n + 1) / 2, tid = threadIdx.x, nt = blockDim.x;
     __shared__ unsigned long long s_pos;
     char *slot = a.scratch + (size_t)blockIdx.x * a.slot_bytes;
@@ -1086,7 +1172,6 @@ __global__ void __launch_bounds__(BLOCK_THREADS, 1) k_casci_block(BatchArgs a, i
         const ClassInfo ci = a.cls[k];
         const BlockSlot L = block_slot(ci.ns);
         BlockProblem B;
-        B.smem = smem;
         B.S = block_mem(n, a.gemm, ci.ns, ci.r, a.rdm);
         B.gemm = a.gemm;
         B.E = 0;
@@ -1248,13 +1333,12 @@ __global__ void __launch_bounds__(BLOCK_THREADS, 1) k_casci_block(BatchArgs a, i
                         double *s0 = W64 + (MMAX / 2) * (L.vec / 8);
                         sigma_block<double>(B, x0, s0);
                         ++n64;
-                        double q[KRED];
-                        q[0] = q[1] = 0.0;
+                        double q[2] = {0.0, 0.0};
                         for (int d = tid; d < pb.N; d += nt) {
                             q[0] += x0[d] * s0[d];
                             q[1] += x0[d] * x0[d];
                         }
-                        block_sums<double>(q, 2, red);
+                        block_sums(q, red);
                         const double th = q[0] / q[1], inv = 1.0 / sqrt(q[1]);
                         for (int d = tid; d < pb.N; d += nt) {
                             V32[d] = (float)(x0[d] * inv);
