@@ -1449,7 +1449,7 @@ int block_grid(mbe_ctx *ctx, BatchArgs &a, const bool (&in)[MBE_MAX_CAS + 1], in
     *smem = block_smem_bytes(ctx, a.n, a, in, rdm, &a.gemm);
     MBE_CHECK(*smem <= ctx->smem_optin, MBE_EUNSUPPORTED, "casci_batch: block solver needs %zu B shared memory",
               *smem);
-    MBE_CU(cudaFuncSetAttribute(k_casci_block, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)*smem));
+    MBE_CU(allow_smem(k_casci_block, ctx->smem_optin));
     *grid = (int)std::min<int64_t>(ctx->sm_count, a.n_tuples);
     int ns = 0;
     for (int k = 0; k <= a.n; ++k)

@@ -670,19 +670,16 @@ static int large_setup(mbe_ctx *ctx, int norb, const double *h1, const double *e
     plan->smem_ab64 = (size_t)P * P * 8;
     MBE_CHECK(plan->smem_ab64 <= ctx->smem_optin, MBE_EUNSUPPORTED, "large CASCI: V needs %zu B shared memory",
               plan->smem_ab64);
-    MBE_CU(cudaFuncSetAttribute(k_large_ab64<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)plan->smem_ab64));
-    MBE_CU(cudaFuncSetAttribute(k_large_ab64<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)plan->smem_ab64));
+    MBE_CU(allow_smem(k_large_ab64<false>, ctx->smem_optin));
+    MBE_CU(allow_smem(k_large_ab64<true>, ctx->smem_optin));
     int b = 0;
     MBE_CU(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_large_ab64<false>, SIGMA_THREADS, plan->smem_ab64));
     plan->grid_ab64 = ctx->sm_count * (b > 0 ? b : 1);
     plan->smem_ss64 = (size_t)SS_ROWS * (SS_TK + 1) * 8;
     plan->smem_ss32 = (size_t)SS_ROWS * (SS_TK + 1) * 4;
-    MBE_CU(cudaFuncSetAttribute(k_large_ss<double, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                (int)plan->smem_ss64));
-    MBE_CU(cudaFuncSetAttribute(k_large_ss<double, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                (int)plan->smem_ss64));
-    MBE_CU(cudaFuncSetAttribute(k_large_ss<double, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                (int)plan->smem_ss64));
+    MBE_CU(allow_smem(k_large_ss<double, false>, ctx->smem_optin));
+    MBE_CU(allow_smem(k_large_ss<double, true>, ctx->smem_optin));
+    MBE_CU(allow_smem(k_large_ss<double, false, true>, ctx->smem_optin));
     MBE_CU(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_large_ss<double, false>, SS_THREADS, plan->smem_ss64));
     plan->grid_ss64 = ctx->sm_count * (b > 0 ? b : 1);
     MBE_CU(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_large_ss<float, false>, SS_THREADS, plan->smem_ss32));

@@ -9,7 +9,7 @@ static int launch_warp_mixed_t(mbe_ctx *ctx, const BatchArgs &a, int b, const Mi
     const size_t smem = (size_t)L.bytes * a.warps;
     MBE_CHECK(smem <= ctx->smem_optin, MBE_EUNSUPPORTED, "casci_batch: mixed warp solver needs %zu B shared memory",
               smem);
-    MBE_CU(cudaFuncSetAttribute(k_casci_warp_mixed<DPL>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    MBE_CU(allow_smem(k_casci_warp_mixed<DPL>, ctx->smem_optin));
     int per_sm = 0;
     MBE_CU(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_casci_warp_mixed<DPL>, a.warps * 32, smem));
     if (per_sm < 1) per_sm = 1;

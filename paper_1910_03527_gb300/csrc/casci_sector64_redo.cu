@@ -9,7 +9,7 @@ static int launch_class(mbe_ctx *ctx, const BatchArgs &a, int b)
 {
     using C = Cls<N, K>;
     const size_t smem = al16((int)sizeof(SectorTables<C>)) + sizeof(Sector64<C>) * a.warps;
-    MBE_CU(cudaFuncSetAttribute(k_sector64<C, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    MBE_CU(allow_smem(k_sector64<C, true>, ctx->smem_optin));
     int per_sm = 0;
     MBE_CU(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_sector64<C, true>, a.warps * 32, smem));
     if (per_sm < 1) per_sm = 1;

@@ -7,7 +7,7 @@ namespace mbe {
 template <int DPL, int MODE>
 static int launch_warp_mode(mbe_ctx *ctx, const BatchArgs &a, int b, const WarpLayout &L, size_t smem)
 {
-    MBE_CU(cudaFuncSetAttribute(k_casci_warp<DPL, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    MBE_CU(allow_smem(k_casci_warp<DPL, MODE>, ctx->smem_optin));
     int per_sm = 0;
     MBE_CU(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_casci_warp<DPL, MODE>, a.warps * 32, smem));
     if (per_sm < 1) per_sm = 1;

@@ -144,6 +144,15 @@ struct Bump {
     }
 };
 
+// Lets a kernel use dynamic shared memory up to the device's limit (less what kernels have
+// statically).  Always the same value: the attribute belongs to the process, and a caller that
+// set it to its own smaller size between another thread's call and launch made that launch fail.
+template <typename F>
+inline cudaError_t allow_smem(F *kernel, size_t smem_optin)
+{
+    return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_optin - 1024);
+}
+
 inline size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
 
 // Position of the m-tuple `key` in a lexicographically sorted list, or -1.

@@ -382,7 +382,7 @@ int mbe::large_ab_tc(cudaStream_t st, int sm_count, size_t smem_optin, int P, in
     }
     MBE_CHECK(S.bytes + 1024 <= smem_optin, MBE_EUNSUPPORTED, "large CASCI: tensor-core sigma needs %u B shared memory",
               S.bytes);
-    MBE_CU(cudaFuncSetAttribute(k_large_ab_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)S.bytes));
+    MBE_CU(allow_smem(k_large_ab_tc, smem_optin));
     const int grid = std::min(sm_count, Ns);
     k_large_ab_tc<<<grid, TC_THREADS, S.bytes, st>>>(a);
     MBE_CU(cudaGetLastError());
