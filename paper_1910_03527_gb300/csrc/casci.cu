@@ -61,7 +61,7 @@ __global__ void k_core_gradient(int norb, const uint8_t *occ, const double *core
 }
 
 struct ClassifyArgs {
-    int bucket_of_k[MBE_MAX_CAS + 1];
+    int bucket_of_k[MBE_MAX_LARGE_CAS + 1];
     int nbuckets;
 };
 
@@ -69,7 +69,7 @@ __global__ void k_classify(BatchArgs a, ClassifyArgs c, int32_t *key, int64_t *c
 {
     int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= a.n_tuples) return;
-    int A[MBE_MAX_CAS];
+    int A[MBE_MAX_LARGE_CAS];
     int b = -1;
     if (build_A(a, t, A)) {
         int k = 0;
@@ -114,11 +114,14 @@ __global__ void k_scatter(int64_t n_tuples, int nbuckets, const int32_t *key, co
 using namespace mbe;
 
 // casci_batch and casci_rdm_batch: rdm = 0 energies only, 1 = + weighted 1-RDM
-// gradients, 2 = + weighted 1- and 2-RDM gradients.
+// gradients, 2 = + weighted 1- and 2-RDM gradients.  classes: the electron pairs k that
+// the tuples have (bit k); a tuple of another class gets MBE_STATUS_BADINPUT.  max_n: the
+// largest active space taken.
 static int run_casci(mbe_ctx *ctx, int norb, const double *h1, const double *eri, const uint8_t *occ, int n_ref,
                      const int32_t *ref_orbs, double e_ref_corr, int order, int64_t n_tuples, const int32_t *tuples,
                      const mbe_opts *opts, double *eps_out, int32_t *status_out, int32_t *iters_out, int rdm,
-                     const double *weights, double *grad_h1, double *grad_eri)
+                     const double *weights, double *grad_h1, double *grad_eri, uint32_t classes = ~0u,
+                     int max_n = MBE_MAX_CAS)
 {
     MBE_CHECK(ctx != nullptr && h1 != nullptr && eri != nullptr && occ != nullptr, MBE_EINVAL,
               "casci_batch: NULL argument");
@@ -130,7 +133,7 @@ static int run_casci(mbe_ctx *ctx, int norb, const double *h1, const double *eri
               "casci_batch: order 0 computes the reference space alone (n_tuples <= 1)");
     const int n = n_ref + order;
     MBE_CHECK(n >= 1, MBE_EINVAL, "casci_batch: empty active space");
-    MBE_CHECK(n <= MBE_MAX_CAS, MBE_EUNSUPPORTED, "casci_batch: |R| + order = %d > %d", n, MBE_MAX_CAS);
+    MBE_CHECK(n <= max_n, MBE_EUNSUPPORTED, "casci_batch: |R| + order = %d > %d", n, max_n);
     MBE_CHECK(n_tuples < (1LL << 31), MBE_EUNSUPPORTED, "casci_batch: n_tuples >= 2^31");
     mbe_opts o;
     if (opts) o = *opts; else mbe_default_opts(&o);
@@ -171,7 +174,7 @@ static int run_casci(mbe_ctx *ctx, int norb, const double *h1, const double *eri
     a.min_fp64 = o.fp64_final_iters;
     a.even_only = o.sectors == MBE_SECTORS_EVEN ? 1 : 0;
     a.s2mu = o.s2_penalty;
-    const mbe_tuning tu = ctx->tune[o.precision == MBE_PREC_MIXED ? 1 : 0][n];
+    const mbe_tuning tu = ctx->tune[o.precision == MBE_PREC_MIXED ? 1 : 0][std::min(n, MBE_MAX_CAS)];
     a.warps = tu.warp_warps;
     a.block_basis = tu.block_basis;
     a.eps = eps_out;
@@ -183,8 +186,10 @@ static int run_casci(mbe_ctx *ctx, int norb, const double *h1, const double *eri
     std::vector<Bucket> buckets;
     int warp_bucket_of_dpl[5] = {-1, -1, -1, -1, -1};
     int block_bucket = -1;
-    bool in_block[MBE_MAX_CAS + 1] = {};
+    bool in_block[MBE_MAX_STRING_ORB + 1] = {};
     for (int k = 0; k <= n; ++k) {
+        cl.bucket_of_k[k] = -1;
+        if (!(classes >> k & 1u)) continue;
         const StringTable *st = nullptr;
         int rc = get_table(ctx, n, k, &st);
         if (rc) return rc;
@@ -314,6 +319,17 @@ static int run_casci(mbe_ctx *ctx, int norb, const double *h1, const double *eri
         ++ctx->launches;
     }
     return MBE_OK;
+}
+
+// casci_batch for active spaces of up to MBE_MAX_LARGE_CAS orbitals whose classes the caller
+// knows (casci_batch_routed).
+int mbe::casci_batch_wide(mbe_ctx *ctx, int norb, const double *h1, const double *eri, const uint8_t *occ, int n_ref,
+                          const int32_t *ref_orbs, double e_ref_corr, int order, int64_t n_tuples,
+                          const int32_t *tuples, const mbe_opts *opts, double *eps_out, int32_t *status_out,
+                          int32_t *iters_out, uint32_t classes)
+{
+    return run_casci(ctx, norb, h1, eri, occ, n_ref, ref_orbs, e_ref_corr, order, n_tuples, tuples, opts, eps_out,
+                     status_out, iters_out, 0, nullptr, nullptr, nullptr, classes, MBE_MAX_LARGE_CAS);
 }
 
 extern "C" int casci_batch(mbe_ctx *ctx, int norb, const double *h1, const double *eri, const uint8_t *occ,

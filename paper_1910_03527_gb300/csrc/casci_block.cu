@@ -32,15 +32,24 @@ __device__ __forceinline__ char *block_shared()
 constexpr int BLOCK_THREADS = 512;  // one block per SM: 128 registers a thread, up to 227 KB
 constexpr int GEMM_MAX_N = 9;       // orbitals up to which sigma is the tiled product
 constexpr int GEMM_T_BYTES = 48 * 1024;
+constexpr int LIST_MAX_NS = 128;    // strings up to which larger orbital counts keep c in shared memory
+
+// Forms of sigma: c in global memory and both lists walked per element; the tiled product; c and
+// V in shared memory and the off-diagonal lists walked (10-16 orbitals with few strings).
+enum { SIGMA_GLOBAL = 0, SIGMA_TILED = 1, SIGMA_LIST = 2 };
+__host__ __device__ inline int sigma_form(int n, int ns)
+{
+    return n <= GEMM_MAX_N ? SIGMA_TILED : ns <= LIST_MAX_NS ? SIGMA_LIST : SIGMA_GLOBAL;
+}
 
 // Per-block slot of the workspace.
 struct BlockSlot {
-    size_t off_V, off_W, off_x, off_t, off_diag, off_Hs64, off_Hs32, off_x2, off_x0, off_full, vec, bytes;
+    size_t off_V, off_W, off_x, off_t, off_diag, off_Hs64, off_Hs32, off_x2, off_x0, off_full, off_V64, off_U, vec, bytes;
 };
 
 __host__ __device__ inline int hs_stride(int ns) { return (ns + 3) / 4 * 4; }
 
-__host__ __device__ inline BlockSlot block_slot(int ns)
+__host__ __device__ inline BlockSlot block_slot(int n, int ns)
 {
     BlockSlot L;
     size_t o = 0;
@@ -57,6 +66,10 @@ __host__ __device__ inline BlockSlot block_slot(int ns)
     L.off_Hs64 = o; o += mat;
     L.off_Hs32 = o; o += mat / 2;
     L.off_full = o; o += mat;  // the product C Hs, or the whole coefficient matrix
+    // SIGMA_LIST: the float64 V, and sums of V over each string's orbitals
+    const size_t P = (size_t)n * (n + 1) / 2, list = sigma_form(n, ns) == SIGMA_LIST ? 1 : 0;
+    L.off_V64 = o; o += list * ((P * P * 8 + 255) & ~(size_t)255);
+    L.off_U = o; o += list * ((ns * P * 4 + 255) & ~(size_t)255);
     L.bytes = o;
     return L;
 }
@@ -91,22 +104,26 @@ __host__ __device__ inline GemmShape gemm_shape(int n, int ns, int r)
     return s;
 }
 
+// Row stride of the float32 c of SIGMA_LIST
+__host__ __device__ inline int list_stride(int ns) { return hs_stride(ns) % 32 == 0 ? hs_stride(ns) + 4 : hs_stride(ns); }
+
 struct BlockMem {  // dynamic shared memory
     int off_A, off_pp, off_h, off_V64, off_V32, off_red, off_G, off_J, off_ev, off_y, off_yp, off_r, off_misc,
         off_hd, off_list, off_c, off_T, off_g1, bytes;
 };
 
-// gemm: the tiled sigma's lists, c (8 bytes an element) and T; else those are absent.
+// The tiled sigma's lists, c and T; the lists and c of SIGMA_LIST; else those are absent.
 // rdm: density matrices follow the solve.
-__host__ __device__ inline BlockMem block_mem(int n, bool gemm, int ns, int r, int rdm)
+__host__ __device__ inline BlockMem block_mem(int n, int form, int ns, int r, int rdm)
 {
     BlockMem S;
     const int P = n * (n + 1) / 2;
+    const bool gemm = form == SIGMA_TILED;
     int o = 0;
-    S.off_A = o; o = al16(o + 4 * MBE_MAX_CAS);
+    S.off_A = o; o = al16(o + 4 * MBE_MAX_STRING_ORB);
     S.off_pp = o; o = al16(o + 4 * P);
     S.off_h = o; o = al16(o + 8 * n * n);
-    S.off_V64 = o; o = al16(o + 8 * P * P);
+    S.off_V64 = o; o = al16(o + (form == SIGMA_LIST ? 0 : 8 * P * P));  // (SIGMA_LIST: in the slot)
     S.off_V32 = o; o = al16(o + 4 * P * ((P + 5) / 6 * 6));
     S.off_red = o; o = al16(o + 8 * 32 * KRED);
     S.off_G = o; o = al16(o + 8 * MMAX * MMAX);
@@ -118,8 +135,9 @@ __host__ __device__ inline BlockMem block_mem(int n, bool gemm, int ns, int r, i
     S.off_misc = o; o = al16(o + 8 * 4);
     S.off_g1 = o; o = al16(o + 8 * n * n);
     S.off_hd = o; o = al16(o + (gemm ? 8 * ns : 0));
-    S.off_list = o; o = al16(o + (gemm ? 2 * ns * (r | 1) : 0));
+    S.off_list = o; o = al16(o + (gemm ? 2 * ns * (r | 1) : form == SIGMA_LIST ? 4 * ns * (r + 1) : 0));
     S.off_c = o;
+    if (form == SIGMA_LIST) o = al16(o + 4 * ns * list_stride(ns));
     if (gemm) {
         // fixed point: c; float32: c, V twice over with both signs, list offsets (see sigma_gemm)
         const GemmShape a = gemm_shape<float>(n, ns, r);
@@ -140,7 +158,8 @@ __host__ __device__ inline BlockMem block_mem(int n, bool gemm, int ns, int r, i
 
 struct BlockProblem {
     Problem pb;       // N: packed elements; diag: packed
-    bool gemm;
+    int form;         // of sigma
+    const float *U;   // SIGMA_LIST: U[I][p] = sum over the orbitals q of string I of V[qq][p]
     bool bad;         // an element of V or Hs is not finite (float64 sigma: fixed point cannot hold it)
     int E;            // fixed-point exponent
     BlockMem S;
@@ -409,13 +428,103 @@ __device__ __noinline__ void sigma_gemm(const BlockProblem &B, const T *src, T *
     }
 }
 
+// Float32 sigma of 10-16 orbitals with few strings: c and V in shared memory, one element per
+// thread.  The diagonal replacements are summed beforehand (U), so that k (n - k) entries of
+// each list are left, and each string's entries are sorted by sign: (k (n - k))^2 multiply-adds
+// per element instead of R^2 (676 for 1,521 at 13 electron pairs in 15 orbitals), two shared
+// gathers each; four entries of Ib share the decoding of one of Ia.
+__device__ __noinline__ void sigma_list(const BlockProblem &B, const float *src, float *dst)
+{
+    const Problem &pb = B.pb;
+    const BlockMem &S = B.S;
+    char *smem = block_shared();
+    const int Ns = pb.Ns, P = pb.P, tid = threadIdx.x, nt = blockDim.x, sgn = pb.sector, ld = list_stride(Ns), vs = P | 1;
+    const int ro = pb.k * (pb.n - pb.k);  // entries; word ro of a list holds the number of positive ones
+    float *c = (float *)(smem + S.off_c);
+    const char *V = smem + S.off_V32;
+    const uint32_t *list = (const uint32_t *)(smem + S.off_list);
+    float *M = (float *)B.full;
+    {
+        int ia = 0, ib = 0;
+        tri_advance(ia, ib, tid, Ns);
+        for (int h = tid; h < pb.N; h += nt) {
+            const float f = ia == ib ? src[h] : 0.70710678118654752f * src[h];
+            c[ia * ld + ib] = f;
+            c[ib * ld + ia] = sgn > 0 ? f : -f;
+            tri_advance(ia, ib, nt, Ns);
+        }
+        for (int q = tid; q < Ns * (ld - Ns); q += nt) c[q / (ld - Ns) * ld + Ns + q % (ld - Ns)] = 0.f;
+    }
+    __syncthreads();
+    same_spin(pb, hs_stride(Ns), ld, c, pb.Hs32, M);
+    __syncthreads();
+    int ia = 0, ib = 0;
+    tri_advance(ia, ib, tid, Ns);
+    for (int h = tid; h < pb.N; h += nt) {
+        const uint32_t *la = list + ia * (ro + 1), *lb = list + ib * (ro + 1);
+        const float *Ua = B.U + ia * P, *Ub = B.U + ib * P;
+        const int ap = la[ro], bp = lb[ro];
+        float acc = 0.f;
+        // both replacements off the diagonal; a list word is 4 pair | (4 ld J) << 12
+        for (int y0 = 0; y0 < ro; y0 += 4) {
+            const char *v[4], *cc[4];
+            float s[4];
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                const uint32_t e = lb[y0 + i < ro ? y0 + i : ro - 1];
+                v[i] = V + (e & 0xfffu) * vs;            // row pair(e)
+                cc[i] = (const char *)c + (e >> 12) / ld;  // column J(e)
+                s[i] = 0.f;
+            }
+#pragma unroll 2
+            for (int x = 0; x < ap; ++x) {
+                const uint32_t e = la[x], p = e & 0xfffu, j = e >> 12;
+#pragma unroll
+                for (int i = 0; i < 4; ++i) s[i] = fmaf(*(const float *)(v[i] + p), *(const float *)(cc[i] + j), s[i]);
+            }
+#pragma unroll 2
+            for (int x = ap; x < ro; ++x) {
+                const uint32_t e = la[x], p = e & 0xfffu, j = e >> 12;
+#pragma unroll
+                for (int i = 0; i < 4; ++i) s[i] = fmaf(-*(const float *)(v[i] + p), *(const float *)(cc[i] + j), s[i]);
+            }
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+                if (y0 + i < ro) acc += y0 + i < bp ? s[i] : -s[i];
+        }
+        // one of them on the diagonal, then both
+        float one = 0.f;
+        for (int x = 0; x < ro; ++x) {
+            const uint32_t a = la[x], b = lb[x];
+            const float u = Ub[(a & 0xfffu) >> 2] * *(const float *)((const char *)(c + ib) + (a >> 12));
+            const float w = Ua[(b & 0xfffu) >> 2] * *(const float *)((const char *)(c + ia * ld) + (b >> 12) / ld);
+            one += x < ap ? u : -u;
+            one += x < bp ? w : -w;
+        }
+        float dd = 0.f;
+        for (uint32_t m = pb.str[ib]; m; m &= m - 1u) {
+            const int q = __ffs((int)m) - 1;
+            dd += Ua[pair_index(q, q)];
+        }
+        acc += one + dd * c[ia * ld + ib];
+        const float mt = M[ib * hs_stride(Ns) + ia];
+        acc += M[ia * hs_stride(Ns) + ib] + (sgn > 0 ? mt : -mt);
+        dst[h] = ia == ib ? (sgn > 0 ? acc : 0.f) : 1.41421356f * acc;
+        tri_advance(ia, ib, nt, Ns);
+    }
+    __syncthreads();
+}
+
 // sigma of a packed sector vector; ends with a barrier.
 template <typename T>
 __device__ __noinline__ void sigma_block(const BlockProblem &B, const T *src, T *dst)
 {
     const Problem &pb = B.pb;
-    if (B.gemm) sigma_gemm<T>(B, src, dst);
-    if (B.gemm && pb.s2mu == 0.0) return;
+    const bool done = B.form == SIGMA_TILED || (B.form == SIGMA_LIST && sizeof(T) == 4);  // but for the penalty
+    if (B.form == SIGMA_TILED) sigma_gemm<T>(B, src, dst);
+    if constexpr (sizeof(T) == 4)
+        if (B.form == SIGMA_LIST) sigma_list(B, src, dst);
+    if (done && pb.s2mu == 0.0) return;
     T *full = (T *)B.full;
     expand_full<T>(pb, src, full, pb.Ns);
     __syncthreads();
@@ -424,7 +533,7 @@ __device__ __noinline__ void sigma_block(const BlockProblem &B, const T *src, T 
     for (int h = threadIdx.x; h < pb.N; h += blockDim.x) {
         T v = (T)0;
         if (!(pb.sector < 0 && ia == ib)) {
-            if (!B.gemm) {
+            if (!done) {
                 if constexpr (sizeof(T) == 4)
                     v = sigma_elem_ashared<T>(pb, pb.V32, pb.Hs32, full, ia, ib);
                 else
@@ -433,7 +542,7 @@ __device__ __noinline__ void sigma_block(const BlockProblem &B, const T *src, T 
             if (pb.s2mu != 0.0) v += (T)pb.s2mu * s2_elem<T, T>(pb, full, ia, ib);
             if (ia != ib) v *= (T)1.4142135623730951;
         }
-        dst[h] = B.gemm ? dst[h] + v : v;
+        dst[h] = done ? dst[h] + v : v;
         tri_advance(ia, ib, blockDim.x, pb.Ns);
     }
     __syncthreads();
@@ -983,7 +1092,7 @@ __device__ void block_setup(const BatchArgs &a, BlockProblem &B, const ClassInfo
         pb.h[e] = v;
     }
     __syncthreads();
-    const int vs = B.gemm ? (P + 5) / 6 * 6 : P;
+    const int vs = B.form == SIGMA_TILED ? (P + 5) / 6 * 6 : B.form == SIGMA_LIST ? P | 1 : P;
     double big = 0.0;
     bool bad = false;
     for (int e = tid; e < P * vs; e += nt) {
@@ -998,7 +1107,24 @@ __device__ void block_setup(const BatchArgs &a, BlockProblem &B, const ClassInfo
         }
         pb.V32[e] = (float)v;
     }
-    if (B.gemm) {
+    if (B.form == SIGMA_LIST) {
+        // off-diagonal replacements, the positive ones first, then their number
+        uint32_t *list = (uint32_t *)(block_shared() + B.S.off_list);
+        const int ro = pb.k * (n - pb.k), ld = list_stride(Ns);
+        for (int I = tid; I < Ns; I += nt) {
+            int at = 0, positive = 0;
+            for (int neg = 0; neg < 2; ++neg) {
+                for (int x = 0; x < pb.R; ++x) {
+                    const int t = ci.table[I * pb.R + x];
+                    if (entry_J(t) != I && entry_neg(t) == neg)
+                        list[I * (ro + 1) + at++] = (uint32_t)(4 * entry_pair(t)) | (uint32_t)(4 * ld * entry_J(t)) << 12;
+                }
+                if (neg == 0) positive = at;
+            }
+            list[I * (ro + 1) + ro] = (uint32_t)positive;
+        }
+    }
+    if (B.form == SIGMA_TILED) {
         uint16_t *list = (uint16_t *)(block_shared() + B.S.off_list);
         const int rs = pb.R | 1;
         for (int e = tid; e < Ns * pb.R; e += nt) {
@@ -1028,6 +1154,13 @@ __device__ void block_setup(const BatchArgs &a, BlockProblem &B, const ClassInfo
         }
     }
     B.bad = __syncthreads_or(bad);
+    if (B.form == SIGMA_LIST)
+        for (int e = tid; e < Ns * P; e += nt) {
+            const int I = e / P, p = e - I * P;
+            double u = 0.0;
+            for (uint32_t m = pb.str[I]; m; m &= m - 1u) u += pb.V64[pair_index(__ffs((int)m) - 1, __ffs((int)m) - 1) * P + p];
+            ((float *)B.U)[e] = (float)u;
+        }
     {
         int ia = 0, ib = 0;
         tri_advance(ia, ib, tid, Ns);
@@ -1043,7 +1176,7 @@ __device__ void block_setup(const BatchArgs &a, BlockProblem &B, const ClassInfo
         }
         if (tid < (4 - pb.N % 4) % 4) pb.diag[pb.N + tid] = 1.0;
     }
-    if (B.gemm) {
+    if (B.form == SIGMA_TILED) {
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) big = fmax(big, __shfl_xor_sync(FULL, big, o));
         if ((tid & 31) == 0) red[tid >> 5] = big;
@@ -1170,10 +1303,11 @@ __global__ void __launch_bounds__(BLOCK_THREADS, 1) k_casci_block(BatchArgs a, i
                 mphi |= 1u << i;
             }
         const ClassInfo ci = a.cls[k];
-        const BlockSlot L = block_slot(ci.ns);
+        const BlockSlot L = block_slot(n, ci.ns);
         BlockProblem B;
-        B.S = block_mem(n, a.gemm, ci.ns, ci.r, a.rdm);
-        B.gemm = a.gemm;
+        B.form = a.tiled ? sigma_form(n, ci.ns) : SIGMA_GLOBAL;
+        B.S = block_mem(n, B.form, ci.ns, ci.r, a.rdm);
+        B.U = (const float *)(slot + L.off_U);
         B.E = 0;
         B.full = (double *)(slot + L.off_full);
         const BlockMem &S = B.S;
@@ -1192,7 +1326,7 @@ __global__ void __launch_bounds__(BLOCK_THREADS, 1) k_casci_block(BatchArgs a, i
         pb.pp = (const short *)(smem + S.off_pp);
         pb.h = (double *)(smem + S.off_h);
         pb.hp = nullptr;
-        pb.V64 = (double *)(smem + S.off_V64);
+        pb.V64 = (double *)(B.form == SIGMA_LIST ? slot + L.off_V64 : smem + S.off_V64);
         pb.V32 = (float *)(smem + S.off_V32);
         pb.Hs64 = (double *)(slot + L.off_Hs64);
         pb.Hs32 = (float *)(slot + L.off_Hs32);
@@ -1429,32 +1563,24 @@ __global__ void __launch_bounds__(BLOCK_THREADS, 1) k_casci_block(BatchArgs a, i
     }
 }
 
-// Shared memory of a bucket's block launch, and whether its sigma is the tiled product.
-static size_t block_smem_bytes(const mbe_ctx *ctx, int n, const BatchArgs &a, const bool (&in)[MBE_MAX_CAS + 1], int rdm,
-                               int *gemm)
-{
-    size_t need[2] = {0, 0};
-    for (int k = 0; k <= n; ++k)
-        if (in[k])
-            for (int g = 0; g < 2; ++g)
-                if (g == 0 || n <= GEMM_MAX_N)
-                    need[g] = std::max(need[g], (size_t)block_mem(n, g, a.cls[k].ns, a.cls[k].r, rdm).bytes);
-    *gemm = n <= GEMM_MAX_N && need[1] <= ctx->smem_optin ? 1 : 0;
-    return need[*gemm];
-}
-
-int block_grid(mbe_ctx *ctx, BatchArgs &a, const bool (&in)[MBE_MAX_CAS + 1], int rdm, int *grid, size_t *smem,
+// Shared memory and slot size of a bucket's block launch (the classes `in`); a.tiled is cleared
+// when the shared-memory forms of sigma do not fit.
+int block_grid(mbe_ctx *ctx, BatchArgs &a, const bool (&in)[MBE_MAX_STRING_ORB + 1], int rdm, int *grid, size_t *smem,
                size_t *slot)
 {
-    *smem = block_smem_bytes(ctx, a.n, a, in, rdm, &a.gemm);
-    MBE_CHECK(*smem <= ctx->smem_optin, MBE_EUNSUPPORTED, "casci_batch: block solver needs %zu B shared memory",
-              *smem);
+    for (a.tiled = 1; a.tiled >= 0; --a.tiled) {
+        *smem = *slot = 0;
+        for (int k = 0; k <= a.n; ++k)
+            if (in[k]) {
+                const int form = a.tiled ? sigma_form(a.n, a.cls[k].ns) : SIGMA_GLOBAL;
+                *smem = std::max(*smem, (size_t)block_mem(a.n, form, a.cls[k].ns, a.cls[k].r, rdm).bytes);
+                *slot = std::max(*slot, block_slot(a.n, a.cls[k].ns).bytes);
+            }
+        if (*smem <= ctx->smem_optin - 1024) break;  // (some static shared memory besides)
+    }
+    MBE_CHECK(a.tiled >= 0, MBE_EUNSUPPORTED, "casci_batch: block solver needs %zu B shared memory", *smem);
     MBE_CU(allow_smem(k_casci_block, ctx->smem_optin));
     *grid = (int)std::min<int64_t>(ctx->sm_count, a.n_tuples);
-    int ns = 0;
-    for (int k = 0; k <= a.n; ++k)
-        if (in[k]) ns = std::max(ns, a.cls[k].ns);
-    *slot = block_slot(ns).bytes;
     return MBE_OK;
 }
 

@@ -60,13 +60,13 @@ struct BatchArgs {
     const double *eri;
     const double *F;
     const uint8_t *occ;
-    int ref[MBE_MAX_CAS];
+    int ref[MBE_MAX_LARGE_CAS];
     const int32_t *tuples;
     int64_t n_tuples;
     const int32_t *perm;
     const int64_t *bucket_off;
     unsigned long long *counters;
-    ClassInfo cls[MBE_MAX_CAS + 1];
+    ClassInfo cls[MBE_MAX_LARGE_CAS + 1];
     double e_ref_corr;
     int precision;
     double tol, tol_switch;
@@ -84,7 +84,7 @@ struct BatchArgs {
     int32_t *pstate;
     // tuned launch choices (mbe_tuning): warps per warp-solver block, block-solver basis
     int warps, block_basis;
-    int gemm;  // block solver: sigma by the tiled product
+    int tiled;  // block solver: the shared-memory forms of sigma fit
     // adjoint (casci_rdm_batch): 0 = energies only, 1 = + 1-RDM, 2 = + 1- and 2-RDM
     int rdm;
     const double *weights;
@@ -2025,7 +2025,7 @@ int launch_sector_mixed(mbe_ctx *ctx, const BatchArgs &a, int b, int k);        
 int launch_sector64(mbe_ctx *ctx, const BatchArgs &a, int b, int k);                     // casci_sector64.cu
 int launch_sector64_redo(mbe_ctx *ctx, const BatchArgs &a, int b, int k);                // casci_sector64_redo.cu
 int launch_warp_mixed_dpl(mbe_ctx *ctx, const BatchArgs &a, int b, const MixLayout &L, int dpl);  // casci_mixed.cu
-int block_grid(mbe_ctx *ctx, BatchArgs &a, const bool (&in)[MBE_MAX_CAS + 1], int rdm, int *grid, size_t *smem,
+int block_grid(mbe_ctx *ctx, BatchArgs &a, const bool (&in)[MBE_MAX_STRING_ORB + 1], int rdm, int *grid, size_t *smem,
                size_t *slot);                                                            // casci_block.cu
 int launch_block(mbe_ctx *ctx, const BatchArgs &a, int b, int grid, size_t smem);        // casci_block.cu
 __global__ void k_core_fock(int norb, const double *h1, const double *eri, const uint8_t *occ, double *F);

@@ -175,6 +175,12 @@ __device__ inline int64_t find_tuple(const int32_t *list, int64_t len, int m, co
     return -1;
 }
 
+// casci_batch for up to MBE_MAX_LARGE_CAS orbitals; classes: bit k set for the electron pairs
+// that occur (casci.cu).
+int casci_batch_wide(mbe_ctx *ctx, int norb, const double *h1, const double *eri, const uint8_t *occ, int n_ref,
+                     const int32_t *ref_orbs, double e_ref_corr, int order, int64_t n_tuples, const int32_t *tuples,
+                     const mbe_opts *opts, double *eps_out, int32_t *status_out, int32_t *iters_out, uint32_t classes);
+
 // Exclusive scan of per-block counts into offsets[0..nblocks] (one block).
 __global__ void k_scan_counts(const int32_t *counts, int64_t nblocks, int64_t *offsets);
 

@@ -3,8 +3,9 @@
 // occupied orbital (Type-2) makes R u Omega large at every order, up to the
 // sizes of a single big CASCI.  The tuples of one order are split on the host:
 // the ones the batched solvers take (at most MBE_MAX_CAS orbitals, at most
-// `large_ndet` determinants) go to casci_batch in one call; each other tuple is
-// solved by casci_solve with the whole GPU.  Both write eps = E_CAS(R u Omega) -
+// `large_ndet` determinants) go to casci_batch in one call, and so do tuples of more orbitals
+// that have few strings (ROUTE_BLOCK_NS), which a thread block solves alone; each other tuple
+// is solved by casci_solve with the whole GPU.  Both write eps = E_CAS(R u Omega) -
 // E_Phi - E_ref,corr (Eq. 1), so the routed results are interchangeable.
 #include <algorithm>
 #include <atomic>
@@ -51,6 +52,13 @@ __global__ void k_route_direct(int64_t n, const int64_t *rows, const int32_t *st
 // caller's context.
 constexpr int ROUTE_WORKERS = 4;
 constexpr int64_t ROUTE_CONCURRENT_NDET = 4000000;
+
+// Strings per spin up to which a tuple of more than MBE_MAX_CAS orbitals goes to the block
+// solver (c and V fit in shared memory: SIGMA_LIST).  A casci_solve of such a space (at most
+// 16,384 determinants) takes about 9 ms whatever its size, in launches and read-backs, four at a
+// time; a block solves one per SM.  91 spaces of 14 orbitals and at most 91 strings (the 26-site
+// ring's Type-2 expansion at order 2): 210 ms by casci_solve, 23 ms by the block solver.
+constexpr int64_t ROUTE_BLOCK_NS = 128;
 
 // Makes sure the context has k worker contexts.
 static int route_workers(mbe_ctx *ctx, int k)
@@ -128,7 +136,10 @@ extern "C" int casci_batch_routed(mbe_ctx *ctx, int norb, const double *h1, cons
     MBE_CU(cudaStreamSynchronize(ctx->stream));
 
     // Classify: batched (B), one whole-GPU solve each (L), or a one-determinant
-    // or malformed active space written directly (D).
+    // or malformed active space written directly (D).  Above MBE_MAX_CAS orbitals the
+    // batched ones are those of ROUTE_BLOCK_NS.
+    const bool wide = n_cas > MBE_MAX_CAS, penalty = opts && opts->s2_penalty != 0.0;
+    uint32_t classes = 0;
     std::vector<int64_t> rows_b, rows_l, rows_d, ndet_l;
     std::vector<int32_t> tup_b;
     std::vector<uint8_t> in_ref(norb, 0);
@@ -143,8 +154,11 @@ extern "C" int casci_batch_routed(mbe_ctx *ctx, int norb, const double *h1, cons
         }
         for (int i = 0; i < n_ref; ++i) k += occ_h[ref_orbs[i]];
         const int64_t ndet = ok ? binom(n_cas, k) * binom(n_cas, k) : 0;
-        const bool batched = n_cas <= MBE_MAX_CAS && (large_ndet <= 0 || ndet <= large_ndet || !ok);
+        const bool batched = wide ? ok && ndet > 1 && binom(n_cas, k) <= ROUTE_BLOCK_NS &&
+                                        (large_ndet <= 0 || ndet <= large_ndet) && !penalty
+                                  : large_ndet <= 0 || ndet <= large_ndet || !ok;
         if (batched) {
+            classes |= 1u << k;
             rows_b.push_back(t);
             tup_b.insert(tup_b.end(), tp, tp + order);
         } else if (!ok || ndet == 1) {
@@ -158,9 +172,14 @@ extern "C" int casci_batch_routed(mbe_ctx *ctx, int norb, const double *h1, cons
     RouteBuffers buf(ctx->stream);
     if (!rows_b.empty()) {
         const int64_t nb = (int64_t)rows_b.size();
+        auto batch = [&](int64_t n, const int32_t *tup, double *eps, int32_t *st, int32_t *it) {
+            return wide ? casci_batch_wide(ctx, norb, h1, eri, occ, n_ref, ref_orbs, e_ref_corr, order, n, tup, opts, eps,
+                                           st, it, classes)
+                        : casci_batch(ctx, norb, h1, eri, occ, n_ref, ref_orbs, e_ref_corr, order, n, tup, opts, eps, st,
+                                      it);
+        };
         if (nb == n_tuples) {
-            int rc = casci_batch(ctx, norb, h1, eri, occ, n_ref, ref_orbs, e_ref_corr, order, n_tuples, tuples,
-                                 opts, eps_out, status_out, iters_out);
+            int rc = batch(n_tuples, tuples, eps_out, status_out, iters_out);
             if (rc) return rc;
         } else {
             void *d_tup = nullptr, *d_rows = nullptr, *d_eps = nullptr, *d_st = nullptr, *d_it = nullptr;
@@ -173,9 +192,8 @@ extern "C" int casci_batch_routed(mbe_ctx *ctx, int norb, const double *h1, cons
                                    ctx->stream));
             MBE_CU(cudaMemcpyAsync(d_rows, rows_b.data(), (size_t)nb * sizeof(int64_t), cudaMemcpyHostToDevice,
                                    ctx->stream));
-            int rc = casci_batch(ctx, norb, h1, eri, occ, n_ref, ref_orbs, e_ref_corr, order, nb,
-                                 order > 0 ? (const int32_t *)d_tup : nullptr, opts, (double *)d_eps,
-                                 (int32_t *)d_st, (int32_t *)d_it);
+            int rc = batch(nb, order > 0 ? (const int32_t *)d_tup : nullptr, (double *)d_eps, (int32_t *)d_st,
+                           (int32_t *)d_it);
             if (rc) return rc;
             k_route_scatter<<<(unsigned)((nb + 255) / 256), 256, 0, ctx->stream>>>(
                 nb, (const int64_t *)d_rows, (const double *)d_eps, (const int32_t *)d_st, (const int32_t *)d_it,

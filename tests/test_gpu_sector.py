@@ -115,3 +115,24 @@ def test_integrals_that_are_not_finite(eng, ctx):
             eps, st, _ = ctx.casci_batch(dev(h1), dev(bad), dev(occ), [], 0.0, n, dev(np.array([t], dtype=np.int32)),
                                          eng.Opts(precision=prec))
             assert int(st[0]) == 2 and np.isnan(float(eps[0]))
+
+
+@pytest.mark.parametrize("prec", ["fp64", "mixed"])
+@pytest.mark.parametrize("n,k", [(13, 1), (13, 2), (13, 11), (14, 13), (15, 2), (15, 13), (16, 14), (16, 15)])
+def test_wide_spaces_of_few_strings(eng, ctx, n, k, prec):
+    """Tuple spaces of 13-16 orbitals with at most 128 strings go to the block solver; with a
+    determinant limit of one they go to casci_solve. One order-1 tuple of each kind in the list
+    where the space allows it, so that the lists are gathered and scattered."""
+    h1, eri, occ = random_system(18, 15 if k > 2 else 3, seed=n + k, eri_scale=0.2)
+    nocc = int(occ.sum())
+    ref = list(range(nocc - k, nocc)) + list(range(nocc, nocc + n - k - 1))
+    if len([p for p in ref if p < 18]) < n - 1:  # not enough virtuals: fill with lower occupied ones
+        ref = list(range(18 - (n - 1), 18))
+    ref = sorted(p for p in ref if p < 18)[:n - 1]
+    exp = [p for p in range(18) if p not in ref]
+    tup = dev(np.array([[p] for p in exp], dtype=np.int32))
+    args = (dev(h1), dev(eri), dev(occ), ref, 0.0, 1, tup, eng.Opts(precision=prec, tol=1e-8))
+    a, sa, _ = ctx.casci_batch_routed(*args)
+    b, sb, _ = ctx.casci_batch_routed(*args, large_ndet=1)
+    assert np.isin(sa.cpu().numpy(), (0, 4)).all() and np.isin(sb.cpu().numpy(), (0, 4)).all()
+    assert np.abs((a - b).cpu().numpy()).max() <= 2 * TOL[prec]
