@@ -25,6 +25,7 @@
 //     iteration to decide convergence.
 
 #include "casci_sector.cuh"
+#include "large_digits.cuh"
 
 using namespace mbe;
 
@@ -194,9 +195,11 @@ __global__ void k_large_diag(LargeCas L)
 // the odd sector vanishes).  Otherwise every element, in row-major order.
 template <bool SECTOR>
 __global__ void __launch_bounds__(SIGMA_THREADS) k_large_ab64(LargeCas L, const double *__restrict__ c,
-                                                               double *__restrict__ sigma, int sgn)
+                                                               double *__restrict__ sigma, int sgn,
+                                                               const unsigned long long *digits)
 {
     extern __shared__ __align__(16) char smem[];
+    if (digits && digits_usable(digits)) return;
     double *Vs = (double *)smem;
     const int P = L.P, Ns = L.Ns, R = L.R;
     for (int e = threadIdx.x; e < P * P; e += blockDim.x) Vs[e] = L.V[e];
@@ -257,9 +260,11 @@ constexpr int SS_ROWS = 32, SS_TK = 256, SS_THREADS = 256;
 // STORE: out[I][K] = (Hs X)[I][K] instead of adding it (TRANS false only).
 template <typename T, bool TRANS, bool STORE = false>
 __global__ void __launch_bounds__(SS_THREADS) k_large_ss(LargeCas L, const T *__restrict__ X,
-                                                          double *__restrict__ sigma)
+                                                          double *__restrict__ sigma,
+                                                          const unsigned long long *digits)
 {
     extern __shared__ __align__(16) char smem[];
+    if (digits && digits_usable(digits)) return;
     T *out = (T *)smem;  // [SS_ROWS][SS_TK + 1]
     const int Ns = L.Ns, lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const T *val = sizeof(T) == 8 ? (const T *)L.val : (const T *)L.val32;
@@ -305,8 +310,10 @@ __global__ void __launch_bounds__(SS_THREADS) k_large_ss(LargeCas L, const T *__
 // sigma += A + sgn A^T for an Ns x Ns matrix A (32 x 32 tiles through shared
 // memory): the same-spin terms of a vector in the spin-flip sector sgn, whose
 // beta term is sgn times the transpose of the alpha term A = Hs C.
-__global__ void k_sym_add(const double *__restrict__ A, int Ns, int sgn, double *__restrict__ sigma)
+__global__ void k_sym_add(const double *__restrict__ A, int Ns, int sgn, double *__restrict__ sigma,
+                          const unsigned long long *digits)
 {
+    if (digits && digits_usable(digits)) return;
     __shared__ double tile[32][33];
     const int nt = (Ns + 31) / 32;
     for (int64_t t = blockIdx.x; t < (int64_t)nt * nt; t += gridDim.x) {
@@ -584,6 +591,8 @@ struct LargePlan {
     int grid_ab64, grid_ss64, grid_ss32, grid_vec, grid_tr;
     size_t smem_ab64, smem_ss64, smem_ss32;
     void *cT;      // transposed coefficients (room for N float64)
+    DigitsArgs dg;  // float64 sigma on the tensor cores
+    int dg_chunk;   // 0: not used
 };
 
 
@@ -640,6 +649,22 @@ static int large_setup(mbe_ctx *ctx, int norb, const double *h1, const double *e
     L.tabT = tabT;
     plan->cT = bump.take<double>((size_t)L.N);  // float32 or float64 use
     L.Hd = dense_at ? dense_at : bump.take<double>((size_t)L.Ns * L.Ns);
+    plan->dg_chunk = large_digits_chunk(ctx->smem_optin, P, L.Ns, L.R);
+    double *hd = nullptr;
+    if (plan->dg_chunk) {
+        DigitsArgs &g = plan->dg;
+        g.P = P;
+        g.Ns = L.Ns;
+        g.R = L.R;
+        g.nsp = (L.Ns + 63) / 64 * 64;
+        g.tab = L.tab;
+        g.V = L.V;
+        g.hd = hd = bump.take<double>((size_t)L.Ns);
+        g.inv = bump.take<int32_t>((size_t)P * g.nsp);
+        g.maxb = bump.take<unsigned long long>(3);
+        g.planes = bump.take<uint16_t>((size_t)DIGITS * L.Ns * g.nsp);
+        g.hplanes = bump.take<uint16_t>((size_t)DIGITS * L.Ns * g.nsp);
+    }
     // (all of the above fits: the caller sized the workspace with large_bytes)
     k_core_fock<<<(norb * norb + 127) / 128, 128, 0, ctx->stream>>>(norb, h1, eri, occ, F);
     LargeSetupArgs sa;
@@ -661,6 +686,11 @@ static int large_setup(mbe_ctx *ctx, int norb, const double *h1, const double *e
     k_large_tables<<<(L.Ns + 255) / 256, 256, 0, ctx->stream>>>(L, tabT);
     MBE_CU(cudaGetLastError());
     ctx->launches += 8;
+    if (plan->dg_chunk) {
+        rc = large_digits_setup(ctx->stream, ctx->sm_count, plan->dg, L.Hd, hd);
+        if (rc) return rc;
+        ctx->launches += 4;
+    }
     *k_out = k;
     int iphi = string_rank(mphi);
     *dphi_out = (int64_t)iphi * L.Ns + iphi;
@@ -688,7 +718,7 @@ static int large_setup(mbe_ctx *ctx, int norb, const double *h1, const double *e
 }
 
 // Workspace bytes of large_setup (and the dense Hs unless aliased).
-static size_t large_bytes(int norb, int n, int k, bool dense_separate, bool fp32)
+static size_t large_bytes(const mbe_ctx *ctx, int norb, int n, int k, bool dense_separate, bool fp32)
 {
     const int64_t ns = binom(n, k), N = ns * ns;
     const int P = n * (n + 1) / 2;
@@ -699,6 +729,10 @@ static size_t large_bytes(int norb, int n, int k, bool dense_separate, bool fp32
                align256((ns + 1) * 8) + 4096;
     b += align256((size_t)k * (n - k + 1) * ns * 4) + align256((size_t)N * 8);
     if (dense_separate) b += align256((size_t)ns * ns * 8);
+    if (large_digits_chunk(ctx->smem_optin, P, (int)ns, k * (n - k + 1))) {
+        const size_t nsp = (size_t)(ns + 63) / 64 * 64;
+        b += align256(ns * 8) + align256(P * nsp * 4) + 256 + 2 * align256((size_t)DIGITS * ns * nsp * 2);
+    }
     return b;
 }
 
@@ -710,13 +744,23 @@ static int large_sigma_launch(mbe_ctx *ctx, const LargePlan &pl, const T *c, dou
 {
     TimedLaunch tl(ctx, order_tag, 2, sizeof(T) == 8 ? 64 : 32);
     const int Ns = pl.L.Ns;
+    const unsigned long long *digits = nullptr;
     if (sizeof(T) == 8) {
+        if (pl.dg_chunk) {
+            DigitsArgs g = pl.dg;
+            g.c = (const double *)c;
+            g.sigma = sigma;
+            const int rc = large_sigma_digits(ctx->stream, ctx->sm_count, ctx->smem_optin, g, pl.dg_chunk);
+            if (rc) return rc;
+            ctx->launches += 4;
+            digits = pl.dg.maxb;  // the kernels below return at once, unless the scales are extreme
+        }
         if (sgn == 0)
             k_large_ab64<false><<<pl.grid_ab64, SIGMA_THREADS, pl.smem_ab64, ctx->stream>>>(pl.L, (const double *)c,
-                                                                                          sigma, 0);
+                                                                                          sigma, 0, digits);
         else
             k_large_ab64<true><<<pl.grid_ab64, SIGMA_THREADS, pl.smem_ab64, ctx->stream>>>(pl.L, (const double *)c,
-                                                                                         sigma, sgn);
+                                                                                         sigma, sgn, digits);
     } else {
         // the dense product on the tensor cores (large_tc.cu)
         const int rc = large_ab_tc(ctx->stream, ctx->sm_count, ctx->smem_optin, pl.L.P, pl.L.Ns, pl.L.R, pl.L.tab,
@@ -727,16 +771,16 @@ static int large_sigma_launch(mbe_ctx *ctx, const LargePlan &pl, const T *c, dou
     const size_t smem_ss = sizeof(T) == 8 ? pl.smem_ss64 : pl.smem_ss32;
     if (sgn == 0) {
         T *cT = (T *)pl.cT;
-        k_large_ss<T, false><<<grid_ss, SS_THREADS, smem_ss, ctx->stream>>>(pl.L, c, sigma);
+        k_large_ss<T, false><<<grid_ss, SS_THREADS, smem_ss, ctx->stream>>>(pl.L, c, sigma, digits);
         k_large_transpose<T><<<pl.grid_tr, dim3(32, 8), 0, ctx->stream>>>(c, Ns, cT);
-        k_large_ss<T, true><<<grid_ss, SS_THREADS, smem_ss, ctx->stream>>>(pl.L, cT, sigma);
+        k_large_ss<T, true><<<grid_ss, SS_THREADS, smem_ss, ctx->stream>>>(pl.L, cT, sigma, digits);
     } else {
         // c in the sector sgn: the beta same-spin term is sgn times the transpose
         // of the alpha one, so one product (into the spare buffer) and a
         // transposing add replace the second product and the transpose of c
         double *A = (double *)pl.cT;
-        k_large_ss<T, false, true><<<grid_ss, SS_THREADS, smem_ss, ctx->stream>>>(pl.L, c, A);
-        k_sym_add<<<pl.grid_tr, dim3(32, 8), 0, ctx->stream>>>(A, Ns, sgn, sigma);
+        k_large_ss<T, false, true><<<grid_ss, SS_THREADS, smem_ss, ctx->stream>>>(pl.L, c, A, digits);
+        k_sym_add<<<pl.grid_tr, dim3(32, 8), 0, ctx->stream>>>(A, Ns, sgn, sigma, digits);
     }
     MBE_CU(cudaGetLastError());
     ctx->launches += sgn == 0 ? 4 : 3;
@@ -764,7 +808,7 @@ extern "C" int casci_sigma_large(mbe_ctx *ctx, int norb, const double *h1, const
     for (int i = 0; i < n_cas; ++i) k0 += (cas_orbs[i] >= 0 && cas_orbs[i] < norb && occ_h[cas_orbs[i]]) ? 1 : 0;
     const int64_t N = binom(n_cas, k0) * binom(n_cas, k0);
     const bool fp32 = precision == MBE_PREC_MIXED;
-    size_t bytes = large_bytes(norb, n_cas, k0, true, fp32) + (fp32 ? align256(N * 4) : 0);
+    size_t bytes = large_bytes(ctx, norb, n_cas, k0, true, fp32) + (fp32 ? align256(N * 4) : 0);
     void *ws = nullptr;
     int rc = workspace(ctx, bytes, &ws);
     if (rc) return rc;
@@ -1108,7 +1152,7 @@ extern "C" int casci_solve(mbe_ctx *ctx, int norb, const double *h1, const doubl
     D.ld = vec / 8;
     D.nblk = ctx->sm_count * 4;
     const bool mixed = o.precision == MBE_PREC_MIXED;
-    size_t bytes = large_bytes(norb, n_cas, k0, false, mixed) + vec * (2 * MLARGE + 6) + align256((size_t)N * 4) +
+    size_t bytes = large_bytes(ctx, norb, n_cas, k0, false, mixed) + vec * (2 * MLARGE + 6) + align256((size_t)N * 4) +
                    align256((size_t)D.nblk * LRED * 8) + 8 * 256 + 4096;
     void *ws = nullptr;
     int rc = workspace(ctx, bytes, &ws);

@@ -8,6 +8,7 @@ in fixed point with a scale taken from them.
 """
 
 import itertools
+import math
 
 import numpy as np
 import pytest
@@ -17,6 +18,7 @@ torch = pytest.importorskip("torch")
 pytestmark = pytest.mark.gpu
 
 from oracle import adjoint as oad  # noqa: E402
+from oracle import fci  # noqa: E402
 from oracle import mbe as omb  # noqa: E402
 from workloads import random_system  # noqa: E402
 
@@ -136,3 +138,34 @@ def test_wide_spaces_of_few_strings(eng, ctx, n, k, prec):
     b, sb, _ = ctx.casci_batch_routed(*args, large_ndet=1)
     assert np.isin(sa.cpu().numpy(), (0, 4)).all() and np.isin(sb.cpu().numpy(), (0, 4)).all()
     assert np.abs((a - b).cpu().numpy()).max() <= 2 * TOL[prec]
+
+
+@pytest.mark.parametrize("n,k", [(1, 1), (3, 1), (5, 2), (7, 4), (9, 3), (10, 8), (11, 5), (13, 2), (14, 3)])
+@pytest.mark.parametrize("scale", [1.0, 1e-150, 1e150])
+def test_large_sigma_on_digits(eng, ctx, n, k, scale):
+    # float64 sigma of one large space from products of 8-bit digits; integrals whose scale is
+    # near the ends of the range (1e-150, 1e150) stay on the plain float64 kernels.  Per term the
+    # operands are rounded to 2^-56 of their largest and what is left out is below 2^-53.
+    h1, eri, occ = random_system(n + 1, k, seed=n)
+    h1, eri = h1 * scale, eri * scale
+    A = list(range(k)) + list(range(k + 1, n + 1)) if n > k else list(range(n))
+    rng = np.random.default_rng(k)
+    N = math.comb(n, k) ** 2
+    c = rng.normal(size=N)
+    got = ctx.casci_sigma_large(dev(h1), dev(eri), dev(occ), A, dev(c), "fp64")[0].cpu().numpy()
+    rows = rng.choice(N, size=min(N, 200), replace=False)
+    _, h_eff, eri_a = omb.frozen_core(h1, eri, occ, A)
+    want = fci.sigma_rows(h_eff, eri_a, k, k, c, rows)
+    terms = (k * (n - k + 1)) ** 2 + 2 * (1 + k * (n - k) + math.comb(k, 2) * math.comb(n - k, 2))
+    bound = terms * 2.0 ** -50 * max(np.abs(eri_a).max(), np.abs(h_eff).max()) * np.abs(c).max()
+    assert np.abs(got[rows] - want).max() <= bound
+
+
+def test_large_sigma_keeps_a_nan_where_it_belongs(eng, ctx):
+    # a NaN in c reaches the determinants that it is connected to, and only those
+    n, k = 8, 4
+    h1, eri, occ = random_system(n, k, seed=1)
+    c = np.random.default_rng(1).normal(size=math.comb(n, k) ** 2)
+    c[0] = np.nan
+    got = ctx.casci_sigma_large(dev(h1), dev(eri), dev(occ), list(range(n)), dev(c), "fp64")[0].cpu().numpy()
+    assert np.isnan(got[0]) and np.isfinite(got).sum() > got.size // 4
