@@ -32,6 +32,7 @@ __device__ __forceinline__ char *block_shared()
 constexpr int BLOCK_THREADS = 512;  // one block per SM: 128 registers a thread, up to 227 KB
 constexpr int GEMM_MAX_N = 9;       // orbitals up to which sigma is the tiled product
 constexpr int GEMM_T_BYTES = 48 * 1024;
+constexpr int LIST_STAGE = 16 * 1024;  // bytes of Hs staged by SIGMA_LIST
 constexpr int LIST_MAX_NS = 128;    // strings up to which larger orbital counts keep c in shared memory
 
 // Forms of sigma: c in global memory and both lists walked per element; the tiled product; c and
@@ -80,7 +81,7 @@ struct GemmShape {
     int fst;        // row stride of the float32 c (not a multiple of 32: its columns are written too)
     int pst;        // row stride of the float32 V (pairs, padded to 6)
     int rs;         // row stride of the lists
-    int np, tiles;  // pair groups, tiles per alpha string
+    int nj, np, tiles;  // string and pair groups, tiles per alpha string
     int g;          // alpha strings per stage
 };
 
@@ -88,15 +89,18 @@ template <typename T>
 __host__ __device__ inline GemmShape gemm_shape(int n, int ns, int r)
 {
     GemmShape s;
-    const int P = n * (n + 1) / 2, tp = sizeof(T) == 8 ? 3 : 6;
+    const int P = n * (n + 1) / 2, tp = sizeof(T) == 8 ? 3 : 6, tj = sizeof(T) == 8 ? 4 : 8;
     s.cst = hs_stride(ns);
     s.fst = s.cst % 32 == 0 ? s.cst + 4 : s.cst;
+    if (s.fst % 8) s.fst += 4;  // (whole tiles of 8)
+    if (s.fst % 32 == 0) s.fst += 8;
     s.pst = (P + 5) / 6 * 6;
     s.rs = r | 1;
     s.np = (P + tp - 1) / tp;
-    s.tiles = s.np * (s.cst / 4);
+    s.nj = (s.cst + tj - 1) / tj;
+    s.tiles = s.np * s.nj;
     s.g = BLOCK_THREADS / s.tiles;
-    const int fit = GEMM_T_BYTES / (P * s.cst * (int)sizeof(T));
+    const int fit = (n < GEMM_MAX_N ? 2 : 1) * GEMM_T_BYTES / (P * s.cst * (int)sizeof(T));
     if (s.g > fit) s.g = fit;
     if (s.g > ns) s.g = ns;
     if (s.g > 1) s.g &= ~1;  // (strings are taken in pairs)
@@ -105,7 +109,11 @@ __host__ __device__ inline GemmShape gemm_shape(int n, int ns, int r)
 }
 
 // Row stride of the float32 c of SIGMA_LIST
-__host__ __device__ inline int list_stride(int ns) { return hs_stride(ns) % 32 == 0 ? hs_stride(ns) + 4 : hs_stride(ns); }
+__host__ __device__ inline int list_stride(int ns)
+{
+    const int s = (ns + 7) / 8 * 8;  // (whole tiles of the same-spin product)
+    return s % 32 == 0 ? s + 8 : s;
+}
 
 struct BlockMem {  // dynamic shared memory
     int off_A, off_pp, off_h, off_V64, off_V32, off_red, off_G, off_J, off_ev, off_y, off_yp, off_r, off_misc,
@@ -138,10 +146,11 @@ __host__ __device__ inline BlockMem block_mem(int n, int form, int ns, int r, in
     S.off_list = o; o = al16(o + (gemm ? 2 * ns * (r | 1) : form == SIGMA_LIST ? 4 * ns * (r + 1) : 0));
     S.off_c = o;
     if (form == SIGMA_LIST) o = al16(o + 4 * ns * list_stride(ns));
+    const int stage = form == SIGMA_LIST ? LIST_STAGE : 0;
     if (gemm) {
         // fixed point: c; float32: c, V twice over with both signs, list offsets (see sigma_gemm)
         const GemmShape a = gemm_shape<float>(n, ns, r);
-        const int f = al16(4 * ns * a.fst) + 16 * P * a.pst + 4 * ns * r;
+        const int f = al16(4 * ns * a.fst) + 8 * P * a.pst + 4 * ns * r;
         o = al16(o + (f > 8 * ns * a.cst ? f : 8 * ns * a.cst));
     }
     S.off_T = o;
@@ -150,6 +159,7 @@ __host__ __device__ inline BlockMem block_mem(int n, int form, int ns, int r, in
         const int ta = a.g * P * a.cst * 4, tb = b.g * P * b.cst * 8;
         o = al16(o + (ta > tb ? ta : tb));
     }
+    o = al16(o + stage);
     // the density matrices' vectors lie over c and T
     const int d = rdm ? S.off_c + 8 * 33 * (n * n + 1) : 0;
     S.bytes = al16(o > d ? o : d);
@@ -187,33 +197,48 @@ __device__ inline void expand_full(const Problem &pb, const T *v, T *full, int l
 }
 
 // M = C Hs for the float32 product: 8 x 4 tiles, c from shared memory by its rows (C[i][J] is
-// sgn C[J][i]), Hs through L1.
-__device__ inline void same_spin(const Problem &pb, int ld, int fst, const float *c, const float *Hs, float *M)
+// sgn C[J][i]), Hs in chunks of rows through shared memory (buf: bytes of it that are free; Hs is
+// larger than what is left of L1, and one row of it per step left the warps waiting for L2).
+// Ends without a barrier.
+__device__ inline void same_spin(const Problem &pb, int ld, int fst, const float *c, const float *Hs, float *M, char *buf,
+                                 int bytes)
 {
-    const int nj = ld / 4, ni = (pb.Ns + 7) / 8;
-    for (int q = threadIdx.x; q < ni * nj; q += blockDim.x) {
-        const int i0 = q / nj * 8, j0 = (q - q / nj * nj) * 4;
+    const int nj = ld / 4, ni = (pb.Ns + 7) / 8, tid = threadIdx.x, nt = blockDim.x;
+    const int rows = min(pb.Ns, bytes / (4 * ld));
+    float *hs = (float *)buf;
+    for (int q0 = 0; q0 < ni * nj; q0 += nt) {
+        const int q = q0 + tid, i0 = q / nj * 8, j0 = (q - q / nj * nj) * 4;
+        const bool on = q < ni * nj;
         const int i1 = i0 + 4 < fst ? i0 + 4 : i0;  // (past the last string: not stored)
         uint64_t a[4][4];
 #pragma unroll
         for (int i = 0; i < 4; ++i)
 #pragma unroll
             for (int j = 0; j < 4; ++j) a[i][j] = 0ull;
+        for (int J0 = 0; J0 < pb.Ns; J0 += rows) {
+            const int jn = min(rows, pb.Ns - J0);
+            __syncthreads();
 #pragma unroll 4
-        for (int J = 0; J < pb.Ns; ++J) {
-            const float4 h = *(const float4 *)(Hs + J * ld + j0);
-            const ulonglong2 c0 = *(const ulonglong2 *)(c + J * fst + i0), c1 = *(const ulonglong2 *)(c + J * fst + i1);
-            const uint64_t cc[4] = {c0.x, c0.y, c1.x, c1.y};
-            const uint64_t hh[4] = {dup2(h.x), dup2(h.y), dup2(h.z), dup2(h.w)};
+            for (int e = tid; e < jn * nj; e += nt) ((float4 *)hs)[e] = ((const float4 *)(Hs + J0 * ld))[e];
+            __syncthreads();
+            if (on)
+#pragma unroll 2
+                for (int J = 0; J < jn; ++J) {
+                    const float4 h = *(const float4 *)(hs + J * ld + j0);
+                    const ulonglong2 c0 = *(const ulonglong2 *)(c + (J0 + J) * fst + i0),
+                                     c1 = *(const ulonglong2 *)(c + (J0 + J) * fst + i1);
+                    const uint64_t cc[4] = {c0.x, c0.y, c1.x, c1.y};
+                    const uint64_t hh[4] = {dup2(h.x), dup2(h.y), dup2(h.z), dup2(h.w)};
 #pragma unroll
-            for (int i = 0; i < 4; ++i)
+                    for (int i = 0; i < 4; ++i)
 #pragma unroll
-                for (int j = 0; j < 4; ++j) ffma2(a[i][j], cc[i], hh[j]);
+                        for (int j = 0; j < 4; ++j) ffma2(a[i][j], cc[i], hh[j]);
+                }
         }
         const float sg = pb.sector > 0 ? 1.f : -1.f;
 #pragma unroll
         for (int i = 0; i < 8; ++i)
-            if (i0 + i < pb.Ns) {
+            if (on && i0 + i < pb.Ns) {
                 float4 o;
                 const int h = 32 * (i & 1);
                 o.x = sg * __uint_as_float((uint32_t)(a[i >> 1][0] >> h));
@@ -226,7 +251,7 @@ __device__ inline void same_spin(const Problem &pb, int ld, int fst, const float
 }
 
 // The same on integers (Hs without its diagonal): 2 x 2 tiles, one int64 per element.
-__device__ inline void same_spin(const Problem &pb, int ld, int, const int2 *c, const int2 *Hs, long long *M)
+__device__ inline void same_spin(const Problem &pb, int ld, int, const int2 *c, const int2 *Hs, long long *M, char *, int)
 {
     const int nt = ld / 2;
     for (int q = threadIdx.x; q < nt * nt; q += blockDim.x) {
@@ -254,38 +279,44 @@ __device__ inline void same_spin(const Problem &pb, int ld, int, const int2 *c, 
     }
 }
 
-// One tile of T in float32: 4 strings x 6 pairs, two strings per instruction (fma.rn.f32x2).
-// Per list entry one offset pair, the four strings and six pairs (V holds each value twice).
+// One tile of T in float32: 8 strings x 6 pairs, two strings per instruction (fma.rn.f32x2).  A
+// 16-byte shared load takes four cycles of the SM's load path even when all lanes read the same
+// address, so the tile is chosen for few bytes per multiply-add: 56 for 48 (at 4 x 6 with V
+// stored twice over, 64 for 24, the load path was the bound).
 __device__ __forceinline__ void gemm_tile(const Problem &pb, const GemmShape &s, const uint32_t *la, const char *c,
                                           const char *V, int j0, int pg, float *T)
 {
-    uint64_t a[6][2];
+    uint64_t a[6][4];
 #pragma unroll
-    for (int k = 0; k < 6; ++k) a[k][0] = a[k][1] = 0ull;
+    for (int k = 0; k < 6; ++k)
+#pragma unroll
+        for (int i = 0; i < 4; ++i) a[k][i] = 0ull;
     c += 4 * j0;
-    V += 48 * pg;
-#pragma unroll 4
+    V += 24 * pg;
+#pragma unroll 2
     for (int x = 0; x < pb.R; ++x) {
         const uint32_t e = la[x];
-        const ulonglong2 cv = *(const ulonglong2 *)(c + ((e & 0xffffu) << 4));
-        const ulonglong2 *v = (const ulonglong2 *)(V + (e >> 16 << 4));
-        const ulonglong2 v0 = v[0], v1 = v[1], v2 = v[2];
-        ffma2(a[0][0], v0.x, cv.x);
-        ffma2(a[0][1], v0.x, cv.y);
-        ffma2(a[1][0], v0.y, cv.x);
-        ffma2(a[1][1], v0.y, cv.y);
-        ffma2(a[2][0], v1.x, cv.x);
-        ffma2(a[2][1], v1.x, cv.y);
-        ffma2(a[3][0], v1.y, cv.x);
-        ffma2(a[3][1], v1.y, cv.y);
-        ffma2(a[4][0], v2.x, cv.x);
-        ffma2(a[4][1], v2.x, cv.y);
-        ffma2(a[5][0], v2.y, cv.x);
-        ffma2(a[5][1], v2.y, cv.y);
+        const ulonglong2 *cp = (const ulonglong2 *)(c + ((e & 0xffffu) << 4));
+        const ulonglong2 c0 = cp[0], c1 = cp[1];
+        const float2 *v = (const float2 *)(V + (e >> 16 << 3));
+        const float2 v0 = v[0], v1 = v[1], v2 = v[2];
+        const float vv[6] = {v0.x, v0.y, v1.x, v1.y, v2.x, v2.y};
+#pragma unroll
+        for (int k = 0; k < 6; ++k) {
+            const uint64_t d = dup2(vv[k]);
+            ffma2(a[k][0], d, c0.x);
+            ffma2(a[k][1], d, c0.y);
+            ffma2(a[k][2], d, c1.x);
+            ffma2(a[k][3], d, c1.y);
+        }
     }
 #pragma unroll
     for (int k = 0; k < 6; ++k)
-        if (pg * 6 + k < pb.P) *(ulonglong2 *)(T + (pg * 6 + k) * s.cst + j0) = make_ulonglong2(a[k][0], a[k][1]);
+        if (pg * 6 + k < pb.P) {
+            float *t = T + (pg * 6 + k) * s.cst + j0;
+            *(ulonglong2 *)t = make_ulonglong2(a[k][0], a[k][1]);
+            if (j0 + 4 < s.cst) *(ulonglong2 *)(t + 4) = make_ulonglong2(a[k][2], a[k][3]);
+        }
 }
 
 // One tile of T in fixed point: 4 strings x 3 pairs.
@@ -340,10 +371,10 @@ __device__ __noinline__ void sigma_gemm(const BlockProblem &B, const T *src, T *
     const double *hd = (const double *)(block_shared() + B.S.off_hd);
     A *M = (A *)B.full;
     const int cld = F64 ? s.cst : s.fst;
-    // float32: behind c, V with every value twice (rows 2 pair + neg), and the lists as offsets
-    // of the rows of c (low half) and V (high half) in units of 16 bytes
+    // float32: behind c, V with both signs (rows 2 pair + neg), and the lists as offsets of the
+    // rows of c (low half, in units of 16 bytes) and V (high half, 8 bytes)
     char *Vd = block_shared() + B.S.off_c + al16(4 * Ns * s.fst);
-    uint32_t *list32 = (uint32_t *)(Vd + 16 * pb.P * s.pst);
+    uint32_t *list32 = (uint32_t *)(Vd + 8 * pb.P * s.pst);
     {
         int ia = 0, ib = 0;
         tri_advance(ia, ib, tid, Ns);
@@ -364,8 +395,8 @@ __device__ __noinline__ void sigma_gemm(const BlockProblem &B, const T *src, T *
             const float *V32 = (const float *)(block_shared() + B.S.off_V32);
             for (int q = tid; q < pb.P * s.pst; q += nt) {
                 const int x = q / s.pst, y = q - x * s.pst;
-                ((float2 *)Vd)[2 * x * s.pst + y] = make_float2(V32[q], V32[q]);
-                ((float2 *)Vd)[(2 * x + 1) * s.pst + y] = make_float2(-V32[q], -V32[q]);
+                ((float *)Vd)[2 * x * s.pst + y] = V32[q];
+                ((float *)Vd)[(2 * x + 1) * s.pst + y] = -V32[q];
             }
             for (int q = tid; q < Ns * R; q += nt) {
                 const int e = list[q / R * s.rs + q % R];
@@ -374,20 +405,21 @@ __device__ __noinline__ void sigma_gemm(const BlockProblem &B, const T *src, T *
         }
     }
     __syncthreads();
-    same_spin(pb, s.cst, cld, c, F64 ? (const E *)pb.Hs64 : (const E *)pb.Hs32, M);
-    const int nj = s.cst / 4;
+    same_spin(pb, s.cst, cld, c, F64 ? (const E *)pb.Hs64 : (const E *)pb.Hs32, M, (char *)Tm,
+              s.g * pb.P * s.cst * (int)sizeof(A));
+    if constexpr (!F64) __syncthreads();  // (Hs was staged over T)
     // Strings are taken from both ends of the list, so that each pair of them has Ns + 1 elements
     // with Ia <= Ib.
     for (int I0 = 0; I0 < Ns; I0 += s.g) {
         const int gc = min(s.g, Ns - I0);
         auto string = [&](int i) { return i & 1 ? Ns - 1 - (i >> 1) : i >> 1; };
         for (int q = tid; q < gc * s.tiles; q += nt) {
-            const int g = q / s.tiles, r = q - g * s.tiles, pg = r / nj, jj = r - pg * nj, Ia = string(I0 + g);
+            const int g = q / s.tiles, r = q - g * s.tiles, pg = r / s.nj, jj = r - pg * s.nj, Ia = string(I0 + g);
             if constexpr (F64)
                 gemm_tile(pb, s, list + Ia * s.rs, c, (const int2 *)(block_shared() + B.S.off_V64), 4 * jj, pg,
                           Tm + g * pb.P * s.cst);
             else
-                gemm_tile(pb, s, list32 + Ia * R, (const char *)c, Vd, 4 * jj, pg, Tm + g * pb.P * s.cst);
+                gemm_tile(pb, s, list32 + Ia * R, (const char *)c, Vd, 8 * jj, pg, Tm + g * pb.P * s.cst);
         }
         __syncthreads();  // (also orders M, written above, before its first use)
         const int n1 = Ns + 1, ne = (gc + 1) / 2 * n1;
@@ -397,7 +429,9 @@ __device__ __noinline__ void sigma_gemm(const BlockProblem &B, const T *src, T *
             const int q = q0 + tid, el = q >> split, pr = el / n1, r = el - pr * n1;
             const int first = string(I0 + 2 * pr), len = Ns - first;  // elements of the pair's first string
             const int g = 2 * pr + (r < len ? 0 : 1), Ia = r < len ? first : string(I0 + g), Ib = Ia + r - (r < len ? 0 : len);
-            const bool on = g < gc && Ib < Ns;
+            const bool on = g < gc && Ib < Ns, last = on && (q & ((1 << split) - 1)) == 0;
+            // (the same-spin terms come from L2: asked for before the walk over the list)
+            const A m0 = last ? M[Ia * s.cst + Ib] : (A)0, m1 = last ? M[Ib * s.cst + Ia] : (A)0;
             A acc = 0;
             if (on) {
                 const A *t = Tm + g * pb.P * s.cst;
@@ -410,10 +444,9 @@ __device__ __noinline__ void sigma_gemm(const BlockProblem &B, const T *src, T *
                 }
             }
             for (int o = 1; o < 1 << split; o <<= 1) acc += __shfl_xor_sync(FULL, acc, o);
-            if (on && (q & ((1 << split) - 1)) == 0) {
-                const A mt = M[Ib * s.cst + Ia];
+            if (last) {
                 const int h = Ia * Ns - Ia * (Ia - 1) / 2 + Ib - Ia;
-                acc += M[Ia * s.cst + Ib] + (sgn > 0 ? mt : -mt);
+                acc += m0 + (sgn > 0 ? m1 : -m1);
                 T v;
                 if constexpr (F64) {
                     v = fma(hd[Ia] + hd[Ib], src[h], (double)acc * (pow2(B.E - 54) * (Ia == Ib ? 1.0 : 1.4142135623730951)));
@@ -456,7 +489,7 @@ __device__ __noinline__ void sigma_list(const BlockProblem &B, const float *src,
         for (int q = tid; q < Ns * (ld - Ns); q += nt) c[q / (ld - Ns) * ld + Ns + q % (ld - Ns)] = 0.f;
     }
     __syncthreads();
-    same_spin(pb, hs_stride(Ns), ld, c, pb.Hs32, M);
+    same_spin(pb, hs_stride(Ns), ld, c, pb.Hs32, M, smem + S.off_T, LIST_STAGE);
     __syncthreads();
     int ia = 0, ib = 0;
     tri_advance(ia, ib, tid, Ns);
@@ -557,8 +590,10 @@ __device__ __noinline__ void sigma_block(const BlockProblem &B, const T *src, T 
 // theta = y.G y, which make the lowest pair float64-accurate (one warp).
 // Output: y[0..m) (unit norm), y2 (the second lowest, which seeds the thick restart), and
 // misc[0] = theta; ends with a barrier.
+// warm: the last call was on the leading (m - 1) x (m - 1) part of G, and its eigenbasis is the
+// start of this one (an arrow matrix is left to diagonalise).
 template <bool REFINE>
-__device__ __noinline__ void small_eig_block(const BlockMem &S, int m)
+__device__ __noinline__ void small_eig_block(const BlockMem &S, int m, bool warm)
 {
     char *smem = block_shared();
     const double *G = (const double *)(smem + S.off_G);
@@ -570,7 +605,20 @@ __device__ __noinline__ void small_eig_block(const BlockMem &S, int m)
     const bool on = i < m && j < m;
     const double shift = G[0];
     float *A = buf, *E = buf + MMAX * MMAX, *A2 = buf + 2 * MMAX * MMAX, *E2 = buf + 3 * MMAX * MMAX;
-    if (on) {
+    if (warm) {
+        // in the last call's eigenbasis: its eigenvalues, and the new row
+        if (tid < m - 1) {
+            float b = 0.f;
+            for (int k = 0; k < m - 1; ++k) b += E[k * MMAX + tid] * (float)G[k * MMAX + m - 1];
+            rot[tid].x = b;
+        }
+        __syncthreads();
+        if (on) {
+            const bool last = i == m - 1 || j == m - 1;
+            A[tid] = i == j ? (last ? (float)(G[i * MMAX + i] - shift) : ev[i]) : last ? rot[i < j ? i : j].x : 0.f;
+            if (last) E[tid] = i == j ? 1.0f : 0.0f;
+        }
+    } else if (on) {
         A[tid] = (float)(G[i * MMAX + j] - (i == j ? shift : 0.0));
         E[tid] = i == j ? 1.0f : 0.0f;
     }
@@ -599,8 +647,10 @@ __device__ __noinline__ void small_eig_block(const BlockMem &S, int m)
                     float c = 1.f, sn = 0.f;
                     const float apq = v < m ? A[tid * MMAX + v] : 0.f;
                     if (fabsf(apq) >= 1e-36f) {
-                        const float th = (A[v * MMAX + v] - A[tid * MMAX + tid]) / (2.0f * apq);
-                        float t = 1.0f / (fabsf(th) + sqrtf(th * th + 1.0f));
+                        // (fast division and root: a rotation that is off by a rounding error leaves
+                        // that much for the next sweep)
+                        const float th = __fdividef(A[v * MMAX + v] - A[tid * MMAX + tid], 2.0f * apq), q = th * th + 1.0f;
+                        float t = q < 1e30f ? __fdividef(1.0f, fabsf(th) + q * rsqrtf(q)) : 0.5f / fabsf(th);
                         if (th < 0.0f) t = -t;
                         c = rsqrtf(t * t + 1.0f);
                         sn = t * c;
@@ -627,6 +677,11 @@ __device__ __noinline__ void small_eig_block(const BlockMem &S, int m)
             E = E2;
             E2 = z;
         }
+    }
+    if (E != buf + MMAX * MMAX) {
+        if (on) E2[tid] = E[tid];
+        __syncthreads();
+        E = buf + MMAX * MMAX;
     }
     if (tid < 32) {
         float best = (lane < m) ? A[lane * MMAX + lane] : 3.0e38f;
@@ -658,6 +713,34 @@ __device__ __noinline__ void small_eig_block(const BlockMem &S, int m)
         }
         __syncwarp();
         double theta = shift + (double)best;
+        __syncwarp();
+        if (!REFINE) {
+            // one such step in float32, which also takes out what the warm starts have gathered in E
+            float row[MMAX];
+#pragma unroll
+            for (int k = 0; k < MMAX; ++k)
+                row[k] = lane < m && k < m ? (float)(k == lane ? G[k * MMAX + k] - shift : G[lane * MMAX + k]) : 0.f;
+            float yi = lane < m ? E[lane * MMAX + bi] : 0.f;
+            float th = 0.f;
+#pragma unroll 1
+            for (int step = 0; step < 2; ++step) {
+                float g = 0.f;
+#pragma unroll
+                for (int k = 0; k < MMAX; ++k) g += row[k] * __shfl_sync(FULL, yi, k);
+                th = warp_sum(yi * g) / warp_sum(yi * yi);
+                if (step == 1) break;
+                const float ri = g - th * yi;
+                float ck = 0.f;
+                for (int k = 0; k < m; ++k) ck += (lane < m ? E[k * MMAX + lane] : 0.f) * __shfl_sync(FULL, ri, k);
+                const float den = lane < m ? ev[lane] - th : 0.f;
+                ck = lane != bi && fabsf(den) > 1e-30f ? ck / den : 0.f;
+                float z = yi;
+                for (int k = 0; k < m; ++k) z -= (lane < m ? E[lane * MMAX + k] : 0.f) * __shfl_sync(FULL, ck, k);
+                yi = z * rsqrtf(warp_sum(z * z));
+            }
+            if (lane < m) y[lane] = (double)yi;
+            theta = shift + (double)th;
+        }
         if (REFINE) {
             for (int step = 0; step < 2; ++step) {
                 double g = 0.0, yi = (lane < m) ? y[lane] : 0.0;
@@ -825,14 +908,15 @@ __device__ __noinline__ PhaseOut davidson_block(const BlockProblem &B, T *Vp, T 
         G[0] = 0.0;  // x0.r0 = 0: shift is x0's Rayleigh quotient
     }
     __syncthreads();
-    int m = 1;
+    int m = 1, warm = 0;
     double theta = 0.0;
     T rn = 0;
     T best = (T)3e38;
     int stall = 0;
     for (int it = 0;; ++it) {
         anch = opaque(anchored);
-        small_eig_block<sizeof(T) == 8>(S, m);
+        small_eig_block<sizeof(T) == 8>(S, m, opaque(warm));
+        warm = 1;
         theta = misc[0];
         const T th = (T)theta;
         K *tdst = (m < mmax) ? V + (size_t)m * ld : tx;
@@ -956,6 +1040,7 @@ __device__ __noinline__ PhaseOut davidson_block(const BlockProblem &B, T *Vp, T 
                 ys[b + 1] = 0.0;
             }
             m = b + (keep ? 2 : 1);
+            warm = 0;
         }
         // Correction: orthogonalise against V[0..m) into V[m]; a second pass when the first
         // one cancelled (less than half of |t|^2 left; with more left, one pass is orthogonal
