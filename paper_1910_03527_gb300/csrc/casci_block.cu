@@ -1517,6 +1517,7 @@ __global__ void __launch_bounds__(BLOCK_THREADS, 1) k_casci_block(BatchArgs a, i
             const int g = sector == 0 ? bi : bj;
             if (sector == 1 && a.rdm)
                 for (int d = tid; d < pb.N; d += nt) x2[d] = x64[d];
+            __syncthreads();  // (the float32 padding zeroed below lies inside x64)
             pb.sector = sector == 0 ? 1 : -1;
             if (mixed) zero_padding(true);
             __syncthreads();
