@@ -164,24 +164,35 @@ __global__ void k_large_hs_fill(LargeCas L, const int64_t *off)
     }
 }
 
-__global__ void k_large_diag(LargeCas L)
+// Diagonal of H, a row per block: V's part of a string is the sum of two table entries, one for
+// its lower and one for its upper 8 orbitals (the double loop over both strings' orbitals took
+// 1.1 ms at 14 orbitals).
+__global__ void __launch_bounds__(256) k_large_diag(LargeCas L)
 {
-    const int Ns = L.Ns, P = L.P;
-    for (int64_t d = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; d < L.N; d += (int64_t)gridDim.x * blockDim.x) {
-        int ia = (int)(d / Ns), ib = (int)(d - (int64_t)ia * Ns);
-        double v = L.Hd[(size_t)ia * Ns + ia] + L.Hd[(size_t)ib * Ns + ib];
-        uint32_t sa = L.str[ia];
-        while (sa) {
-            int p = __ffs((int)sa) - 1;
-            sa &= sa - 1;
-            uint32_t sb = L.str[ib];
-            while (sb) {
-                int q = __ffs((int)sb) - 1;
-                sb &= sb - 1;
-                v += L.V[pair_index(p, p) * P + pair_index(q, q)];
-            }
+    __shared__ double u[16], part[2][256];
+    const int Ns = L.Ns, P = L.P, tid = threadIdx.x;
+    for (int ia = blockIdx.x; ia < Ns; ia += gridDim.x) {
+        __syncthreads();
+        if (tid < 16) {
+            double v = 0.0;
+            if (tid < L.n)
+                for (uint32_t s = L.str[ia]; s; s &= s - 1)
+                    v += L.V[pair_index(__ffs((int)s) - 1, __ffs((int)s) - 1) * P + pair_index(tid, tid)];
+            u[tid] = v;
         }
-        L.diag[d] = v;
+        __syncthreads();
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            double v = 0.0;
+            for (uint32_t s = tid; s; s &= s - 1) v += u[8 * h + __ffs((int)s) - 1];
+            part[h][tid] = v;
+        }
+        __syncthreads();
+        const double ha = L.Hd[(size_t)ia * Ns + ia];
+        for (int ib = tid; ib < Ns; ib += blockDim.x) {
+            const uint32_t s = L.str[ib];
+            L.diag[(size_t)ia * Ns + ib] = ha + L.Hd[(size_t)ib * Ns + ib] + (part[0][s & 255] + part[1][s >> 8]);
+        }
     }
 }
 
@@ -305,6 +316,96 @@ __global__ void __launch_bounds__(SS_THREADS) k_large_ss(LargeCas L, const T *__
         }
         __syncthreads();
     }
+}
+
+// The same in float32 while a slab of TK columns of X fits in shared memory (up to 14 orbitals):
+// there the rows of X are gathered from shared memory instead of L2, whose rate bounded
+// k_large_ss (11.5 of ~12 TB/s).  A row of Hs per TK / 4 lanes, four columns a lane, the entries
+// loaded one per lane and handed round; the padding of the last ones reads a row of zeros.  Work
+// items are slabs x blocks of rows.
+constexpr int SLAB_THREADS = 1024;
+
+template <int TK, bool TRANS, bool STORE>
+__global__ void __launch_bounds__(SLAB_THREADS) k_large_ss_slab(LargeCas L, const float *__restrict__ X,
+                                                                double *__restrict__ sigma, int blocks)
+{
+    extern __shared__ __align__(16) char smem[];
+    constexpr int LPR = TK / 4, RPW = 32 / LPR;
+    float *slab = (float *)smem;  // [Ns + 1][TK]
+    const int Ns = L.Ns, lane = threadIdx.x & 31, warp = threadIdx.x >> 5, l = lane % LPR;
+    const int nslab = (Ns + TK - 1) / TK, per = ((Ns + blocks - 1) / blocks + RPW - 1) / RPW * RPW;
+    for (int item = blockIdx.x; item < nslab * blocks; item += gridDim.x) {
+        const int K0 = item / blocks * TK, b = item % blocks;
+        __syncthreads();  // the last slab is done with
+#pragma unroll 8
+        for (int q = threadIdx.x; q < (Ns + 1) * TK; q += SLAB_THREADS) {
+            const int J = q / TK, K = K0 + q % TK;
+            slab[q] = J < Ns && K < Ns ? X[(size_t)J * Ns + K] : 0.f;
+        }
+        __syncthreads();
+        const int I1 = min((b + 1) * per, Ns);
+        for (int r = b * per + warp * RPW; r < I1; r += SLAB_THREADS / 32 * RPW) {
+            const int I = r + lane / LPR;
+            const int64_t e0 = I < I1 ? L.roff[I] : 0;
+            const int n = I < I1 ? (int)(L.roff[I + 1] - e0) : 0;
+            const int most = __reduce_max_sync(FULL, n);
+            float a0 = 0.f, a1 = 0.f, a2 = 0.f, a3 = 0.f;
+            int col = l < n ? L.col[e0 + l] : Ns;
+            float val = l < n ? L.val32[e0 + l] : 0.f;
+            for (int e = 0; e < most; e += LPR) {
+                const int cc = col;
+                const float cv = val;
+                const int next = e + LPR + l;
+                col = next < n ? L.col[e0 + next] : Ns;
+                val = next < n ? L.val32[e0 + next] : 0.f;
+#pragma unroll
+                for (int i = 0; i < LPR; ++i) {
+                    const int J = __shfl_sync(FULL, cc, i, LPR);
+                    const float v = __shfl_sync(FULL, cv, i, LPR);
+                    const float4 x = *(const float4 *)(slab + J * TK + 4 * l);
+                    a0 = fmaf(v, x.x, a0);
+                    a1 = fmaf(v, x.y, a1);
+                    a2 = fmaf(v, x.z, a2);
+                    a3 = fmaf(v, x.w, a3);
+                }
+            }
+            const float out[4] = {a0, a1, a2, a3};
+            if (I < I1)
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    const int K = K0 + 4 * l + j;
+                    if (K >= Ns) continue;
+                    double *o = sigma + (TRANS ? (size_t)K * Ns + I : (size_t)I * Ns + K);
+                    if (STORE)
+                        *o = (double)out[j];
+                    else
+                        *o += (double)out[j];
+                }
+        }
+    }
+}
+
+// Launch shape of k_large_ss_slab: columns per slab (0: none fits), row blocks that fill the last
+// wave best (a slab's load counted as 2% of a whole product with it).
+static int slab_columns(size_t smem_optin, int Ns)
+{
+    for (int tk = 32; tk >= 16; tk /= 2)
+        if ((size_t)(Ns + 1) * tk * 4 + 1024 <= smem_optin) return tk;
+    return 0;
+}
+static int slab_blocks(int sm_count, int Ns, int tk)
+{
+    const int nslab = (Ns + tk - 1) / tk;
+    int best = 1;
+    double cost = 1e300;
+    for (int b = 1; b <= 16 && b * 32 <= Ns + 31; ++b) {
+        const double c = (double)((nslab * b + sm_count - 1) / sm_count) * (1.0 / b + 0.02);
+        if (c < cost) {
+            cost = c;
+            best = b;
+        }
+    }
+    return best;
 }
 
 // sigma += A + sgn A^T for an Ns x Ns matrix A (32 x 32 tiles through shared
@@ -593,6 +694,7 @@ struct LargePlan {
     void *cT;      // transposed coefficients (room for N float64)
     DigitsArgs dg;  // float64 sigma on the tensor cores
     int dg_chunk;   // 0: not used
+    int slab_tk, slab_blocks;  // k_large_ss_slab (0: k_large_ss)
 };
 
 
@@ -712,6 +814,8 @@ static int large_setup(mbe_ctx *ctx, int norb, const double *h1, const double *e
     plan->grid_ss64 = ctx->sm_count * (b > 0 ? b : 1);
     MBE_CU(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_large_ss<float, false>, SS_THREADS, plan->smem_ss32));
     plan->grid_ss32 = ctx->sm_count * (b > 0 ? b : 1);
+    plan->slab_tk = slab_columns(ctx->smem_optin, L.Ns);
+    plan->slab_blocks = plan->slab_tk ? slab_blocks(ctx->sm_count, L.Ns, plan->slab_tk) : 0;
     plan->grid_tr = ctx->sm_count * 8;
     plan->grid_vec = ctx->sm_count * 4;
     return MBE_OK;
@@ -734,6 +838,19 @@ static size_t large_bytes(const mbe_ctx *ctx, int norb, int n, int k, bool dense
         b += align256(ns * 8) + align256(P * nsp * 4) + 256 + 2 * align256((size_t)DIGITS * ns * nsp * 2);
     }
     return b;
+}
+
+template <bool TRANS, bool STORE>
+static int large_ss_slab(mbe_ctx *ctx, const LargePlan &pl, const float *X, double *out)
+{
+    const int Ns = pl.L.Ns, items = (Ns + pl.slab_tk - 1) / pl.slab_tk * pl.slab_blocks;
+    const int grid = std::min(items, ctx->sm_count), smem = (Ns + 1) * pl.slab_tk * 4;
+    auto launch = [&](auto *kernel) -> int {
+        MBE_CU(allow_smem(kernel, ctx->smem_optin));
+        kernel<<<grid, SLAB_THREADS, smem, ctx->stream>>>(pl.L, X, out, pl.slab_blocks);
+        return MBE_OK;
+    };
+    return pl.slab_tk == 32 ? launch(k_large_ss_slab<32, TRANS, STORE>) : launch(k_large_ss_slab<16, TRANS, STORE>);
 }
 
 // sigma = H c: the opposite-spin term written first, then Hs C added, then C Hs^T
@@ -766,6 +883,23 @@ static int large_sigma_launch(mbe_ctx *ctx, const LargePlan &pl, const T *c, dou
         const int rc = large_ab_tc(ctx->stream, ctx->sm_count, ctx->smem_optin, pl.L.P, pl.L.Ns, pl.L.R, pl.L.tab,
                                    pl.L.V32, (const float *)c, sigma, ctx->dev_err);
         if (rc) return rc;
+    }
+    if (sizeof(T) == 4 && pl.slab_tk) {
+        if (sgn == 0) {
+            float *cT = (float *)pl.cT;
+            int rc = large_ss_slab<false, false>(ctx, pl, (const float *)c, sigma);
+            k_large_transpose<float><<<pl.grid_tr, dim3(32, 8), 0, ctx->stream>>>((const float *)c, Ns, cT);
+            if (!rc) rc = large_ss_slab<true, false>(ctx, pl, cT, sigma);
+            if (rc) return rc;
+        } else {
+            double *A = (double *)pl.cT;
+            const int rc = large_ss_slab<false, true>(ctx, pl, (const float *)c, A);
+            if (rc) return rc;
+            k_sym_add<<<pl.grid_tr, dim3(32, 8), 0, ctx->stream>>>(A, Ns, sgn, sigma, nullptr);
+        }
+        MBE_CU(cudaGetLastError());
+        ctx->launches += sgn == 0 ? 4 : 3;
+        return tl.done();
     }
     const int grid_ss = sizeof(T) == 8 ? pl.grid_ss64 : pl.grid_ss32;
     const size_t smem_ss = sizeof(T) == 8 ? pl.smem_ss64 : pl.smem_ss32;
