@@ -17,6 +17,7 @@
 // see casci_sector64.cuh), because a float64 multiply-add costs 36 integer ones here.
 // Beyond 9 orbitals c does not fit, and sigma walks both lists per element.
 #include "casci_sector.cuh"
+#include "digits.cuh"
 
 namespace mbe {
 
@@ -108,6 +109,32 @@ __host__ __device__ inline GemmShape gemm_shape(int n, int ns, int r)
     return s;
 }
 
+// Float64 operands of the tiled sigma as digits (sigma_digits), from off_c on.
+constexpr int DIGITS_SMEM = 226 * 1024;  // used where all of the block's shared memory fits in this
+struct DigitShape {
+    int c8, cs, vs, mt;  // tiles of 8 strings; row strides (16-bit words) of c and V; tiles of 16 pairs
+    int g;               // strings per round: as many as the float32 T has room for
+    int off_v, off_l, off_rows, bytes;
+};
+
+__host__ __device__ inline DigitShape digit_shape(int n, int ns, int r)
+{
+    DigitShape d;
+    const int P = n * (n + 1) / 2;
+    const GemmShape a = gemm_shape<float>(n, ns, r), b = gemm_shape<double>(n, ns, r);
+    d.g = a.g / 2 > b.g ? a.g / 2 : b.g;
+    if (d.g > 1) d.g &= ~1;
+    d.c8 = (ns + 7) / 8;
+    d.cs = 8 * (d.c8 | 1);  // (odd multiples of 16 bytes: the 8 rows of a matrix in different banks)
+    d.mt = (P + 15) / 16;
+    d.vs = d.mt * 16 + 8;
+    d.off_v = 2 * DIGITS * (ns + 1) * d.cs;  // (row ns of c is zero)
+    d.off_l = d.off_v + 2 * DIGITS * P * d.vs;
+    d.off_rows = al16(d.off_l + 2 * ns * ((r + 15) / 16 * 16));
+    d.bytes = d.off_rows + 8 * d.g * (d.cs + d.mt * 16);
+    return d;
+}
+
 // Row stride of the float32 c of SIGMA_LIST
 __host__ __device__ inline int list_stride(int ns)
 {
@@ -117,14 +144,15 @@ __host__ __device__ inline int list_stride(int ns)
 
 struct BlockMem {  // dynamic shared memory
     int off_A, off_pp, off_h, off_V64, off_V32, off_red, off_G, off_J, off_ev, off_y, off_yp, off_r, off_misc,
-        off_hd, off_list, off_c, off_T, off_g1, bytes;
+        off_hd, off_list, off_c, off_T, off_g1, bytes, digits;
 };
 
 // The tiled sigma's lists, c and T; the lists and c of SIGMA_LIST; else those are absent.
 // rdm: density matrices follow the solve.
-__host__ __device__ inline BlockMem block_mem(int n, int form, int ns, int r, int rdm)
+__host__ __device__ inline BlockMem block_mem(int n, int form, int ns, int r, int rdm, int digits = 1)
 {
     BlockMem S;
+    S.digits = form == SIGMA_TILED ? digits : 0;
     const int P = n * (n + 1) / 2;
     const bool gemm = form == SIGMA_TILED;
     int o = 0;
@@ -151,19 +179,21 @@ __host__ __device__ inline BlockMem block_mem(int n, int form, int ns, int r, in
         // fixed point: c; float32: c, V twice over with both signs, list offsets (see sigma_gemm)
         const GemmShape a = gemm_shape<float>(n, ns, r);
         const int f = al16(4 * ns * a.fst) + 8 * P * a.pst + 4 * ns * r;
-        o = al16(o + (f > 8 * ns * a.cst ? f : 8 * ns * a.cst));
+        const int c = S.digits ? digit_shape(n, ns, r).bytes : 8 * ns * a.cst;
+        o = al16(o + (f > c ? f : c));
     }
     S.off_T = o;
     if (gemm) {
         const GemmShape a = gemm_shape<float>(n, ns, r), b = gemm_shape<double>(n, ns, r);
         const int ta = a.g * P * a.cst * 4, tb = b.g * P * b.cst * 8;
-        o = al16(o + (ta > tb ? ta : tb));
+        const int th = S.digits ? 2 * DIGITS * 16 * digit_shape(n, ns, r).cs : 0;  // (16 rows of Hs)
+        o = al16(o + (ta > tb ? ta > th ? ta : th : tb > th ? tb : th));
     }
     o = al16(o + stage);
     // the density matrices' vectors lie over c and T
     const int d = rdm ? S.off_c + 8 * 33 * (n * n + 1) : 0;
     S.bytes = al16(o > d ? o : d);
-    return S;
+    return S.digits && S.bytes > DIGITS_SMEM ? block_mem(n, form, ns, r, rdm, 0) : S;
 }
 
 struct BlockProblem {
@@ -355,6 +385,264 @@ __device__ __forceinline__ void gemm_tile(const Problem &pb, const GemmShape &s,
             for (int i = 0; i < 4; ++i) T[(p0 + k) * s.cst + j0 + i] = hi[i][k] + ((lo[i][k] + (1LL << 27)) >> 28);
 }
 
+// The strings are taken from both ends of the list, so that each pair of them has Ns + 1 elements
+// with Ia <= Ib.
+__device__ __forceinline__ int tail_string(int Ns, int i) { return i & 1 ? Ns - 1 - (i >> 1) : i >> 1; }
+
+// sigma of the elements of gc strings from their T and the same-spin terms M.
+template <typename T, typename A>
+__device__ __forceinline__ void gather_strings(const BlockProblem &B, const GemmShape &s, const A *Tm, const A *M, int I0, int gc,
+                                               const T *src, T *dst)
+{
+    constexpr bool F64 = sizeof(T) == 8;
+    const Problem &pb = B.pb;
+    const int Ns = pb.Ns, tid = threadIdx.x, nt = blockDim.x, R = pb.R, sgn = pb.sector;
+    const uint16_t *list = (const uint16_t *)(block_shared() + B.S.off_list);
+    const double *hd = (const double *)(block_shared() + B.S.off_hd);
+            const int n1 = Ns + 1, ne = (gc + 1) / 2 * n1;
+            int split = 0;  // 2^split threads per element, where they fit
+            while (split < 3 && (ne << (split + 1)) <= nt) ++split;
+            for (int q0 = 0; q0 < ne << split; q0 += nt) {
+                const int q = q0 + tid, el = q >> split, pr = el / n1, r = el - pr * n1;
+                const int first = tail_string(Ns, I0 + 2 * pr), len = Ns - first;  // elements of the pair's first string
+                const int g = 2 * pr + (r < len ? 0 : 1), Ia = r < len ? first : tail_string(Ns, I0 + g), Ib = Ia + r - (r < len ? 0 : len);
+                const bool on = g < gc && Ib < Ns, last = on && (q & ((1 << split) - 1)) == 0;
+                // (the same-spin terms come from L2: asked for before the walk over the list)
+                const A m0 = last ? M[Ia * s.cst + Ib] : (A)0, m1 = last ? M[Ib * s.cst + Ia] : (A)0;
+                A acc = 0;
+                if (on) {
+                    const A *t = Tm + g * pb.P * s.cst;
+                    const uint16_t *lb = list + Ib * s.rs;
+    #pragma unroll 4
+                    for (int y = q & ((1 << split) - 1); y < R; y += 1 << split) {
+                        const int e = lb[y];
+                        const A v = t[((e >> 1) & 63) * s.cst + (e >> 7)];
+                        acc += e & 1 ? -v : v;
+                    }
+                }
+                for (int o = 1; o < 1 << split; o <<= 1) acc += __shfl_xor_sync(FULL, acc, o);
+                if (last) {
+                    const int h = Ia * Ns - Ia * (Ia - 1) / 2 + Ib - Ia;
+                    acc += m0 + (sgn > 0 ? m1 : -m1);
+                    T v;
+                    if constexpr (F64) {
+                        v = fma(hd[Ia] + hd[Ib], src[h], (double)acc * (pow2(B.E - 54) * (Ia == Ib ? 1.0 : 1.4142135623730951)));
+                        if (B.bad) v = __longlong_as_double(0x7ff8000000000000LL);
+                    } else {
+                        v = Ia == Ib ? acc : 1.41421356f * acc;
+                    }
+                    dst[h] = sgn < 0 && Ia == Ib ? (T)0 : v;
+                }
+            }
+}
+
+// float64 sigma of a packed sector vector with the products on the tensor cores, in exact digits
+// (digits.cuh: 32 multiply-adds per clock and SM, where three wide integer ones per product reach
+// 7).  T per alpha string Ia as mma.sync tiles of 16 pairs x 8 strings: the rows of V and c that
+// the off-diagonal replacements name are gathered by ldmatrix, the signs are flipped in c's
+// fragments, and the k diagonal replacements, all of which keep J = Ia, enter as one row, their
+// sum U of V, in integers: k (n - k) <= 16 list entries up to 8 orbitals, one mma step.  The sums
+// of up to 32 products stay within 2^22, so the accumulators start at 1.5 * 2^23 and hold
+// their integers in the low bits.  A warp takes a run of consecutive tiles.  Tm: [P][cst]
+// per string as in sigma_gemm, the same units; the rest of sigma is that of sigma_gemm.
+__device__ __noinline__ void sigma_digits(const BlockProblem &B, const double *src, double *dst)
+{
+    const Problem &pb = B.pb;
+    const int n = pb.n, P = pb.P, Ns = pb.Ns, R = pb.R, sgn = pb.sector, tid = threadIdx.x, nt = blockDim.x;
+    const int lane = tid & 31, warp = tid >> 5, nw = nt >> 5;
+    const DigitShape d = digit_shape(n, Ns, R);
+    GemmShape s = gemm_shape<double>(n, Ns, R);
+    s.g = d.g;
+    char *at = block_shared() + B.S.off_c;
+    uint16_t *cd = (uint16_t *)at, *vd = (uint16_t *)(at + d.off_v), *off = (uint16_t *)(at + d.off_l);
+    int2 *rows = (int2 *)(at + d.off_rows);  // per string of a round: its row of c, and U
+    const int rst = d.cs + d.mt * 16;
+    long long *Tm = (long long *)(block_shared() + B.S.off_T), *M = (long long *)B.full;
+    const uint16_t *list = (const uint16_t *)(block_shared() + B.S.off_list);
+    const int2 *Vf = (const int2 *)(block_shared() + B.S.off_V64), *Hf = (const int2 *)pb.Hs64;
+    const int cplane = (Ns + 1) * d.cs, vplane = P * d.vs, ro = pb.k * (n - pb.k), nks = (ro + 15) / 16, kx = 16 * nks;
+    const double one = 36028797018963968.0, root = 0.70710678118654752 * 36028797018963968.0;  // 2^55
+    auto joined = [](int2 f) { return ((long long)f.x << 28) + f.y; };
+    {
+        int ia = 0, ib = 0;
+        tri_advance(ia, ib, tid, Ns);
+        for (int h = tid; h < pb.N; h += nt) {
+            uint16_t f[DIGITS];
+            to_digits(__double2ll_rn(src[h] * (ia == ib ? one : root)), f);
+#pragma unroll
+            for (int i = 0; i < DIGITS; ++i) {
+                cd[i * cplane + ia * d.cs + ib] = f[i];
+                cd[i * cplane + ib * d.cs + ia] = sgn > 0 ? f[i] : f[i] ^ 0x8000;
+            }
+            tri_advance(ia, ib, nt, Ns);
+        }
+        const int pad = d.cs - Ns;
+        for (int q = tid; q < Ns * pad + d.cs; q += nt) {
+            const int to = q < Ns * pad ? q / pad * d.cs + Ns + q % pad : Ns * d.cs + q - Ns * pad;
+#pragma unroll
+            for (int i = 0; i < DIGITS; ++i) cd[i * cplane + to] = 0;
+        }
+        for (int q = tid; q < vplane; q += nt) {
+            const int x = q / d.vs, y = q - x * d.vs;
+            uint16_t f[DIGITS];
+            to_digits(y < P ? joined(Vf[x * P + y]) : 0, f);
+#pragma unroll
+            for (int i = 0; i < DIGITS; ++i) vd[i * vplane + q] = f[i];
+        }
+        for (int I = tid; I < Ns; I += nt) {
+            int to = 0;
+            for (int x = 0; x < R; ++x) {
+                const int e = list[I * s.rs + x];
+                if (e >> 7 != I) off[I * kx + to++] = (uint16_t)e;
+            }
+            for (; to < kx; ++to) off[I * kx + to] = (uint16_t)(Ns << 7);
+        }
+    }
+    auto stage_rows = [&](int I0) {
+        for (int q = tid; q < min(s.g, Ns - I0) * rst; q += nt) {
+            const int g = q / rst, x = q - g * rst, Ia = tail_string(Ns, I0 + g);
+            int2 f = make_int2(0, 0);
+            if (x < Ns) {
+                const int lo = min(Ia, x), hi = max(Ia, x);
+                f = to_fixed(src[lo * Ns - lo * (lo - 1) / 2 + hi - lo], Ia == x ? one : root);
+                if (sgn < 0 && x < Ia) f = make_int2(-f.x, -f.y);
+            } else if (x >= d.cs && x - d.cs < P) {
+                for (uint32_t m = pb.str[Ia]; m; m &= m - 1u) {
+                    const int2 v = Vf[pair_index(__ffs((int)m) - 1, __ffs((int)m) - 1) * P + x - d.cs];
+                    f.x += v.x;
+                    f.y += v.y;
+                }
+            }
+            rows[q] = f;
+        }
+    };
+    stage_rows(0);
+    // same-spin terms: M = c Hs, the digits of Hs made in chunks of rows where T will be
+    const int hr = min(min((Ns + 15) / 16 * 16, 128), (B.S.bytes - B.S.off_T) / (2 * DIGITS * d.cs) / 16 * 16);
+    uint16_t *hs = (uint16_t *)Tm;
+    for (int J0 = 0; J0 < Ns; J0 += hr) {
+        const int jn = min(hr, (Ns - J0 + 15) / 16 * 16), hplane = jn * d.cs;
+        __syncthreads();
+        for (int q = tid; q < hplane; q += nt) {
+            const int J = J0 + q / d.cs, j = q % d.cs;
+            uint16_t f[DIGITS];
+            to_digits(J < Ns && j < s.cst ? joined(Hf[J * s.cst + j]) : 0, f);
+#pragma unroll
+            for (int i = 0; i < DIGITS; ++i) hs[i * hplane + q] = f[i];
+        }
+        __syncthreads();
+        for (int t = warp; t < (Ns + 15) / 16 * d.c8; t += nw) {
+            const int m = t / d.c8, jt = t - m * d.c8;
+            // (rows and columns of c beyond Ns are whatever digits follow: such rows are not
+            // stored, such columns meet zeros of Hs)
+            const uint32_t aa = shared_u32(cd + (m * 16 + (lane & 15)) * d.cs + (lane >> 4) * 8 + J0);
+            const uint32_t ba = shared_u32(hs + (lane & 15) * d.cs + jt * 8);
+            float acc[DIGITS][4];
+#pragma unroll
+            for (int i = 0; i < DIGITS; ++i) acc[i][0] = acc[i][1] = acc[i][2] = acc[i][3] = 0.f;
+#pragma unroll 1
+            for (int k = 0; k < jn; k += 16) {
+                uint32_t bf[DIGITS][2];
+#pragma unroll
+                for (int j = 0; j < DIGITS; ++j) ldsm_x2_trans(bf[j], ba + 2 * (j * hplane + k * d.cs));
+#pragma unroll
+                for (int i = 0; i < DIGITS; ++i) {
+                    uint32_t af[4];
+                    ldsm_x4(af, aa + 2 * (i * cplane + k));
+#pragma unroll
+                    for (int j = 0; i + j < DIGITS; ++j) mma_bf16(acc[i + j], af, bf[j][0], bf[j][1]);
+                }
+            }
+            const int i = m * 16 + (lane >> 2), j = jt * 8 + (lane & 3) * 2;
+#pragma unroll
+            for (int h = 0; h < 2; ++h)
+                if (i + 8 * h < Ns && j < s.cst) {
+                    longlong2 *o = (longlong2 *)(M + (i + 8 * h) * s.cst + j);
+                    const longlong2 old = J0 ? *o : make_longlong2(0, 0);
+                    *o = make_longlong2(old.x + join_digits(acc, 2 * h), old.y + join_digits(acc, 2 * h + 1));
+                }
+        }
+    }
+    __syncthreads();  // (Hs was staged over T)
+    for (int I0 = 0; I0 < Ns; I0 += s.g) {
+        const int gc = min(s.g, Ns - I0), tiles = gc * d.mt * d.c8, last = (warp + 1) * tiles / nw;
+        int now = -1, g = 0, m = 0;
+        uint32_t aa[2] = {0, 0}, ba[2] = {0, 0}, flip[2][2] = {{0, 0}, {0, 0}};
+        for (int t = warp * tiles / nw; t < last; ++t) {
+            const int gm = t / d.c8, jt = t - gm * d.c8;
+            if (gm != now) {
+                now = gm;
+                g = gm / d.mt;
+                m = gm - g * d.mt;
+                const uint16_t *l = off + tail_string(Ns, I0 + g) * kx;
+#pragma unroll
+                for (int k = 0; k < 2; ++k)
+                    if (k < nks) {
+                        ba[k] = shared_u32(cd + (l[16 * k + (lane & 15)] >> 7) * d.cs);
+                        aa[k] = shared_u32(vd + (l[16 * k + (lane & 7) + (lane >> 4) * 8] >> 1 & 63) * d.vs + m * 16 + (lane >> 3 & 1) * 8);
+                        const uint16_t *x = l + 16 * k + (lane & 3) * 2;
+                        flip[k][0] = (x[0] & 1u) << 15 | (x[1] & 1u) << 31;
+                        flip[k][1] = (x[8] & 1u) << 15 | (x[9] & 1u) << 31;
+                    }
+            }
+            float acc[DIGITS][4];
+#pragma unroll
+            for (int i = 0; i < DIGITS; ++i) acc[i][0] = acc[i][1] = acc[i][2] = acc[i][3] = 12582912.f;
+            uint32_t av = aa[0], bv = ba[0] + 16 * jt, f0 = flip[0][0], f1 = flip[0][1];
+#pragma unroll 1
+            for (int k = 0; k < nks; ++k) {
+                uint32_t bf[DIGITS][2];
+#pragma unroll
+                for (int j = 0; j < DIGITS; ++j) {
+                    ldsm_x2_trans(bf[j], bv + 2 * j * cplane);
+                    bf[j][0] ^= f0;
+                    bf[j][1] ^= f1;
+                }
+#pragma unroll
+                for (int i = 0; i < DIGITS; ++i) {
+                    uint32_t af[4];
+                    ldsm_x4_trans(af, av + 2 * i * vplane);
+#pragma unroll
+                    for (int j = 0; i + j < DIGITS; ++j) mma_bf16(acc[i + j], af, bf[j][0], bf[j][1]);
+                }
+                av = aa[1];
+                bv = ba[1] + 16 * jt;
+                f0 = flip[1][0];
+                f1 = flip[1][1];
+            }
+            const int p0 = m * 16 + (lane >> 2), J = jt * 8 + (lane & 3) * 2;
+            const int4 cr = *(const int4 *)(rows + g * rst + J);
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const int p = p0 + 8 * h;
+                if (p >= P || J >= s.cst) continue;
+                const int2 u = rows[g * rst + d.cs + p];
+                long long v[2];
+#pragma unroll
+                for (int e = 0; e < 2; ++e) {
+                    // (the joins of two sums fit in 32 bits, and the offsets cancel modulo 2^32)
+                    auto pair = [&](int i) {
+                        return (int)((__float_as_uint(acc[i][2 * h + e]) << 8) + __float_as_uint(acc[i + 1][2 * h + e]) -
+                                     0x4b400000u * 257u);
+                    };
+                    const int rest = ((int)(__float_as_uint(acc[6][2 * h + e]) - 0x4b400000u) + 128) >> 8;
+                    const int cx = e ? cr.z : cr.x, cy = e ? cr.w : cr.y;
+                    long long lo = 1LL << 27;
+                    lo += (long long)u.x * cy;
+                    lo += (long long)u.y * cx;
+                    v[e] = ((long long)pair(0) << 32) + (long long)pair(2) * 65536 + pair(4) + rest;
+                    v[e] += (long long)u.x * cx + (lo >> 28);
+                }
+                *(longlong2 *)(Tm + (g * P + p) * s.cst + J) = make_longlong2(v[0], v[1]);
+            }
+        }
+        __syncthreads();  // (also orders M, written above, before its first use)
+        gather_strings<double>(B, s, Tm, M, I0, gc, src, dst);
+        if (I0 + s.g < Ns) stage_rows(I0 + s.g);
+        __syncthreads();
+    }
+}
+
 // sigma of a packed sector vector, tiled product.
 template <typename T>
 __device__ __noinline__ void sigma_gemm(const BlockProblem &B, const T *src, T *dst)
@@ -408,13 +696,10 @@ __device__ __noinline__ void sigma_gemm(const BlockProblem &B, const T *src, T *
     same_spin(pb, s.cst, cld, c, F64 ? (const E *)pb.Hs64 : (const E *)pb.Hs32, M, (char *)Tm,
               s.g * pb.P * s.cst * (int)sizeof(A));
     if constexpr (!F64) __syncthreads();  // (Hs was staged over T)
-    // Strings are taken from both ends of the list, so that each pair of them has Ns + 1 elements
-    // with Ia <= Ib.
     for (int I0 = 0; I0 < Ns; I0 += s.g) {
         const int gc = min(s.g, Ns - I0);
-        auto string = [&](int i) { return i & 1 ? Ns - 1 - (i >> 1) : i >> 1; };
         for (int q = tid; q < gc * s.tiles; q += nt) {
-            const int g = q / s.tiles, r = q - g * s.tiles, pg = r / s.nj, jj = r - pg * s.nj, Ia = string(I0 + g);
+            const int g = q / s.tiles, r = q - g * s.tiles, pg = r / s.nj, jj = r - pg * s.nj, Ia = tail_string(Ns, I0 + g);
             if constexpr (F64)
                 gemm_tile(pb, s, list + Ia * s.rs, c, (const int2 *)(block_shared() + B.S.off_V64), 4 * jj, pg,
                           Tm + g * pb.P * s.cst);
@@ -422,41 +707,7 @@ __device__ __noinline__ void sigma_gemm(const BlockProblem &B, const T *src, T *
                 gemm_tile(pb, s, list32 + Ia * R, (const char *)c, Vd, 8 * jj, pg, Tm + g * pb.P * s.cst);
         }
         __syncthreads();  // (also orders M, written above, before its first use)
-        const int n1 = Ns + 1, ne = (gc + 1) / 2 * n1;
-        int split = 0;  // 2^split threads per element, where they fit
-        while (split < 3 && (ne << (split + 1)) <= nt) ++split;
-        for (int q0 = 0; q0 < ne << split; q0 += nt) {
-            const int q = q0 + tid, el = q >> split, pr = el / n1, r = el - pr * n1;
-            const int first = string(I0 + 2 * pr), len = Ns - first;  // elements of the pair's first string
-            const int g = 2 * pr + (r < len ? 0 : 1), Ia = r < len ? first : string(I0 + g), Ib = Ia + r - (r < len ? 0 : len);
-            const bool on = g < gc && Ib < Ns, last = on && (q & ((1 << split) - 1)) == 0;
-            // (the same-spin terms come from L2: asked for before the walk over the list)
-            const A m0 = last ? M[Ia * s.cst + Ib] : (A)0, m1 = last ? M[Ib * s.cst + Ia] : (A)0;
-            A acc = 0;
-            if (on) {
-                const A *t = Tm + g * pb.P * s.cst;
-                const uint16_t *lb = list + Ib * s.rs;
-#pragma unroll 4
-                for (int y = q & ((1 << split) - 1); y < R; y += 1 << split) {
-                    const int e = lb[y];
-                    const A v = t[((e >> 1) & 63) * s.cst + (e >> 7)];
-                    acc += e & 1 ? -v : v;
-                }
-            }
-            for (int o = 1; o < 1 << split; o <<= 1) acc += __shfl_xor_sync(FULL, acc, o);
-            if (last) {
-                const int h = Ia * Ns - Ia * (Ia - 1) / 2 + Ib - Ia;
-                acc += m0 + (sgn > 0 ? m1 : -m1);
-                T v;
-                if constexpr (F64) {
-                    v = fma(hd[Ia] + hd[Ib], src[h], (double)acc * (pow2(B.E - 54) * (Ia == Ib ? 1.0 : 1.4142135623730951)));
-                    if (B.bad) v = __longlong_as_double(0x7ff8000000000000LL);
-                } else {
-                    v = Ia == Ib ? acc : 1.41421356f * acc;
-                }
-                dst[h] = sgn < 0 && Ia == Ib ? (T)0 : v;
-            }
-        }
+        gather_strings<T>(B, s, Tm, M, I0, gc, src, dst);
         __syncthreads();
     }
 }
@@ -554,7 +805,14 @@ __device__ __noinline__ void sigma_block(const BlockProblem &B, const T *src, T 
 {
     const Problem &pb = B.pb;
     const bool done = B.form == SIGMA_TILED || (B.form == SIGMA_LIST && sizeof(T) == 4);  // but for the penalty
-    if (B.form == SIGMA_TILED) sigma_gemm<T>(B, src, dst);
+    if (B.form == SIGMA_TILED) {
+        bool digits = false;
+        if constexpr (sizeof(T) == 8) {
+            digits = B.S.digits;
+            if (digits) sigma_digits(B, src, dst);
+        }
+        if (!digits) sigma_gemm<T>(B, src, dst);
+    }
     if constexpr (sizeof(T) == 4)
         if (B.form == SIGMA_LIST) sigma_list(B, src, dst);
     if (done && pb.s2mu == 0.0) return;

@@ -1,10 +1,10 @@
 #pragma once
 // The float64 sigma of one large space on the tensor cores (large_digits.cu).
 #include "common.cuh"
+#include "digits.cuh"
 
 namespace mbe {
 
-constexpr int DIGITS = 7;  // of base 256
 constexpr int DIGITS_EXP = 450;  // largest |exponent| of an operand's scale
 
 struct DigitsArgs {
