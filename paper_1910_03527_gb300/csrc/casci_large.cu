@@ -320,7 +320,8 @@ __global__ void __launch_bounds__(SS_THREADS) k_large_ss(LargeCas L, const T *__
 
 // The same in float32 while a slab of TK columns of X fits in shared memory (up to 14 orbitals):
 // there the rows of X are gathered from shared memory instead of L2, whose rate bounded
-// k_large_ss (11.5 of ~12 TB/s).  A row of Hs per TK / 4 lanes, four columns a lane, the entries
+// k_large_ss (11.5 of ~12 TB/s): 334 -> 57 us at 12 orbitals; at 14, where only 16 columns fit
+// and half of the paired rows share banks, 2.0 -> 1.65 ms (the shared-memory pipe).  A row of Hs per TK / 4 lanes, four columns a lane, the entries
 // loaded one per lane and handed round; the padding of the last ones reads a row of zeros.  Work
 // items are slabs x blocks of rows.
 constexpr int SLAB_THREADS = 1024;
@@ -695,6 +696,7 @@ struct LargePlan {
     DigitsArgs dg;  // float64 sigma on the tensor cores
     int dg_chunk;   // 0: not used
     int slab_tk, slab_blocks;  // k_large_ss_slab (0: k_large_ss)
+    uint32_t *tc_lists;        // of large_ab_tc
 };
 
 
@@ -751,6 +753,7 @@ static int large_setup(mbe_ctx *ctx, int norb, const double *h1, const double *e
     L.tabT = tabT;
     plan->cT = bump.take<double>((size_t)L.N);  // float32 or float64 use
     L.Hd = dense_at ? dense_at : bump.take<double>((size_t)L.Ns * L.Ns);
+    plan->tc_lists = fp32 ? (uint32_t *)bump.take<char>(large_tc_list_bytes(ctx->smem_optin, P, L.Ns, L.R)) : nullptr;
     plan->dg_chunk = large_digits_chunk(ctx->smem_optin, P, L.Ns, L.R);
     double *hd = nullptr;
     if (plan->dg_chunk) {
@@ -788,6 +791,10 @@ static int large_setup(mbe_ctx *ctx, int norb, const double *h1, const double *e
     k_large_tables<<<(L.Ns + 255) / 256, 256, 0, ctx->stream>>>(L, tabT);
     MBE_CU(cudaGetLastError());
     ctx->launches += 8;
+    if (fp32) {
+        if ((rc = large_tc_lists(ctx->stream, ctx->smem_optin, P, L.Ns, L.R, L.tab, plan->tc_lists))) return rc;
+        ++ctx->launches;
+    }
     if (plan->dg_chunk) {
         rc = large_digits_setup(ctx->stream, ctx->sm_count, plan->dg, L.Hd, hd);
         if (rc) return rc;
@@ -833,6 +840,7 @@ static size_t large_bytes(const mbe_ctx *ctx, int norb, int n, int k, bool dense
                align256((ns + 1) * 8) + 4096;
     b += align256((size_t)k * (n - k + 1) * ns * 4) + align256((size_t)N * 8);
     if (dense_separate) b += align256((size_t)ns * ns * 8);
+    if (fp32) b += align256(large_tc_list_bytes(ctx->smem_optin, P, (int)ns, k * (n - k + 1)));
     if (large_digits_chunk(ctx->smem_optin, P, (int)ns, k * (n - k + 1))) {
         const size_t nsp = (size_t)(ns + 63) / 64 * 64;
         b += align256(ns * 8) + align256(P * nsp * 4) + 256 + 2 * align256((size_t)DIGITS * ns * nsp * 2);
@@ -881,7 +889,7 @@ static int large_sigma_launch(mbe_ctx *ctx, const LargePlan &pl, const T *c, dou
     } else {
         // the dense product on the tensor cores (large_tc.cu)
         const int rc = large_ab_tc(ctx->stream, ctx->sm_count, ctx->smem_optin, pl.L.P, pl.L.Ns, pl.L.R, pl.L.tab,
-                                   pl.L.V32, (const float *)c, sigma, ctx->dev_err);
+                                   pl.tc_lists, pl.L.V32, (const float *)c, sigma, ctx->dev_err);
         if (rc) return rc;
     }
     if (sizeof(T) == 4 && pl.slab_tk) {

@@ -190,6 +190,9 @@ __global__ void k_scan_counts(const int32_t *counts, int64_t nblocks, int64_t *o
 // float32 packed-pair integrals V32 [P][P].  *err (device) is set to 1 if a
 // bounded wait runs out.
 int large_ab_tc(cudaStream_t st, int sm_count, size_t smem_optin, int P, int Ns, int R, const int32_t *tab,
-                const float *V32, const float *c, double *sigma, int *err);
+                const uint32_t *lists, const float *V32, const float *c, double *sigma, int *err);
+// Its scatter lists, made once per space: their bytes, and the kernel that makes them.
+size_t large_tc_list_bytes(size_t smem_optin, int P, int Ns, int R);
+int large_tc_lists(cudaStream_t st, size_t smem_optin, int P, int Ns, int R, const int32_t *tab, uint32_t *lists);
 
 }  // namespace mbe
