@@ -1907,6 +1907,34 @@ __global__ void __launch_bounds__(BLOCK_THREADS, 1) k_casci_block(BatchArgs a, i
     }
 }
 
+// small_eig_block on a Rayleigh matrix in global memory (the large-CAS solver's).  col: its new last
+// column, put in first (m values; may be NULL).
+__global__ void __launch_bounds__(416) k_small_eig(double *Gd, int m, const double *col, BlockMem S, double *ys, double *y2s,
+                                                          double *misc)
+{
+    const int tid = threadIdx.x;
+    double *G = (double *)(block_shared() + S.off_G);
+    if (col && tid < m) Gd[tid * MMAX + m - 1] = Gd[(m - 1) * MMAX + tid] = col[tid];
+    __syncthreads();
+    if (tid < MMAX * MMAX) G[tid] = Gd[tid];
+    __syncthreads();
+    small_eig_block<true>(S, m, false);
+    if (tid < m) {
+        ys[tid] = ((double *)(block_shared() + S.off_y))[tid];
+        y2s[tid] = ((double *)(block_shared() + S.off_yp))[tid];
+    }
+    if (tid == 0) misc[0] = *(double *)(block_shared() + S.off_misc);
+}
+
+int launch_small_eig(cudaStream_t st, double *Gd, int m, const double *col, double *ys, double *y2s,
+                     double *misc)
+{
+    const BlockMem S = block_mem(2, SIGMA_GLOBAL, 1, 1, 0);
+    k_small_eig<<<1, 416, S.bytes, st>>>(Gd, m, col, S, ys, y2s, misc);
+    MBE_CU(cudaGetLastError());
+    return MBE_OK;
+}
+
 // Shared memory and slot size of a bucket's block launch (the classes `in`); a.tiled is cleared
 // when the shared-memory forms of sigma do not fit.
 int block_grid(mbe_ctx *ctx, BatchArgs &a, const bool (&in)[MBE_MAX_STRING_ORB + 1], int rdm, int *grid, size_t *smem,

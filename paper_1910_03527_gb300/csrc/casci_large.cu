@@ -468,11 +468,52 @@ __global__ void k_large_tables(LargeCas L, int32_t *tabT)
 
 // ---- grid-wide vector algebra of the large Davidson (all float64)
 
-// partial[b*K + i] = block b's share of sum_d A_i[d] * u[d], i < K; A_i = A + i*ld.
-__global__ void __launch_bounds__(LARGE_THREADS) k_multidot(const double *A, size_t ld, int K, const double *u,
-                                                            int64_t N, double *partial)
+// out[i] = sum of v[i] over the grid, i < K (fixed order): each block's sums to partial, and the
+// block that finishes last (ticket, back at 0 afterwards) adds them up.
+template <int L>
+__device__ __forceinline__ void grid_sums(double (&v)[L], int K, double *partial, unsigned *ticket, double *out)
 {
-    __shared__ double red[32 * LRED];
+    __shared__ double red[32 * L];
+    __shared__ bool last;
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
+#pragma unroll
+    for (int i = 0; i < L; ++i)
+        if (i < K) v[i] = warp_sum(v[i]);
+    if (lane == 0)
+#pragma unroll
+        for (int i = 0; i < L; ++i)
+            if (i < K) red[w * L + i] = v[i];
+    __syncthreads();
+    if (threadIdx.x < K) {
+        double s = 0.0;
+        for (int j = 0; j < nw; ++j) s += red[j * L + threadIdx.x];
+        __stcg(partial + (size_t)blockIdx.x * K + threadIdx.x, s);
+        __threadfence();
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) last = atomicInc(ticket, gridDim.x - 1) == gridDim.x - 1;
+    __syncthreads();
+    if (!last) return;
+    __threadfence();
+    for (int i = w; i < K; i += nw) {
+        double s = 0.0;
+        for (int b = lane; b < gridDim.x; b += 32) s += __ldcg(partial + (size_t)b * K + i);
+        s = warp_sum(s);
+        if (lane == 0) out[i] = s;
+    }
+}
+
+// Whether the second orthogonalisation pass is needed: the first one left less than half of
+// |t|^2 (with more left, one pass is orthogonal to within a few rounding errors).
+__device__ __forceinline__ bool cancelled(const double *left, const double *t2) { return !(*left >= 0.5 * *t2); }
+
+// out[i] = sum_d A_i[d] * u[d], i < K; A_i = A + i*ld.  Bound by the FP64 pipe.  left, t2: of a
+// second pass, see cancelled.
+__global__ void __launch_bounds__(LARGE_THREADS) k_multidot(const double *A, size_t ld, int K, const double *u,
+                                                            int64_t N, double *partial, unsigned *ticket, double *out,
+                                                            const double *left, const double *t2)
+{
+    if (left && !cancelled(left, t2)) return;
     double v[LRED];
 #pragma unroll
     for (int i = 0; i < LRED; ++i) v[i] = 0.0;
@@ -482,46 +523,44 @@ __global__ void __launch_bounds__(LARGE_THREADS) k_multidot(const double *A, siz
         for (int i = 0; i < LRED; ++i)
             if (i < K) v[i] += A[i * ld + d] * ud;
     }
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
-#pragma unroll
-    for (int i = 0; i < LRED; ++i)
-        if (i < K) v[i] = warp_sum(v[i]);
-    if (lane == 0)
-#pragma unroll
-        for (int i = 0; i < LRED; ++i)
-            if (i < K) red[w * LRED + i] = v[i];
-    __syncthreads();
-    if (threadIdx.x < K) {
-        double s = 0.0;
-        for (int j = 0; j < nw; ++j) s += red[j * LRED + threadIdx.x];
-        partial[(size_t)blockIdx.x * K + threadIdx.x] = s;
-    }
+    grid_sums(v, K, partial, ticket, out);
 }
 
-// out[i] = sum over blocks of partial (fixed order); one warp per value.
-__global__ void k_multidot_final(const double *partial, int nblocks, int K, double *out)
+// u -= sum_{i<K} coef[i] A_i and out = |u|^2.  A second pass that is not needed only passes the
+// norm on.
+__global__ void __launch_bounds__(LARGE_THREADS) k_orthogonalise(const double *A, size_t ld, int K, const double *coef,
+                                                                 int64_t N, double *u, double *partial, unsigned *ticket,
+                                                                 double *out, const double *left, const double *t2)
 {
-    const int i = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    if (i >= K) return;
-    double s = 0.0;
-    for (int b = lane; b < nblocks; b += 32) s += partial[(size_t)b * K + i];
-    s = warp_sum(s);
-    if (lane == 0) out[i] = s;
+    if (left && !cancelled(left, t2)) {
+        if (blockIdx.x == 0 && threadIdx.x == 0) *out = *left;
+        return;
+    }
+    double cf[MLARGE], v[1] = {0.0};
+#pragma unroll
+    for (int i = 0; i < MLARGE; ++i) cf[i] = (i < K) ? coef[i] : 0.0;
+    for (int64_t d = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; d < N; d += (int64_t)gridDim.x * blockDim.x) {
+        double s = u[d];
+#pragma unroll
+        for (int i = 0; i < MLARGE; ++i)
+            if (i < K) s -= cf[i] * A[i * ld + d];
+        u[d] = s;
+        v[0] += s * s;
+    }
+    grid_sums(v, 1, partial, ticket, out);
 }
 
-// x = V y, hx = W y, r = hx - theta x, t = r / clamp(diag - theta); partial sums of
-// |r|^2 and |t|^2 (two values per block).
+// x = V y, hx = W y, r = hx - theta x, t = r / clamp(diag - theta); out = |r|^2, |t|^2.
 __global__ void __launch_bounds__(LARGE_THREADS) k_ritz(const double *V, const double *W, size_t ld, int m,
                                                         const double *ys, const double *misc, const double *diag,
                                                         double shift, int64_t N, double *x, double *hx, double *t,
-                                                        double *partial)
+                                                        double *partial, unsigned *ticket, double *out)
 {
-    __shared__ double red[64];
     const double th = misc[0];
     double y[MLARGE];
 #pragma unroll
     for (int i = 0; i < MLARGE; ++i) y[i] = (i < m) ? ys[i] : 0.0;
-    double rr = 0.0, tt = 0.0;
+    double v2[2] = {0.0, 0.0};
     for (int64_t d = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; d < N; d += (int64_t)gridDim.x * blockDim.x) {
         double xs = 0.0, hs = 0.0;
 #pragma unroll
@@ -537,26 +576,13 @@ __global__ void __launch_bounds__(LARGE_THREADS) k_ritz(const double *V, const d
         if (fabs(den) < 1e-4) den = den >= 0.0 ? 1e-4 : -1e-4;
         double td = r / den;
         t[d] = td;
-        rr += r * r;
-        tt += td * td;
+        v2[0] += r * r;
+        v2[1] += td * td;
     }
-    rr = warp_sum(rr);
-    tt = warp_sum(tt);
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    if (lane == 0) {
-        red[w] = rr;
-        red[32 + w] = tt;
-    }
-    __syncthreads();
-    if (threadIdx.x < 2) {
-        double s = 0.0;
-        for (int j = 0; j < nw; ++j) s += red[threadIdx.x * 32 + j];
-        partial[(size_t)blockIdx.x * 2 + threadIdx.x] = s;
-    }
+    grid_sums(v2, 2, partial, ticket, out);
 }
 
-// u -= sum_{i<K} coef[i] A_i  (and the same on a second pair when B is not NULL:
-// ub -= sum coef[i] B_i), coefficients read on the device.
+// u -= sum_{i<K} coef[i] A_i and ub -= sum coef[i] B_i, coefficients read on the device.
 __global__ void k_subtract(const double *A, const double *B, size_t ld, int K, const double *coef, int64_t N,
                            double *u, double *ub)
 {
@@ -564,28 +590,26 @@ __global__ void k_subtract(const double *A, const double *B, size_t ld, int K, c
 #pragma unroll
     for (int i = 0; i < LRED; ++i) cf[i] = (i < K) ? coef[i] : 0.0;
     for (int64_t d = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; d < N; d += (int64_t)gridDim.x * blockDim.x) {
-        double s = u[d], sb = ub ? ub[d] : 0.0;
+        double s = u[d], sb = ub[d];
 #pragma unroll
         for (int i = 0; i < LRED; ++i)
             if (i < K) {
                 s -= cf[i] * A[i * ld + d];
-                if (ub) sb -= cf[i] * B[i * ld + d];
+                sb -= cf[i] * B[i * ld + d];
             }
         u[d] = s;
-        if (ub) ub[d] = sb;
+        ub[d] = sb;
     }
 }
 
 // u = src * scale(norm2), scale = 1/sqrt(norm2[0]); optional second vector.
 __global__ void k_scale_copy(const double *src, const double *src2, const double *norm2, int64_t N, double *u,
-                             double *u2, float *u32)
+                             double *u2)
 {
     const double s = 1.0 / sqrt(norm2[0]);
     for (int64_t d = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; d < N; d += (int64_t)gridDim.x * blockDim.x) {
-        double v = src[d] * s;
-        u[d] = v;
+        u[d] = src[d] * s;
         if (u2) u2[d] = src2[d] * s;
-        if (u32) u32[d] = (float)v;
     }
 }
 
@@ -603,12 +627,92 @@ __global__ void k_copy2(const double *a, const double *b, int64_t N, double *ca,
     }
 }
 
-// start vector: lowest diagonal element (index given) + fixed admixture
-__global__ void k_large_guess(const int64_t *best, int Ns, int sgn, int64_t N, double *x)
+// Row of element h of a packed sector vector (the upper triangle row by row, row i starting at
+// i Ns - i (i - 1) / 2).
+__device__ __forceinline__ int64_t packed_at(int Ns, int i, int j) { return (int64_t)i * Ns - (int64_t)i * (i - 1) / 2 + j - i; }
+
+// Tiles of 32 x 32 on and above the diagonal of an Ns x Ns matrix, one per block and step.
+template <typename F>
+__device__ __forceinline__ void upper_tiles(int Ns, F f)
+{
+    const int nt = (Ns + 31) / 32;
+    for (int64_t t = blockIdx.x; t < (int64_t)nt * nt; t += gridDim.x) {
+        const int bi = (int)(t / nt), bj = (int)(t - (int64_t)bi * nt);
+        if (bi > bj) continue;
+        __syncthreads();
+        f(bi * 32, bj * 32);
+    }
+}
+
+constexpr double ROOT_HALF = 0.70710678118654752440, ROOT_2 = 1.41421356237309504880;
+
+// full = the coefficient matrix of a packed vector v of the sector sgn; norm2: v is divided by
+// its norm first, in place.
+template <typename T>
+__global__ void k_unpack(double *v, const double *norm2, int Ns, int sgn, T *full)
+{
+    __shared__ T tile[32][33];
+    const double s = norm2 ? 1.0 / sqrt(*norm2) : 1.0;
+    upper_tiles(Ns, [&](int i0, int j0) {
+        for (int r = threadIdx.y; r < 32; r += blockDim.y) {
+            const int i = i0 + r, j = j0 + threadIdx.x;
+            if (i > j || j >= Ns) continue;
+            double x = v[packed_at(Ns, i, j)];
+            if (norm2) v[packed_at(Ns, i, j)] = x *= s;
+            const T c = (T)(i == j ? x : ROOT_HALF * x);
+            full[(size_t)i * Ns + j] = c;
+            tile[r][threadIdx.x] = c;
+        }
+        __syncthreads();
+        for (int r = threadIdx.y; r < 32; r += blockDim.y) {
+            const int i = i0 + threadIdx.x, j = j0 + r;
+            if (i < j && j < Ns) full[(size_t)j * Ns + i] = sgn > 0 ? tile[threadIdx.x][r] : -tile[threadIdx.x][r];
+        }
+    });
+}
+
+// The packed form of the sector's part of S + A + sgn A^T (A: may be NULL), less shift v (v: may be
+// NULL): S and its mirror image are averaged, since its rounding is not symmetric and would let the
+// other sector's lower states leak in.
+__global__ void k_pack(const double *__restrict__ S, const double *__restrict__ A, int Ns, int sgn, const double *v,
+                       double shift, double *__restrict__ out)
+{
+    __shared__ double tile[32][33];
+    auto at = [&](int i, int j) { return 0.5 * S[(size_t)i * Ns + j] + (A ? A[(size_t)i * Ns + j] : 0.0); };
+    upper_tiles(Ns, [&](int i0, int j0) {
+        for (int r = threadIdx.y; r < 32; r += blockDim.y) {
+            const int j = j0 + r, i = i0 + threadIdx.x;
+            tile[threadIdx.x][r] = i <= j && j < Ns ? at(j, i) : 0.0;
+        }
+        __syncthreads();
+        for (int r = threadIdx.y; r < 32; r += blockDim.y) {
+            const int i = i0 + r, j = j0 + threadIdx.x;
+            if (i > j || j >= Ns) continue;
+            double x = at(i, j) + (sgn > 0 ? tile[r][threadIdx.x] : -tile[r][threadIdx.x]);
+            if (i == j)
+                x = sgn > 0 ? x : 0.0;
+            else
+                x *= ROOT_2;
+            const int64_t h = packed_at(Ns, i, j);
+            out[h] = v ? x - shift * v[h] : x;
+        }
+    });
+}
+
+// start vector (packed): lowest diagonal element (index given) + fixed admixture
+__global__ void k_large_guess(const int64_t *best, int Ns, int sgn, double *x)
 {
     const SectorGuess sg{(int)best[0], sgn};
-    for (int64_t d = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; d < N; d += (int64_t)gridDim.x * blockDim.x)
-        x[d] = sector_guess((int)d, Ns, sg);
+    for (int i = blockIdx.x; i < Ns; i += gridDim.x)
+        for (int j = i + threadIdx.x; j < Ns; j += blockDim.x)
+            x[packed_at(Ns, i, j)] = i == j && sgn < 0 ? 0.0 : (i == j ? 1.0 : ROOT_2) * sector_guess(i * Ns + j, Ns, sg);
+}
+
+// the packed vector's elements of the diagonal of H
+__global__ void k_pack_diag(const double *diag, int Ns, double *out)
+{
+    for (int i = blockIdx.x; i < Ns; i += gridDim.x)
+        for (int j = i + threadIdx.x; j < Ns; j += blockDim.x) out[packed_at(Ns, i, j)] = diag[(size_t)i * Ns + j];
 }
 
 // index of the smallest diagonal element (ties -> lowest index), optionally
@@ -652,27 +756,7 @@ __global__ void k_argmin(const double *diag, int64_t N, int Ns, int open_only, i
     }
 }
 
-// Projected eigenproblem (one warp) and bookkeeping of G on the device.
-__global__ void k_large_small_eig(const double *Gd, int m, double *ys, double *y2s, double *misc)
-{
-    __shared__ double G[MMAX * MMAX];
-    __shared__ float A[MMAX * MMAX], E[MMAX * MMAX], ev[MMAX];
-    __shared__ double r[MMAX];
-    for (int e = threadIdx.x; e < MMAX * MMAX; e += 32) G[e] = Gd[e];
-    __syncwarp();
-    small_eig_warp<true>(G, m, A, E, ev, ys, y2s, r, misc);
-}
-
-// G column m (and row m) from the dots in `dots` (m + 1 values)
-__global__ void k_set_gcol(double *Gd, int m, const double *dots)
-{
-    int i = threadIdx.x;
-    if (i <= m) {
-        Gd[i * MMAX + m] = dots[i];
-        Gd[m * MMAX + i] = dots[i];
-    }
-}
-
+// Bookkeeping of G on the device.
 __global__ void k_set_g2(double *Gd, const double *dots, int two)
 {
     if (threadIdx.x == 0) {
@@ -865,7 +949,7 @@ static int large_ss_slab(mbe_ctx *ctx, const LargePlan &pl, const float *X, doub
 // added through the transposed copy of c.
 template <typename T>
 static int large_sigma_launch(mbe_ctx *ctx, const LargePlan &pl, const T *c, double *sigma, int order_tag,
-                              int sgn = 0)
+                              int sgn = 0, double *packed = nullptr, const double *v = nullptr, double shift = 0.0)
 {
     TimedLaunch tl(ctx, order_tag, 2, sizeof(T) == 8 ? 64 : 32);
     const int Ns = pl.L.Ns;
@@ -903,7 +987,7 @@ static int large_sigma_launch(mbe_ctx *ctx, const LargePlan &pl, const T *c, dou
             double *A = (double *)pl.cT;
             const int rc = large_ss_slab<false, true>(ctx, pl, (const float *)c, A);
             if (rc) return rc;
-            k_sym_add<<<pl.grid_tr, dim3(32, 8), 0, ctx->stream>>>(A, Ns, sgn, sigma, nullptr);
+            k_pack<<<pl.grid_tr, dim3(32, 8), 0, ctx->stream>>>(sigma, A, Ns, sgn, v, shift, packed);
         }
         MBE_CU(cudaGetLastError());
         ctx->launches += sgn == 0 ? 4 : 3;
@@ -922,7 +1006,11 @@ static int large_sigma_launch(mbe_ctx *ctx, const LargePlan &pl, const T *c, dou
         // transposing add replace the second product and the transpose of c
         double *A = (double *)pl.cT;
         k_large_ss<T, false, true><<<grid_ss, SS_THREADS, smem_ss, ctx->stream>>>(pl.L, c, A, digits);
-        k_sym_add<<<pl.grid_tr, dim3(32, 8), 0, ctx->stream>>>(A, Ns, sgn, sigma, digits);
+        if (sizeof(T) == 8) {
+            k_sym_add<<<pl.grid_tr, dim3(32, 8), 0, ctx->stream>>>(A, Ns, sgn, sigma, digits);
+            ++ctx->launches;
+        }
+        k_pack<<<pl.grid_tr, dim3(32, 8), 0, ctx->stream>>>(sigma, sizeof(T) == 8 ? nullptr : A, Ns, sgn, v, shift, packed);
     }
     MBE_CU(cudaGetLastError());
     ctx->launches += sgn == 0 ? 4 : 3;
@@ -992,24 +1080,6 @@ __global__ void k_lincomb2(const double *V, const double *W, size_t ld, int m, c
     }
 }
 
-// Projects v onto the spin-flip sector sgn (v[Ia][Ib] = sgn v[Ib][Ia]), pairs
-// (d, P d) averaged: the large solver's sigma is not formed over a half space,
-// so its rounding would otherwise let the other sector's lower states leak in.
-__global__ void k_project_sector(double *v, int Ns, int sgn, int64_t N)
-{
-    for (int64_t d = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; d < N; d += (int64_t)gridDim.x * blockDim.x) {
-        const int ia = (int)(d / Ns), ib = (int)(d - (int64_t)ia * Ns);
-        if (ia == ib) {
-            if (sgn < 0) v[d] = 0.0;
-        } else if (ia < ib) {
-            const int64_t pd = (int64_t)ib * Ns + ia;
-            const double m = 0.5 * (v[d] + sgn * v[pd]);
-            v[d] = m;
-            v[pd] = sgn * m;
-        }
-    }
-}
-
 // w -= shift * v  (the image of a correction under H - theta0)
 __global__ void k_shift_image(const double *v, double shift, int64_t N, double *w)
 {
@@ -1062,29 +1132,34 @@ __global__ void k_set_g3(double *Gd, const double *dots, int two)
 }
 
 struct LargeDav {
-    double *V, *W, *x, *hx, *t, *x2, *hx2, *xs, *partial, *dots, *Gd, *ys, *y2s, *misc;
-    float *c32;
+    // vectors are packed: the elements Ia <= Ib of a sector vector, those with Ia != Ib times
+    // sqrt 2 (half the work of the vector algebra, which the FP64 pipe bounds, and of its memory)
+    double *V, *W, *x, *hx, *t, *x2, *hx2, *xs, *diag, *partial, *dots, *Gd, *ys, *y2s, *misc;
+    double *full, *S;  // coefficient matrix (also as float32) and sigma of the sigma in work
+    unsigned *ticket;
     int64_t *best;
+    int64_t N;  // packed elements
     size_t ld;
     int nblk;
 };
+// places in LargeDav::dots besides the sums of a call: |r|^2, |t|^2; |u|^2 after one pass and two
+constexpr int DOT_R = 24, DOT_T = 25, DOT_U1 = 26, DOT_U2 = 27;
 
-static void dot_to(mbe_ctx *ctx, const LargePlan &pl, const LargeDav &D, const double *A, int K, const double *u,
-                   double *out)
+static void dot_to(mbe_ctx *ctx, const LargeDav &D, const double *A, int K, const double *u, double *out,
+                   const double *left = nullptr)
 {
-    k_multidot<<<D.nblk, LARGE_THREADS, 0, ctx->stream>>>(A, D.ld, K, u, pl.L.N, D.partial);
-    k_multidot_final<<<1, 32 * K, 0, ctx->stream>>>(D.partial, D.nblk, K, out);
-    ctx->launches += 2;
+    k_multidot<<<D.nblk, LARGE_THREADS, 0, ctx->stream>>>(A, D.ld, K, u, D.N, D.partial, D.ticket, out, left, D.dots + DOT_T);
+    ++ctx->launches;
 }
 
+// wout = (H - shift) vin, both packed; norm2: vin is normalised first, in place.
 template <typename T>
-static int large_apply(mbe_ctx *ctx, const LargePlan &pl, const LargeDav &D, const double *vin, double *wout,
-                       int sgn)
+static int large_apply(mbe_ctx *ctx, const LargePlan &pl, const LargeDav &D, double *vin, const double *norm2, double *wout,
+                       int sgn, double shift)
 {
-    if (sizeof(T) == 8) return large_sigma_launch<double>(ctx, pl, vin, wout, pl.L.n, sgn);
-    k_to_float<<<pl.grid_vec, 256, 0, ctx->stream>>>(vin, pl.L.N, D.c32);
+    k_unpack<T><<<pl.grid_tr, dim3(32, 8), 0, ctx->stream>>>(vin, norm2, pl.L.Ns, sgn, (T *)D.full);
     ++ctx->launches;
-    return large_sigma_launch<float>(ctx, pl, D.c32, wout, pl.L.n, sgn);
+    return large_sigma_launch<T>(ctx, pl, (const T *)D.full, D.S, pl.L.n, sgn, wout, shift != 0.0 ? vin : nullptr, shift);
 }
 
 // One Davidson phase on the large space (T = sigma arithmetic).  D.x: start
@@ -1100,7 +1175,7 @@ static int large_phase(mbe_ctx *ctx, const LargePlan &pl, const LargeDav &D, int
                        int max_iter, int steer, double *lambda, double *rnorm, int *nsig, int *status,
                        int *nsig64 = nullptr, double *anchor_y0 = nullptr)
 {
-    const int64_t N = pl.L.N;
+    const int64_t N = D.N;
     const size_t ld = D.ld;
     cudaStream_t st = ctx->stream;
     const int g = pl.grid_vec;
@@ -1110,42 +1185,36 @@ static int large_phase(mbe_ctx *ctx, const LargePlan &pl, const LargeDav &D, int
     *status = MBE_STATUS_OK;
     int rc;
     double shift = 0.0;
-    const int Ns = pl.L.Ns;
-    k_project_sector<<<g, 256, 0, st>>>(D.x, Ns, sgn, N);
-    dot_to(ctx, pl, D, D.x, 1, D.x, D.dots);
-    k_scale_copy<<<g, 256, 0, st>>>(D.x, nullptr, D.dots, N, D.V, nullptr, nullptr);
-    ctx->launches += 2;
+    dot_to(ctx, D, D.x, 1, D.x, D.dots);
+    k_scale_copy<<<g, 256, 0, st>>>(D.x, nullptr, D.dots, N, D.V, nullptr);
+    ++ctx->launches;
     if (anch) {
-        if ((rc = large_sigma_launch<double>(ctx, pl, D.V, D.W, pl.L.n, sgn))) return rc;
+        if ((rc = large_apply<double>(ctx, pl, D, D.V, nullptr, D.W, sgn, 0.0))) return rc;
         ++*nsig64;
-        k_project_sector<<<g, 256, 0, st>>>(D.W, Ns, sgn, N);
-        ++ctx->launches;
-        dot_to(ctx, pl, D, D.W, 1, D.V, D.dots);
+        dot_to(ctx, D, D.W, 1, D.V, D.dots);
         MBE_CU(cudaMemcpyAsync(&shift, D.dots, 8, cudaMemcpyDeviceToHost, st));
         MBE_CU(cudaStreamSynchronize(st));
         k_shift_image<<<g, 256, 0, st>>>(D.V, shift, N, D.W);
         ++ctx->launches;
     } else {
-        if ((rc = large_apply<T>(ctx, pl, D, D.V, D.W, sgn))) return rc;
+        if ((rc = large_apply<T>(ctx, pl, D, D.V, nullptr, D.W, sgn, 0.0))) return rc;
         ++*nsig;
     }
-    k_project_sector<<<g, 256, 0, st>>>(D.W, Ns, sgn, N);
-    ++ctx->launches;
-    dot_to(ctx, pl, D, D.W, 1, D.V, D.dots);
+    dot_to(ctx, D, D.W, 1, D.V, D.dots);
     k_set_g2<<<1, 32, 0, st>>>(D.Gd, D.dots, 0);
     ++ctx->launches;
     int m = 1;
     double best = 3e38;
     int stall = 0;
+    const double *col = nullptr;  // the new column of G
     for (int it = 0;; ++it) {
-        k_large_small_eig<<<1, 32, 0, st>>>(D.Gd, m, D.ys, D.y2s, D.misc);
+        if ((rc = launch_small_eig(st, D.Gd, m, col, D.ys, D.y2s, D.misc))) return rc;
         double *tdst = (m < MLARGE) ? D.V + (size_t)m * ld : D.t;
-        k_ritz<<<D.nblk, LARGE_THREADS, 0, st>>>(D.V, D.W, ld, m, D.ys, D.misc, pl.L.diag, shift, N, D.x, D.hx,
-                                                 tdst, D.partial);
-        k_multidot_final<<<1, 64, 0, st>>>(D.partial, D.nblk, 2, D.dots);
-        ctx->launches += 3;
+        k_ritz<<<D.nblk, LARGE_THREADS, 0, st>>>(D.V, D.W, ld, m, D.ys, D.misc, D.diag, shift, N, D.x, D.hx, tdst,
+                                                 D.partial, D.ticket, D.dots + DOT_R);
+        ctx->launches += 2;
         int herr = 0;
-        MBE_CU(cudaMemcpyAsync(h3, D.dots, 16, cudaMemcpyDeviceToHost, st));
+        MBE_CU(cudaMemcpyAsync(h3, D.dots + DOT_R, 16, cudaMemcpyDeviceToHost, st));
         MBE_CU(cudaMemcpyAsync(h3 + 2, D.misc, 8, cudaMemcpyDeviceToHost, st));
         MBE_CU(cudaMemcpyAsync(h3 + 3, D.ys, 8, cudaMemcpyDeviceToHost, st));
         MBE_CU(cudaMemcpyAsync(&herr, ctx->dev_err, sizeof(int), cudaMemcpyDeviceToHost, st));
@@ -1179,30 +1248,29 @@ static int large_phase(mbe_ctx *ctx, const LargePlan &pl, const LargeDav &D, int
             k_anchor_restart<<<g, 256, 0, st>>>(D.V, D.W, ld, m, D.ys, D.y2s, N, D.x2, D.hx2, D.x, D.hx);
             k_copy2<<<g, 256, 0, st>>>(D.x2, D.hx2, N, D.V + ld, D.W + ld);
             ctx->launches += 2;
-            dot_to(ctx, pl, D, D.V + ld, 1, D.V + ld, D.dots);
-            k_scale_copy<<<g, 256, 0, st>>>(D.V + ld, D.W + ld, D.dots, N, D.V + ld, D.W + ld, nullptr);
+            dot_to(ctx, D, D.V + ld, 1, D.V + ld, D.dots);
+            k_scale_copy<<<g, 256, 0, st>>>(D.V + ld, D.W + ld, D.dots, N, D.V + ld, D.W + ld);
             k_copy2<<<g, 256, 0, st>>>(D.x, D.hx, N, D.V + 2 * ld, D.W + 2 * ld);
             ctx->launches += 2;
             for (int pass = 0; pass < 2; ++pass) {
-                dot_to(ctx, pl, D, D.V + ld, 1, D.V + 2 * ld, D.dots);
+                dot_to(ctx, D, D.V + ld, 1, D.V + 2 * ld, D.dots);
                 k_subtract<<<g, 256, 0, st>>>(D.V + ld, D.W + ld, ld, 1, D.dots, N, D.V + 2 * ld, D.W + 2 * ld);
                 ++ctx->launches;
             }
-            dot_to(ctx, pl, D, D.V + 2 * ld, 1, D.V + 2 * ld, D.dots);
+            dot_to(ctx, D, D.V + 2 * ld, 1, D.V + 2 * ld, D.dots);
             MBE_CU(cudaMemcpyAsync(h3, D.dots, 8, cudaMemcpyDeviceToHost, st));
             MBE_CU(cudaStreamSynchronize(st));
             const int two = sqrt(h3[0]) > 1e-3 ? 1 : 0;
             if (two) {
-                k_scale_copy<<<g, 256, 0, st>>>(D.V + 2 * ld, D.W + 2 * ld, D.dots, N, D.V + 2 * ld, D.W + 2 * ld,
-                                                 nullptr);
+                k_scale_copy<<<g, 256, 0, st>>>(D.V + 2 * ld, D.W + 2 * ld, D.dots, N, D.V + 2 * ld, D.W + 2 * ld);
                 ++ctx->launches;
             }
-            dot_to(ctx, pl, D, D.W, 1, D.V + ld, D.dots);               // W0.V1
-            dot_to(ctx, pl, D, D.V + ld, 1, D.W + ld, D.dots + 1);      // V1.W1
+            dot_to(ctx, D, D.W, 1, D.V + ld, D.dots);               // W0.V1
+            dot_to(ctx, D, D.V + ld, 1, D.W + ld, D.dots + 1);      // V1.W1
             if (two) {
-                dot_to(ctx, pl, D, D.W, 1, D.V + 2 * ld, D.dots + 2);   // W0.V2
-                dot_to(ctx, pl, D, D.V + ld, 1, D.W + 2 * ld, D.dots + 3);  // V1.W2
-                dot_to(ctx, pl, D, D.V + 2 * ld, 1, D.W + 2 * ld, D.dots + 4);  // V2.W2
+                dot_to(ctx, D, D.W, 1, D.V + 2 * ld, D.dots + 2);   // W0.V2
+                dot_to(ctx, D, D.V + ld, 1, D.W + 2 * ld, D.dots + 3);  // V1.W2
+                dot_to(ctx, D, D.V + 2 * ld, 1, D.W + 2 * ld, D.dots + 4);  // V2.W2
             }
             k_set_g3<<<1, 32, 0, st>>>(D.Gd, D.dots, two);
             ++ctx->launches;
@@ -1216,49 +1284,39 @@ static int large_phase(mbe_ctx *ctx, const LargePlan &pl, const LargeDav &D, int
             k_copy2<<<g, 256, 0, st>>>(D.x2, D.hx2, N, D.V + ld, D.W + ld);
             ctx->launches += 3;
             for (int pass = 0; pass < 2; ++pass) {
-                dot_to(ctx, pl, D, D.V, 1, D.V + ld, D.dots);
+                dot_to(ctx, D, D.V, 1, D.V + ld, D.dots);
                 k_subtract<<<g, 256, 0, st>>>(D.V, D.W, ld, 1, D.dots, N, D.V + ld, D.W + ld);
                 ++ctx->launches;
             }
-            dot_to(ctx, pl, D, D.V + ld, 1, D.V + ld, D.dots);
-            k_scale_copy<<<g, 256, 0, st>>>(D.V + ld, D.W + ld, D.dots, N, D.V + ld, D.W + ld, nullptr);
-            dot_to(ctx, pl, D, D.W, 2, D.V, D.dots);
-            dot_to(ctx, pl, D, D.W + ld, 1, D.V + ld, D.dots + 2);
+            dot_to(ctx, D, D.V + ld, 1, D.V + ld, D.dots);
+            k_scale_copy<<<g, 256, 0, st>>>(D.V + ld, D.W + ld, D.dots, N, D.V + ld, D.W + ld);
+            dot_to(ctx, D, D.W, 2, D.V, D.dots);
+            dot_to(ctx, D, D.W + ld, 1, D.V + ld, D.dots + 2);
             k_set_g2<<<1, 32, 0, st>>>(D.Gd, D.dots, 1);
             ctx->launches += 2;
             m = 2;
             u = D.V + (size_t)m * ld;
             MBE_CU(cudaMemcpyAsync(u, D.t, (size_t)N * 8, cudaMemcpyDeviceToDevice, st));
         }
-        k_project_sector<<<g, 256, 0, st>>>(u, Ns, sgn, N);
-        ++ctx->launches;
         for (int pass = 0; pass < 2; ++pass) {
-            dot_to(ctx, pl, D, D.V, m, u, D.dots);
-            k_subtract<<<g, 256, 0, st>>>(D.V, nullptr, ld, m, D.dots, N, u, nullptr);
+            const double *left = pass ? D.dots + DOT_U1 : nullptr;
+            dot_to(ctx, D, D.V, m, u, D.dots, left);
+            k_orthogonalise<<<D.nblk, LARGE_THREADS, 0, st>>>(D.V, ld, m, D.dots, N, u, D.partial, D.ticket,
+                                                              D.dots + (pass ? DOT_U2 : DOT_U1), left, D.dots + DOT_T);
             ++ctx->launches;
         }
-        dot_to(ctx, pl, D, u, 1, u, D.dots);
-        MBE_CU(cudaMemcpyAsync(h3, D.dots, 8, cudaMemcpyDeviceToHost, st));
+        MBE_CU(cudaMemcpyAsync(h3, D.dots + DOT_U2, 8, cudaMemcpyDeviceToHost, st));
         MBE_CU(cudaStreamSynchronize(st));
         const double tn = sqrt(h3[0]);
         if (!(tn > 1e-12 * t0n) || !(tn > 0.0)) {
             if (!steer && rn > tol) *status = MBE_STATUS_MAXITER;
             break;
         }
-        k_scale_copy<<<g, 256, 0, st>>>(u, nullptr, D.dots, N, u, nullptr, nullptr);
-        ++ctx->launches;
-        if ((rc = large_apply<T>(ctx, pl, D, u, D.W + (size_t)m * ld, sgn))) return rc;
+        if ((rc = large_apply<T>(ctx, pl, D, u, D.dots + DOT_U2, D.W + (size_t)m * ld, sgn, anch ? shift : 0.0))) return rc;
         ++*nsig;
-        k_project_sector<<<g, 256, 0, st>>>(D.W + (size_t)m * ld, Ns, sgn, N);
-        ++ctx->launches;
-        if (anch) {
-            k_shift_image<<<g, 256, 0, st>>>(u, shift, N, D.W + (size_t)m * ld);
-            ++ctx->launches;
-        }
-        dot_to(ctx, pl, D, D.V, m + 1, D.W + (size_t)m * ld, D.dots);
-        if (anch) dot_to(ctx, pl, D, D.W, 1, u, D.dots);  // x0.(A u) as u.r0
-        k_set_gcol<<<1, 32, 0, st>>>(D.Gd, m, D.dots);
-        ++ctx->launches;
+        dot_to(ctx, D, D.V, m + 1, D.W + (size_t)m * ld, D.dots);
+        if (anch) dot_to(ctx, D, D.W, 1, u, D.dots);  // x0.(A u) as u.r0
+        col = D.dots;
         ++m;
     }
     return MBE_OK;
@@ -1289,12 +1347,14 @@ extern "C" int casci_solve(mbe_ctx *ctx, int norb, const double *h1, const doubl
     int k0 = 0;
     for (int i = 0; i < n_cas; ++i) k0 += (cas_orbs[i] >= 0 && cas_orbs[i] < norb && occ_h[cas_orbs[i]]) ? 1 : 0;
     const int64_t N = binom(n_cas, k0) * binom(n_cas, k0);
-    const size_t vec = align256((size_t)N * 8);
+    const int64_t ns0 = binom(n_cas, k0);
     LargeDav D;
+    D.N = ns0 * (ns0 + 1) / 2;
+    const size_t vec = align256((size_t)D.N * 8);
     D.ld = vec / 8;
     D.nblk = ctx->sm_count * 4;
     const bool mixed = o.precision == MBE_PREC_MIXED;
-    size_t bytes = large_bytes(ctx, norb, n_cas, k0, false, mixed) + vec * (2 * MLARGE + 6) + align256((size_t)N * 4) +
+    size_t bytes = large_bytes(ctx, norb, n_cas, k0, false, mixed) + vec * (2 * MLARGE + 7) + 2 * align256((size_t)N * 8) +
                    align256((size_t)D.nblk * LRED * 8) + 8 * 256 + 4096;
     void *ws = nullptr;
     int rc = workspace(ctx, bytes, &ws);
@@ -1308,7 +1368,10 @@ extern "C" int casci_solve(mbe_ctx *ctx, int norb, const double *h1, const doubl
     D.x2 = bump.take<double>(D.ld);
     D.hx2 = bump.take<double>(D.ld);
     D.xs = bump.take<double>(D.ld);
-    D.c32 = bump.take<float>((size_t)N);
+    D.diag = bump.take<double>(D.ld);
+    D.full = bump.take<double>((size_t)N);
+    D.S = bump.take<double>((size_t)N);
+    D.ticket = bump.take<unsigned>(1);
     D.partial = bump.take<double>((size_t)D.nblk * LRED);
     D.dots = bump.take<double>(32);
     D.Gd = bump.take<double>(MMAX * MMAX);
@@ -1325,9 +1388,12 @@ extern "C" int casci_solve(mbe_ctx *ctx, int norb, const double *h1, const doubl
     const int Ns = pl.L.Ns;
     k_argmin<<<1, 1024, 0, ctx->stream>>>(pl.L.diag, N, Ns, 0, D.best);
     k_argmin<<<1, 1024, 0, ctx->stream>>>(pl.L.diag, N, Ns, 1, D.best + 1);
-    ctx->launches += 2;
+    k_pack_diag<<<std::min(Ns, ctx->sm_count * 8), 256, 0, ctx->stream>>>(pl.L.diag, Ns, D.diag);
+    MBE_CU(cudaMemsetAsync(D.ticket, 0, sizeof(unsigned), ctx->stream));
+    ctx->launches += 3;
     double lam = 0.0, rn = 0.0;
     int n32 = 0, n64 = 0, st = 0;
+    int won = 1;
     bool degen = false;
     // the two spin-flip sectors (see sector_guess); each runs the float32 phase
     // (mixed mode) and the float64 phase; the second sector first runs a float64
@@ -1335,8 +1401,8 @@ extern "C" int casci_solve(mbe_ctx *ctx, int norb, const double *h1, const doubl
     for (int sector = 0; sector < 2; ++sector) {
         if (sector == 1 && (Ns < 2 || st != MBE_STATUS_OK || o.sectors == MBE_SECTORS_EVEN)) break;
         const int sgn = sector == 0 ? 1 : -1;
-        if (sector == 1) MBE_CU(cudaMemcpyAsync(D.xs, D.x, (size_t)N * 8, cudaMemcpyDeviceToDevice, ctx->stream));
-        k_large_guess<<<pl.grid_vec, 256, 0, ctx->stream>>>(D.best + sector, Ns, sgn, N, D.x);
+        if (sector == 1) MBE_CU(cudaMemcpyAsync(D.xs, D.x, (size_t)D.N * 8, cudaMemcpyDeviceToDevice, ctx->stream));
+        k_large_guess<<<std::min(Ns, ctx->sm_count * 8), 256, 0, ctx->stream>>>(D.best + sector, Ns, sgn, D.x);
         ++ctx->launches;
         double l = 0.0, r = 0.0;
         int s64 = 0, s32 = 0, ss = MBE_STATUS_OK;
@@ -1352,7 +1418,7 @@ extern "C" int casci_solve(mbe_ctx *ctx, int norb, const double *h1, const doubl
             s32 += n;
             bool decided = sector == 0;
             if (ss == MBE_STATUS_NONFINITE) {
-                k_large_guess<<<pl.grid_vec, 256, 0, ctx->stream>>>(D.best + sector, Ns, sgn, N, D.x);
+                k_large_guess<<<std::min(Ns, ctx->sm_count * 8), 256, 0, ctx->stream>>>(D.best + sector, Ns, sgn, D.x);
                 ++ctx->launches;
             } else {
                 for (int anc = 0; anc < LARGE_ANCHORS && !lose && !refined; ++anc) {
@@ -1402,14 +1468,19 @@ extern "C" int casci_solve(mbe_ctx *ctx, int norb, const double *h1, const doubl
             lam = l;
             rn = r;
             st = ss;
+            won = sgn;
         } else {
             degen = degen || (!lose && ss == MBE_STATUS_OK && st == MBE_STATUS_OK && fabs(l - lam) <= DEGEN_TOL);
-            MBE_CU(cudaMemcpyAsync(D.x, D.xs, (size_t)N * 8, cudaMemcpyDeviceToDevice, ctx->stream));
+            MBE_CU(cudaMemcpyAsync(D.x, D.xs, (size_t)D.N * 8, cudaMemcpyDeviceToDevice, ctx->stream));
         }
     }
     double ephi = 0.0;
     MBE_CU(cudaMemcpyAsync(&ephi, pl.L.diag + dphi, 8, cudaMemcpyDeviceToHost, ctx->stream));
-    if (cvec) MBE_CU(cudaMemcpyAsync(cvec, D.x, (size_t)N * 8, cudaMemcpyDeviceToDevice, ctx->stream));
+    if (cvec) {
+        k_unpack<double><<<pl.grid_tr, dim3(32, 8), 0, ctx->stream>>>(D.x, nullptr, Ns, won, cvec);
+        MBE_CU(cudaGetLastError());
+        ++ctx->launches;
+    }
     MBE_CU(cudaStreamSynchronize(ctx->stream));
     result[0] = lam;
     result[1] = lam - ephi;
