@@ -840,16 +840,16 @@ __device__ __noinline__ void sigma_block(const BlockProblem &B, const T *src, T 
 }
 
 // Lowest eigenpair of the m x m symmetric Rayleigh matrix G (shared memory, float64, row
-// stride MMAX) by the whole block: a float32 Jacobi on G - G00 I in round-robin order, m / 2
-// disjoint rotations at a time (one lane each), then one element of the matrix and of the
-// eigenvectors per thread (m - 1 steps per sweep, where rotating one pair after the other in one warp took m (m - 1)
-// / 2 of about the same length); in float64 then two Newton steps in that eigenbasis,
-// z = y - sum_{k != 0} e_k (e_k . r) / (theta_k - theta),  r = G y - theta y,
-// theta = y.G y, which make the lowest pair float64-accurate (one warp).
+// stride MMAX) by the whole block.  warm: the last call was on the leading (m - 1) x (m - 1) part
+// of G; in its eigenbasis an arrow matrix is left, whose eigenvalues are the roots of a secular
+// equation (one lane each) and whose eigenvectors have a closed form, with the couplings recomputed
+// from the roots, which keeps them orthogonal (Gu and Eisenstat, SIAM J. Matrix Anal. Appl. 16,
+// 172, 1995).  Otherwise a float32 Jacobi on G - G00 I in round-robin order, m / 2 disjoint
+// rotations at a time, EIGNOTE.  In float64 then two Newton steps in that
+// eigenbasis, z = y - sum_{k != 0} e_k (e_k . r) / (theta_k - theta),  r = G y - theta y,
+// theta = y.G y, which make the lowest pair float64-accurate; in float32 one (one warp).
 // Output: y[0..m) (unit norm), y2 (the second lowest, which seeds the thick restart), and
 // misc[0] = theta; ends with a barrier.
-// warm: the last call was on the leading (m - 1) x (m - 1) part of G, and its eigenbasis is the
-// start of this one (an arrow matrix is left to diagonalise).
 template <bool REFINE>
 __device__ __noinline__ void small_eig_block(const BlockMem &S, int m, bool warm)
 {
@@ -864,25 +864,132 @@ __device__ __noinline__ void small_eig_block(const BlockMem &S, int m, bool warm
     const double shift = G[0];
     float *A = buf, *E = buf + MMAX * MMAX, *A2 = buf + 2 * MMAX * MMAX, *E2 = buf + 3 * MMAX * MMAX;
     if (warm) {
-        // in the last call's eigenbasis: its eigenvalues, and the new row
-        if (tid < m - 1) {
-            float b = 0.f;
-            for (int k = 0; k < m - 1; ++k) b += E[k * MMAX + tid] * (float)G[k * MMAX + m - 1];
-            rot[tid].x = b;
+        // half a warp per pole or root, its lanes share the terms of every sum
+        const int q = m - 1, half = tid >> 4, l0 = tid & 15;
+        const bool work = half < MMAX;  // (whole warps)
+        float *sd = A2, *sb = sd + MMAX, *sp = sb + MMAX, *st = sp + MMAX, *sn = st + MMAX;  // poles, couplings, a root's
+                                                                                            // pole and offset, norms
+        auto sum16 = [](float v) {
+#pragma unroll
+            for (int o = 8; o > 0; o >>= 1) v += __shfl_xor_sync(FULL, v, o);
+            return v;
+        };
+        auto over = [](float x, float y) {  // x / y, y a normal number
+            float r;
+            asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(y));
+            return x * r;
+        };
+        auto gap = [&](int k, int l) { return (sp[k] - sd[l]) + st[k]; };  // root k - pole l
+        if (work) {
+            float b = 0.f;  // the new row in the last basis
+            for (int k = l0; k < q; k += 16) b += half < q ? E[k * MMAX + half] * (float)G[k * MMAX + q] : 0.f;
+            b = sum16(b);
+            if (l0 == 0) sb[half] = b;
         }
         __syncthreads();
-        if (on) {
-            const bool last = i == m - 1 || j == m - 1;
-            A[tid] = i == j ? (last ? (float)(G[i * MMAX + i] - shift) : ev[i]) : last ? rot[i < j ? i : j].x : 0.f;
-            if (last) E[tid] = i == j ? 1.0f : 0.0f;
+        // the arrow matrix: diagonal d = ev, row b, corner a
+        const float a = (float)(G[q * MMAX + q] - shift);
+        float b = lane < q ? sb[lane] : 0.f, d = lane < q ? ev[lane] : 0.f;  // (in every warp)
+        float scale = fmaxf(fabsf(a), fmaxf(fabsf(d), fabsf(b)));
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) scale = fmaxf(scale, __shfl_xor_sync(FULL, scale, o));
+        // poles apart and couplings nonzero by a rounding error of the matrix
+        const float eps = fmaxf(1.2e-7f * scale, 1e-15f);
+        if (lane < q && fabsf(b) < eps) b = copysignf(eps, b);
+        d = lane < q ? d - lane * 2.f * eps : -3e38f;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const float u = __shfl_up_sync(FULL, d, o);
+            if (lane >= o && lane < q) d = fmaxf(d, u);
         }
-    } else if (on) {
-        A[tid] = (float)(G[i * MMAX + j] - (i == j ? shift : 0.0));
-        E[tid] = i == j ? 1.0f : 0.0f;
+        d += lane * 2.f * eps;
+        const float nb = sqrtf(warp_sum(b * b)) * 1.001f;
+        if (tid < q) sd[tid] = d;
+        __syncthreads();  // (sb has been read)
+        if (tid < q) sb[tid] = b;
+        __syncthreads();
+        if (work) {
+            const int l1 = l0 + 16;
+            const float d0 = l0 < q ? sd[l0] : 0.f, b0 = l0 < q ? sb[l0] * sb[l0] : 0.f;
+            const float d1 = l1 < q ? sd[l1] : 0.f, b1 = l1 < q ? sb[l1] * sb[l1] : 0.f;
+            auto secular = [&](float pole, float t) {  // falls from pole to pole
+                float f = l0 < q ? over(b0, (d0 - pole) - t) : 0.f;
+                if (l1 < q) f += over(b1, (d1 - pole) - t);
+                return ((a - pole) - t) - sum16(f);
+            };
+            // root `half` lies between poles half - 1 and half: as a distance from the nearer one, by
+            // bisection on its bits
+            const int k = min(half, q), lp = max(k - 1, 0), rp = min(k, q - 1);
+            const float mid2 = 0.5f * (sd[rp] - sd[lp]);
+            const float fm = secular(sd[lp], mid2 > 0.f ? mid2 : nb);
+            const bool left = k == q || (k > 0 && !(fm > 0.f));
+            const float pole = sd[left ? lp : rp];
+            const float lim = k == 0 ? fmaxf(pole - a, 0.f) + nb : k == q ? fmaxf(a - pole, 0.f) + nb : mid2;
+            int lo = 0x00800000, hi = max(__float_as_int(lim), lo);
+#pragma unroll 1
+            for (int it = 0; it < 31; ++it) {
+                const int mid = lo + ((hi - lo) >> 1);
+                const float t = __int_as_float(mid);
+                if ((secular(pole, left ? t : -t) > 0.f) == left)
+                    lo = mid;
+                else
+                    hi = mid;
+            }
+            if (l0 == 0 && half <= q) {
+                sp[half] = pole;
+                st[half] = left ? __int_as_float(hi) : -__int_as_float(hi);
+            }
+        }
+        __syncthreads();
+        float bh = 0.f;
+        if (work) {
+            // the couplings whose arrow matrix has exactly these roots
+            float p = 1.f;
+            for (int l = l0; l < q; l += 16)
+                if (half < q) p *= l == half ? -gap(l, half) * gap(l + 1, half) : over(gap(l < half ? l : l + 1, half), sd[l] - sd[half]);
+#pragma unroll
+            for (int o = 8; o > 0; o >>= 1) p *= __shfl_xor_sync(FULL, p, o);
+            bh = half < q ? copysignf(sqrtf(fmaxf(p, 0.f)), sb[half]) : 0.f;
+        }
+        __syncthreads();
+        if (work && l0 == 0 && half < q) sb[half] = bh;
+        __syncthreads();
+        if (work) {
+            float z = 0.f;
+            for (int l = l0; l < q; l += 16)
+                if (half <= q) {
+                    const float v = over(sb[l], gap(half, l));
+                    z += v * v;
+                }
+            z = sum16(z);
+            if (l0 == 0 && half <= q) {
+                sn[half] = rsqrtf(1.f + z);
+                ev[half] = sp[half] + st[half];
+            }
+        }
+        __syncthreads();
+        if (on) A[tid] = sn[j] * (i < q ? over(sb[i], gap(j, i)) : 1.f);
+        __syncthreads();
+        float e = 0.f;
+        if (on) {
+            if (i < q)
+                for (int l = 0; l < q; ++l) e += E[i * MMAX + l] * A[l * MMAX + j];
+            else
+                e = A[tid];
+        }
+        __syncthreads();
+        if (on) E[tid] = e;
+        __syncthreads();
     }
-    __syncthreads();
+    if (!warm) {
+        if (on) {
+            A[tid] = (float)(G[i * MMAX + j] - (i == j ? shift : 0.0));
+            E[tid] = i == j ? 1.0f : 0.0f;
+        }
+        __syncthreads();
+    }
     const int M = m + (m & 1);  // an odd matrix gets an idle partner
-    for (int sweep = 0; sweep < 10 && m > 1; ++sweep) {
+    for (int sweep = 0; sweep < 10 && m > 1 && !warm; ++sweep) {
         float dia = 0.f;
         bool big = false;
         if (on) {
@@ -936,41 +1043,33 @@ __device__ __noinline__ void small_eig_block(const BlockMem &S, int m, bool warm
             E2 = z;
         }
     }
-    if (E != buf + MMAX * MMAX) {
-        if (on) E2[tid] = E[tid];
+    if (!warm) {
+        // eigenvalues in ascending order, into ev and the place of E
+        int *rank = (int *)rot;
+        if (tid < m) {
+            const float x = A[tid * MMAX + tid];
+            int r = 0;
+            for (int k = 0; k < m; ++k) {
+                const float v = A[k * MMAX + k];
+                r += v < x || (v == x && k < tid) ? 1 : 0;
+            }
+            rank[tid] = min(r, m - 1);
+            ev[min(r, m - 1)] = x;
+        }
+        const float e = on ? E[tid] : 0.f;
         __syncthreads();
         E = buf + MMAX * MMAX;
+        if (on) E[i * MMAX + rank[j]] = e;
+        __syncthreads();
     }
     if (tid < 32) {
-        float best = (lane < m) ? A[lane * MMAX + lane] : 3.0e38f;
-        int bi = lane;
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            float ov = __shfl_xor_sync(FULL, best, o);
-            int oi = __shfl_xor_sync(FULL, bi, o);
-            if (ov < best || (ov == best && oi < bi)) {
-                best = ov;
-                bi = oi;
-            }
-        }
-        float best2 = (lane < m && lane != bi) ? A[lane * MMAX + lane] : 3.0e38f;
-        int b2 = (lane < m && lane != bi) ? lane : 0x7fffffff;
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            float ov = __shfl_xor_sync(FULL, best2, o);
-            int oi = __shfl_xor_sync(FULL, b2, o);
-            if (ov < best2 || (ov == best2 && oi < b2)) {
-                best2 = ov;
-                b2 = oi;
-            }
-        }
+        constexpr int bi = 0;
         if (lane < m) {
-            ev[lane] = A[lane * MMAX + lane];
-            y[lane] = (double)E[lane * MMAX + bi];
-            y2[lane] = (b2 < m) ? (double)E[lane * MMAX + b2] : 0.0;
+            y[lane] = (double)E[lane * MMAX];
+            y2[lane] = m > 1 ? (double)E[lane * MMAX + 1] : 0.0;
         }
         __syncwarp();
-        double theta = shift + (double)best;
+        double theta = shift + (double)ev[0];
         __syncwarp();
         if (!REFINE) {
             // one such step in float32, which also takes out what the warm starts have gathered in E
@@ -1908,17 +2007,25 @@ __global__ void __launch_bounds__(BLOCK_THREADS, 1) k_casci_block(BatchArgs a, i
 }
 
 // small_eig_block on a Rayleigh matrix in global memory (the large-CAS solver's).  col: its new last
-// column, put in first (m values; may be NULL).
-__global__ void __launch_bounds__(416) k_small_eig(double *Gd, int m, const double *col, BlockMem S, double *ys, double *y2s,
-                                                          double *misc)
+// column, put in first (m values, or NULL).  basis: the eigenbasis and eigenvalues of the
+// last call, read if warm ([MMAX + 1][MMAX]), replaced.
+__global__ void __launch_bounds__(416) k_small_eig(double *Gd, int m, const double *col, int warm, BlockMem S, float *basis, double *ys,
+                                                   double *y2s, double *misc)
 {
     const int tid = threadIdx.x;
     double *G = (double *)(block_shared() + S.off_G);
+    float *E = (float *)(block_shared() + S.off_J) + MMAX * MMAX, *ev = (float *)(block_shared() + S.off_ev);
     if (col && tid < m) Gd[tid * MMAX + m - 1] = Gd[(m - 1) * MMAX + tid] = col[tid];
     __syncthreads();
-    if (tid < MMAX * MMAX) G[tid] = Gd[tid];
+    if (tid < MMAX * MMAX) {
+        G[tid] = Gd[tid];
+        if (warm) E[tid] = basis[tid];
+    }
+    if (warm && tid < MMAX) ev[tid] = basis[MMAX * MMAX + tid];
     __syncthreads();
-    small_eig_block<true>(S, m, false);
+    small_eig_block<true>(S, m, warm);
+    if (tid < MMAX * MMAX) basis[tid] = E[tid];
+    if (tid < MMAX) basis[MMAX * MMAX + tid] = ev[tid];
     if (tid < m) {
         ys[tid] = ((double *)(block_shared() + S.off_y))[tid];
         y2s[tid] = ((double *)(block_shared() + S.off_yp))[tid];
@@ -1926,11 +2033,11 @@ __global__ void __launch_bounds__(416) k_small_eig(double *Gd, int m, const doub
     if (tid == 0) misc[0] = *(double *)(block_shared() + S.off_misc);
 }
 
-int launch_small_eig(cudaStream_t st, double *Gd, int m, const double *col, double *ys, double *y2s,
+int launch_small_eig(cudaStream_t st, double *Gd, int m, const double *col, int warm, float *basis, double *ys, double *y2s,
                      double *misc)
 {
     const BlockMem S = block_mem(2, SIGMA_GLOBAL, 1, 1, 0);
-    k_small_eig<<<1, 416, S.bytes, st>>>(Gd, m, col, S, ys, y2s, misc);
+    k_small_eig<<<1, 416, S.bytes, st>>>(Gd, m, col, warm, S, basis, ys, y2s, misc);
     MBE_CU(cudaGetLastError());
     return MBE_OK;
 }

@@ -2026,7 +2026,7 @@ int launch_sector64(mbe_ctx *ctx, const BatchArgs &a, int b, int k);            
 int launch_sector64_redo(mbe_ctx *ctx, const BatchArgs &a, int b, int k);                // casci_sector64_redo.cu
 int launch_warp_mixed_dpl(mbe_ctx *ctx, const BatchArgs &a, int b, const MixLayout &L, int dpl);  // casci_mixed.cu
 // Projected eigenproblem of the large-CAS Davidson (casci_block.cu).
-int launch_small_eig(cudaStream_t st, double *Gd, int m, const double *col, double *ys, double *y2s,
+int launch_small_eig(cudaStream_t st, double *Gd, int m, const double *col, int warm, float *basis, double *ys, double *y2s,
                      double *misc);
 int block_grid(mbe_ctx *ctx, BatchArgs &a, const bool (&in)[MBE_MAX_STRING_ORB + 1], int rdm, int *grid, size_t *smem,
                size_t *slot);                                                            // casci_block.cu

@@ -1137,6 +1137,7 @@ struct LargeDav {
     double *V, *W, *x, *hx, *t, *x2, *hx2, *xs, *diag, *partial, *dots, *Gd, *ys, *y2s, *misc;
     double *full, *S;  // coefficient matrix (also as float32) and sigma of the sigma in work
     unsigned *ticket;
+    float *basis;  // of launch_small_eig
     int64_t *best;
     int64_t N;  // packed elements
     size_t ld;
@@ -1207,8 +1208,10 @@ static int large_phase(mbe_ctx *ctx, const LargePlan &pl, const LargeDav &D, int
     double best = 3e38;
     int stall = 0;
     const double *col = nullptr;  // the new column of G
+    int warm = 0;                 // G grew by it since the last eigenproblem
     for (int it = 0;; ++it) {
-        if ((rc = launch_small_eig(st, D.Gd, m, col, D.ys, D.y2s, D.misc))) return rc;
+        if ((rc = launch_small_eig(st, D.Gd, m, col, warm, D.basis, D.ys, D.y2s, D.misc))) return rc;
+        warm = 1;
         double *tdst = (m < MLARGE) ? D.V + (size_t)m * ld : D.t;
         k_ritz<<<D.nblk, LARGE_THREADS, 0, st>>>(D.V, D.W, ld, m, D.ys, D.misc, D.diag, shift, N, D.x, D.hx, tdst,
                                                  D.partial, D.ticket, D.dots + DOT_R);
@@ -1275,6 +1278,7 @@ static int large_phase(mbe_ctx *ctx, const LargePlan &pl, const LargeDav &D, int
             k_set_g3<<<1, 32, 0, st>>>(D.Gd, D.dots, two);
             ++ctx->launches;
             m = 2 + two;
+            warm = 0;
             u = D.V + (size_t)m * ld;
             MBE_CU(cudaMemcpyAsync(u, D.t, (size_t)N * 8, cudaMemcpyDeviceToDevice, st));
         } else if (m == MLARGE) {
@@ -1295,6 +1299,7 @@ static int large_phase(mbe_ctx *ctx, const LargePlan &pl, const LargeDav &D, int
             k_set_g2<<<1, 32, 0, st>>>(D.Gd, D.dots, 1);
             ctx->launches += 2;
             m = 2;
+            warm = 0;
             u = D.V + (size_t)m * ld;
             MBE_CU(cudaMemcpyAsync(u, D.t, (size_t)N * 8, cudaMemcpyDeviceToDevice, st));
         }
@@ -1355,7 +1360,7 @@ extern "C" int casci_solve(mbe_ctx *ctx, int norb, const double *h1, const doubl
     D.nblk = ctx->sm_count * 4;
     const bool mixed = o.precision == MBE_PREC_MIXED;
     size_t bytes = large_bytes(ctx, norb, n_cas, k0, false, mixed) + vec * (2 * MLARGE + 7) + 2 * align256((size_t)N * 8) +
-                   align256((size_t)D.nblk * LRED * 8) + 8 * 256 + 4096;
+                   align256((size_t)D.nblk * LRED * 8) + 8 * 256 + 8192;
     void *ws = nullptr;
     int rc = workspace(ctx, bytes, &ws);
     if (rc) return rc;
@@ -1372,6 +1377,7 @@ extern "C" int casci_solve(mbe_ctx *ctx, int norb, const double *h1, const doubl
     D.full = bump.take<double>((size_t)N);
     D.S = bump.take<double>((size_t)N);
     D.ticket = bump.take<unsigned>(1);
+    D.basis = bump.take<float>((MMAX + 1) * MMAX);
     D.partial = bump.take<double>((size_t)D.nblk * LRED);
     D.dots = bump.take<double>(32);
     D.Gd = bump.take<double>(MMAX * MMAX);
