@@ -399,41 +399,41 @@ __device__ __forceinline__ void gather_strings(const BlockProblem &B, const Gemm
     const int Ns = pb.Ns, tid = threadIdx.x, nt = blockDim.x, R = pb.R, sgn = pb.sector;
     const uint16_t *list = (const uint16_t *)(block_shared() + B.S.off_list);
     const double *hd = (const double *)(block_shared() + B.S.off_hd);
-            const int n1 = Ns + 1, ne = (gc + 1) / 2 * n1;
-            int split = 0;  // 2^split threads per element, where they fit
-            while (split < 3 && (ne << (split + 1)) <= nt) ++split;
-            for (int q0 = 0; q0 < ne << split; q0 += nt) {
-                const int q = q0 + tid, el = q >> split, pr = el / n1, r = el - pr * n1;
-                const int first = tail_string(Ns, I0 + 2 * pr), len = Ns - first;  // elements of the pair's first string
-                const int g = 2 * pr + (r < len ? 0 : 1), Ia = r < len ? first : tail_string(Ns, I0 + g), Ib = Ia + r - (r < len ? 0 : len);
-                const bool on = g < gc && Ib < Ns, last = on && (q & ((1 << split) - 1)) == 0;
-                // (the same-spin terms come from L2: asked for before the walk over the list)
-                const A m0 = last ? M[Ia * s.cst + Ib] : (A)0, m1 = last ? M[Ib * s.cst + Ia] : (A)0;
-                A acc = 0;
-                if (on) {
-                    const A *t = Tm + g * pb.P * s.cst;
-                    const uint16_t *lb = list + Ib * s.rs;
-    #pragma unroll 4
-                    for (int y = q & ((1 << split) - 1); y < R; y += 1 << split) {
-                        const int e = lb[y];
-                        const A v = t[((e >> 1) & 63) * s.cst + (e >> 7)];
-                        acc += e & 1 ? -v : v;
-                    }
-                }
-                for (int o = 1; o < 1 << split; o <<= 1) acc += __shfl_xor_sync(FULL, acc, o);
-                if (last) {
-                    const int h = Ia * Ns - Ia * (Ia - 1) / 2 + Ib - Ia;
-                    acc += m0 + (sgn > 0 ? m1 : -m1);
-                    T v;
-                    if constexpr (F64) {
-                        v = fma(hd[Ia] + hd[Ib], src[h], (double)acc * (pow2(B.E - 54) * (Ia == Ib ? 1.0 : 1.4142135623730951)));
-                        if (B.bad) v = __longlong_as_double(0x7ff8000000000000LL);
-                    } else {
-                        v = Ia == Ib ? acc : 1.41421356f * acc;
-                    }
-                    dst[h] = sgn < 0 && Ia == Ib ? (T)0 : v;
-                }
+    const int n1 = Ns + 1, ne = (gc + 1) / 2 * n1;
+    int split = 0;  // 2^split threads per element, where they fit
+    while (split < 3 && (ne << (split + 1)) <= nt) ++split;
+    for (int q0 = 0; q0 < ne << split; q0 += nt) {
+        const int q = q0 + tid, el = q >> split, pr = el / n1, r = el - pr * n1;
+        const int first = tail_string(Ns, I0 + 2 * pr), len = Ns - first;  // elements of the pair's first string
+        const int g = 2 * pr + (r < len ? 0 : 1), Ia = r < len ? first : tail_string(Ns, I0 + g), Ib = Ia + r - (r < len ? 0 : len);
+        const bool on = g < gc && Ib < Ns, last = on && (q & ((1 << split) - 1)) == 0;
+        // (the same-spin terms come from L2: asked for before the walk over the list)
+        const A m0 = last ? M[Ia * s.cst + Ib] : (A)0, m1 = last ? M[Ib * s.cst + Ia] : (A)0;
+        A acc = 0;
+        if (on) {
+            const A *t = Tm + g * pb.P * s.cst;
+            const uint16_t *lb = list + Ib * s.rs;
+#pragma unroll 4
+            for (int y = q & ((1 << split) - 1); y < R; y += 1 << split) {
+                const int e = lb[y];
+                const A v = t[((e >> 1) & 63) * s.cst + (e >> 7)];
+                acc += e & 1 ? -v : v;
             }
+        }
+        for (int o = 1; o < 1 << split; o <<= 1) acc += __shfl_xor_sync(FULL, acc, o);
+        if (last) {
+            const int h = Ia * Ns - Ia * (Ia - 1) / 2 + Ib - Ia;
+            acc += m0 + (sgn > 0 ? m1 : -m1);
+            T v;
+            if constexpr (F64) {
+                v = fma(hd[Ia] + hd[Ib], src[h], (double)acc * (pow2(B.E - 54) * (Ia == Ib ? 1.0 : 1.4142135623730951)));
+                if (B.bad) v = __longlong_as_double(0x7ff8000000000000LL);
+            } else {
+                v = Ia == Ib ? acc : 1.41421356f * acc;
+            }
+            dst[h] = sgn < 0 && Ia == Ib ? (T)0 : v;
+        }
+    }
 }
 
 // float64 sigma of a packed sector vector with the products on the tensor cores, in exact digits
@@ -845,7 +845,8 @@ __device__ __noinline__ void sigma_block(const BlockProblem &B, const T *src, T 
 // equation (one lane each) and whose eigenvectors have a closed form, with the couplings recomputed
 // from the roots, which keeps them orthogonal (Gu and Eisenstat, SIAM J. Matrix Anal. Appl. 16,
 // 172, 1995).  Otherwise a float32 Jacobi on G - G00 I in round-robin order, m / 2 disjoint
-// rotations at a time, EIGNOTE.  In float64 then two Newton steps in that
+// rotations at a time (60-90 thousand cycles where the arrow takes 19, or 33 in
+// float64).  In float64 then two Newton steps in that
 // eigenbasis, z = y - sum_{k != 0} e_k (e_k . r) / (theta_k - theta),  r = G y - theta y,
 // theta = y.G y, which make the lowest pair float64-accurate; in float32 one (one warp).
 // Output: y[0..m) (unit norm), y2 (the second lowest, which seeds the thick restart), and
@@ -1623,7 +1624,7 @@ __device__ void block_setup(const BatchArgs &a, BlockProblem &B, const ClassInfo
         for (int o = 16; o > 0; o >>= 1) big = fmax(big, __shfl_xor_sync(FULL, big, o));
         if ((tid & 31) == 0) red[tid >> 5] = big;
         __syncthreads();
-        B.E = fixed_exponent((tid & 31) < (nt >> 5) ? red[tid & 31] : 0.0);
+        B.E = fixed_exponent((tid & 31) < (nt >> 5) ? high_word(red[tid & 31]) : 0);
         const double scale = pow2(55 - B.E);
         int2 *Vf = (int2 *)pb.V64, *Hf = (int2 *)pb.Hs64;
         for (int e = tid; e < P * P; e += nt) Vf[e] = to_fixed(pb.V64[e], scale);

@@ -229,12 +229,14 @@ __device__ inline int2 to_fixed(double v, double scale)
 // 2^e as a double (e within the normal range)
 __device__ inline double pow2(int e) { return __longlong_as_double((long long)(e + 1023) << 52); }
 
-// Exponent E of the fixed-point scale: 2^E is the power of two above the warp's largest v.
-__device__ inline int fixed_exponent(double v)
+// |v|'s high word: ordered like |v| (a warp's double fmax is 19 cycles of the FP64 pipe).
+__device__ inline int high_word(double v) { return __double2hiint(v) & 0x7fffffff; }
+
+// Exponent E of the fixed-point scale: 2^E is the power of two above the warp's largest value,
+// from its high words.
+__device__ inline int fixed_exponent(int hi)
 {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v = fmax(v, __shfl_xor_sync(FULL, v, o));
-    const int E = (int)((__double_as_longlong(v) >> 52) & 0x7ff) - 1022;
+    const int E = (__reduce_max_sync(FULL, hi) >> 20) - 1022;
     return E < -900 ? -900 : E > 900 ? 900 : E;
 }
 
@@ -293,7 +295,13 @@ __device__ SectorStart sector_setup(const BatchArgs &a, const SectorTables<C> &T
         if (ij.x == ij.y) hd[ij.x] = v;
     }
     __syncwarp();
-    double best = 1e300, best_o = 1e300;
+    // (compared as integers that are ordered like the values: a warp's float64 comparison holds the
+    // FP64 pipe for 19 cycles)
+    auto ordered = [](double v) {
+        const long long b = __double_as_longlong(v);
+        return b ^ ((b >> 63) & 0x7fffffffffffffffLL);
+    };
+    long long best = ordered(1e300), best_o = best;
     SectorStart st;
     st.g = st.go = 0x7fffffff;
 #pragma unroll 1
@@ -303,18 +311,19 @@ __device__ SectorStart sector_setup(const BatchArgs &a, const SectorTables<C> &T
 #pragma unroll 1
         for (uint32_t m = T.str[ij.y]; m; m &= m - 1u) v += dsum[ij.x * C::n + __ffs((int)m) - 1];
         diag[e] = v;
-        if (v < best) {
-            best = v;
+        const long long u = ordered(v);
+        if (u < best) {
+            best = u;
             st.g = e;
         }
-        if (ij.x != ij.y && v < best_o) {
-            best_o = v;
+        if (ij.x != ij.y && u < best_o) {
+            best_o = u;
             st.go = e;
         }
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {  // the lowest element, ties to the lowest index
-        double ov = __shfl_xor_sync(FULL, best, o);
+        long long ov = __shfl_xor_sync(FULL, best, o);
         int oi = __shfl_xor_sync(FULL, st.g, o);
         if (ov < best || (ov == best && oi < st.g)) {
             best = ov;
@@ -856,7 +865,7 @@ __global__ void __launch_bounds__(SECTOR_WARPS * 32, C::DH > 4 ? 3 : 4) k_sector
         double *Vp = W.Vp, *Hsp = (double *)W.Hsf;
         const SectorStart st =
             sector_setup<C>(a, T, W.A, Vp, Hsp, W.hd, W.s.su.h, W.c.dsum, W.s.su.diag);
-        double vmax = 0.0;
+        int vmax = 0;
 #pragma unroll 1
         for (int e = lane; e < C::PT; e += 32) {
             const uchar2 xy = T.ptri[e];
@@ -869,7 +878,7 @@ __global__ void __launch_bounds__(SECTOR_WARPS * 32, C::DH > 4 ? 3 : 4) k_sector
             s = W.Vs + xy.x * VR + 2 * xy.y;
             s[0] = f;
             s[1] = -f;
-            vmax = fmax(vmax, fabs(v));
+            vmax = max(vmax, high_word(v));
         }
 #pragma unroll 1
         for (int e = lane; e < C::NH; e += 32) {
@@ -878,7 +887,7 @@ __global__ void __launch_bounds__(SECTOR_WARPS * 32, C::DH > 4 ? 3 : 4) k_sector
             float *hs = (float *)W.Hs2;
             hs[((ij.x >> 1) * C::NSP + ij.y) * 2 + (ij.x & 1)] = (float)v;
             hs[((ij.y >> 1) * C::NSP + ij.x) * 2 + (ij.y & 1)] = (float)v;
-            if (ij.x != ij.y) vmax = fmax(vmax, fabs(v));
+            if (ij.x != ij.y) vmax = max(vmax, high_word(v));
             W.dg[e] = (float)W.s.su.diag[e];
         }
         for (int p = lane; p < C::P; p += 32) W.Vs[p * (2 * C::P + 1) + 2 * C::P] = 0.f;

@@ -430,25 +430,27 @@ __global__ void __launch_bounds__(SECTOR_WARPS * 32, C::DH > 4 ? 2 : 3) k_sector
         __syncwarp();
         double *Vp = W.m.s.u.su.Vp, *Hsp = W.m.s.u.su.Hsp;
         const SectorStart st = sector_setup<C>(a, T, W.A, Vp, Hsp, W.hd, W.m.s.u.su.h, W.m.s.u.su.dsum, W.dg);
-        double vmax = 0.0;
+        int vmax = 0;
         bool bad = false;
 #pragma unroll 1
         for (int e = lane; e < C::PT; e += 32) {
-            vmax = fmax(vmax, 0.5 * fabs(Vp[e]));
-            bad = bad || !isfinite(Vp[e]);
+            const int hi = high_word(Vp[e]);
+            vmax = max(vmax, hi - 0x00100000);  // (of 1/2 V)
+            bad = bad || hi >= 0x7ff00000;
         }
 #pragma unroll 1
         for (int e = lane; e < C::NH; e += 32) {
             const uchar2 ij = T.tri[e];
-            if (ij.x != ij.y) vmax = fmax(vmax, fabs(Hsp[e]));
-            bad = bad || !isfinite(Hsp[e]);
+            const int hi = high_word(Hsp[e]);
+            if (ij.x != ij.y) vmax = max(vmax, hi);
+            bad = bad || hi >= 0x7ff00000;
         }
         const int E = fixed_exponent(vmax);
         const double scale = pow2(55 - E);
 #pragma unroll 1
         for (int e = lane; e < C::PT; e += 32) {
             const uchar2 xy = T.ptri[e];
-            W.m.s.Vf[xy.x * C::P + xy.y] = W.m.s.Vf[xy.y * C::P + xy.x] = to_fixed(0.5 * Vp[e], scale);
+            W.m.s.Vf[xy.x * C::P + xy.y] = W.m.s.Vf[xy.y * C::P + xy.x] = to_fixed(Vp[e], 0.5 * scale);
         }
 #pragma unroll 1
         for (int e = lane; e < C::NH; e += 32) {
