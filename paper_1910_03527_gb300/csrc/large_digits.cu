@@ -22,8 +22,8 @@
 // Same-spin terms: Hs (symmetric, its diagonal kept out and added in float64: it would set the
 // scale) and c as dense matrices of digits.
 //
-// casci_sigma_large in float64, with its set-up: 12 orbitals 5.6 -> 1.4 ms, 13 orbitals 18.0 -> 5.2,
-// 14 orbitals 88 -> 34, 10 orbitals 1.37 -> 0.24; largest error against 64-bit sums at 12 orbitals
+// casci_sigma_large in float64, with its set-up: 12 orbitals 5.6 -> 1.3 ms, 13 orbitals 18.0 -> 4.8,
+// 14 orbitals 88 -> 30, 10 orbitals 1.37 -> 0.24; largest error against 64-bit sums at 12 orbitals
 // 5.6e-16 of the largest element, 6.0e-16 before.
 #include <algorithm>
 
@@ -165,6 +165,12 @@ __global__ void __launch_bounds__(DG_THREADS, 1) k_large_ab_digits(DigitsArgs a)
             const uint16_t *buf = B + (ch & 1) * DIGITS * bplane;
             for (int t = warp; t < S.mt * (DG_CHUNK / 8); t += DG_THREADS / 32) {
                 const int mt = t / (DG_CHUNK / 8), nt = t - mt * (DG_CHUNK / 8);
+                int to[4];  // where the tile's elements go (asked for before the product)
+#pragma unroll
+                for (int e = 0; e < 4; ++e) {
+                    const int p = mt * 16 + (lane >> 2) + (e >> 1) * 8, J = ch * DG_CHUNK + nt * 8 + (lane & 3) * 2 + (e & 1);
+                    to[e] = p < P && J < Ns ? a.inv[(size_t)p * a.nsp + J] : -1;
+                }
                 float acc[DIGITS][4];
 #pragma unroll
                 for (int d = 0; d < DIGITS; ++d) acc[d][0] = acc[d][1] = acc[d][2] = acc[d][3] = 0.f;
@@ -175,24 +181,22 @@ __global__ void __launch_bounds__(DG_THREADS, 1) k_large_ab_digits(DigitsArgs a)
                     uint32_t bf[DIGITS][2];
 #pragma unroll
                     for (int j = 0; j < DIGITS; ++j) ldsm_x2_trans(bf[j], ba + 2 * (j * bplane + k * DG_BS));
+                    uint32_t af[2][4];
+                    ldsm_x4(af[0], aa + 2 * k);
 #pragma unroll
                     for (int i = 0; i < DIGITS; ++i) {
-                        uint32_t af[4];
-                        ldsm_x4(af, aa + 2 * (i * aplane + k));
+                        if (i + 1 < DIGITS) ldsm_x4(af[(i + 1) & 1], aa + 2 * ((i + 1) * aplane + k));
 #pragma unroll
-                        for (int j = 0; i + j < DIGITS; ++j) mma_bf16(acc[i + j], af, bf[j][0], bf[j][1]);
+                        for (int j = 0; i + j < DIGITS; ++j) mma_bf16(acc[i + j], af[i & 1], bf[j][0], bf[j][1]);
                     }
                 }
                 // scatter
 #pragma unroll
                 for (int e = 0; e < 4; ++e) {
-                    const int p = mt * 16 + (lane >> 2) + (e >> 1) * 8, J = ch * DG_CHUNK + nt * 8 + (lane & 3) * 2 + (e & 1);
-                    if (p >= P || J >= Ns) continue;
-                    const int to = a.inv[(size_t)p * a.nsp + J];
-                    if (to < 0) continue;
+                    if (to[e] < 0) continue;
                     long long s = join_digits(acc, e);
-                    if (to & 1) s = -s;
-                    int *r = row + (to >> 1);
+                    if (to[e] & 1) s = -s;
+                    int *r = row + (to[e] >> 1);
                     atomicAdd(r, (int)(s & 0x1fffff));
                     atomicAdd(r + Ns, (int)(s >> 21 & 0x1fffff));
                     atomicAdd(r + 2 * Ns, (int)(s >> 42));
@@ -278,14 +282,15 @@ __global__ void __launch_bounds__(GM_THREADS, 2) k_large_ss_digits(DigitsArgs a)
                 uint32_t bf[DIGITS][4];
 #pragma unroll
                 for (int j = 0; j < DIGITS; ++j) ldsm_x4_trans(bf[j], ba + 2 * (j * GM_K + k) * GM_S);
+                uint32_t af[2][4];
+                ldsm_x4(af[0], aa + 2 * k);
 #pragma unroll
                 for (int i = 0; i < DIGITS; ++i) {
-                    uint32_t af[4];
-                    ldsm_x4(af, aa + 2 * (i * GM_M * GM_S + k));
+                    if (i + 1 < DIGITS) ldsm_x4(af[(i + 1) & 1], aa + 2 * ((i + 1) * GM_M * GM_S + k));
 #pragma unroll
                     for (int j = 0; i + j < DIGITS; ++j) {
-                        mma_bf16(acc[0][i + j], af, bf[j][0], bf[j][1]);
-                        mma_bf16(acc[1][i + j], af, bf[j][2], bf[j][3]);
+                        mma_bf16(acc[0][i + j], af[i & 1], bf[j][0], bf[j][1]);
+                        mma_bf16(acc[1][i + j], af[i & 1], bf[j][2], bf[j][3]);
                     }
                 }
             }
