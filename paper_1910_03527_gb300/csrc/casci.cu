@@ -438,7 +438,7 @@ __global__ void __launch_bounds__(CTA_THREADS)
 {
     extern __shared__ __align__(16) char smem[];
     const int n = a.n, P = n * (n + 1) / 2;
-    const BlockSmem S = block_smem(n);
+    const SetupSmem S = setup_smem(n);
     int *A = (int *)(smem + S.off_A);
     if (threadIdx.x == 0) build_A(a, 0, A);
     __syncthreads();
@@ -539,11 +539,11 @@ extern "C" int casci_sigma(mbe_ctx *ctx, int norb, const double *h1, const doubl
     a.F = F;
     a.n_tuples = 1;
     k_core_fock<<<(norb * norb + 127) / 128, 128, 0, ctx->stream>>>(norb, h1, eri, occ, F);
-    BlockSmem S = block_smem(n_cas);
-    MBE_CU(cudaFuncSetAttribute(k_sigma_setup, cudaFuncAttributeMaxDynamicSharedMemorySize, S.bytes));
+    SetupSmem S = setup_smem(n_cas);
+    MBE_CU(allow_smem(k_sigma_setup, ctx->smem_optin));
     k_sigma_setup<<<1, CTA_THREADS, S.bytes, ctx->stream>>>(a, ci, V, Hs, dg);
     size_t smem = (size_t)P * P * 8;
-    MBE_CU(cudaFuncSetAttribute(k_sigma_apply, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    MBE_CU(allow_smem(k_sigma_apply, ctx->smem_optin));
     int64_t blocks = (N + CTA_THREADS - 1) / CTA_THREADS;
     int grid = (int)std::min<int64_t>(blocks, (int64_t)ctx->sm_count * 8);
     k_sigma_apply<<<grid, CTA_THREADS, smem, ctx->stream>>>(n_cas, ci, V, Hs, c, sigma);
@@ -638,19 +638,13 @@ extern "C" int casci_sigma_noalloc(int device, void *cuda_stream, int norb, cons
         ClassInfo ci{strings, table, (int)ns, r};
         k_string_table<<<(unsigned)((ns + 127) / 128), 128, 0, st>>>(n_cas, n_el, ns, r, strings, table);
         k_core_fock<<<(norb * norb + 127) / 128, 128, 0, st>>>(norb, h1, eri, occ, F);
-        BlockSmem S = block_smem(n_cas);
-        cudaError_t e = cudaFuncSetAttribute(k_sigma_setup, cudaFuncAttributeMaxDynamicSharedMemorySize, S.bytes);
-        if (e == cudaSuccess) {
-            k_sigma_setup<<<1, CTA_THREADS, S.bytes, st>>>(a, ci, V, Hs, dg);
-            int smem = P * P * 8;
-            e = cudaFuncSetAttribute(k_sigma_apply, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-        }
-        if (e == cudaSuccess) {
-            int64_t blocks = (N + CTA_THREADS - 1) / CTA_THREADS;
-            int grid = (int)std::min<int64_t>(blocks, 4096);
-            k_sigma_apply<<<grid, CTA_THREADS, P * P * 8, st>>>(n_cas, ci, V, Hs, c, sigma);
-            e = cudaGetLastError();
-        }
+        SetupSmem S = setup_smem(n_cas);
+        // (up to 10 orbitals both kernels stay below the 48 KB that need no attribute)
+        k_sigma_setup<<<1, CTA_THREADS, S.bytes, st>>>(a, ci, V, Hs, dg);
+        int64_t blocks = (N + CTA_THREADS - 1) / CTA_THREADS;
+        int grid = (int)std::min<int64_t>(blocks, 4096);
+        k_sigma_apply<<<grid, CTA_THREADS, P * P * 8, st>>>(n_cas, ci, V, Hs, c, sigma);
+        cudaError_t e = cudaGetLastError();
         if (e != cudaSuccess) rc = cuda_fail(e, "casci_sigma_noalloc launch", __FILE__, __LINE__);
     }
     if (prev != device) cudaSetDevice(prev);

@@ -612,11 +612,10 @@ __device__ inline void entry_orbitals(const Problem &pb, uint32_t s, int32_t e, 
 
 // Accumulates, for the unit vector c of the (k, k) sector, the spin-free
 //   g1[p n + q]           += <c| E_pq |c>
-//   g2[((p n + q) n + r) n + s] += <c| E_pq E_rs |c>        (g2 may be NULL)
-// with E = E^alpha + E^beta, walking the replacement lists: E_rs |J> = s1 |K>,
-// E_pq |K> = s2 |L> contributes c_L s1 s2 c_J.  Shared- or global-memory atomics.
+// with E = E^alpha + E^beta, walking the replacement lists.  Shared-memory atomics.  (Two-body
+// density matrices: sector_rdm and block_rdm.)
 template <class G>
-__device__ void rdm_accumulate(const Problem &pb, const double *c, double *g1, double *g2)
+__device__ void rdm_accumulate(const Problem &pb, const double *c, double *g1)
 {
     const int tid = G::rank(), nt = G::size();
     const int n = pb.n, Ns = pb.Ns, R = pb.R, RS = pb.RS;
@@ -632,48 +631,12 @@ __device__ void rdm_accumulate(const Problem &pb, const double *c, double *g1, d
             int p, q;
             entry_orbitals(pb, sa, e, p, q);
             atomicAdd(&g1[p * n + q], flip_if(c[ka * Ns + jb], entry_neg(e)) * cd);
-            if (!g2) continue;
-            const double s1cd = flip_if(cd, entry_neg(e));
-            const uint32_t ska = pb.str[ka];
-            const int32_t *tka = pb.tab + ka * RS;
-            for (int x2 = 0; x2 < R; ++x2) {
-                const int e2 = tka[x2];
-                int p2, q2;
-                entry_orbitals(pb, ska, e2, p2, q2);
-                atomicAdd(&g2[((p2 * n + q2) * n + p) * n + q],
-                          flip_if(c[entry_J(e2) * Ns + jb], entry_neg(e2)) * s1cd);
-            }
-            for (int y2 = 0; y2 < R; ++y2) {
-                const int e2 = tb[y2];
-                int p2, q2;
-                entry_orbitals(pb, sb, e2, p2, q2);
-                atomicAdd(&g2[((p2 * n + q2) * n + p) * n + q],
-                          flip_if(c[ka * Ns + entry_J(e2)], entry_neg(e2)) * s1cd);
-            }
         }
         for (int y = 0; y < R; ++y) {  // first operator on the beta string
             const int e = tb[y], kb = entry_J(e);
             int p, q;
             entry_orbitals(pb, sb, e, p, q);
             atomicAdd(&g1[p * n + q], flip_if(c[ja * Ns + kb], entry_neg(e)) * cd);
-            if (!g2) continue;
-            const double s1cd = flip_if(cd, entry_neg(e));
-            const uint32_t skb = pb.str[kb];
-            const int32_t *tkb = pb.tab + kb * RS;
-            for (int x2 = 0; x2 < R; ++x2) {
-                const int e2 = ta[x2];
-                int p2, q2;
-                entry_orbitals(pb, sa, e2, p2, q2);
-                atomicAdd(&g2[((p2 * n + q2) * n + p) * n + q],
-                          flip_if(c[entry_J(e2) * Ns + kb], entry_neg(e2)) * s1cd);
-            }
-            for (int y2 = 0; y2 < R; ++y2) {
-                const int e2 = tkb[y2];
-                int p2, q2;
-                entry_orbitals(pb, skb, e2, p2, q2);
-                atomicAdd(&g2[((p2 * n + q2) * n + p) * n + q],
-                          flip_if(c[ja * Ns + entry_J(e2)], entry_neg(e2)) * s1cd);
-            }
         }
     }
 }
@@ -712,9 +675,9 @@ __device__ inline void rdm_two_body(const BatchArgs &a, const int *A, int n, int
 }
 
 // Adds w * (dE_CAS(A)/dtheta - dE_Phi/dtheta) to the gradients from the active
-// density matrices accumulated by rdm_accumulate (Gamma = <E_pq E_rs> - d_qr gamma_ps).
+// one-body density matrix accumulated by rdm_accumulate.
 template <class G>
-__device__ void rdm_flush(const BatchArgs &a, const Problem &pb, const double *g1, const double *g2, double w)
+__device__ void rdm_flush(const BatchArgs &a, const Problem &pb, const double *g1, double w)
 {
     const int tid = G::rank(), nt = G::size();
     const int n = pb.n, norb = a.norb;
@@ -722,17 +685,6 @@ __device__ void rdm_flush(const BatchArgs &a, const Problem &pb, const double *g
     for (int e = tid; e < n * n; e += nt) {
         const int p = e / n, q = e - p * n;
         rdm_one_body(a, A, n, p, q, w * (g1[e] - ((p == q && a.occ[A[p]]) ? 2.0 : 0.0)));
-    }
-    if (!g2) return;
-    for (int e = tid; e < n * n * n * n; e += nt) {
-        const int s = e % n, r = (e / n) % n, q = (e / (n * n)) % n, p = e / (n * n * n);
-        double Gv = g2[e] - (q == r ? g1[p * n + s] : 0.0);
-        const bool op = a.occ[A[p]], oq = a.occ[A[q]], orr = a.occ[A[r]];
-        double phi = 0.0;
-        if (p == q && r == s && op && orr) phi += (p == r) ? 2.0 : 4.0;
-        if (p == s && q == r && p != q && op && oq) phi -= 2.0;
-        const double v = 0.5 * w * (Gv - phi);
-        if (v != 0.0) atomicAdd(&a.grad_eri[eri_index(norb, A[p], A[q], A[r], A[s])], v);
     }
 }
 
@@ -1345,9 +1297,9 @@ __global__ void __launch_bounds__(WARPS_PER_BLOCK * 32)
                 }
                 for (int e = lane; e < n * n; e += 32) g1[e] = 0.0;
                 __syncwarp();
-                rdm_accumulate<WarpGroup>(pb, cv, g1, nullptr);
+                rdm_accumulate<WarpGroup>(pb, cv, g1);
                 __syncwarp();
-                rdm_flush<WarpGroup>(a, pb, g1, nullptr, a.weights ? a.weights[t] : 1.0);
+                rdm_flush<WarpGroup>(a, pb, g1, a.weights ? a.weights[t] : 1.0);
                 __syncwarp();
             }
         }
@@ -1812,14 +1764,13 @@ constexpr int BLOCK_STALL = 3;
 constexpr int BLOCK_ANCHOR_STALL = 25;
 constexpr int BLOCK_ANCHORS = 8;
 
-struct BlockSmem {  // dynamic shared memory of the block solver
-    int off_A, off_pp, off_h, off_hp, off_V64, off_V32, off_red, off_G, off_A32, off_E32, off_ev, off_y,
-        off_yp, off_r, off_misc, off_g1, off_g2, bytes;
+struct SetupSmem {  // dynamic shared memory of casci_sigma's set-up
+    int off_A, off_pp, off_h, off_hp, off_V64, off_V32, bytes;
 };
 
-__host__ __device__ inline BlockSmem block_smem(int n, bool two_body = false)
+__host__ __device__ inline SetupSmem setup_smem(int n)
 {
-    BlockSmem S;
+    SetupSmem S;
     int P = n * (n + 1) / 2, o = 0;
     S.off_A = o; o = al16(o + 4 * MBE_MAX_CAS);
     S.off_pp = o; o = al16(o + 4 * P);
@@ -1827,149 +1778,8 @@ __host__ __device__ inline BlockSmem block_smem(int n, bool two_body = false)
     S.off_hp = o; o = al16(o + 8 * P);
     S.off_V64 = o; o = al16(o + 8 * P * P);
     S.off_V32 = o; o = al16(o + 4 * P * P);
-    S.off_red = o; o = al16(o + 8 * 32 * KRED);
-    S.off_G = o; o = al16(o + 8 * MMAX * MMAX);
-    S.off_A32 = o; o = al16(o + 4 * MMAX * MMAX);
-    S.off_E32 = o; o = al16(o + 4 * MMAX * MMAX);
-    S.off_ev = o; o = al16(o + 4 * MMAX);
-    S.off_y = o; o = al16(o + 8 * MMAX);
-    S.off_yp = o; o = al16(o + 8 * MMAX);
-    S.off_r = o; o = al16(o + 8 * MMAX);
-    S.off_misc = o; o = al16(o + 8 * 4);
-    S.off_g1 = o; o = al16(o + 8 * n * n);
-    S.off_g2 = o; o = al16(o + (two_body ? 8 * n * n * n * n : 0));
     S.bytes = o;
     return S;
-}
-
-// Lowest eigenpair of the m x m symmetric Rayleigh matrix G (shared memory,
-// float64, row stride MMAX), computed by one warp: a float32 cyclic Jacobi on
-// G - G00 I gives all eigenpairs; in the float64 phase two Newton steps in that
-// eigenbasis,  z = y - sum_{k != 0} e_k (e_k . r) / (theta_k - theta),
-// r = G y - theta y,  theta = y.G y, make the lowest pair float64-accurate.
-// Output: y[0..m) (shared, float64, unit norm) and misc[0] = theta.
-template <bool REFINE>
-__device__ void small_eig_warp(const double *G, int m, float *A, float *E, float *ev, double *y, double *y2,
-                               double *r, double *misc)
-{
-    const int lane = threadIdx.x & 31;
-    const double shift = G[0];
-    for (int e = lane; e < m * m; e += 32) {
-        int i = e / m, j = e - i * m;
-        A[i * MMAX + j] = (float)(G[i * MMAX + j] - (i == j ? shift : 0.0));
-        E[i * MMAX + j] = (i == j) ? 1.0f : 0.0f;
-    }
-    __syncwarp();
-    for (int sweep = 0; sweep < 10; ++sweep) {
-        float off = 0.0f, dia = 0.0f;
-        if (lane < m)
-            for (int j = 0; j < m; ++j) {
-                float v = A[lane * MMAX + j];
-                if (j == lane) dia += v * v; else off += v * v;
-            }
-        off = warp_sum(off);
-        dia = warp_sum(dia);
-        if (off <= 1e-14f * dia || off < 1e-36f) break;
-        for (int p = 0; p < m - 1; ++p)
-            for (int q = p + 1; q < m; ++q) {
-                float apq = A[p * MMAX + q];
-                if (fabsf(apq) < 1e-36f) continue;
-                float app = A[p * MMAX + p], aqq = A[q * MMAX + q];
-                float th = (aqq - app) / (2.0f * apq);
-                float t = 1.0f / (fabsf(th) + sqrtf(th * th + 1.0f));
-                if (th < 0.0f) t = -t;
-                float c = rsqrtf(t * t + 1.0f), s = t * c;
-                float ajp = 0.f, ajq = 0.f, ejp = 0.f, ejq = 0.f;
-                if (lane < m) {
-                    ajp = A[lane * MMAX + p];
-                    ajq = A[lane * MMAX + q];
-                    ejp = E[lane * MMAX + p];
-                    ejq = E[lane * MMAX + q];
-                }
-                __syncwarp();
-                if (lane < m) {
-                    if (lane != p && lane != q) {
-                        float np_ = c * ajp - s * ajq, nq = s * ajp + c * ajq;
-                        A[lane * MMAX + p] = np_;
-                        A[p * MMAX + lane] = np_;
-                        A[lane * MMAX + q] = nq;
-                        A[q * MMAX + lane] = nq;
-                    } else if (lane == p) {
-                        A[p * MMAX + p] = app - t * apq;
-                        A[p * MMAX + q] = 0.0f;
-                        A[q * MMAX + p] = 0.0f;
-                    } else {
-                        A[q * MMAX + q] = aqq + t * apq;
-                    }
-                    E[lane * MMAX + p] = c * ejp - s * ejq;
-                    E[lane * MMAX + q] = s * ejp + c * ejq;
-                }
-                __syncwarp();
-            }
-    }
-    float best = (lane < m) ? A[lane * MMAX + lane] : 3.0e38f;
-    int bi = lane;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        float ov = __shfl_xor_sync(FULL, best, o);
-        int oi = __shfl_xor_sync(FULL, bi, o);
-        if (ov < best || (ov == best && oi < bi)) {
-            best = ov;
-            bi = oi;
-        }
-    }
-    // second-lowest eigenvalue (its eigenvector seeds the thick restart)
-    float best2 = (lane < m && lane != bi) ? A[lane * MMAX + lane] : 3.0e38f;
-    int b2 = (lane < m && lane != bi) ? lane : 0x7fffffff;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        float ov = __shfl_xor_sync(FULL, best2, o);
-        int oi = __shfl_xor_sync(FULL, b2, o);
-        if (ov < best2 || (ov == best2 && oi < b2)) {
-            best2 = ov;
-            b2 = oi;
-        }
-    }
-    if (lane < m) {
-        ev[lane] = A[lane * MMAX + lane];
-        y[lane] = (double)E[lane * MMAX + bi];
-        y2[lane] = (b2 < m) ? (double)E[lane * MMAX + b2] : 0.0;
-    }
-    __syncwarp();
-    double theta = shift + (double)best;
-    if (REFINE) {
-        for (int step = 0; step < 2; ++step) {
-            double g = 0.0, yi = (lane < m) ? y[lane] : 0.0;
-            if (lane < m)
-                for (int j = 0; j < m; ++j) g += G[lane * MMAX + j] * y[j];
-            double yy = warp_sum(yi * yi), ygy = warp_sum(yi * g);
-            theta = ygy / yy;
-            if (lane < m) r[lane] = g - theta * yi;
-            __syncwarp();
-            // coefficient of eigenvector k (lane k)
-            double ck = 0.0;
-            if (lane < m && lane != bi) {
-                for (int i = 0; i < m; ++i) ck += (double)E[i * MMAX + lane] * r[i];
-                double den = shift + (double)ev[lane] - theta;
-                ck = (fabs(den) > 1e-300) ? ck / den : 0.0;
-            }
-            __syncwarp();
-            if (lane < m) r[lane] = ck;  // reuse r for the coefficients
-            __syncwarp();
-            double z = yi;
-            if (lane < m)
-                for (int k = 0; k < m; ++k) z -= (double)E[lane * MMAX + k] * r[k];
-            double zz = warp_sum(z * z);
-            if (lane < m) y[lane] = z / sqrt(zz);
-            __syncwarp();
-        }
-        double g = 0.0, yi = (lane < m) ? y[lane] : 0.0;
-        if (lane < m)
-            for (int j = 0; j < m; ++j) g += G[lane * MMAX + j] * y[j];
-        theta = warp_sum(yi * g);
-    }
-    if (lane == 0) misc[0] = theta;
-    __syncwarp();
 }
 
 // Optional event pair around one solver launch (mbe_ctx_set_timing).
