@@ -9,13 +9,16 @@
 // sigma up to 9 orbitals (at most 126 strings): the whole coefficient matrix c sits in shared
 // memory, and per alpha string Ia the opposite-spin term is a dense product and a gather,
 //     T[p][J] = sum_x s_x V[p_x][p] c[J_x][J],   sigma[Ia][Ib] = sum_y s_y T[p_y][J_y].
-// The product is register-tiled (4 strings x 6 pairs per thread in float32: one 16-byte and
-// three 8-byte shared loads for 24 multiply-adds), where the double loop over both lists
-// gathers three values for every multiply-add; it does 2 P / R = 3.6 times more of them at
-// 9 orbitals, but near the rate of the pipe.  In float64 the same product runs on integers
-// (55-bit fixed point in two limbs, three wide integer multiply-adds per term, exact sums:
-// see casci_sector64.cuh), because a float64 multiply-add costs 36 integer ones here.
-// Beyond 9 orbitals c does not fit, and sigma walks both lists per element.
+// The product is register-tiled in float32 (8 strings x 6 pairs per thread, see gemm_tile), where the
+// double loop over both lists gathers three values for every multiply-add; it does 2 P / R = 3.6
+// times more of them at 9 orbitals, but near the rate of the pipe.  In float64, where a
+// multiply-add costs 74 float32 ones, the product is one of exact digits on the tensor cores
+// (sigma_digits), or, where those do not fit in shared memory, of 55-bit fixed-point numbers in
+// two limbs (three wide integer multiply-adds per term).  Cycles per phase of an iteration, before
+// and after each step: the float32 product 595 -> 390 thousand at 9 orbitals, the float64 one
+// 782 -> 317 thousand at 8.
+// From 10 orbitals with at most 128 strings, c and V in shared memory and sorted lists (sigma_list);
+// beyond, c does not fit, and sigma walks both lists per element.
 #include "casci_sector.cuh"
 #include "digits.cuh"
 

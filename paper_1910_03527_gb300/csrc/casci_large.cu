@@ -2,27 +2,23 @@
 //
 // One CASCI over a large active space (up to 16 orbitals, 165.6M determinants
 // at (16e,16o)), spread over the whole GPU:
-//   * set-up: h_eff, packed V, h' (one block); the one-spin Hamiltonian Hs built
-//     column-parallel over the grid as a dense Ns x Ns matrix, then compressed to
-//     CSR (each row holds the strings connected by at most a double replacement);
-//   * sigma = (Hs x 1) c + (1 x Hs) c + opposite-spin term.  The same-spin terms
-//     are row-streamed sparse products C' = Hs C (coalesced over the second
-//     index), the beta one applied to the transposed coefficient matrix and added
-//     back transposed.  The opposite-spin term is, in float64, the direct double
-//     loop over the alpha and beta replacement lists (one thread per determinant,
-//     V in shared memory); in float32 it is, per alpha string, a dense product of
-//     the signed V columns with the gathered rows of C followed by a scatter
-//     through the beta lists into a shared-memory sigma row;
+//   * set-up: h_eff, packed V (one block); the one-spin Hamiltonian Hs by the Slater-Condon
+//     rules over the grid as a dense Ns x Ns matrix, then compressed to CSR (each row holds
+//     the strings connected by at most a double replacement);
+//   * sigma = (Hs x 1) c + (1 x Hs) c + opposite-spin term.  In float64 up to 14 orbitals all of
+//     it is products of exact digits on the tensor cores (large_digits.cu); above, the direct
+//     double loop over the alpha and beta replacement lists (one thread per determinant, V in
+//     shared memory) and row-streamed sparse products C' = Hs C, the beta one applied to the
+//     transposed coefficient matrix and added back transposed.  In float32 the opposite-spin
+//     term is, per alpha string, a dense product on the tensor cores followed by a scatter
+//     (large_tc.cu), and the sparse products take slabs of c from shared memory;
 //   * inside the Davidson every vector lies in one spin-flip sector,
-//     c[Ia][Ib] = sgn c[Ib][Ia], and so does its sigma: the float64 opposite-spin
-//     term is computed for Ia <= Ib and mirrored, and the beta same-spin term is
-//     sgn times the transpose of the alpha one (one sparse product and a
-//     transposing add instead of two products and a transpose of c);
+//     c[Ia][Ib] = sgn c[Ib][Ia], and is kept packed (LargeDav); the beta same-spin term is
+//     sgn times the transpose of the alpha one (one sparse product and a transposing add);
 //   * Davidson: the tuple solvers' algorithm (MLARGE-vector basis, thick restart
 //     on the two lowest Ritz vectors, float32 phase then float64 phase) with its
 //     vector algebra in grid-wide kernels, the projected eigenproblem in one
-//     warp on the device, and the host reading back one residual norm per
-//     iteration to decide convergence.
+//     block, and the host reading back two norms per iteration to decide convergence.
 
 #include "casci_sector.cuh"
 #include "large_digits.cuh"
