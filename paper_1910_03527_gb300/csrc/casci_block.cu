@@ -1738,8 +1738,8 @@ __global__ void __launch_bounds__(BLOCK_THREADS, 1) k_casci_block(BatchArgs a, i
                 if (!lose && finite) {
                     // Anchored refinement (struct Anchor): a float64 sigma of the float64
                     // anchor x0, then the float32 Davidson on H - theta0 with x0 as its
-                    // first basis vector; x0 <- x0 + d after each pass, re-anchoring while
-                    // the residual stays above tol.
+                    // first basis vector; x0 <- (x0 + d) / |x0 + d| after each pass, re-anchoring
+                    // while the residual stays above tol.
                     for (int d = tid; d < pb.N; d += nt) x0[d] = (double)x32[d];
                     __syncthreads();
                     bool done = false, bad = false;
@@ -1769,8 +1769,19 @@ __global__ void __launch_bounds__(BLOCK_THREADS, 1) k_casci_block(BatchArgs a, i
                         lam_s = th + o.lambda;
                         bad = o.status == MBE_STATUS_NONFINITE;
                         done = !bad && o.rnorm <= a.tol && o.dnorm <= MIX_DMAX;
-                        if (!bad)
-                            for (int d = tid; d < pb.N; d += nt) x0[d] = x0[d] * inv + (double)x32[d];
+                        // x0 <- x0 + d as a unit vector: |d| may be anything until a pass is accepted,
+                        // and the fixed-point sigma holds elements of at most 1
+                        if (!bad) {
+                            double nn[1] = {0.0};
+                            for (int d = tid; d < pb.N; d += nt) {
+                                const double v = x0[d] * inv + (double)x32[d];
+                                x0[d] = v;
+                                nn[0] += v * v;
+                            }
+                            block_sums(nn, red);
+                            const double unit = 1.0 / sqrt(nn[0]);
+                            for (int d = tid; d < pb.N; d += nt) x0[d] *= unit;
+                        }
                         __syncthreads();
                     }
                     // the refined vector (or the start of the float64 fallback) as x64
