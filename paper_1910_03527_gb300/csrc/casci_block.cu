@@ -39,7 +39,7 @@ struct BlockProblem {
     int form;         // of sigma
     const float *U;   // SIGMA_LIST: U[I][p] = sum over the orbitals q of string I of V[qq][p]
     bool bad;         // an element of V or Hs is not finite (float64 sigma: fixed point cannot hold it)
-    int E;            // fixed-point exponent
+    int E;            // 2^E: the power of two above the largest element of V and (off-diagonal) Hs
     BlockMem S;
     double *full;     // [Ns][stride] scratch of the slot
 };
@@ -687,6 +687,9 @@ __device__ __noinline__ void sigma_block(const BlockProblem &B, const T *src, T 
 // float64).  In float64 then two Newton steps in that
 // eigenbasis, z = y - sum_{k != 0} e_k (e_k . r) / (theta_k - theta),  r = G y - theta y,
 // theta = y.G y, which make the lowest pair float64-accurate; in float32 one (one warp).
+// All float32 work is on (G - G00 I) 2^-e, e from its largest element, so that neither its squares
+// nor the absolute floors below depend on the unit of the integrals; ev is kept in that unit, e
+// (which may change from call to call) in misc[1].
 // Output: y[0..m) (unit norm), y2 (the second lowest, which seeds the thick restart), and
 // misc[0] = theta; ends with a barrier.
 template <bool REFINE>
@@ -701,6 +704,12 @@ __device__ __noinline__ void small_eig_block(const BlockMem &S, int m, bool warm
     const int tid = threadIdx.x, i = tid / MMAX, j = tid - i * MMAX, lane = tid & 31;
     const bool on = i < m && j < m;
     const double shift = G[0];
+    int top = lane < m ? high_word(G[lane * MMAX + lane] - shift) : 0;  // (in every warp)
+    for (int q = lane; q < m * MMAX; q += 32)
+        if (q % MMAX < q / MMAX) top = max(top, high_word(G[q]));
+    top = __reduce_max_sync(FULL, top);
+    const int e2 = top == 0 ? 0 : max(-1000, min(1000, (top >> 20) - 1023));
+    const double down = pow2(-e2), up = pow2(e2);
     float *A = buf, *E = buf + MMAX * MMAX, *A2 = buf + 2 * MMAX * MMAX, *E2 = buf + 3 * MMAX * MMAX;
     if (warm) {
         // half a warp per pole or root, its lanes share the terms of every sum
@@ -721,14 +730,15 @@ __device__ __noinline__ void small_eig_block(const BlockMem &S, int m, bool warm
         auto gap = [&](int k, int l) { return (sp[k] - sd[l]) + st[k]; };  // root k - pole l
         if (work) {
             float b = 0.f;  // the new row in the last basis
-            for (int k = l0; k < q; k += 16) b += half < q ? E[k * MMAX + half] * (float)G[k * MMAX + q] : 0.f;
+            for (int k = l0; k < q; k += 16) b += half < q ? E[k * MMAX + half] * (float)(G[k * MMAX + q] * down) : 0.f;
             b = sum16(b);
             if (l0 == 0) sb[half] = b;
         }
         __syncthreads();
         // the arrow matrix: diagonal d = ev, row b, corner a
-        const float a = (float)(G[q * MMAX + q] - shift);
-        float b = lane < q ? sb[lane] : 0.f, d = lane < q ? ev[lane] : 0.f;  // (in every warp)
+        const float a = (float)((G[q * MMAX + q] - shift) * down);
+        const float unit = (float)pow2(max(-126, min(126, (int)misc[1] - e2)));  // of the last ev
+        float b = lane < q ? sb[lane] : 0.f, d = lane < q ? ev[lane] * unit : 0.f;  // (in every warp)
         float scale = fmaxf(fabsf(a), fmaxf(fabsf(d), fabsf(b)));
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) scale = fmaxf(scale, __shfl_xor_sync(FULL, scale, o));
@@ -822,7 +832,7 @@ __device__ __noinline__ void small_eig_block(const BlockMem &S, int m, bool warm
     }
     if (!warm) {
         if (on) {
-            A[tid] = (float)(G[i * MMAX + j] - (i == j ? shift : 0.0));
+            A[tid] = (float)((G[i * MMAX + j] - (i == j ? shift : 0.0)) * down);
             E[tid] = i == j ? 1.0f : 0.0f;
         }
         __syncthreads();
@@ -908,14 +918,15 @@ __device__ __noinline__ void small_eig_block(const BlockMem &S, int m, bool warm
             y2[lane] = m > 1 ? (double)E[lane * MMAX + 1] : 0.0;
         }
         __syncwarp();
-        double theta = shift + (double)ev[0];
+        double theta = shift + (double)ev[0] * up;
         __syncwarp();
         if (!REFINE) {
             // one such step in float32, which also takes out what the warm starts have gathered in E
             float row[MMAX];
+            const double own = lane < m ? G[lane * MMAX + lane] - shift : 0.0;
 #pragma unroll
             for (int k = 0; k < MMAX; ++k)
-                row[k] = lane < m && k < m ? (float)(k == lane ? G[k * MMAX + k] - shift : G[lane * MMAX + k]) : 0.f;
+                row[k] = lane < m && k < m ? (float)((k == lane ? own : G[lane * MMAX + k]) * down) : 0.f;
             float yi = lane < m ? E[lane * MMAX + bi] : 0.f;
             float th = 0.f;
 #pragma unroll 1
@@ -935,7 +946,7 @@ __device__ __noinline__ void small_eig_block(const BlockMem &S, int m, bool warm
                 yi = z * rsqrtf(warp_sum(z * z));
             }
             if (lane < m) y[lane] = (double)yi;
-            theta = shift + (double)th;
+            theta = shift + (double)th * up;
         }
         if (REFINE) {
             for (int step = 0; step < 2; ++step) {
@@ -950,7 +961,7 @@ __device__ __noinline__ void small_eig_block(const BlockMem &S, int m, bool warm
                 double ck = 0.0;
                 if (lane < m && lane != bi) {
                     for (int k = 0; k < m; ++k) ck += (double)E[k * MMAX + lane] * r[k];
-                    double den = shift + (double)ev[lane] - theta;
+                    double den = shift + (double)ev[lane] * up - theta;
                     ck = (fabs(den) > 1e-300) ? ck / den : 0.0;
                 }
                 __syncwarp();
@@ -968,7 +979,10 @@ __device__ __noinline__ void small_eig_block(const BlockMem &S, int m, bool warm
                 for (int k = 0; k < m; ++k) g += G[lane * MMAX + k] * y[k];
             theta = warp_sum(yi * g);
         }
-        if (lane == 0) misc[0] = theta;
+        if (lane == 0) {
+            misc[0] = theta;
+            misc[1] = (double)e2;
+        }
     }
     __syncthreads();
 }
@@ -1064,6 +1078,10 @@ __device__ __noinline__ PhaseOut davidson_block(const BlockProblem &B, T *Vp, T 
     o.status = MBE_STATUS_OK;
     o.dnorm = 0.0;
     const T shT = (T)shift, shT_lo = (T)(shift - (double)shT);
+    // float32 residuals are squared in the unit 2^E and the corrections kept near |r| 2^-E (the floor
+    // of the preconditioner's denominator is 1e-4 in any unit): integrals of 1e-18 would underflow
+    const int Ec = sizeof(T) == 8 ? 0 : max(-100, min(100, B.E));
+    const T per_unit = (T)pow2(-Ec), unit = (T)pow2(Ec), lift = (T)pow2(Ec < -13 ? -13 - Ec : 0);
     T v1[1], v2[2];
     auto dot = [&](const K &a, const K &b, T s) {
 #pragma unroll
@@ -1129,17 +1147,17 @@ __device__ __noinline__ PhaseOut davidson_block(const BlockProblem &B, T *Vp, T 
             }
 #pragma unroll
             for (int l = 0; l < VL; ++l) {
-                const T r = hs.e[l] - th * xs.e[l];
-                v2[0] += r * r;
+                const T r = hs.e[l] - th * xs.e[l], ru = r * per_unit;
+                v2[0] += ru * ru;
                 T den = (T)(pb.diag[d * VL + l] - shift) - th;
                 if (fabs(den) < (T)1e-4) den = den >= (T)0 ? (T)1e-4 : (T)-1e-4;
-                td.e[l] = r / den;
+                td.e[l] = r * lift / den;
                 v2[1] += td.e[l] * td.e[l];
             }
             tdst[d] = td;
         }
         block_sums(v2, red);
-        rn = sqrt(v2[0]);
+        rn = sqrt(v2[0]) * unit;
         const T t0n = sqrt(v2[1]);
         if (!isfinite(rn) || !isfinite(theta)) {
             o.status = MBE_STATUS_NONFINITE;
@@ -1457,12 +1475,12 @@ __device__ void block_setup(const BatchArgs &a, BlockProblem &B, const ClassInfo
         }
         if (tid < (4 - pb.N % 4) % 4) pb.diag[pb.N + tid] = 1.0;
     }
-    if (B.form == SIGMA_TILED) {
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) big = fmax(big, __shfl_xor_sync(FULL, big, o));
-        if ((tid & 31) == 0) red[tid >> 5] = big;
-        __syncthreads();
-        B.E = fixed_exponent((tid & 31) < (nt >> 5) ? high_word(red[tid & 31]) : 0);
+    for (int o = 16; o > 0; o >>= 1) big = fmax(big, __shfl_xor_sync(FULL, big, o));
+    if ((tid & 31) == 0) red[tid >> 5] = big;
+    __syncthreads();
+    B.E = fixed_exponent((tid & 31) < (nt >> 5) ? high_word(red[tid & 31]) : 0);
+    if (B.form == SIGMA_TILED) {
         const double scale = pow2(55 - B.E);
         int2 *Vf = (int2 *)pb.V64, *Hf = (int2 *)pb.Hs64;
         for (int e = tid; e < P * P; e += nt) Vf[e] = to_fixed(pb.V64[e], scale);
@@ -1858,7 +1876,7 @@ __global__ void __launch_bounds__(BLOCK_THREADS, 1) k_casci_block(BatchArgs a, i
 
 // small_eig_block on a Rayleigh matrix in global memory (the large-CAS solver's).  col: its new last
 // column, put in first (m values, or NULL).  basis: the eigenbasis and eigenvalues of the
-// last call, read if warm ([MMAX + 1][MMAX]), replaced.
+// last call, read if warm ([MMAX + 1][MMAX], then their unit's exponent), replaced.
 __global__ void __launch_bounds__(416) k_small_eig(double *Gd, int m, const double *col, int warm, BlockMem S, float *basis, double *ys,
                                                    double *y2s, double *misc)
 {
@@ -1872,10 +1890,13 @@ __global__ void __launch_bounds__(416) k_small_eig(double *Gd, int m, const doub
         if (warm) E[tid] = basis[tid];
     }
     if (warm && tid < MMAX) ev[tid] = basis[MMAX * MMAX + tid];
+    double *unit = (double *)(block_shared() + S.off_misc) + 1;
+    if (warm && tid == 0) *unit = (double)basis[(MMAX + 1) * MMAX];
     __syncthreads();
     small_eig_block<true>(S, m, warm);
     if (tid < MMAX * MMAX) basis[tid] = E[tid];
     if (tid < MMAX) basis[MMAX * MMAX + tid] = ev[tid];
+    if (tid == 0) basis[(MMAX + 1) * MMAX] = (float)*unit;
     if (tid < m) {
         ys[tid] = ((double *)(block_shared() + S.off_y))[tid];
         y2s[tid] = ((double *)(block_shared() + S.off_yp))[tid];

@@ -1373,7 +1373,7 @@ extern "C" int casci_solve(mbe_ctx *ctx, int norb, const double *h1, const doubl
     D.full = bump.take<double>((size_t)N);
     D.S = bump.take<double>((size_t)N);
     D.ticket = bump.take<unsigned>(1);
-    D.basis = bump.take<float>((MMAX + 1) * MMAX);
+    D.basis = bump.take<float>((MMAX + 1) * MMAX + 1);
     D.partial = bump.take<double>((size_t)D.nblk * LRED);
     D.dots = bump.take<double>(32);
     D.Gd = bump.take<double>(MMAX * MMAX);
