@@ -409,7 +409,12 @@ int mbe_phi_gradient(mbe_ctx *ctx, int norb, const uint8_t *occ, double scale, d
  * determinants), spread over the whole GPU.  Same operator, determinant order
  * and layouts as casci_sigma; the same-spin part uses a compressed (CSR) copy
  * of the one-spin Hamiltonian.
- *   precision   MBE_PREC_FP64: float64 arithmetic; MBE_PREC_MIXED: float32
+ *   precision   MBE_PREC_FP64: float64 accuracy element by element: float64
+ *               arithmetic, or, up to 14 orbitals and where the elements of c and of
+ *               the integrals are even enough for it to be no less accurate, sums of
+ *               exact products of 8-bit digits on the tensor cores, whose error is
+ *               below 2^-52 (R^2 max|V| + 2 C max|Hs|) max|c| (R replacements of a
+ *               string, C strings that Hs connects); MBE_PREC_MIXED: float32
  *               arithmetic on a float32 copy of c (result written as float64), the
  *               opposite-spin product on the tensor cores (tcgen05, TF32 split into
  *               hi + lo pairs, hi*hi + hi*lo + lo*hi accumulated in float32)

@@ -842,11 +842,13 @@ static int large_setup(mbe_ctx *ctx, int norb, const double *h1, const double *e
         g.Ns = L.Ns;
         g.R = L.R;
         g.nsp = (L.Ns + 63) / 64 * 64;
+        g.n = 0;
         g.tab = L.tab;
+        g.tabT = L.tabT;
         g.V = L.V;
         g.hd = hd = bump.take<double>((size_t)L.Ns);
         g.inv = bump.take<int32_t>((size_t)P * g.nsp);
-        g.maxb = bump.take<unsigned long long>(3);
+        g.maxb = bump.take<unsigned long long>(4);
         g.planes = bump.take<uint16_t>((size_t)DIGITS * L.Ns * g.nsp);
         g.hplanes = bump.take<uint16_t>((size_t)DIGITS * L.Ns * g.nsp);
     }
@@ -957,8 +959,8 @@ static int large_sigma_launch(mbe_ctx *ctx, const LargePlan &pl, const T *c, dou
             g.sigma = sigma;
             const int rc = large_sigma_digits(ctx->stream, ctx->sm_count, ctx->smem_optin, g, pl.dg_chunk);
             if (rc) return rc;
-            ctx->launches += 4;
-            digits = pl.dg.maxb;  // the kernels below return at once, unless the scales are extreme
+            ctx->launches += g.n ? 6 : 4;
+            digits = pl.dg.maxb;  // the kernels below return at once, unless digits_usable() says no
         }
         if (sgn == 0)
             k_large_ab64<false><<<pl.grid_ab64, SIGMA_THREADS, pl.smem_ab64, ctx->stream>>>(pl.L, (const double *)c,
@@ -1045,7 +1047,10 @@ extern "C" int casci_sigma_large(mbe_ctx *ctx, int norb, const double *h1, const
     rc = large_setup(ctx, norb, h1, eri, occ, n_cas, cas_orbs, bump, nullptr, fp32, &pl, &k, &dphi);
     if (rc) return rc;
     if (diag) MBE_CU(cudaMemcpyAsync(diag, pl.L.diag, N * 8, cudaMemcpyDeviceToDevice, ctx->stream));
-    if (precision == MBE_PREC_FP64) return large_sigma_launch<double>(ctx, pl, c, sigma, n_cas);
+    if (precision == MBE_PREC_FP64) {
+        pl.dg.n = n_cas;  // (a caller's vector may have any spread; inside the eigensolver the norm of the error counts)
+        return large_sigma_launch<double>(ctx, pl, c, sigma, n_cas);
+    }
     float *c32 = bump.take<float>((size_t)N);
     k_to_float<<<pl.grid_vec, 256, 0, ctx->stream>>>(c, N, c32);
     ++ctx->launches;

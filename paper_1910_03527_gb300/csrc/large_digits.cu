@@ -9,22 +9,25 @@
 // and c as fixed-point numbers of 55 bits and sign below their largest elements, in seven signed
 // digits of base 256, each exact in bfloat16.  The products of digits i of one and j of the other
 // operand with the same i + j = d add up in one float32 accumulator, exactly (at most 1,023 of
-// them, each at most 2^14); the pairs with i + j > 6, below 2^-54 of the largest term, are left
-// out: 28 products of mma.sync.m16n8k16, 32 exact multiply-adds per clock and SM.  The seven
-// sums of an element are joined in a 64-bit integer and rounded to 2^-54 of the largest term.
+// them, each at most 2^14); the pairs with i + j > 7, below 2^-61 of the largest term, are left
+// out: 34 products of mma.sync.m16n8k16.  The eight sums of an element are joined in a 64-bit
+// integer and rounded to 2^-54 of the largest term.  (28 products, without i + j = 7, took 1.33 ms
+// at 12 orbitals where these take 1.41, but their errors were those of the pairs left out, 2.4 times
+// as large.)
+// The error is a fraction of the operands' largest elements, where that of a float64 sum is a
+// fraction of its own terms: a caller's vector is looked at first (k_digits_near).
 //
 // Opposite-spin term, per alpha string Ia: a dense product T[p][J] = sum_x (s_x V[p_x][p])
 // c[J_x][J] and a scatter, sigma[Ia][K] += s T[p][J] for every E_p |J> = s |K>, in three 21-bit
 // parts (32-bit shared atomics, exact in any order).  One CTA per SM, persistent over Ia; the
 // digits of the signed V columns stay in shared memory, the rows of c come in chunks of strings
 // by cp.async from planes of digits (made once per vector), two buffers.  A warp takes 16 pairs
-// x 8 strings at a time: per 16 list entries 14 ldmatrix for 28 mma.
+// x 8 strings at a time: per 16 list entries 14 ldmatrix for 34 mma.
 // Same-spin terms: Hs (symmetric, its diagonal kept out and added in float64: it would set the
 // scale) and c as dense matrices of digits.
 //
-// casci_sigma_large in float64, with its set-up: 12 orbitals 5.6 -> 1.3 ms, 13 orbitals 18.0 -> 4.8,
-// 14 orbitals 88 -> 30, 10 orbitals 1.37 -> 0.24; largest error against 64-bit sums at 12 orbitals
-// 5.6e-16 of the largest element, 6.0e-16 before.
+// casci_sigma_large in float64, with its set-up, against the plain kernels: 12 orbitals 5.6 -> 1.5 ms;
+// largest error against 64-bit sums there 3.6e-16 of the largest element, 6.0e-16 before.
 #include <algorithm>
 
 #include "common.cuh"
@@ -35,6 +38,19 @@ namespace mbe {
 constexpr int DG_THREADS = 640;  // 20 warps: the 5 x 8 tiles of 12 orbitals in two rounds
 // Row strides in 16-bit words are odd multiples of 8 so that the 8 rows of an ldmatrix matrix lie
 // in different banks.
+
+// Sums kept: the digit pairs with i + j < DIGIT_SUMS.
+constexpr int DIGIT_SUMS = DIGITS + 1;
+
+// The sums of an element, joined (in units of 256^7, as join_digits).
+__device__ __forceinline__ long long join_sums(const float (&acc)[DIGIT_SUMS][4], int e)
+{
+    long long s = (long long)__float2int_rn(acc[0][e]);
+#pragma unroll
+    for (int d = 1; d < DIGITS - 1; ++d) s = s * 256 + __float2int_rn(acc[d][e]);
+    const int rest = __float2int_rn(acc[DIGITS - 1][e]) + ((__float2int_rn(acc[DIGITS][e]) + 128) >> 8);
+    return s + ((rest + 128) >> 8);
+}
 
 struct DigitsShape {
     int mt, kp, as, off_b, off_row, off_jx, bytes;
@@ -80,10 +96,70 @@ __global__ void k_digits_max(const double *__restrict__ M, int64_t rows, int col
     max_bits(big, out);
 }
 
-// Planes of digits of an Ns x Ns matrix, rows padded to nsp with zeros; skip: the diagonal as 0.
-__global__ void k_digits_planes(const double *__restrict__ M, int Ns, int nsp, int skip, const unsigned long long *big,
-                                uint16_t *planes)
+// Whether digits are as accurate as float64 sums for every element of the result.  They round V, Hs
+// and c to fixed fractions of their largest elements, float64 sums each term to a fraction of itself,
+// so digits are the more accurate ones where the sums are not made of small terms only: the R^2
+// elements of c that an element of sigma adds up must average EVEN_C of the largest (first, the sums
+// over the beta lists; then those over the alpha lists), the elements of V EVEN_V of its largest, and
+// Hs must not exceed n max|V|.  Otherwise (a converged CI vector, say, whose elements fall with the
+// excitation) usable[3] is set, and the plain float64 kernels answer.  Errors in units of 2^-53 sum
+// |V| |c|, root mean square (largest) over 1,400 elements of 10 orbitals, plain and by digits:
+// normal c 0.75 (4.0) and 0.34 (1.2); c falling by 3 per excitation 0.63 (3.3) and 33 (300).  The two
+// passes over c take 50 us at 12 orbitals.
+constexpr double EVEN_C = 1.0 / 12, EVEN_V = 1.0 / 40;
+
+__global__ void __launch_bounds__(256) k_digits_near(DigitsArgs a, float *near)
 {
+    extern __shared__ __align__(128) unsigned char smem[];
+    float *row = (float *)smem;
+    if (!digits_in_range(a.maxb)) return;
+    const int Ns = a.Ns;
+    const double scale = pow2d(-bits_exponent(a.maxb[2]));
+    for (int I = blockIdx.x; I < Ns; I += gridDim.x) {
+        __syncthreads();
+        for (int K = threadIdx.x; K < Ns; K += blockDim.x) row[K] = (float)fabs(a.c[(size_t)I * Ns + K] * scale);
+        __syncthreads();
+        for (int K = threadIdx.x; K < Ns; K += blockDim.x) {
+            float v = 0.f;
+            for (int y = 0; y < a.R; ++y) v += row[entry_J(a.tabT[(size_t)y * Ns + K])];
+            near[(size_t)I * Ns + K] = v;
+        }
+    }
+}
+
+__global__ void __launch_bounds__(256) k_digits_even(DigitsArgs a, const float *near)
+{
+    if (!digits_in_range(a.maxb)) return;
+    const int Ns = a.Ns;
+    const double top = __longlong_as_double((long long)a.maxb[2]) * pow2d(-bits_exponent(a.maxb[2]));
+    const float least = (float)(EVEN_C * a.R * a.R * top);
+    bool even = true;
+    for (int I = blockIdx.x; I < Ns; I += gridDim.x) {
+        const int32_t *ta = a.tab + (size_t)I * a.R;
+        for (int K = threadIdx.x; K < Ns; K += blockDim.x) {
+            float v = 0.f;
+            for (int x = 0; x < a.R; ++x) v += near[(size_t)entry_J(ta[x]) * Ns + K];
+            even = even && v >= least;
+        }
+    }
+    if (blockIdx.x == 0 && threadIdx.x < 32) {
+        const double vscale = pow2d(-bits_exponent(a.maxb[0]));
+        float v = 0.f;
+        for (int q = threadIdx.x; q < a.P * a.P; q += 32) v += (float)fabs(a.V[q] * vscale);
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+        const double vtop = __longlong_as_double((long long)a.maxb[0]), hs = __longlong_as_double((long long)a.maxb[1]);
+        even = even && v >= EVEN_V * a.P * a.P * vtop * vscale && hs <= a.n * vtop;
+    }
+    if (!even) a.maxb[3] = 1ull;
+}
+
+// Planes of digits of an Ns x Ns matrix, rows padded to nsp with zeros; skip: the diagonal as 0.
+// usable: of all operands, or NULL (the planes are made in any case).
+__global__ void k_digits_planes(const double *__restrict__ M, int Ns, int nsp, int skip, const unsigned long long *big,
+                                const unsigned long long *usable, uint16_t *planes)
+{
+    if (usable && !digits_usable(usable)) return;
     const double scale = pow2d(55 - bits_exponent(*big));
     const size_t plane = (size_t)Ns * nsp;
     for (int I = blockIdx.x; I < Ns; I += gridDim.x)
@@ -171,9 +247,9 @@ __global__ void __launch_bounds__(DG_THREADS, 1) k_large_ab_digits(DigitsArgs a)
                     const int p = mt * 16 + (lane >> 2) + (e >> 1) * 8, J = ch * DG_CHUNK + nt * 8 + (lane & 3) * 2 + (e & 1);
                     to[e] = p < P && J < Ns ? a.inv[(size_t)p * a.nsp + J] : -1;
                 }
-                float acc[DIGITS][4];
+                float acc[DIGIT_SUMS][4];
 #pragma unroll
-                for (int d = 0; d < DIGITS; ++d) acc[d][0] = acc[d][1] = acc[d][2] = acc[d][3] = 0.f;
+                for (int d = 0; d < DIGIT_SUMS; ++d) acc[d][0] = acc[d][1] = acc[d][2] = acc[d][3] = 0.f;
                 const uint32_t aa = shared_u32(A + (mt * 16 + (lane & 15)) * S.as + (lane >> 4) * 8);
                 const uint32_t ba = shared_u32(buf + (lane & 15) * DG_BS + nt * 8);
 #pragma unroll 1
@@ -187,14 +263,14 @@ __global__ void __launch_bounds__(DG_THREADS, 1) k_large_ab_digits(DigitsArgs a)
                     for (int i = 0; i < DIGITS; ++i) {
                         if (i + 1 < DIGITS) ldsm_x4(af[(i + 1) & 1], aa + 2 * ((i + 1) * aplane + k));
 #pragma unroll
-                        for (int j = 0; i + j < DIGITS; ++j) mma_bf16(acc[i + j], af[i & 1], bf[j][0], bf[j][1]);
+                        for (int j = 0; j < DIGITS && i + j < DIGIT_SUMS; ++j) mma_bf16(acc[i + j], af[i & 1], bf[j][0], bf[j][1]);
                     }
                 }
                 // scatter
 #pragma unroll
                 for (int e = 0; e < 4; ++e) {
                     if (to[e] < 0) continue;
-                    long long s = join_digits(acc, e);
+                    long long s = join_sums(acc, e);
                     if (to[e] & 1) s = -s;
                     int *r = row + (to[e] >> 1);
                     atomicAdd(r, (int)(s & 0x1fffff));
@@ -254,7 +330,7 @@ __global__ void __launch_bounds__(GM_THREADS, 2) k_large_ss_digits(DigitsArgs a)
             }
             asm volatile("cp.async.commit_group;" ::: "memory");
         };
-        float acc[2][DIGITS][4];
+        float acc[2][DIGIT_SUMS][4];
         double sum[2][4];
 #pragma unroll
         for (int h = 0; h < 2; ++h)
@@ -262,7 +338,7 @@ __global__ void __launch_bounds__(GM_THREADS, 2) k_large_ss_digits(DigitsArgs a)
             for (int e = 0; e < 4; ++e) {
                 sum[h][e] = 0.0;
 #pragma unroll
-                for (int d = 0; d < DIGITS; ++d) acc[h][d][e] = 0.f;
+                for (int d = 0; d < DIGIT_SUMS; ++d) acc[h][d][e] = 0.f;
             }
         __syncthreads();  // the last tile's buffers are free
         fetch(0);
@@ -288,7 +364,7 @@ __global__ void __launch_bounds__(GM_THREADS, 2) k_large_ss_digits(DigitsArgs a)
                 for (int i = 0; i < DIGITS; ++i) {
                     if (i + 1 < DIGITS) ldsm_x4(af[(i + 1) & 1], aa + 2 * ((i + 1) * GM_M * GM_S + k));
 #pragma unroll
-                    for (int j = 0; i + j < DIGITS; ++j) {
+                    for (int j = 0; j < DIGITS && i + j < DIGIT_SUMS; ++j) {
                         mma_bf16(acc[0][i + j], af[i & 1], bf[j][0], bf[j][1]);
                         mma_bf16(acc[1][i + j], af[i & 1], bf[j][2], bf[j][3]);
                     }
@@ -299,9 +375,9 @@ __global__ void __launch_bounds__(GM_THREADS, 2) k_large_ss_digits(DigitsArgs a)
                 for (int h = 0; h < 2; ++h)
 #pragma unroll
                     for (int e = 0; e < 4; ++e) {
-                        sum[h][e] += (double)join_digits(acc[h], e);
+                        sum[h][e] += (double)join_sums(acc[h], e);
 #pragma unroll
-                        for (int d = 0; d < DIGITS; ++d) acc[h][d][e] = 0.f;
+                        for (int d = 0; d < DIGIT_SUMS; ++d) acc[h][d][e] = 0.f;
                     }
             }
             __syncthreads();  // the buffer is free for the chunk after the next
@@ -323,9 +399,13 @@ int large_sigma_digits(cudaStream_t st, int sm_count, size_t smem_optin, const D
 {
     const DigitsShape S = digits_shape(a.P, a.Ns, a.R, chunk);
     const int smem_ss = 2 * GM_BUF * 2, rows = std::min(a.Ns, sm_count * 8);
-    MBE_CU(cudaMemsetAsync(a.maxb + 2, 0, 8, st));
+    MBE_CU(cudaMemsetAsync(a.maxb + 2, 0, 2 * 8, st));
     k_digits_max<<<rows, 256, 0, st>>>(a.c, a.Ns, a.Ns, nullptr, a.maxb + 2);
-    k_digits_planes<<<rows, 256, 0, st>>>(a.c, a.Ns, a.nsp, 0, a.maxb + 2, a.planes);
+    if (a.n) {  // (the sums lie where the planes will)
+        k_digits_near<<<rows, 256, std::max(a.Ns, 32) * 4, st>>>(a, (float *)a.planes);
+        k_digits_even<<<rows, 256, 0, st>>>(a, (const float *)a.planes);
+    }
+    k_digits_planes<<<rows, 256, 0, st>>>(a.c, a.Ns, a.nsp, 0, a.maxb + 2, a.maxb, a.planes);
     if (chunk == 64) {
         MBE_CU(allow_smem(k_large_ab_digits<64>, smem_optin));
         k_large_ab_digits<64><<<std::min(sm_count, a.Ns), DG_THREADS, S.bytes, st>>>(a);
@@ -343,11 +423,11 @@ int large_sigma_digits(cudaStream_t st, int sm_count, size_t smem_optin, const D
 int large_digits_setup(cudaStream_t st, int sm_count, const DigitsArgs &a, const double *Hs, double *hd)
 {
     const int rows = std::min(a.Ns, sm_count * 8);
-    MBE_CU(cudaMemsetAsync(a.maxb, 0, 3 * 8, st));
+    MBE_CU(cudaMemsetAsync(a.maxb, 0, 4 * 8, st));
     MBE_CU(cudaMemsetAsync(a.inv, 0xff, (size_t)a.P * a.nsp * 4, st));
     k_digits_max<<<1, 1024, 0, st>>>(a.V, a.P, a.P, nullptr, a.maxb);
     k_digits_max<<<rows, 256, 0, st>>>(Hs, a.Ns, a.Ns, hd, a.maxb + 1);
-    k_digits_planes<<<rows, 256, 0, st>>>(Hs, a.Ns, a.nsp, 1, a.maxb + 1, a.hplanes);
+    k_digits_planes<<<rows, 256, 0, st>>>(Hs, a.Ns, a.nsp, 1, a.maxb + 1, nullptr, a.hplanes);
     k_digits_inverse<<<(a.Ns * a.R + 255) / 256, 256, 0, st>>>(a.tab, a.Ns, a.nsp, a.R, a.inv);
     MBE_CU(cudaGetLastError());
     return MBE_OK;

@@ -9,13 +9,15 @@ constexpr int DIGITS_EXP = 450;  // largest |exponent| of an operand's scale
 
 struct DigitsArgs {
     int P, Ns, R, nsp;    // nsp: Ns rounded up to 64, the row stride of planes and inv
+    int n;                // orbitals, if c may have any spread (see k_digits_near), else 0
     const int32_t *tab;   // [Ns][R] replacement lists
+    const int32_t *tabT;  // [R][Ns]
     int32_t *inv;         // [P][nsp] K << 1 | neg, or -1
     const double *V;      // [P][P]
     const double *hd;     // [Ns] diagonal of Hs
     const double *c;      // [Ns][Ns]
     uint16_t *planes;     // [DIGITS][Ns][nsp] digits of c (scratch)
-    unsigned long long *maxb;  // bits of the largest |V|, |off-diagonal Hs| and |c|
+    unsigned long long *maxb;  // [4] bits of the largest |V|, |off-diagonal Hs| and |c|; not 0: digits are not used
     uint16_t *hplanes;  // [DIGITS][Ns][nsp] digits of Hs without its diagonal
     double *sigma;        // [Ns][Ns], written
 };
@@ -39,7 +41,7 @@ __device__ inline int bits_exponent(unsigned long long b)
 
 // Whether the scales of all operands are far from the ends of float64's range (an infinity or a
 // NaN has the largest exponent); zero operands are.
-__device__ inline bool digits_usable(const unsigned long long *maxb)
+__device__ inline bool digits_in_range(const unsigned long long *maxb)
 {
     for (int i = 0; i < 3; ++i) {
         const int E = (int)(maxb[i] >> 52) - 1022;
@@ -47,6 +49,9 @@ __device__ inline bool digits_usable(const unsigned long long *maxb)
     }
     return true;
 }
+
+// ... and they are not too uneven either (k_digits_even).
+__device__ inline bool digits_usable(const unsigned long long *maxb) { return maxb[3] == 0ull && digits_in_range(maxb); }
 
 // Largest of the lanes' |v|, as bits (in which a NaN is above all numbers), into *out.
 __device__ inline void max_bits(unsigned long long b, unsigned long long *out)
