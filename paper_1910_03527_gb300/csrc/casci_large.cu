@@ -436,8 +436,9 @@ __global__ void k_sym_add(const double *__restrict__ A, int Ns, int sgn, double 
 
 // out = in^T for an Ns x Ns matrix, 32 x 32 tiles through shared memory.
 template <typename T>
-__global__ void k_large_transpose(const T *__restrict__ in, int Ns, T *__restrict__ out)
+__global__ void k_large_transpose(const T *__restrict__ in, int Ns, T *__restrict__ out, const unsigned long long *digits)
 {
+    if (digits && digits_usable(digits)) return;
     __shared__ T tile[32][33];
     const int nt = (Ns + 31) / 32;
     for (int64_t t = blockIdx.x; t < (int64_t)nt * nt; t += gridDim.x) {
@@ -780,11 +781,18 @@ struct LargePlan {
 };
 
 
+// Strings from which the float64 sigma is made of digits (six launches more than the plain kernels):
+// in casci_sigma_large 5 of 10 orbitals (Ns = 252) 1002 -> 262 us, (6, 3) with 20 strings 185 -> 158,
+// (6, 2) with 15 147 -> 155, (5, 2) with 10 126 -> 152; inside casci_solve, where the set-up is
+// paid once, 12 strings 5.83 -> 5.74 and 18.2 -> 16.5 ms, 10 strings 3.64 -> 3.85 ms.
+constexpr int DIGITS_SIGMA_NS = 16, DIGITS_SOLVE_NS = 11;
+
 // Sets up one large CAS; the dense Hs may live in `dense_at` (e.g. the Davidson
-// basis region, unused during set-up). `fp32` adds the float32 sigma's tables.
+// basis region, unused during set-up). `fp32` adds the float32 sigma's tables, and `fp64` the
+// digits' from that many strings on (0: never).
 static int large_setup(mbe_ctx *ctx, int norb, const double *h1, const double *eri, const uint8_t *occ, int n_cas,
-                       const int32_t *cas_orbs, Bump &bump, double *dense_at, bool fp32, LargePlan *plan, int *k_out,
-                       int64_t *dphi_out)
+                       const int32_t *cas_orbs, Bump &bump, double *dense_at, bool fp32, int fp64, LargePlan *plan,
+                       int *k_out, int64_t *dphi_out)
 {
     MBE_CHECK(n_cas >= 1 && n_cas <= MBE_MAX_STRING_ORB && n_cas <= norb, MBE_EUNSUPPORTED,
               "large CASCI: n_cas %d outside 1..%d", n_cas, MBE_MAX_STRING_ORB);
@@ -834,7 +842,7 @@ static int large_setup(mbe_ctx *ctx, int norb, const double *h1, const double *e
     plan->cT = bump.take<double>((size_t)L.N);  // float32 or float64 use
     L.Hd = dense_at ? dense_at : bump.take<double>((size_t)L.Ns * L.Ns);
     plan->tc_lists = fp32 ? (uint32_t *)bump.take<char>(large_tc_list_bytes(ctx->smem_optin, P, L.Ns, L.R)) : nullptr;
-    plan->dg_chunk = large_digits_chunk(ctx->smem_optin, P, L.Ns, L.R);
+    plan->dg_chunk = fp64 > 0 && L.Ns >= fp64 ? large_digits_chunk(ctx->smem_optin, P, L.Ns, L.R) : 0;
     double *hd = nullptr;
     if (plan->dg_chunk) {
         DigitsArgs &g = plan->dg;
@@ -911,7 +919,7 @@ static int large_setup(mbe_ctx *ctx, int norb, const double *h1, const double *e
 }
 
 // Workspace bytes of large_setup (and the dense Hs unless aliased).
-static size_t large_bytes(const mbe_ctx *ctx, int norb, int n, int k, bool dense_separate, bool fp32)
+static size_t large_bytes(const mbe_ctx *ctx, int norb, int n, int k, bool dense_separate, bool fp32, int fp64)
 {
     const int64_t ns = binom(n, k), N = ns * ns;
     const int P = n * (n + 1) / 2;
@@ -923,7 +931,7 @@ static size_t large_bytes(const mbe_ctx *ctx, int norb, int n, int k, bool dense
     b += align256((size_t)k * (n - k + 1) * ns * 4) + align256((size_t)N * 8);
     if (dense_separate) b += align256((size_t)ns * ns * 8);
     if (fp32) b += align256(large_tc_list_bytes(ctx->smem_optin, P, (int)ns, k * (n - k + 1)));
-    if (large_digits_chunk(ctx->smem_optin, P, (int)ns, k * (n - k + 1))) {
+    if (fp64 > 0 && ns >= fp64 && large_digits_chunk(ctx->smem_optin, P, (int)ns, k * (n - k + 1))) {
         const size_t nsp = (size_t)(ns + 63) / 64 * 64;
         b += align256(ns * 8) + align256(P * nsp * 4) + 256 + 2 * align256((size_t)DIGITS * ns * nsp * 2);
     }
@@ -978,7 +986,7 @@ static int large_sigma_launch(mbe_ctx *ctx, const LargePlan &pl, const T *c, dou
         if (sgn == 0) {
             float *cT = (float *)pl.cT;
             int rc = large_ss_slab<false, false>(ctx, pl, (const float *)c, sigma);
-            k_large_transpose<float><<<pl.grid_tr, dim3(32, 8), 0, ctx->stream>>>((const float *)c, Ns, cT);
+            k_large_transpose<float><<<pl.grid_tr, dim3(32, 8), 0, ctx->stream>>>((const float *)c, Ns, cT, nullptr);
             if (!rc) rc = large_ss_slab<true, false>(ctx, pl, cT, sigma);
             if (rc) return rc;
         } else {
@@ -996,7 +1004,7 @@ static int large_sigma_launch(mbe_ctx *ctx, const LargePlan &pl, const T *c, dou
     if (sgn == 0) {
         T *cT = (T *)pl.cT;
         k_large_ss<T, false><<<grid_ss, SS_THREADS, smem_ss, ctx->stream>>>(pl.L, c, sigma, digits);
-        k_large_transpose<T><<<pl.grid_tr, dim3(32, 8), 0, ctx->stream>>>(c, Ns, cT);
+        k_large_transpose<T><<<pl.grid_tr, dim3(32, 8), 0, ctx->stream>>>(c, Ns, cT, digits);
         k_large_ss<T, true><<<grid_ss, SS_THREADS, smem_ss, ctx->stream>>>(pl.L, cT, sigma, digits);
     } else {
         // c in the sector sgn: the beta same-spin term is sgn times the transpose
@@ -1036,7 +1044,8 @@ extern "C" int casci_sigma_large(mbe_ctx *ctx, int norb, const double *h1, const
     for (int i = 0; i < n_cas; ++i) k0 += (cas_orbs[i] >= 0 && cas_orbs[i] < norb && occ_h[cas_orbs[i]]) ? 1 : 0;
     const int64_t N = binom(n_cas, k0) * binom(n_cas, k0);
     const bool fp32 = precision == MBE_PREC_MIXED;
-    size_t bytes = large_bytes(ctx, norb, n_cas, k0, true, fp32) + (fp32 ? align256(N * 4) : 0);
+    const int fp64 = fp32 ? 0 : DIGITS_SIGMA_NS;  // (a float32 sigma needs no digits)
+    size_t bytes = large_bytes(ctx, norb, n_cas, k0, true, fp32, fp64) + (fp32 ? align256(N * 4) : 0);
     void *ws = nullptr;
     int rc = workspace(ctx, bytes, &ws);
     if (rc) return rc;
@@ -1044,7 +1053,7 @@ extern "C" int casci_sigma_large(mbe_ctx *ctx, int norb, const double *h1, const
     LargePlan pl;
     int k = 0;
     int64_t dphi = 0;
-    rc = large_setup(ctx, norb, h1, eri, occ, n_cas, cas_orbs, bump, nullptr, fp32, &pl, &k, &dphi);
+    rc = large_setup(ctx, norb, h1, eri, occ, n_cas, cas_orbs, bump, nullptr, fp32, fp64, &pl, &k, &dphi);
     if (rc) return rc;
     if (diag) MBE_CU(cudaMemcpyAsync(diag, pl.L.diag, N * 8, cudaMemcpyDeviceToDevice, ctx->stream));
     if (precision == MBE_PREC_FP64) {
@@ -1360,7 +1369,7 @@ extern "C" int casci_solve(mbe_ctx *ctx, int norb, const double *h1, const doubl
     D.ld = vec / 8;
     D.nblk = ctx->sm_count * 4;
     const bool mixed = o.precision == MBE_PREC_MIXED;
-    size_t bytes = large_bytes(ctx, norb, n_cas, k0, false, mixed) + vec * (2 * MLARGE + 7) + 2 * align256((size_t)N * 8) +
+    size_t bytes = large_bytes(ctx, norb, n_cas, k0, false, mixed, DIGITS_SOLVE_NS) + vec * (2 * MLARGE + 7) + 2 * align256((size_t)N * 8) +
                    align256((size_t)D.nblk * LRED * 8) + 8 * 256 + 8192;
     void *ws = nullptr;
     int rc = workspace(ctx, bytes, &ws);
@@ -1390,7 +1399,7 @@ extern "C" int casci_solve(mbe_ctx *ctx, int norb, const double *h1, const doubl
     int k = 0;
     int64_t dphi = 0;
     // The dense one-spin Hamiltonian of the set-up lives in the (not yet used) basis region.
-    rc = large_setup(ctx, norb, h1, eri, occ, n_cas, cas_orbs, bump, D.V, mixed, &pl, &k, &dphi);
+    rc = large_setup(ctx, norb, h1, eri, occ, n_cas, cas_orbs, bump, D.V, mixed, DIGITS_SOLVE_NS, &pl, &k, &dphi);
     if (rc) return rc;
     const int Ns = pl.L.Ns;
     k_argmin<<<1, 1024, 0, ctx->stream>>>(pl.L.diag, N, Ns, 0, D.best);

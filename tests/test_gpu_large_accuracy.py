@@ -83,3 +83,17 @@ def test_rows_of_graded_vectors(eng, ctx, system, fall):
         e[row] = 1.0
         h = ctx.casci_sigma(*a, dev(e))[0].cpu().numpy()  # (H is symmetric)
         assert abs(got[row] - math.fsum(h * c)) <= terms * 2.0 ** -50 * float(np.abs(h * c).sum()), row
+
+
+def test_no_launches_for_a_form_that_is_not_used(eng, ctx):
+    # set-up: 8 kernels; float64 sigma of few strings: opposite-spin, two same-spin, transpose; float32:
+    # scatter lists, conversion, opposite-spin, two same-spin, transpose
+    h1, eri, occ = random_system(8, 4, seed=2)
+    a = (dev(h1), dev(eri), dev(occ))
+    for A, prec, most in ((list(range(2, 7)), "fp64", 12), (list(range(8)), "mixed", 14)):
+        k = int(sum(occ[p] for p in A))
+        c = dev(np.random.default_rng(1).normal(size=math.comb(len(A), k) ** 2))
+        ctx.casci_sigma_large(*a, A, c, prec)
+        before = ctx.launches()
+        ctx.casci_sigma_large(*a, A, c, prec)
+        assert ctx.launches() - before <= most
