@@ -451,10 +451,12 @@ int casci_solve(mbe_ctx *ctx, int norb, const double *h1, const double *eri, con
  * arguments, output and meaning as casci_batch (eps_out[t] = E_CAS(R u tuple_t)
  * - E_Phi - e_ref_corr), with |R| + order up to MBE_MAX_LARGE_CAS and one more:
  *   large_ndet   a tuple whose active space has more than large_ndet determinants
- *                (large_ndet > 0), or more than MBE_MAX_CAS orbitals and more than
- *                128 strings per spin, is solved by casci_solve with the whole
- *                GPU; the others go to casci_batch's solvers in one call
- *                (gathered to a temporary list when the order is mixed).
+ *                (large_ndet > 0), or more than MBE_MAX_CAS orbitals, is solved by
+ *                casci_solve with the whole GPU; the others go to casci_batch's
+ *                solvers in one call (gathered to a temporary list when the order
+ *                is mixed), and so do tuples of more than MBE_MAX_CAS orbitals and
+ *                at most 128 strings per spin where there are enough of one class
+ *                for that to be the faster way in the precision asked for.
  *                With large_ndet <= 0 and |R| + order <= MBE_MAX_CAS this is
  *                casci_batch itself.
  * A routed tuple's iters_out holds casci_solve's sigma counts in the casci_batch

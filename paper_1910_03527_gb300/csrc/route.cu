@@ -4,8 +4,8 @@
 // sizes of a single big CASCI.  The tuples of one order are split on the host:
 // the ones the batched solvers take (at most MBE_MAX_CAS orbitals, at most
 // `large_ndet` determinants) go to casci_batch in one call, and so do tuples of more orbitals
-// that have few strings (ROUTE_BLOCK_NS), which a thread block solves alone; each other tuple
-// is solved by casci_solve with the whole GPU.  Both write eps = E_CAS(R u Omega) -
+// that have few strings and are many (route_block), which a thread block solves alone; each other
+// tuple is solved by casci_solve with the whole GPU.  Both write eps = E_CAS(R u Omega) -
 // E_Phi - E_ref,corr (Eq. 1), so the routed results are interchangeable.
 #include <algorithm>
 #include <atomic>
@@ -53,12 +53,27 @@ __global__ void k_route_direct(int64_t n, const int64_t *rows, const int32_t *st
 constexpr int ROUTE_WORKERS = 4;
 constexpr int64_t ROUTE_CONCURRENT_NDET = 4000000;
 
-// Strings per spin up to which a tuple of more than MBE_MAX_CAS orbitals goes to the block
-// solver (c and V fit in shared memory: SIGMA_LIST).  A casci_solve of such a space (at most
-// 16,384 determinants) takes about 9 ms whatever its size, in launches and read-backs, four at a
-// time; a block solves one per SM.  91 spaces of 14 orbitals and at most 91 strings (the 26-site
-// ring's Type-2 expansion at order 2): 210 ms by casci_solve, 23 ms by the block solver.
+// Strings per spin up to which the block solver may take a tuple of more than MBE_MAX_CAS orbitals
+// (c and V fit in shared memory: SIGMA_LIST).
 constexpr int64_t ROUTE_BLOCK_NS = 128;
+
+// Whether `count` such tuples of one class are solved sooner by the block solver, one per SM at a
+// time, than by casci_solve, ROUTE_WORKERS at a time.  Both take the same iterations.  One of
+// casci_solve costs 0.2 ms whatever the size (launches and read-backs), 0.27 with four at once; one of
+// a block costs its multiply-adds on one SM: N (k (n - k))^2 of them in mixed mode (with a share of the
+// float64 anchors), N R^2 on the float64 pipe in float64.  Measured, block solver against casci_solve
+// in ms (13-16 orbitals, 13-120 strings):
+//   mixed    (13,2): 1 tuple 17 and 18, 8: 23 and 54;  (15,13): 1: 101 and 40, 4: 106 and 55, 8: 106
+//            and 111, 64: 106 and 703;  (16,2): 8: 121 and 96, 16: 128 and 195
+//   float64  (14,13): 1: 7.8 and 19.7;  (13,2): 8: 94 and 61, 16: 94 and 115;  (15,13): 32: 514 and
+//            335, 64: 513 and 615;  (16,14): 64: 706 and 464
+static bool route_block(int n, int k, int64_t count, int sm_count, bool fp64)
+{
+    const double ns = (double)binom(n, k), N = ns * (ns + 1) / 2, r = fp64 ? k * (n - k + 1) : k * (n - k);
+    const double block = fp64 ? 0.03 + 0.42e-6 * N * r * r : 0.05 + 0.1e-6 * N * r * r;
+    const double solve = count == 1 ? 0.2 : 0.27 * (double)((count + ROUTE_WORKERS - 1) / ROUTE_WORKERS);
+    return block * (double)((count + sm_count - 1) / sm_count) <= solve;
+}
 
 // Makes sure the context has k worker contexts.
 static int route_workers(mbe_ctx *ctx, int k)
@@ -136,27 +151,45 @@ extern "C" int casci_batch_routed(mbe_ctx *ctx, int norb, const double *h1, cons
     MBE_CU(cudaStreamSynchronize(ctx->stream));
 
     // Classify: batched (B), one whole-GPU solve each (L), or a one-determinant
-    // or malformed active space written directly (D).  Above MBE_MAX_CAS orbitals the
-    // batched ones are those of ROUTE_BLOCK_NS.
+    // or malformed active space written directly (D).  Above MBE_MAX_CAS orbitals route_block
+    // decides, class by class.
     const bool wide = n_cas > MBE_MAX_CAS, penalty = opts && opts->s2_penalty != 0.0;
     uint32_t classes = 0;
     std::vector<int64_t> rows_b, rows_l, rows_d, ndet_l;
     std::vector<int32_t> tup_b;
     std::vector<uint8_t> in_ref(norb, 0);
     for (int i = 0; i < n_ref; ++i) in_ref[ref_orbs[i]] = 1;
+    int k_ref = 0;
+    for (int i = 0; i < n_ref; ++i) k_ref += occ_h[ref_orbs[i]];
+    // electron pairs of a tuple's active space, or -1
+    auto pairs = [&](const int32_t *tp) {
+        int k = k_ref;
+        for (int i = 0; i < order; ++i) {
+            if (!(tp[i] >= 0 && tp[i] < norb && !in_ref[tp[i]] && (i == 0 || tp[i] > tp[i - 1]))) return -1;
+            k += occ_h[tp[i]];
+        }
+        return k;
+    };
+    bool block[MBE_MAX_LARGE_CAS + 1] = {};
+    if (wide && !penalty) {
+        int64_t count[MBE_MAX_LARGE_CAS + 1] = {};
+        for (int64_t t = 0; t < n_tuples; ++t) {
+            const int k = pairs(tup_h.data() + (size_t)t * order);
+            if (k >= 0) ++count[k];
+        }
+        const bool fp64 = !opts || opts->precision == MBE_PREC_FP64;
+        for (int k = 1; k < n_cas; ++k) {
+            const int64_t ns = binom(n_cas, k);
+            block[k] = ns <= ROUTE_BLOCK_NS && (large_ndet <= 0 || ns * ns <= large_ndet) &&
+                       route_block(n_cas, k, count[k], ctx->sm_count, fp64);
+        }
+    }
     for (int64_t t = 0; t < n_tuples; ++t) {
         const int32_t *tp = tup_h.data() + (size_t)t * order;
-        bool ok = true;
-        int k = 0;
-        for (int i = 0; i < order; ++i) {
-            ok = ok && tp[i] >= 0 && tp[i] < norb && !in_ref[tp[i]] && (i == 0 || tp[i] > tp[i - 1]);
-            if (ok) k += occ_h[tp[i]];
-        }
-        for (int i = 0; i < n_ref; ++i) k += occ_h[ref_orbs[i]];
+        const int k = pairs(tp);
+        const bool ok = k >= 0;
         const int64_t ndet = ok ? binom(n_cas, k) * binom(n_cas, k) : 0;
-        const bool batched = wide ? ok && ndet > 1 && binom(n_cas, k) <= ROUTE_BLOCK_NS &&
-                                        (large_ndet <= 0 || ndet <= large_ndet) && !penalty
-                                  : large_ndet <= 0 || ndet <= large_ndet || !ok;
+        const bool batched = wide ? ok && block[k] : large_ndet <= 0 || ndet <= large_ndet || !ok;
         if (batched) {
             classes |= 1u << k;
             rows_b.push_back(t);
