@@ -410,7 +410,7 @@ __device__ __noinline__ void sector_rdm(const BatchArgs &a, const SectorTables<C
 // One warp per tuple of the class (n, k); REDO: only the tuples that the mixed solver
 // flagged.  Density matrices when a.rdm is set.
 template <class C, bool REDO>
-__global__ void __launch_bounds__(SECTOR_WARPS * 32, C::DH > 4 ? 2 : 3) k_sector64(BatchArgs a, int bucket)
+__device__ __forceinline__ void sector64_tuples(const BatchArgs &a, int bucket)
 {
     extern __shared__ __align__(16) char smem[];
     SectorTables<C> &T = *(SectorTables<C> *)smem;
@@ -519,6 +519,27 @@ __global__ void __launch_bounds__(SECTOR_WARPS * 32, C::DH > 4 ? 2 : 3) k_sector
         }
         if (a.rdm) sector_rdm<C>(a, T, W, won, x, a.weights ? a.weights[t] : 1.0);
         __syncwarp();
+    }
+}
+
+template <class C, bool REDO>
+__global__ void __launch_bounds__(SECTOR_WARPS * 32, C::DH > 4 ? 2 : 3) k_sector64(BatchArgs a, int bucket)
+{
+    sector64_tuples<C, REDO>(a, bucket);
+}
+
+// Two classes in one launch, as k_sector_mixed_pair.
+template <class C0, class C1, bool REDO>
+__global__ void __launch_bounds__(SECTOR_WARPS * 32, 3) k_sector64_pair(BatchArgs a, int b)
+{
+#pragma unroll 1
+    for (int pass = 0; pass < 2; ++pass) {
+        const unsigned half = gridDim.x / 2, second = (blockIdx.x >= half) != (pass == 1);
+        if (!bucket_open(a, REDO ? a.counters2 : a.counters, b + second, pass ? half * (blockDim.x >> 5) : 0)) continue;
+        if (second)
+            sector64_tuples<C1, REDO>(a, b + 1);
+        else
+            sector64_tuples<C0, REDO>(a, b);
     }
 }
 

@@ -41,6 +41,7 @@ static int launch_warp(mbe_ctx *ctx, const BatchArgs &a, int b, const Bucket &bk
 // The same for a sector-solver bucket (one string class).
 static int launch_sector(mbe_ctx *ctx, const BatchArgs &a, int b, const Bucket &bk)
 {
+    if (a.n == 3 && bk.k == 2) return MBE_OK;  // (launched with k = 1, the bucket before)
     TimedLaunch tl(ctx, a.order, 0, bk.dpl);
     int rc;
     if (a.pstate != nullptr) {
