@@ -199,8 +199,10 @@ static int run_casci(mbe_ctx *ctx, int norb, const double *h1, const double *eri
         a.cls[k].r = st->r;
         int64_t N = st->ns * st->ns;
         int b;
-        // the sector solvers: energies in both precisions, density matrices in float64
-        const bool sector = sector_class(n, k) && o.s2_penalty == 0.0 && (rdm == 0 || o.precision == MBE_PREC_FP64);
+        // the sector solvers: energies in both precisions, density matrices in float64, the two-body
+        // ones of up to SECTOR_RDM_NDET determinants in mixed mode too
+        const bool sector = sector_class(n, k) && o.s2_penalty == 0.0 &&
+                            (rdm == 0 || o.precision == MBE_PREC_FP64 || (rdm == 2 && N <= SECTOR_RDM_NDET));
         if (n <= WARP_MAX_N && N <= tu.warp_max_ndet && (rdm != 2 || sector)) {
             int di = 0;
             while (DPL_SET[di] * 32 < N) ++di;

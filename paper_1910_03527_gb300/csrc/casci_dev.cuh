@@ -1820,6 +1820,10 @@ struct Bucket {
 // nor full.  The S^2 penalty keeps the list-driven warp solver.
 constexpr int SECTOR_MAX_N = 6;
 inline bool sector_class(int n, int k) { return n >= 2 && n <= SECTOR_MAX_N && k >= 1 && k < n; }
+// Two-body density matrices in mixed mode: up to this size the float64 sector solver is the faster one
+// (and the more accurate), beyond it the block solver's mixed form.  700 tuples of (3,1) 1.67 -> 0.43
+// ms (1.20 by blocks of half the size), 2,000 of (5,2) 12.2 -> 2.3; but 100 of (6,3) 2.7 and 3.9.
+constexpr int64_t SECTOR_RDM_NDET = 100;
 
 // Grid of a sector-solver launch: a persistent grid, or fewer blocks when the whole batch
 // has fewer tuples than warps in it.

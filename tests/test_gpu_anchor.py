@@ -68,3 +68,18 @@ def test_mixed_density_matrix_belongs_to_a_unit_vector(eng, ctx, n, k):
                                  eng.Opts(precision="mixed"))
         assert int(st[0]) in (0, 4)
         assert abs(float(gh.trace())) <= 1e-13 * 2 * k
+
+
+@pytest.mark.parametrize("n,k", [(2, 1), (3, 1), (3, 2), (4, 2), (5, 2), (5, 4), (6, 1)])
+def test_two_body_density_matrices_of_small_spaces(eng, ctx, n, k):
+    """Mixed mode takes the float64 solver there: the same gradients, up to the order of the sums."""
+    h1, eri, occ = random_system(20, 10, seed=n, eri_scale=0.3)
+    t = dev(np.array([list(range(i, i + k)) + list(range(10 + i, 10 + i + n - k)) for i in range(0, 5)], dtype=np.int32))
+    got = []
+    for prec in ("fp64", "mixed"):
+        gh = torch.zeros((20,) * 2, dtype=torch.float64, device="cuda")
+        ge = torch.zeros((20,) * 4, dtype=torch.float64, device="cuda")
+        st = ctx.casci_rdm_batch(dev(h1), dev(eri), dev(occ), [], n, t, None, gh, ge, eng.Opts(precision=prec, tol=1e-9))
+        assert np.isin(st.cpu().numpy(), (0, 4)).all()
+        got.append((gh, ge))
+    assert float((got[0][0] - got[1][0]).abs().max()) <= 1e-13 and float((got[0][1] - got[1][1]).abs().max()) <= 1e-13
