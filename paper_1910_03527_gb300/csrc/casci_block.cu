@@ -742,9 +742,11 @@ __device__ __noinline__ void small_eig_block(const BlockMem &S, int m, bool warm
         float scale = fmaxf(fabsf(a), fmaxf(fabsf(d), fabsf(b)));
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) scale = fmaxf(scale, __shfl_xor_sync(FULL, scale, o));
-        // poles apart and couplings nonzero by a rounding error of the matrix
+        // poles apart by a rounding error of the matrix; couplings nonzero, their squares in float32's
+        // range (and no larger: those of an anchored basis to x0 are of the size of its residual, and
+        // whatever is added to them bounds the residual that a refinement can reach)
         const float eps = fmaxf(1.2e-7f * scale, 1e-15f);
-        if (lane < q && fabsf(b) < eps) b = copysignf(eps, b);
+        if (lane < q && fabsf(b) < 1e-17f) b = copysignf(1e-17f, b);
         d = lane < q ? d - lane * 2.f * eps : -3e38f;
 #pragma unroll
         for (int o = 1; o < 32; o <<= 1) {
