@@ -47,3 +47,9 @@ def test_mixed_refinements_reach_1e12(eng, ctx, n, k, count):
     st, it = _solve(eng, ctx, n, k, count, 1.0, "mixed", 1e-12)
     assert np.isin(st, (0, 4)).all()
     assert (it >> 16).max() <= 16 and (it >> 16).mean() <= 8
+
+
+@pytest.mark.parametrize("n,k,count,scale,tol", [(10, 2, 76, 1.0, 1e-13), (8, 4, 76, 0.5, 5e-14)])
+def test_float64_reaches_its_rounding_error(eng, ctx, n, k, count, scale, tol):
+    st, _ = _solve(eng, ctx, n, k, count, scale, "fp64", tol)
+    assert np.isin(st, (0, 4)).all()
