@@ -39,7 +39,8 @@ struct BlockProblem {
     int form;         // of sigma
     const float *U;   // SIGMA_LIST: U[I][p] = sum over the orbitals q of string I of V[qq][p]
     bool bad;         // an element of V or Hs is not finite (float64 sigma: fixed point cannot hold it)
-    int E;            // 2^E: the power of two above the largest element of V and (off-diagonal) Hs
+    int E;            // fixed-point exponent: 2^E is above the elements of V and (off-diagonal) Hs
+    int Eh;           // the same with the diagonal of H: the unit of residuals (0 if H is zero)
     BlockMem S;
     double *full;     // [Ns][stride] scratch of the slot
 };
@@ -1080,9 +1081,9 @@ __device__ __noinline__ PhaseOut davidson_block(const BlockProblem &B, T *Vp, T 
     o.status = MBE_STATUS_OK;
     o.dnorm = 0.0;
     const T shT = (T)shift, shT_lo = (T)(shift - (double)shT);
-    // float32 residuals are squared in the unit 2^E and the corrections kept near |r| 2^-E (the floor
+    // float32 residuals are squared in the unit 2^Eh and the corrections kept near |r| 2^-Eh (the floor
     // of the preconditioner's denominator is 1e-4 in any unit): integrals of 1e-18 would underflow
-    const int Ec = sizeof(T) == 8 ? 0 : max(-100, min(100, B.E));
+    const int Ec = sizeof(T) == 8 ? 0 : max(-100, min(100, B.Eh));
     const T per_unit = (T)pow2(-Ec), unit = (T)pow2(Ec), lift = (T)pow2(Ec < -13 ? -13 - Ec : 0);
     T v1[1], v2[2];
     auto dot = [&](const K &a, const K &b, T s) {
@@ -1263,7 +1264,7 @@ __device__ __noinline__ PhaseOut davidson_block(const BlockProblem &B, T *Vp, T 
         // to within a few rounding errors), and in float64 near the end of what it can reach, where
         // those few add up in the residual (integrals of 5: 95% of the (8,4) tuples got to 1e-13
         // with two passes, 76% without).
-        const bool twice = sizeof(T) == 8 && rn < (T)1e-12 * (T)pow2(B.E);
+        const bool twice = sizeof(T) == 8 && rn < (T)1e-12 * (T)pow2(B.Eh);
         K *tv = V + (size_t)m * ld;
         const K *tsrc = (tdst == tx) ? tx : tv;
         T tn = t0n;
@@ -1458,6 +1459,7 @@ __device__ void block_setup(const BatchArgs &a, BlockProblem &B, const ClassInfo
         }
     }
     B.bad = __syncthreads_or(bad);
+    int top = 0;
     if (B.form == SIGMA_LIST)
         for (int e = tid; e < Ns * P; e += nt) {
             const int I = e / P, p = e - I * P;
@@ -1476,15 +1478,23 @@ __device__ void block_setup(const BatchArgs &a, BlockProblem &B, const ClassInfo
             }
             v += pb.s2mu * __popc(pb.str[ia] & ~pb.str[ib]);
             pb.diag[h] = v;
+            top = max(top, high_word(v));
             tri_advance(ia, ib, nt, Ns);
         }
         if (tid < (4 - pb.N % 4) % 4) pb.diag[pb.N + tid] = 1.0;
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) big = fmax(big, __shfl_xor_sync(FULL, big, o));
-    if ((tid & 31) == 0) red[tid >> 5] = big;
+    top = __reduce_max_sync(FULL, top);
+    if ((tid & 31) == 0) {
+        red[tid >> 5] = big;
+        red[32 + (tid >> 5)] = (double)top;
+    }
     __syncthreads();
-    B.E = fixed_exponent((tid & 31) < (nt >> 5) ? high_word(red[tid & 31]) : 0);
+    big = (tid & 31) < (nt >> 5) ? red[tid & 31] : 0.0;
+    top = (tid & 31) < (nt >> 5) ? max((int)red[32 + (tid & 31)], high_word(big)) : 0;
+    B.E = fixed_exponent(high_word(big));
+    B.Eh = __reduce_max_sync(FULL, top) == 0 ? 0 : fixed_exponent(top);
     if (B.form == SIGMA_TILED) {
         const double scale = pow2(55 - B.E);
         int2 *Vf = (int2 *)pb.V64, *Hf = (int2 *)pb.Hs64;
@@ -1612,7 +1622,7 @@ __global__ void __launch_bounds__(BLOCK_THREADS, 1) k_casci_block(BatchArgs a, i
         B.form = a.tiled ? sigma_form(n, ci.ns) : SIGMA_GLOBAL;
         B.S = block_mem(n, B.form, ci.ns, ci.r, a.rdm);
         B.U = (const float *)(slot + L.off_U);
-        B.E = 0;
+        B.E = B.Eh = 0;
         B.full = (double *)(slot + L.off_full);
         const BlockMem &S = B.S;
         Problem &pb = B.pb;

@@ -61,3 +61,16 @@ def test_large_solver_in_any_unit(eng, ctx, unit, prec):
                           eng.Opts(precision=prec, tol=1e-7 * unit, tol_switch=1e-5 * unit))
     assert want["status"] in VALID and got["status"] in VALID
     assert abs(got["lam"] / unit - want["lam"]) <= 1e-9
+
+
+@pytest.mark.parametrize("n,k", [(7, 3), (9, 5), (10, 2)])
+def test_no_interaction(eng, ctx, n, k):
+    # a diagonal h and no (pq|rs): the unit of the float32 residuals is the diagonal's.  The lowest energy
+    # is that of the lowest k orbitals, Phi's (h rises with the orbital)
+    h1, eri, occ = random_system(18, 9, seed=3)
+    t = np.array([list(range(9 - k, 9)) + list(range(9, 9 + n - k)), list(range(0, k)) + list(range(18 - n + k, 18))],
+                 dtype=np.int32)
+    eps, st, _ = ctx.casci_batch(dev(np.diag(np.diag(h1))), dev(0.0 * eri), dev(occ), [], 0.0, n, dev(t),
+                                 eng.Opts(precision="mixed"))
+    assert np.isin(st.cpu().numpy(), VALID).all()
+    assert float(eps.abs().max()) <= 1e-9
