@@ -48,7 +48,11 @@ static int launch_sector(mbe_ctx *ctx, const BatchArgs &a, int b, const Bucket &
         if ((rc = launch_sector_mixed(ctx, a, b, bk.k))) return rc;
         if ((rc = launch_sector64_redo(ctx, a, b, bk.k))) return rc;
     } else {
-        if ((rc = launch_sector64(ctx, a, b, bk.k))) return rc;
+        // two-body density matrices: the cap is in iterations of the block solver's basis of 20 (and, in
+        // mixed mode, in up to nine phases of them), each worth several of this solver's three vectors
+        BatchArgs d = a;
+        if (a.rdm == 2) d.max_iter = (int)std::min<int64_t>(8LL * a.max_iter, 1 << 30);
+        if ((rc = launch_sector64(ctx, d, b, bk.k))) return rc;
     }
     return tl.done();
 }

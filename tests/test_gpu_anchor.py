@@ -83,3 +83,16 @@ def test_two_body_density_matrices_of_small_spaces(eng, ctx, n, k):
         assert np.isin(st.cpu().numpy(), (0, 4)).all()
         got.append((gh, ge))
     assert float((got[0][0] - got[1][0]).abs().max()) <= 1e-13 and float((got[0][1] - got[1][1]).abs().max()) <= 1e-13
+
+
+@pytest.mark.parametrize("prec", ["fp64", "mixed"])
+@pytest.mark.parametrize("n,k", [(3, 1), (4, 2), (5, 2), (6, 1)])
+def test_density_matrices_within_few_iterations(eng, ctx, n, k, prec):
+    """20 iterations are enough for these spaces with a Davidson basis of 20 vectors, and so for the
+    solver of three that takes their two-body density matrices."""
+    h1, eri, occ = random_system(20, 10, seed=n, eri_scale=0.3)
+    t = dev(np.array([list(range(i, i + k)) + list(range(10 + i, 10 + i + n - k)) for i in range(0, 5)], dtype=np.int32))
+    gh = torch.zeros((20,) * 2, dtype=torch.float64, device="cuda")
+    ge = torch.zeros((20,) * 4, dtype=torch.float64, device="cuda")
+    st = ctx.casci_rdm_batch(dev(h1), dev(eri), dev(occ), [], n, t, None, gh, ge, eng.Opts(precision=prec, tol=1e-9, max_iter=20))
+    assert np.isin(st.cpu().numpy(), (0, 4)).all()
