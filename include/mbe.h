@@ -67,7 +67,12 @@ extern "C" {
                                      the statement after Eq. 3) */
 
 /* Precision modes of casci_batch. */
-#define MBE_PREC_FP64 0  /* every sigma and every Davidson step in float64             */
+#define MBE_PREC_FP64 0  /* every sigma and every Davidson step to float64 accuracy: in
+                            float64, or the products of a sigma in fixed point of 55
+                            bits below the largest element of V and Hs and below 1 for
+                            the unit vector, each within 2^-52 of the largest element.
+                            Residuals down to about 1e-13 of the largest element of H
+                            can be asked for                                       */
 #define MBE_PREC_MIXED 1 /* float32 sigma and Davidson until the residual reaches
                             tol_switch; then an anchored refinement in every solver
                             (warp, block and single large CAS): one float64 sigma of

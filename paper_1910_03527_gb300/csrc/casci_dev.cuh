@@ -1756,8 +1756,9 @@ __global__ void __launch_bounds__(WARPS_PER_BLOCK * 32, DPL <= 8 ? 4 : 3)
 constexpr int MMAX = 20;  // Davidson subspace of the block solver
 constexpr int KRED = 24;  // values per block reduction (>= MMAX + 1)
 // float32 iterations without a 10% residual drop that end the block solver's float32
-// phase (a window of 10 moved work into float32 on the 40-orbital molecule but took
-// longer: this solver's float32 sigma is not much cheaper than its float64 one)
+// phase.  Chosen when a float32 sigma cost nearly as much as a float64 one (a window of 10 took
+// longer then); with the tiled products it costs a fifth, and 10 would take 75 ms for 95 on the
+// 40-orbital molecule's orders 1-2 and 340 for 355 on the 20-orbital one's orders 1-3
 constexpr int BLOCK_STALL = 3;
 // anchored refinement of the block solver: iterations without a 10% residual drop
 // before it re-anchors, and the number of anchors before the float64 fallback

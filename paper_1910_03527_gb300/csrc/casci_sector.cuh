@@ -535,9 +535,10 @@ __device__ __forceinline__ void sigma_sector(const SectorTables<C> &Tb, const fl
 // ------------------------------------------------------------------ sigma of an anchor, integers
 
 // H x0 of an anchor to float64 accuracy on the integer pipe.  A float64 multiply-add costs
-// about 36 times a wide integer one here (1.67 against 60 lanes per clock and SM, measured),
-// so V and Hs are kept as 55-bit fixed-point numbers in two limbs (to_fixed) and the anchor
-// as integers c 2^28: each term is two 32 x 32 + 64 -> 64 bit multiply-adds, exact.  The sums
+// about 12 times a wide integer one here (1.67 against 18-23 lanes per clock and SM, measured with
+// operands that change), so V and Hs are kept as 55-bit fixed-point numbers in two limbs (to_fixed)
+// and the anchor as integers c 2^28 (it may be any vector near the float32 one: r0 belongs to the
+// integer one): each term is two 32 x 32 + 64 -> 64 bit multiply-adds, exact.  The sums
 // cannot overflow: by Cauchy-Schwarz the absolute terms of one element add up to at most
 // (12 * 3 + 9) |c| |V|max < 2^5.5 * 2^28 * 2^27 for a unit vector (a list of 12 entries holds
 // its own string 3 times, every other string once).  The result is rounded once, to 2^-55 of
