@@ -451,7 +451,7 @@ def run_ours(args):
                 "kernel": kname, "launch": f"order {order} solver launch",
                 "ms_per_launch": launch_ms, "fp64_flop_per_launch": f64, "fp32_flop_per_launch": f32,
                 "fp64_tflops": f64 / t_s / 1e12, "fp32_tflops": f32 / t_s / 1e12,
-                "note": "the float64 products of tuples of 2-6 orbitals run in exact fixed point on the integer pipe, "
+                "note": "the float64 products of tuples of 2-6 orbitals run in fixed point on the integer pipe, "
                         "so the fraction of the FP64 pipe's peak may exceed 1",
                 "share_of_step": sum(per_bucket[key]) / total_ms}
 

@@ -105,7 +105,7 @@ __global__ void k_digits_max(const double *__restrict__ M, int64_t rows, int col
 // excitation) usable[3] is set, and the plain float64 kernels answer.  Errors in units of 2^-53 sum
 // |V| |c|, root mean square (largest) over 1,400 elements of 10 orbitals, plain and by digits:
 // normal c 0.75 (4.0) and 0.34 (1.2); c falling by 3 per excitation 0.63 (3.3) and 33 (300).  The two
-// passes over c take 50 us at 12 orbitals.
+// passes over c take 45 us at 12 orbitals.
 constexpr double EVEN_C = 1.0 / 12, EVEN_V = 1.0 / 40;
 
 __global__ void __launch_bounds__(256) k_digits_near(DigitsArgs a, float *near)
@@ -127,29 +127,37 @@ __global__ void __launch_bounds__(256) k_digits_near(DigitsArgs a, float *near)
     }
 }
 
+// (The last block looks at the integrals.)
 __global__ void __launch_bounds__(256) k_digits_even(DigitsArgs a, const float *near)
 {
     if (!digits_in_range(a.maxb)) return;
-    const int Ns = a.Ns;
+    const int Ns = a.Ns, last = gridDim.x - 1;
+    if (blockIdx.x == last) {
+        __shared__ float part[8];
+        const double vscale = pow2d(-bits_exponent(a.maxb[0]));
+        float v = 0.f;
+        for (int q = threadIdx.x; q < a.P * a.P; q += blockDim.x) v += (float)fabs(a.V[q] * vscale);
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+        if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = v;
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            for (int w = 1; w < 8; ++w) v += part[w];
+            const double top = __longlong_as_double((long long)a.maxb[0]), hs = __longlong_as_double((long long)a.maxb[1]);
+            if (!(v >= EVEN_V * a.P * a.P * top * vscale) || !(hs <= a.n * top)) a.maxb[3] = 1ull;
+        }
+        return;
+    }
     const double top = __longlong_as_double((long long)a.maxb[2]) * pow2d(-bits_exponent(a.maxb[2]));
     const float least = (float)(EVEN_C * a.R * a.R * top);
     bool even = true;
-    for (int I = blockIdx.x; I < Ns; I += gridDim.x) {
+    for (int I = blockIdx.x; I < Ns; I += last) {
         const int32_t *ta = a.tab + (size_t)I * a.R;
         for (int K = threadIdx.x; K < Ns; K += blockDim.x) {
             float v = 0.f;
             for (int x = 0; x < a.R; ++x) v += near[(size_t)entry_J(ta[x]) * Ns + K];
             even = even && v >= least;
         }
-    }
-    if (blockIdx.x == 0 && threadIdx.x < 32) {
-        const double vscale = pow2d(-bits_exponent(a.maxb[0]));
-        float v = 0.f;
-        for (int q = threadIdx.x; q < a.P * a.P; q += 32) v += (float)fabs(a.V[q] * vscale);
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-        const double vtop = __longlong_as_double((long long)a.maxb[0]), hs = __longlong_as_double((long long)a.maxb[1]);
-        even = even && v >= EVEN_V * a.P * a.P * vtop * vscale && hs <= a.n * vtop;
     }
     if (!even) a.maxb[3] = 1ull;
 }
@@ -403,7 +411,7 @@ int large_sigma_digits(cudaStream_t st, int sm_count, size_t smem_optin, const D
     k_digits_max<<<rows, 256, 0, st>>>(a.c, a.Ns, a.Ns, nullptr, a.maxb + 2);
     if (a.n) {  // (the sums lie where the planes will)
         k_digits_near<<<rows, 256, std::max(a.Ns, 32) * 4, st>>>(a, (float *)a.planes);
-        k_digits_even<<<rows, 256, 0, st>>>(a, (const float *)a.planes);
+        k_digits_even<<<rows + 1, 256, 0, st>>>(a, (const float *)a.planes);
     }
     k_digits_planes<<<rows, 256, 0, st>>>(a.c, a.Ns, a.nsp, 0, a.maxb + 2, a.maxb, a.planes);
     if (chunk == 64) {
