@@ -6,7 +6,8 @@
 //     rules over the grid as a dense Ns x Ns matrix, then compressed to CSR (each row holds
 //     the strings connected by at most a double replacement);
 //   * sigma = (Hs x 1) c + (1 x Hs) c + opposite-spin term.  In float64 up to 14 orbitals all of
-//     it is products of exact digits on the tensor cores (large_digits.cu); above, the direct
+//     it is products of exact digits on the tensor cores (large_digits.cu); above, with few strings and
+//     for operands that digits do not suit, the direct
 //     double loop over the alpha and beta replacement lists (one thread per determinant, V in
 //     shared memory) and row-streamed sparse products C' = Hs C, the beta one applied to the
 //     transposed coefficient matrix and added back transposed.  In float32 the opposite-spin
